@@ -557,6 +557,14 @@ def nnz_of(H) -> int:
     return int(sum(nb[K] * nb[col[e]] for K in range(len(nb)) for e in range(rp[K], rp[K + 1])))
 
 
+def slice_pairs(s: int) -> int:
+    """BF16 products that the dense sliced form runs for s 6-bit slices: pairs
+    i + j < w of d 9-bit digits per operand (csrc/sliced.cu, digits_for and weights_for)."""
+    d = (6 * s + 9) // 9
+    w = min(max(d, (min(6 * (s + 1), 53) + 18) // 9 - 1), max(s, d))
+    return sum(max(0, min(t, d - 1) - max(0, t - d + 1) + 1) for t in range(w))
+
+
 def measure_sliced(ctx, X_warm, state, cycle, vd, Ns, N, m, Ne, kT, args, dev, bf16_peak):
     """Mixed cycles with the Rayleigh-Ritz products rebuilt from exact BF16
     slices, started from the warm block the timed cycles left; one filtered warm
@@ -568,7 +576,7 @@ def measure_sliced(ctx, X_warm, state, cycle, vd, Ns, N, m, Ne, kT, args, dev, b
     stream = torch.cuda.current_stream()
     ev = lambda: torch.cuda.Event(enable_timing=True)  # noqa: E731
     s = args.slices
-    pairs = s * (s + 1) // 2
+    pairs = slice_pairs(s)
     warm_prev = state["prev"]
     out = {"slices": s, "slice_pairs": pairs}
     b, _ = ctx.bounds(vd, 10)
@@ -668,7 +676,7 @@ def run_sliced_only(args):
         e_.record()
         torch.cuda.synchronize()
         ms = s_.elapsed_time(e_) / max(args.steps, 1)
-    pairs = args.slices * (args.slices + 1) // 2
+    pairs = slice_pairs(args.slices)
     print(json.dumps({"mode": "sliced-only", "M": M, "K": K, "slices": args.slices, "ms": ms,
                       "tensor_tflops": pairs * 2.0 * M * M * K / (ms * 1e-3) / 1e12}), flush=True)
     return 0
@@ -1247,7 +1255,7 @@ def main():
             "bound": "tensor", "achieved": g["tensor_tflops"], "peak": bf16_peak, "unit": "TFLOP/s",
             "frac": g["frac"], "traffic": profiled_pairs_traffic(Ns, N), "kernel": "k_slice_pairs_2sm",
             "ms_per_launch": g["ms"] / max(g["launches"], 1),
-            "work": f"{args.slices * (args.slices + 1) // 2} slice pairs x 2 Ns^2 x 4096 per launch (one K chunk of "
+            "work": f"{slice_pairs(args.slices)} slice pairs x 2 Ns^2 x 4096 per launch (one K chunk of "
                     "the Gram-shaped product)",
             "peak_source": src}
     if not args.no_next_rows and args.prec != "f64":

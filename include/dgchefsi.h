@@ -255,11 +255,12 @@ dgchefsi_status dgchefsi_set_orthonormalisation(dgchefsi_ctx* ctx, int mode);
  *   DGCHEFSI_PRODUCTS_F64          FP64 operands, FP64 accumulation on the
  *                                  CUDA cores (default)
  *   DGCHEFSI_PRODUCTS_SLICED_BF16  each FP64 operand split exactly into
- *                                  `slices` BF16 integer slices of 6 bits per
- *                                  row (column) and 4096-long K chunk, the
- *                                  slice pairs multiplied on the BF16 tensor
- *                                  cores with exact FP32 accumulation, summed
- *                                  and rescaled in FP64 (the Ozaki scheme; see
+ *                                  BF16 integer slices worth `slices` 6-bit
+ *                                  ones (60 bits at 10) per row (column) and
+ *                                  4096-long K chunk, the slice pairs
+ *                                  multiplied on the BF16 tensor cores with
+ *                                  exact accumulation, summed and rescaled in
+ *                                  FP64 (the Ozaki scheme; see
  *                                  dgchefsi_sliced_gemm)
  *   slices  2..16 for the sliced form (ignored for FP64); 10 gives an error
  *           below the FP64 worst-case bound for rows of similar magnitude
@@ -419,12 +420,13 @@ dgchefsi_status dgchefsi_eigensolver_stats(const dgchefsi_ctx* ctx, int* used, i
  * With row maxima m_r of A and column maxima n_c of the product's right
  * operand over each 4096-long chunk of K (length L), the error of C[r, c] is at
  * most the sum over chunks of L m_r n_c (2^{-6 slices} (slices + 4) + (5 + chunks) 2^{-53}).
- * The slice pairs run on this library's tcgen05 kernel on pairs of SMs, all
- * pairs of a K chunk in one launch; their FP32 results go to up to 8 GB of
- * workspace (two buffers when there are several chunks or column panels, so
- * that the FP64 reduction of one runs on a second library stream beside the
- * next one's pairs), plus the slices (2 bytes x slices per operand entry) and,
- * for b_rows = 0, a transposed FP64 copy of B. Synchronises;
+ * The slices are held as 9-bit digits, as many as keep that bound (7 at 10
+ * slices). Their pairs run on this library's tcgen05 kernel on pairs of SMs,
+ * all pairs of a K chunk in one launch; their exact INT32 sums per digit weight
+ * go to up to 8 GB of workspace (two buffers when there are several chunks or
+ * column panels, so that the FP64 reduction of one runs on a second library
+ * stream beside the next one's pairs), plus the digits (2 bytes x digits per
+ * operand entry) and, for b_rows = 0, a transposed FP64 copy of B. Synchronises;
  * ERR_NONFINITE if A or B holds NaN/Inf (C is then unspecified), ERR_ARG on bad
  * sizes, ERR_UNSUPPORTED when K / 4096 > 65535 or M, Nc > 2^31 - 1. */
 dgchefsi_status dgchefsi_sliced_gemm(dgchefsi_ctx* ctx, int b_rows, int a_lower, int64_t M, int64_t Nc, int64_t K,

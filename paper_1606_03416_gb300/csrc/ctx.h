@@ -191,17 +191,27 @@ dgchefsi_status reduce_pair_slabs(const float* Pw, int64_t rows, int64_t cols, c
                                   cudaStream_t st);
 // The slice-pair products of the dense sliced GEMM (pair_gemm.cu: tcgen05 on
 // pairs of SMs, cta_group::2, all pairs of the chunk in one persistent
-// launch): for every pair i + j < s, Pw[pair i*s - i(i-1)/2 + j] (M x pn,
-// row-major FP32) = Qa_i[:, k0:k0+kc] times Qb_j[n0:n0+pn, k0:k0+kc]^T, with
-// Qa_i = Qa + i*sa (M x K, row stride lqa), Qb_j = Qb + j*sb (Nc x K, row
-// stride lqb), entries k >= K read as zero; a_lower: A is lower triangular,
-// so a row tile skips the K slices past its last row. Enqueued only.
+// launch). s digit slices per operand; the pairs i + j = t < nw (nw <= s + 1) of
+// one weight t are summed exactly in
+// count[t] INT32 slabs (total over all t), t descending: slab = sum of
+// Qa_i[:, k0:k0+kc] times Qb_j[n0:n0+pn, k0:k0+kc]^T, M rows of pn entries at
+// a row pitch of pn rounded up to 4, with Qa_i = Qa + i*sa (M x K, row stride
+// lqa), Qb_j = Qb + j*sb (Nc x K, row stride lqb), entries k >= K read as zero
+// and kc <= 4096; a_lower: A is lower triangular, so a row tile skips the K
+// slices past its last row. norm_a, norm_b (device, s entries): the largest sum
+// of squares of digit i over an aligned 512-entry block of a row. Enqueued only.
+// pair_groups: how many slabs each weight is split into for an M x Nc output.
 // pair_products_begin clears the kernel's error word; pair_products_status
 // synchronises and reports a pipeline timeout.
+struct PairGroups {
+  uint8_t count[16];
+  int total;
+};
+PairGroups pair_groups(int s, int nw, int64_t M, int64_t Nc, int nsm);
 dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, int64_t lqa, int64_t sa, int64_t M,
                                   const __nv_bfloat16* Qb, int64_t lqb, int64_t sb, int64_t Nc, int64_t K, int64_t k0,
-                                  int64_t kc, int64_t n0, int64_t pn, int s, float* Pw, bool a_lower,
-                                  int64_t tri = 0);
+                                  int64_t kc, int64_t n0, int64_t pn, int s, int nw, const PairGroups& groups,
+                                  const uint32_t* norm_a, const uint32_t* norm_b, int32_t* Pw, bool a_lower, int64_t tri = 0);
 dgchefsi_status pair_products_begin(dgchefsi_ctx* ctx);
 dgchefsi_status pair_products_status(dgchefsi_ctx* ctx);
 // Y = H X (X, Y: Ns x ld state-major FP64) from s BF16 slices of each operand on

@@ -1,27 +1,50 @@
 // Slice-pair products of the FP64-from-BF16-slices GEMM (the Ozaki scheme of
 // sliced.cu; Alg. 1 steps 3-5) on pairs of SMs: tcgen05 with cta_group::2.
 //
-// Every slice pair (i, j) of a K chunk is a plain BF16 GEMM with FP32
-// accumulation, P_ij = A_i B_j^T, written as an FP32 slab. One CTA pair (a
-// cluster of two) computes a 256 x 256 tile of one pair at a time: each CTA
-// stages its own 128 rows of A_i and its own 128 rows of B_j (32 KB per
-// 64-wide K slice), the first CTA of the pair issues 256 x 256 x 16 MMAs that
-// read both CTAs' halves, and each CTA's tensor memory holds its 128 rows of
-// the tile. Per SM that is 8 KB of operands per 128-clock MMA, half of what a
-// single-SM 128 x 256 tile reads, which leaves shared-memory bandwidth for the
-// TMA refills. The kernel is persistent over (pair, tile) units, the tiles of
-// one pair back to back so that the units in flight read the same two slices
-// from L2, and the tensor maps of all slices sit in device memory, so one
-// launch covers every pair of a chunk.
+// The digits of a slice are integers of magnitude at most 256 (9 bits, exact
+// in BF16), so a product summed over 256 terms is an integer of magnitude at
+// most 2^24: the tensor core's FP32 accumulation returns it exactly. The
+// accumulator is drained every 256 terms (four 64-wide K slices), or every 512
+// to 4096 where the digits' norms say that no partial sum can pass 2^24 there
+// (Cauchy-Schwarz; the splitting kernel leaves the largest norms; digits of
+// Gaussian-like entries allow 512, pairs with a leading digit 1024 and more),
+// and the sums go on in INT32 registers of the epilogue warps, over the whole 4096-long K
+// chunk and over all pairs (i, j) of one weight t = i + j (up to 7 pairs:
+// 7 * 2^16 * 4096 < 2^31). So one INT32 slab per weight leaves the kernel
+// where one FP32 slab per pair would with an accumulator that had to hold the
+// whole chunk (6-bit digits: 10 slices, 55 pairs and 55 slabs for the 60 bits
+// that 7 slices, 28 pairs and 7 slabs give here).
 //
-// Roles per CTA (320 threads): warp 0 lane 0 loads its halves with TMA into a
+// One CTA pair (a cluster of two) computes a 256 x 256 tile of one weight at
+// a time: each CTA stages its own 128 rows of A_i and its own 128 rows of B_j
+// (32 KB per 64-wide K slice), the first CTA of the pair issues
+// 256 x 256 x 16 MMAs that read both CTAs' halves, and each CTA's tensor
+// memory holds its 128 rows of the tile. Per SM that is 8 KB of operands per
+// 128-clock MMA, half of what a single-SM 128 x 256 tile reads, which leaves
+// shared-memory bandwidth for the TMA refills. The kernel is persistent over
+// (weight group, tile) units, the tiles of one group back to back and the
+// largest groups first, so that the units in flight read the same slices from
+// L2 and the last wave is of the shortest units; the tensor maps of all slices
+// sit in device memory, so one launch covers every pair of a chunk.
+//
+// What bounds it: the tensor pipe (32 MMAs = 4096 clocks per 512 terms). The
+// drain of those 128 x 256 sums runs beside the next terms in the other
+// accumulator: ~2150 clocks, because the float-to-int conversion runs at 16 per
+// clock and SM; the extra commit and the hand-over cost the tensor pipe a few
+// hundred clocks each, so the fewer the better. Tensor rate of the 28 pairs at
+// 4096^2 x 16384: 990 TFLOP/s with 256 terms per accumulator (the drain sets
+// the time), 1510 with 512, 1660 with the norms' choice for Gaussian entries,
+// 1710 without any drain: 9.3 ms, where 55 pairs of 6-bit digits took ~16.
+//
+// Roles per CTA (576 threads): warp 0 lane 0 loads its halves with TMA into a
 // 6-slot ring and signals the first CTA's "full" barrier (its expect-tx counts
 // both CTAs' bytes); warp 1 lane 0 of the first CTA issues the MMAs, frees
 // ring slots in both CTAs and announces finished accumulators to both
-// (multicast commits); warps 2-9 drain their CTA's accumulator
-// (double-buffered, 2 x 256 columns) and report to the first CTA's "empty"
-// accumulator barrier. Every wait is bounded; on expiry the CTA records an
-// error word and both CTAs still meet at the final cluster barrier.
+// (multicast commits); warps 2-17 drain their CTA's accumulator
+// (double-buffered, 2 x 256 columns; 64 columns of 32 rows each) and report to
+// the first CTA's "empty" accumulator barrier. Every wait is bounded; on
+// expiry the CTA records an error word and both CTAs still meet at the final
+// cluster barrier.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -31,24 +54,30 @@
 namespace dg {
 namespace {
 
-constexpr int PG_THREADS = 320;
+constexpr int PG_EPI_WARPS = 16;
+constexpr int PG_THREADS = 32 * (2 + PG_EPI_WARPS);
 constexpr int PG_HALF = 128 * SLICE_BYTES;  // 128 rows x 64 BF16 of one operand
 constexpr int PG_STAGE = 2 * PG_HALF;       // A half + B half per CTA
 constexpr int PG_STAGES = 6;
+constexpr int PG_DRAIN = 4;       // K slices (64 terms each) per accumulator: 256 * 2^16 = 2^24
+constexpr int PG_MAXPAIRS = 66;   // 11 digits
 
 struct PairJob {
   const CUtensorMap* maps;  // device, 64-byte aligned: [s] maps of A_i, then [s] maps of B_j
-  const int32_t* pair_i;    // [npairs]
+  const int32_t* group;     // [ngroups + 1] first pair of each group; a group's pairs have one weight i + j
+  const int32_t* pair_i;    // [npairs], in group order
   const int32_t* pair_j;
-  int npairs, s;
+  int ngroups, s;
   int64_t M;        // rows of A (the slab's rows)
-  int64_t pn;       // columns of the slab (rows n0 .. n0 + pn - 1 of B)
+  int64_t pitch;    // row pitch of the slab, a multiple of 4
   int n0, k0, nk;   // first B row, first K column, 64-wide K slices of the chunk
   int nmt, nnt;     // 256-row tiles along M and along the panel
   int lower;        // A is lower triangular: a row tile stops at the chunk's last K slice it reaches
   const int2* tiles;  // null: every (row tile, column tile); else the ntl tiles to compute
   int ntl;
-  float* Pw;        // slab of pair p at Pw + p * M * pn, row-major M x pn
+  const uint32_t* norm_a;  // [s] largest sum of squares of digit i over 512 terms of a row of A, of B
+  const uint32_t* norm_b;
+  int32_t* Pw;      // slab of group g at Pw + g * M * pitch, row-major M x pitch
   int* err;
 };
 
@@ -70,6 +99,14 @@ __device__ __forceinline__ void cluster_sync() {
 
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+
+// Adds one to a shared-memory counter; returns its old value. Orders what the
+// warps before it did before what the last one does next.
+__device__ __forceinline__ uint32_t count_acq_rel(uint32_t* p) {
+  uint32_t old;
+  asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(old) : "r"(smem_u32(p)) : "memory");
+  return old;
 }
 
 // TMA load into this CTA's shared memory, completing on a barrier that may sit
@@ -99,23 +136,28 @@ __device__ __forceinline__ void commit_pair(uint32_t bar) {
       : "memory");
 }
 
-// Pair and tile of work unit u: pairs outermost (in the table's order, one
-// slice of A with the slices of B in turn), the tiles of one pair back to back
-// (row tiles fastest), so the units in flight share one A slice and one or two
-// B slices, which stay in L2.
-__device__ __forceinline__ void unit_of(const PairJob& J, int64_t u, int& p, int& mt, int& nt) {
+// Group and tile of work unit u: groups outermost, the tiles of one group back
+// to back (row tiles fastest), so the units in flight walk the same pairs and
+// share their slices in L2.
+__device__ __forceinline__ void unit_of(const PairJob& J, int64_t u, int& g, int& mt, int& nt) {
   if (J.tiles) {
-    p = (int)(u / J.ntl);
-    const int2 t = J.tiles[u - (int64_t)p * J.ntl];
+    g = (int)(u / J.ntl);
+    const int2 t = J.tiles[u - (int64_t)g * J.ntl];
     mt = t.x;
     nt = t.y;
     return;
   }
   const int64_t ntiles = (int64_t)J.nmt * J.nnt;
-  p = (int)(u / ntiles);
-  const int64_t tile = u - (int64_t)p * ntiles;
+  g = (int)(u / ntiles);
+  const int64_t tile = u - (int64_t)g * ntiles;
   mt = (int)(tile % J.nmt);
   nt = (int)(tile / J.nmt);
+}
+
+// The k-th unit of cluster cid: forwards and backwards in turn, so that every
+// cluster gets long and short units alike (units come longest first).
+__device__ __forceinline__ int64_t nth_unit(int64_t k, int cid, int ncl) {
+  return k * ncl + ((k & 1) ? ncl - 1 - cid : cid);
 }
 
 // K slices of the chunk that row tile mt needs: all of them, or for a lower
@@ -133,12 +175,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + PG_STAGES * PG_STAGE);
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
+  __shared__ uint32_t drained_sh[2];       // epilogue warps done with their part, over all uses of a buffer
+  __shared__ int drain_sh[PG_MAXPAIRS];    // K slices per accumulator of each pair
 
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
-  const int64_t nunits = (J.tiles ? (int64_t)J.ntl : (int64_t)J.nmt * J.nnt) * J.npairs;
+  const int64_t nunits = (J.tiles ? (int64_t)J.ntl : (int64_t)J.nmt * J.nnt) * J.ngroups;
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * PG_STAGES;
   const uint32_t accf0 = empty0 + 8 * PG_STAGES, acce0 = accf0 + 16;
 
@@ -149,9 +193,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accf0 + 8 * b, 1);
-      mbar_init(acce0 + 8 * b, 2 * EPI_WARPS);  // the epilogue warps of both CTAs
+      mbar_init(acce0 + 8 * b, 2);  // the last epilogue warp of each CTA
     }
     abort_sh = 0;
+    drained_sh[0] = drained_sh[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -160,6 +205,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
                  "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  // Any partial sum of products over 512 terms is at most |a||b|, over 2^h such
+  // blocks at most 2^h |a||b| with the largest block norms (Cauchy-Schwarz):
+  // exact in FP32 while that is at most 2^24.
+  for (int p = threadIdx.x; p < J.group[J.ngroups]; p += PG_THREADS) {
+    const uint64_t sq = (uint64_t)J.norm_a[J.pair_i[p]] * J.norm_b[J.pair_j[p]];
+    int len = PG_DRAIN;
+    for (int h = 0; h < 4 && sq <= 1ull << (48 - 2 * h); ++h) len *= 2;
+    drain_sh[p] = len;
   }
   tc_fence_before();
   __syncthreads();
@@ -173,27 +227,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
       const uint32_t full_l = map_to_rank(full0, 0);
       int c = 0;
       bool ok = true;
-      for (int64_t u = cid; u < nunits && ok; u += ncl) {
-        int p, mt, nt;
-        unit_of(J, u, p, mt, nt);
-        const CUtensorMap* am = J.maps + J.pair_i[p];
-        const CUtensorMap* bm = J.maps + J.s + J.pair_j[p];
+      for (int64_t k = 0, u; (u = nth_unit(k, cid, ncl)) < nunits && ok; ++k) {
+        int g, mt, nt;
+        unit_of(J, u, g, mt, nt);
         const int ya = mt * 256 + (int)rank * 128;
         const int yb = J.n0 + nt * 256 + (int)rank * 128;
         const int nk = slices_of_tile(J, mt);
-        for (int ks = 0; ks < nk; ++ks) {
-          const int st = c % PG_STAGES;
-          const uint32_t ph = (uint32_t)(c / PG_STAGES) & 1u;
-          if (!mbar_wait(empty0 + 8 * st, ph ^ 1u)) {
-            ok = false;
-            break;
+        for (int p = J.group[g]; p < J.group[g + 1] && ok; ++p) {
+          const CUtensorMap* am = J.maps + J.pair_i[p];
+          const CUtensorMap* bm = J.maps + J.s + J.pair_j[p];
+          for (int ks = 0; ks < nk; ++ks) {
+            const int st = c % PG_STAGES;
+            const uint32_t ph = (uint32_t)(c / PG_STAGES) & 1u;
+            if (!mbar_wait(empty0 + 8 * st, ph ^ 1u)) {
+              ok = false;
+              break;
+            }
+            if (leader) mbar_expect_tx(full0 + 8 * st, (uint32_t)(2 * PG_STAGE));
+            const uint32_t dst = smem_u32(smem + st * PG_STAGE);
+            const int x = J.k0 + ks * (SLICE_BYTES / 2);
+            tma_load_2d_pair(dst, am, x, ya, full_l + 8 * st);
+            tma_load_2d_pair(dst + PG_HALF, bm, x, yb, full_l + 8 * st);
+            ++c;
           }
-          if (leader) mbar_expect_tx(full0 + 8 * st, (uint32_t)(2 * PG_STAGE));
-          const uint32_t dst = smem_u32(smem + st * PG_STAGE);
-          const int x = J.k0 + ks * (SLICE_BYTES / 2);
-          tma_load_2d_pair(dst, am, x, ya, full_l + 8 * st);
-          tma_load_2d_pair(dst + PG_HALF, bm, x, yb, full_l + 8 * st);
-          ++c;
         }
       }
       if (!ok) {
@@ -207,38 +263,46 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
       constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) |
                               ((uint32_t)(256 >> 4) << 24);
       const uint64_t desc0 = sdesc(smem_u32(smem));
-      int c = 0, i = 0;
+      int c = 0, i = 0;  // ring slots and accumulators used so far
       bool ok = true;
-      for (int64_t u = cid; u < nunits && ok; u += ncl, ++i) {
-        const int buf = i & 1;
-        const uint32_t use = (uint32_t)(i >> 1);
-        if (!mbar_wait(acce0 + 8 * buf, (use & 1u) ^ 1u)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(buf * 256);
-        int p_, mt, nt_;
-        unit_of(J, u, p_, mt, nt_);
+      for (int64_t k = 0, u; (u = nth_unit(k, cid, ncl)) < nunits && ok; ++k) {
+        int g, mt, nt_;
+        unit_of(J, u, g, mt, nt_);
         const int nk = slices_of_tile(J, mt);
-        for (int ks = 0; ks < nk && ok; ++ks) {
-          const int st = c % PG_STAGES;
-          const uint32_t ph = (uint32_t)(c / PG_STAGES) & 1u;
-          if (!mbar_wait(full0 + 8 * st, ph)) {
+        for (int p = J.group[g], k0 = 0, len = drain_sh[p]; p < J.group[g + 1] && ok; ++i) {
+          const int buf = i & 1;
+          const uint32_t use = (uint32_t)(i >> 1);
+          if (!mbar_wait(acce0 + 8 * buf, (use & 1u) ^ 1u)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint64_t da = desc0 + (uint64_t)((st * PG_STAGE) >> 4);
-          const uint64_t db = da + (uint64_t)(PG_HALF >> 4);
+          const uint32_t d = tmem + (uint32_t)(buf * 256);
+          const int k1 = min(k0 + len, nk);
+          for (int ks = k0; ks < k1; ++ks) {
+            const int st = c % PG_STAGES;
+            const uint32_t ph = (uint32_t)(c / PG_STAGES) & 1u;
+            if (!mbar_wait(full0 + 8 * st, ph)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t da = desc0 + (uint64_t)((st * PG_STAGE) >> 4);
+            const uint64_t db = da + (uint64_t)(PG_HALF >> 4);
 #pragma unroll
-          for (int kk = 0; kk < SLICE_BYTES / 32; ++kk)
-            mma_bf16_pair(d, da + (uint64_t)((32 * kk) >> 4), db + (uint64_t)((32 * kk) >> 4), ID,
-                          (ks > 0 || kk > 0) ? 1u : 0u);
-          commit_pair(empty0 + 8 * st);
-          ++c;
+            for (int kk = 0; kk < SLICE_BYTES / 32; ++kk)
+              mma_bf16_pair(d, da + (uint64_t)((32 * kk) >> 4), db + (uint64_t)((32 * kk) >> 4), ID,
+                            (ks > k0 || kk > 0) ? 1u : 0u);
+            commit_pair(empty0 + 8 * st);
+            ++c;
+          }
+          if (ok) commit_pair(accf0 + 8 * buf);
+          k0 = k1;
+          if (k0 == nk) {  // an accumulator holds terms of one pair only
+            k0 = 0;
+            if (++p < J.group[g + 1]) len = drain_sh[p];
+          }
         }
-        if (ok) commit_pair(accf0 + 8 * buf);
       }
       if (!ok) {
         atomicOr(J.err, 1);
@@ -246,49 +310,55 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
       }
     }
   } else {
-    // ---------------- epilogue: warps 2..9, lane quarter q = tile rows 32q..32q+31 of this
-    // CTA's half; the two warps of a quarter take alternate 16-column chunks
+    // ---------------- epilogue: warps 2..17, lane quarter q = tile rows 32q..32q+31 of this
+    // CTA's half, columns 64h..64h+63; the running sums stay in registers for the whole unit
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;
     const uint32_t acce_l = map_to_rank(acce0, 0);
     int i = 0;
-    for (int64_t u = cid; u < nunits; u += ncl, ++i) {
-      const int buf = i & 1;
-      const uint32_t use = (uint32_t)(i >> 1);
-      bool ready = mbar_wait(accf0 + 8 * buf, use & 1u);
-      ready = __all_sync(0xffffffffu, ready);
-      if (!ready) {
-        if (lane == 0) atomicOr(J.err, 1);
-        break;
-      }
-      tc_fence_after();
-      int p, mt, nt;
-      unit_of(J, u, p, mt, nt);
-      const int64_t r = (int64_t)mt * 256 + rank * 128 + 32 * q + lane;
-      const bool row_ok = r < J.M && *(volatile int*)&abort_sh == 0;
-      float* out = J.Pw + (size_t)p * (size_t)(J.M * J.pn) + (size_t)(r < J.M ? r : 0) * (size_t)J.pn;
-      const uint32_t ta = tmem + (uint32_t)(buf * 256) + ((uint32_t)(32 * q) << 16);
-#pragma unroll 1
-      for (int cc = 0; cc < 8; ++cc) {
-        const int c0 = 16 * (h + 2 * cc);
-        float v[16];
-        tmem_ld16(ta + (uint32_t)c0, v);
-        const int64_t col = (int64_t)nt * 256 + c0;
-        if (row_ok) {
-          if (col + 16 <= J.pn && (J.pn & 3) == 0) {  // rows start on 16 bytes only when pn % 4 == 0
-            float4* o = reinterpret_cast<float4*>(out + col);
+    bool ready = true;
+    for (int64_t n = 0, u; (u = nth_unit(n, cid, ncl)) < nunits && ready; ++n) {
+      int g, mt, nt;
+      unit_of(J, u, g, mt, nt);
+      const int nk = slices_of_tile(J, mt);
+      int ndrain = 0;
+      for (int p = J.group[g]; p < J.group[g + 1]; ++p) ndrain += (nk + drain_sh[p] - 1) / drain_sh[p];
+      int sum[64];
 #pragma unroll
-            for (int z = 0; z < 4; ++z) o[z] = make_float4(v[4 * z], v[4 * z + 1], v[4 * z + 2], v[4 * z + 3]);
-          } else {
+      for (int z = 0; z < 64; ++z) sum[z] = 0;
+      for (int k = 0; k < ndrain; ++k, ++i) {
+        const int buf = i & 1;
+        const uint32_t use = (uint32_t)(i >> 1);
+        ready = mbar_wait(accf0 + 8 * buf, use & 1u);
+        ready = __all_sync(0xffffffffu, ready);
+        if (!ready) {
+          if (lane == 0) atomicOr(J.err, 1);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t ta = tmem + (uint32_t)(buf * 256 + 64 * h) + ((uint32_t)(32 * q) << 16);
 #pragma unroll
-            for (int z = 0; z < 16; ++z)
-              if (col + z < J.pn) out[col + z] = v[z];
+        for (int cc = 0; cc < 4; ++cc) {
+          float v[16];
+          tmem_ld16(ta + (uint32_t)(16 * cc), v);
+          if (cc == 3) {  // this warp's last read: the CTA's last warp to get here frees the accumulator
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0 && count_acq_rel(&drained_sh[buf]) == PG_EPI_WARPS * (use + 1) - 1)
+              arrive_remote(acce_l + 8 * buf);
           }
+#pragma unroll
+          for (int z = 0; z < 16; ++z) sum[16 * cc + z] += __float2int_rn(v[z]);
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) arrive_remote(acce_l + 8 * buf);
+      const int64_t r = (int64_t)mt * 256 + rank * 128 + 32 * q + lane;
+      if (!ready || r >= J.M || *(volatile int*)&abort_sh != 0) continue;
+      int32_t* out = J.Pw + ((size_t)g * (size_t)J.M + (size_t)r) * (size_t)J.pitch;
+      const int64_t c0 = (int64_t)nt * 256 + 64 * h;
+#pragma unroll
+      for (int z = 0; z < 64; z += 4)  // pitch % 4 == 0: every vector is inside the row or past it
+        if (c0 + z < J.pitch)
+          *reinterpret_cast<int4*>(out + c0 + z) = make_int4(sum[z], sum[z + 1], sum[z + 2], sum[z + 3]);
     }
   }
   tc_fence_before();
@@ -331,13 +401,37 @@ dgchefsi_status slice_map(CUtensorMap* map, const __nv_bfloat16* base, uint64_t 
 
 }  // namespace
 
+// Pairs (i, t - i) of weight t with both digits below s.
+static int pairs_of_weight(int s, int t) { return std::max(0, std::min(t, s - 1) - std::max(0, t - s + 1) + 1); }
+
+PairGroups pair_groups(int s, int nw, int64_t M, int64_t Nc, int nsm) {
+  // pairs per unit: all of a weight (at most 7, the INT32 bound) when there
+  // are many units for the clusters; fewer when a small output would leave
+  // clusters idle or waiting for the longest unit
+  const int64_t tiles = ((M + 255) / 256) * ((Nc + 255) / 256);
+  const int64_t clusters = std::max(nsm / 2, 1);
+  int64_t pairs = 0;
+  for (int t = 0; t < nw; ++t) pairs += pairs_of_weight(s, t);
+  const int64_t avg = (pairs * tiles + clusters - 1) / clusters;
+  const int cap = (int)std::min<int64_t>(7, std::max<int64_t>(1, (avg + 1) / 2));
+  PairGroups g{};
+  for (int t = 0; t < nw; ++t) {
+    g.count[t] = (uint8_t)((pairs_of_weight(s, t) + cap - 1) / cap);
+    g.total += g.count[t];
+  }
+  return g;
+}
+
 dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, int64_t lqa, int64_t sa, int64_t M,
                                   const __nv_bfloat16* Qb, int64_t lqb, int64_t sb, int64_t Nc, int64_t K, int64_t k0,
-                                  int64_t kc, int64_t n0, int64_t pn, int s, float* Pw, bool a_lower, int64_t tri) {
+                                  int64_t kc, int64_t n0, int64_t pn, int s, int nw, const PairGroups& groups,
+                                  const uint32_t* norm_a, const uint32_t* norm_b, int32_t* Pw, bool a_lower, int64_t tri) {
   if (M > 2147483647LL - 256 || Nc > 2147483647LL - 256 || K > 2147483647LL)
     return set_error(DGCHEFSI_ERR_UNSUPPORTED, "slice-pair product too large for 32-bit TMA coordinates");
   cudaStream_t st = ctx->stream;
-  const int npairs = s * (s + 1) / 2;
+  int npairs = 0;
+  for (int t = 0; t < nw; ++t) npairs += pairs_of_weight(s, t);
+  const int ng = groups.total;
   const int nmt = (int)((M + 255) / 256), nnt = (int)((pn + 255) / 256);
   // tri > 0: only entries (r, n0 + c) with n0 + c <= r mod tri are wanted (the
   // lower triangle of a symmetric product, or of each of several stacked
@@ -353,24 +447,31 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
       }
     if (tl.empty()) return DGCHEFSI_OK;
   }
-  // tables: 2s tensor maps (64-byte aligned), then the pair lists, then the tile list
+  // tables: 2s tensor maps (64-byte aligned), then groups and pairs, then the tile list
   const size_t maps_bytes = sizeof(CUtensorMap) * (size_t)(2 * s);
-  const size_t pairs_bytes = sizeof(int32_t) * (size_t)(2 * npairs);
-  const size_t tiles_at = (maps_bytes + pairs_bytes + 15) / 16 * 16;
+  const size_t lists_bytes = sizeof(int32_t) * (size_t)(ng + 1 + 2 * npairs);
+  const size_t tiles_at = (maps_bytes + lists_bytes + 15) / 16 * 16;
   std::vector<uint8_t> host(tiles_at + sizeof(int2) * tl.size());
   CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(host.data());
   for (int i = 0; i < s; ++i) {
     DG_TRY(slice_map(&maps[i], Qa + (size_t)i * sa, (uint64_t)K, (uint64_t)M, (uint64_t)lqa));
     DG_TRY(slice_map(&maps[s + i], Qb + (size_t)i * sb, (uint64_t)K, (uint64_t)Nc, (uint64_t)lqb));
   }
-  int32_t* pi = reinterpret_cast<int32_t*>(host.data() + maps_bytes);
+  int32_t* gp = reinterpret_cast<int32_t*>(host.data() + maps_bytes);
+  int32_t* pi = gp + ng + 1;
   int32_t* pj = pi + npairs;
-  int n = 0;
-  for (int i = 0; i < s; ++i)
-    for (int j = 0; i + j < s; ++j, ++n) {
-      pi[n] = i;
-      pj[n] = j;
+  int n = 0, g = 0;
+  for (int t = nw - 1; t >= 0; --t) {  // the pairs of weight t in count[t] groups of nearly equal size
+    const int np = pairs_of_weight(s, t), i0 = std::max(0, t - s + 1);
+    for (int q = 0, k = 0; q < groups.count[t]; ++q) {
+      gp[g++] = n;
+      for (const int end = np * (q + 1) / groups.count[t]; k < end; ++k, ++n) {
+        pi[n] = i0 + k;
+        pj[n] = t - i0 - k;
+      }
     }
+  }
+  gp[g] = n;
   if (!tl.empty()) std::memcpy(host.data() + tiles_at, tl.data(), sizeof(int2) * tl.size());
   // the context's table buffer (may be regrown here: it holds no state across launches)
   DevBuf& tables = ctx->ws_pairs;
@@ -380,18 +481,21 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
   // the pageable copy above has been staged before it returns, so `host` may go
   PairJob J{};
   J.maps = reinterpret_cast<const CUtensorMap*>(tab);
-  J.pair_i = reinterpret_cast<const int32_t*>(tab + maps_bytes);
+  J.group = reinterpret_cast<const int32_t*>(tab + maps_bytes);
+  J.pair_i = J.group + ng + 1;
   J.pair_j = J.pair_i + npairs;
-  J.npairs = npairs;
+  J.ngroups = ng;
   J.s = s;
   J.M = M;
-  J.pn = pn;
+  J.pitch = (pn + 3) / 4 * 4;
   J.n0 = (int)n0;
   J.k0 = (int)k0;
   J.nk = (int)((kc + 63) / 64);
   J.nmt = nmt;
   J.nnt = nnt;
   J.lower = a_lower ? 1 : 0;
+  J.norm_a = norm_a;
+  J.norm_b = norm_b;
   J.tiles = tl.empty() ? nullptr : reinterpret_cast<const int2*>(tab + tiles_at);
   J.ntl = (int)tl.size();
   J.Pw = Pw;
@@ -399,7 +503,7 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
   J.err = static_cast<int*>(ctx->ws_pairs_err.p);
   int nsm = 0;
   DG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-  const int64_t units = (J.tiles ? (int64_t)J.ntl : (int64_t)J.nmt * J.nnt) * npairs;
+  const int64_t units = (J.tiles ? (int64_t)J.ntl : (int64_t)J.nmt * J.nnt) * ng;
   const int clusters = (int)std::min<int64_t>(units, std::max(nsm / 2, 1));
   const int smem = PG_STAGES * PG_STAGE + (2 * PG_STAGES + 4) * 8 + 1024;
   DG_CUDA(cudaFuncSetAttribute(k_slice_pairs_2sm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));

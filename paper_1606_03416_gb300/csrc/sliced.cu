@@ -5,26 +5,37 @@
 // ISC 2020).
 //
 // Over one K chunk of length L <= 4096, row r of A is written as
-//   a[r,k] = 2^{e_r} sum_{i<s} q_i[r,k] 2^{-6(i+1)},  q_i integer, |q_0| <= 64, |q_i| <= 32,
+//   a[r,k] = 2^{e_r} sum_{i<d} q_i[r,k] 2^{-8-9i},  q_i integer, |q_i| <= 256,
 // with 2^{e_r} > max_k |a[r,k]| (and likewise each column of the product's
-// right operand with exponent f_c). Every q is exact in BF16, every product
-// q_i q_j is at most 2^12, so a slice-pair product summed over L <= 4096 terms
-// is an integer of magnitude <= 2^24: the tensor core's FP32 accumulation
-// returns it exactly, whatever its summation order. The pairs with
-// i + j <= s - 1 are kept; their FP32 results are summed per t = i + j in FP64
-// (exact: integers below 2^53), combined by Horner in 2^{-6}, scaled by
-// 2^{e_r + f_c - 12} and added over the chunks. The slice-pair products run
-// on this library's tcgen05 kernel for pairs of SMs (pair_gemm.cu: 256 x 256
-// tiles, every pair of a chunk in one persistent launch, FP32 slabs);
-// splitting and the FP64 reduction are the kernels below.
+// right operand with exponent f_c). Every q is exact in BF16 (8 significant
+// bits hold the integers up to 256), every product q_i q_j is at most 2^16, so
+// a slice-pair product summed over 256 terms is an integer of magnitude at
+// most 2^24: the tensor core's FP32 accumulation returns it exactly, whatever
+// its summation order. The pair kernel (pair_gemm.cu: tcgen05 on pairs of SMs)
+// drains its accumulators every 256 terms (more where the digits' norms bound
+// the longer sums too) into INT32 sums over the chunk and
+// over the pairs of one weight t = i + j. The pairs with t < w are kept (w = d
+// or d + 1, weights_for); their INT32 slabs are combined four weights at a time in INT64, the blocks
+// meet in FP64, scaled by 2^{e_r + f_c - 16}, and the chunks are added;
+// splitting and that reduction are the kernels below.
+//
+// `slices` s of the callers counts 6-bit digits (60 bits at 10, the splitting
+// of one digit per whole 4096-term FP32 sum); digits_for(s) is the number d of
+// 9-bit digits that keeps at least as much (10: d = w = 7, 28 pairs).
 //
 // Error per chunk (row and column maxima m_r, n_c over the chunk): the
-// remainders after s slices and the dropped pairs contribute at most
-// L 2^{e_r + f_c} 2^{-6s} (s + 4)/4 <= L m_r n_c 2^{-6s} (s + 4); the FP64
-// Horner sum and the sum over chunks add at most (5 + chunks) u L m_r n_c,
-// u = 2^{-53}. For s = 10 the splitting term is below u L m_r n_c, the size of
-// FP64's own worst-case bound. The bound is normwise per row and column:
-// entries far below their row's maximum keep fewer significant bits than FP64.
+// remainders after d digits and the dropped pairs contribute at most
+// L 2^{e_r + f_c} 2^{-9d} (d + 2) <= 4 L m_r n_c 2^{-9d} (d + 2), which
+// digits_for keeps below L m_r n_c 2^{-6s} (s + 4); the FP64 steps and the sum
+// over chunks add at most (5 + chunks) u L m_r n_c, u = 2^{-53}. For s = 10
+// (d = 7) the splitting term is below u L m_r n_c, the size of FP64's own
+// worst-case bound. The bound is normwise per row and column: entries far
+// below their row's maximum keep fewer significant bits than FP64.
+//
+// The block-sparse product H X (below) still multiplies one pair per launch on
+// the filter's step kernel with whole-row FP32 sums, so it keeps the 6-bit
+// digits: a[r,k] = 2^{e_r} sum_{i<s} q_i 2^{-6(i+1)}, |q_0| <= 64, |q_i| <= 32,
+// pair sums over L <= 4096 terms at most 2^24.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -35,8 +46,20 @@
 
 namespace dg {
 
-static constexpr int kBeta = 6;      // bits per slice
-static constexpr int64_t kL = 4096;  // K chunk: 4096 * 2^12 = 2^24
+static constexpr int64_t kL = 4096;     // K chunk: one exponent per row and chunk; INT32 holds 7 pairs of it
+static constexpr int kNormPitch = 16;  // digit norms of a chunk (at most 11 digits)
+// For a request of s 6-bit slices (2 <= s <= 16): the number of 9-bit digits,
+// 9 d >= 6 s + 1, so that their remainders are below those of the slices; and
+// the number of weights t = i + j kept, w >= d. w is d, or d + 1 where integer
+// operands that s slices multiply exactly need it to stay exact: operands of a
+// and b slices, a + b <= s + 1, have at most 6 (a + b) bits between them (53
+// when the result is representable) and ceil((bits + 1) / 9) digits each, and
+// the pair of their last digits is kept when those counts sum to at most w + 1.
+static int digits_for(int s) { return (6 * s + 9) / 9; }
+static int weights_for(int s) {
+  const int bits = std::min(6 * (s + 1), 53);
+  return std::min(std::max(digits_for(s), (bits + 18) / 9 - 1), std::max(s, digits_for(s)));
+}
 
 __device__ __forceinline__ void atomic_flag(int* flag) {
   if (flag) atomicOr(flag, 1);
@@ -104,37 +127,127 @@ __device__ __forceinline__ int warp_max(int v) {
   return v;
 }
 
-// One CTA per (row, chunk), 256 threads, 16 entries each. Q: s slices of
-// rows x ldq BF16 (slice i at Q + i * sstride); E[row * nch + chunk] = e_r, the
-// frexp exponent of the row's largest |entry| in the chunk (0 if all are zero).
-// lower: entries k > row are zero (a lower-triangular operand). bal (may be
-// null): entry k is split as X[row, k] 2^{bal[k]}. A row chunk holding NaN/Inf
-// gets zero slices and raises flag.
-__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X, int64_t ldx, int64_t K, int s,
-                                                    int lower, const int32_t* __restrict__ bal,
+// Four consecutive digits (|x| <= 256) to q as BF16, their squares to *norm.
+__device__ __forceinline__ void put_digits(const int (&x)[4], __nv_bfloat16* __restrict__ q, bool store,
+                                           uint32_t* norm) {
+  if (store) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn((float)x[0], (float)x[1]);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn((float)x[2], (float)x[3]);
+    *reinterpret_cast<uint2*>(q) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+  }
+  const uint32_t sq = __reduce_add_sync(0xffffffffu, (uint32_t)(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]));
+  if ((threadIdx.x & 31) == 0) atomicAdd(norm, sq);
+}
+
+// Digits i = 0 .. d - 1 of four consecutive entries, entry c = (-1)^neg M_c
+// 2^{E_c - 1075}, scaled by 2^{-e}: F = round(v 2^{9d - 1}) as a 64-bit integer
+// (d <= 7: |F| <= 2^62; |v 2^{9d-1} - F| <= 1/2), then its balanced base-512
+// digits from the last one up, the first the rest (|q_0| <= 256). Integer
+// arithmetic only; one 8-byte store per digit (where `store`). norm[i] (shared)
+// collects the squares of digit i; every lane of the warp takes part.
+__device__ __forceinline__ void digits_fixed4(const int64_t (&M)[4], const int (&sh)[4], const bool (&neg)[4], int d,
+                                              __nv_bfloat16* __restrict__ q, int64_t stride, bool store,
+                                              uint32_t* norm) {
+  int64_t F[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    F[c] = 0;
+    if (M[c] != 0) {
+      if (sh[c] >= 0)
+        F[c] = M[c] << sh[c];
+      else if (sh[c] > -54)
+        F[c] = (M[c] + (1LL << (-sh[c] - 1))) >> (-sh[c]);
+    }
+    if (neg[c]) F[c] = -F[c];
+  }
+  for (int i = d - 1; i >= 0; --i) {
+    int x[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      x[c] = (int)(i > 0 ? ((F[c] + 256) & 511) - 256 : F[c]);
+      F[c] = (F[c] - x[c]) >> 9;
+    }
+    put_digits(x, q + i * stride, store, norm + i);
+  }
+}
+
+// The same digits for d > 7 (F would not fit 64 bits): v is scaled in FP64,
+// each digit rounded to nearest and subtracted (every step exact).
+__device__ __forceinline__ void digits_fp64x4(const double (&v)[4], int d, __nv_bfloat16* __restrict__ q,
+                                              int64_t stride, bool store, uint32_t* norm) {
+  double r[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) r[c] = v[c] * 256.0;
+  for (int i = 0; i < d; ++i) {
+    int x[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const double g = rint(r[c]);
+      r[c] = (r[c] - g) * 512.0;
+      x[c] = (int)g;
+    }
+    put_digits(x, q + i * stride, store, norm + i);
+  }
+}
+
+// One CTA per (row, chunk), 256 threads, four groups of four consecutive
+// entries each. Q: d digit slices of rows x ldq BF16 (slice i at Q + i *
+// sstride; ldq a multiple of 8 and at least K, the entries past K written as
+// zero); E[row * nch + chunk] = e_r, the frexp exponent of the row's largest
+// |entry| in the chunk (0 if all are zero). lower: entries k > row are zero (a
+// lower-triangular operand). bal (may be null): entry k is split as
+// X[row, k] 2^{bal[k]}. wide: rows of X start on 16 bytes. A row chunk holding
+// NaN/Inf gets zero slices and raises flag. norm2[chunk * kNormPitch + i] is
+// raised to the largest sum of squares of digit i over a 512-entry block of
+// any row of the chunk (zero before the launch): what lets the pair kernel
+// keep its FP32 sums over 512 terms or more instead of 256.
+// Bound by HBM: 8 bytes read and 2 d written per entry, in 32- and 8-byte
+// pieces per thread (2-byte stores of single entries took twice the time).
+__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X, int64_t ldx, int64_t K, int d,
+                                                    int lower, int wide, const int32_t* __restrict__ bal,
                                                     __nv_bfloat16* __restrict__ Q, int64_t ldq, int64_t sstride,
-                                                    int32_t* __restrict__ E, int nch, int* __restrict__ flag) {
+                                                    int32_t* __restrict__ E, int nch, uint32_t* __restrict__ norm2,
+                                                    int* __restrict__ flag) {
   const int64_t row = blockIdx.x;
   const int chunk = blockIdx.y;
   const int64_t k0 = (int64_t)chunk * kL;
-  double v[16];
+  const int64_t kend = lower && row + 1 < K ? row + 1 : K;  // entries from here on are zero
+  double v[4][4];
   int emax = INT_MIN;
   bool bad = false;
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int64_t k = k0 + threadIdx.x + 256 * u;
-    double x = 0.0;
-    if (k < K && !(lower && k > row)) x = X[row * ldx + k];
-    v[u] = x;
-    int64_t M;
-    int Ex;
-    const int c = decompose(x, M, Ex);
-    if (c == 2) bad = true;
-    if (c == 1) emax = max(emax, Ex + (bal ? bal[k] : 0));
+  for (int u = 0; u < 4; ++u) {
+    const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
+    const double* x = X + row * ldx + k;
+    if (wide && k + 4 <= kend) {
+      const double2 a = *reinterpret_cast<const double2*>(x), b = *reinterpret_cast<const double2*>(x + 2);
+      v[u][0] = a.x;
+      v[u][1] = a.y;
+      v[u][2] = b.x;
+      v[u][3] = b.y;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[u][c] = k + c < kend ? x[c] : 0.0;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      int64_t M;
+      int Ex;
+      const int z = decompose(v[u][c], M, Ex);
+      if (z == 2) bad = true;
+      if (z == 1) emax = max(emax, Ex + (bal ? bal[k + c] : 0));
+    }
   }
   __shared__ int red[8];
   __shared__ int sbad;
+  __shared__ uint32_t norm[8][kNormPitch];  // by 512-entry block and digit
   if (threadIdx.x == 0) sbad = 0;
+  if (threadIdx.x < 8 * kNormPitch) norm[threadIdx.x / kNormPitch][threadIdx.x % kNormPitch] = 0;
   emax = warp_max(emax);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = emax;
@@ -150,19 +263,37 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
     if (zero) atomic_flag(flag);
   }
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int64_t k = k0 + threadIdx.x + 256 * u;
-    if (k >= K) break;
+  for (int u = 0; u < 4; ++u) {
+    const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
+    if (k0 + 1024 * u >= K) break;  // the same for the whole CTA
+    uint32_t* nrm = norm[2 * u + (threadIdx.x >> 7)];
     __nv_bfloat16* q = Q + row * ldq + k;
-    const int b = bal ? bal[k] : 0;
-    if (s <= 10) {
-      int64_t M = 0;
-      int Ex = 0;
-      if (zero || decompose(v[u], M, Ex) != 1) M = 0;
-      slice_fixed(M, Ex + b, v[u] < 0.0, -1075 - e + 6 * s, s, q, sstride);
+    if (d <= 7) {
+      int64_t M[4];
+      int sh[4];
+      bool neg[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        int Ex = 0;
+        if (zero || decompose(v[u][c], M[c], Ex) != 1) M[c] = 0;
+        sh[c] = M[c] != 0 ? Ex + (bal ? bal[k + c] : 0) - 1075 - e + 9 * d - 1 : 0;
+        neg[c] = v[u][c] < 0.0;
+      }
+      digits_fixed4(M, sh, neg, d, q, sstride, k < K, nrm);
     } else {
-      slice_fp64(zero ? 0.0 : ldexp(v[u], b - e), s, q, sstride);
+      double r[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        r[c] = zero || v[u][c] == 0.0 ? 0.0 : ldexp(v[u][c], (bal ? bal[k + c] : 0) - e);
+      digits_fp64x4(r, d, q, sstride, k < K, nrm);
     }
+  }
+  __syncthreads();
+  if (threadIdx.x < d) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) m = max(m, norm[b][threadIdx.x]);
+    atomicMax(norm2 + chunk * kNormPitch + threadIdx.x, m);
   }
 }
 
@@ -336,9 +467,122 @@ static cudaError_t launch_reduce(int s, const float* Pw, int64_t M, int64_t P, c
   return cudaGetLastError();
 }
 
+// h 2^e (one rounding, as ldexp; the power of two is built from its bits when
+// it is a normal number).
+__device__ __forceinline__ double scale_pow2(double h, int e) {
+  if (e > -1000 && e < 1000) return h * __longlong_as_double((long long)(e + 1023) << 52);
+  return ldexp(h, e);
+}
+
+// C[r, n0 + c] (+)= 2^{e_r + f_{n0+c} - 16} sum_t 2^{-9t} g_t for r < M, c < P,
+// g_t the sum of weight t's count[t] INT32 slabs (M rows of `pitch` entries, t
+// descending). Four consecutive t are combined in INT64 (|g_t| < 2^32, so the
+// block is below 2^60) and converted to FP64, and the blocks meet by Horner in
+// 2^{-36}: one rounding of each block and one per step.
+// Four consecutive outputs per thread, one 16-byte load per slab; wide: the
+// rows of C at n0 start on 16 bytes. tri > 0: only the entries with
+// n0 + c <= r mod tri are formed (the slice-pair kernel left the tiles above
+// that line out); the others are not read or written.
+// Bound by HBM: 4 bytes read per slab and entry (28 at w = 7) and 8 written, 16
+// when a chunk is added; it runs on its own stream beside the next chunk's pairs.
+template <int W>
+__global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict__ Pw, int64_t M, int64_t P,
+                                                      int64_t pitch, const PairGroups groups,
+                                                      const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb,
+                                                      int nch, int chunk, int64_t n0, double* __restrict__ C,
+                                                      int64_t ldc, int wide, int accumulate, int64_t tri) {
+  constexpr int NB = (W + 3) / 4;
+  const int64_t slab = M * pitch, quads = pitch / 4, total = M * quads;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = q / quads, c0 = 4 * (q - r * quads);
+    // the four entries share a row and a 256-column tile: when the first is
+    // above the line all are, and otherwise the tile was computed
+    const int64_t rdiag = tri > 0 ? r % tri : 0;
+    if (tri > 0 && n0 + c0 > rdiag) continue;
+    const int4* p = reinterpret_cast<const int4*>(Pw + 4 * q);
+    int64_t g[4][W];
+    if (groups.total == W) {  // one slab per weight: all loads before any use
+      int4 v[W];
+#pragma unroll
+      for (int t = 0; t < W; ++t) v[t] = __ldcs(p + (int64_t)(W - 1 - t) * (slab / 4));
+#pragma unroll
+      for (int t = 0; t < W; ++t) {
+        g[0][t] = v[t].x;
+        g[1][t] = v[t].y;
+        g[2][t] = v[t].z;
+        g[3][t] = v[t].w;
+      }
+    } else {
+#pragma unroll
+      for (int t = W - 1; t >= 0; --t) {
+        g[0][t] = g[1][t] = g[2][t] = g[3][t] = 0;
+        for (int k = 0; k < groups.count[t]; ++k, p += slab / 4) {
+          const int4 v = __ldcs(p);
+          g[0][t] += v.x;
+          g[1][t] += v.y;
+          g[2][t] += v.z;
+          g[3][t] += v.w;
+        }
+      }
+    }
+    const int er = Ea[r * nch + chunk] - 16 - 27;
+    double y[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      // B_b = sum_{t = 4b}^{4b+3} g_t 2^{9(4b + 3 - t)}; sum_t g_t 2^{-9t} = 2^{-27} sum_b B_b 2^{-36b}
+      double h = 0.0;
+#pragma unroll
+      for (int b = NB - 1; b >= 0; --b) {
+        int64_t B = 0;
+#pragma unroll
+        for (int t = 4 * b; t < 4 * b + 4; ++t) B = B * 512 + (t < W ? g[e][t] : 0);
+        h = b == NB - 1 ? (double)B : h * 0x1p-36 + (double)B;
+      }
+      y[e] = c0 + e < P ? scale_pow2(h, er + Eb[(n0 + c0 + e) * nch + chunk]) : 0.0;
+    }
+    double* out = C + r * ldc + n0 + c0;
+    if (wide && c0 + 4 <= P && (tri == 0 || n0 + c0 + 3 <= rdiag)) {
+      double2* o = reinterpret_cast<double2*>(out);
+      if (accumulate) {
+        const double2 a = o[0], b = o[1];
+        y[0] += a.x;
+        y[1] += a.y;
+        y[2] += b.x;
+        y[3] += b.y;
+      }
+      o[0] = make_double2(y[0], y[1]);
+      o[1] = make_double2(y[2], y[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (c0 + e < P && (tri == 0 || n0 + c0 + e <= rdiag)) out[e] = accumulate ? out[e] + y[e] : y[e];
+    }
+  }
+}
+
+typedef void (*DigitReduce)(const int32_t*, int64_t, int64_t, int64_t, const PairGroups, const int32_t*,
+                            const int32_t*, int, int, int64_t, double*, int64_t, int, int, int64_t);
+
+static DigitReduce digit_reduce(int w) {
+  switch (w) {
+    case 2: return k_digit_reduce<2>;
+    case 3: return k_digit_reduce<3>;
+    case 4: return k_digit_reduce<4>;
+    case 5: return k_digit_reduce<5>;
+    case 6: return k_digit_reduce<6>;
+    case 7: return k_digit_reduce<7>;
+    case 8: return k_digit_reduce<8>;
+    case 9: return k_digit_reduce<9>;
+    case 10: return k_digit_reduce<10>;
+    case 11: return k_digit_reduce<11>;
+    default: return nullptr;
+  }
+}
+
 static int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-// Workspace cap of the FP32 slice-pair products; wider outputs run in column panels.
+// Workspace cap of the slabs of the slice-pair products; wider outputs run in column panels.
 static constexpr size_t kPairBytes = size_t(8) << 30;
 
 // T (cols x rows, row-major, ldt) = X^T for X (rows x cols, row-major, ldx);
@@ -369,17 +613,21 @@ static dgchefsi_status transpose_f64(const double* X, int64_t ldx, int64_t rows,
 }
 
 dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_t M, int64_t Nc, int64_t K,
-                            const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc, int s,
-                            int* flag, int64_t tri) {
+                            const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
+                            int slices, int* flag, int64_t tri) {
   if (M <= 0 || Nc <= 0) return DGCHEFSI_OK;
-  if (!reduce_kernel(s)) return set_error(DGCHEFSI_ERR_ARG, "slices = %d outside 2..16", s);
+  if (slices < 2 || slices > 16) return set_error(DGCHEFSI_ERR_ARG, "slices = %d outside 2..16", slices);
+  const int s = digits_for(slices), nw = weights_for(slices);
   cudaStream_t st = ctx->stream;
   if (K <= 0) {
     DG_CUDA(cudaMemset2DAsync(C, sizeof(double) * ldc, 0, sizeof(double) * Nc, M, st));
     return DGCHEFSI_OK;
   }
   const int nch = (int)((K + kL - 1) / kL);
-  const int64_t pairs = (int64_t)s * (s + 1) / 2;
+  int nsm = 0;
+  DG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+  const PairGroups groups = pair_groups(s, nw, M, Nc, nsm);
+  const size_t slab_row = sizeof(int32_t) * (size_t)groups.total * (size_t)M;  // bytes per output column
   // Slices of A: s x M x lqa, of the right operand as rows: s x Nc x lqb (K
   // contiguous in both; the A B form transposes B first).
   const int64_t lqa = round_up(K, 8);
@@ -392,22 +640,21 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
   const size_t ea_bytes = sizeof(int32_t) * (size_t)(M * nch);
   const size_t eb_bytes = sizeof(int32_t) * (size_t)(Nc * nch);
   const size_t bal_bytes = b_rows ? 0 : 2 * sizeof(int32_t) * (size_t)K;
+  const size_t norm_bytes = 2 * sizeof(uint32_t) * (size_t)(kNormPitch * nch);
   const size_t a256 = 256;
   auto up = [&](size_t x) { return (x + a256 - 1) / a256 * a256; };
-  // Column panel of the product (a multiple of the kernel's 128-column tiles)
-  // so that the FP32 pair slabs stay under the cap; two slab buffers when the
-  // product has more than one (panel, chunk) step, so that the reduction of
-  // one step (on the context's reduction stream) overlaps the next step's
-  // slice pairs.
-  const bool multi = nch > 1 || (int64_t)(kPairBytes / (sizeof(float) * (size_t)pairs * (size_t)M)) < Nc;
+  // Column panel of the product (a multiple of the kernel's 256-column tiles)
+  // so that the slabs stay under the cap; two slab buffers when the product
+  // has more than one (panel, chunk) step, so that the reduction of one step
+  // (on the context's reduction stream) overlaps the next step's slice pairs.
+  const bool multi = nch > 1 || (int64_t)(kPairBytes / slab_row) < Nc;
   const int nbuf = multi ? 2 : 1;
-  int64_t P = (int64_t)(kPairBytes / nbuf / (sizeof(float) * (size_t)pairs * (size_t)M));
-  P = std::max<int64_t>(128, P / 128 * 128);
+  int64_t P = std::max<int64_t>(256, (int64_t)(kPairBytes / nbuf / slab_row) / 256 * 256);
   if (P >= Nc) P = Nc;
-  const size_t slab_set = sizeof(float) * (size_t)pairs * (size_t)M * (size_t)P;
+  const size_t slab_set = slab_row * (size_t)round_up(P, 4);
   const size_t pw_bytes = (size_t)nbuf * up(slab_set);
   DG_TRY(ensure(ctx, ctx->ws_sliced,
-                up(qa_bytes) + up(qb_bytes) + up(ea_bytes) + up(eb_bytes) + up(bal_bytes) + up(pw_bytes),
+                up(qa_bytes) + up(qb_bytes) + up(ea_bytes) + up(eb_bytes) + up(bal_bytes) + up(norm_bytes) + up(pw_bytes),
                 "sliced-product workspace"));
   char* base = static_cast<char*>(ctx->ws_sliced.p);
   __nv_bfloat16* Qa = reinterpret_cast<__nv_bfloat16*>(base);
@@ -417,8 +664,11 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
   int32_t* bal = b_rows ? nullptr
                         : reinterpret_cast<int32_t*>(base + up(qa_bytes) + up(qb_bytes) + up(ea_bytes) + up(eb_bytes));
   int32_t* nbal = b_rows ? nullptr : bal + K;
-  float* Pw =
-      reinterpret_cast<float*>(base + up(qa_bytes) + up(qb_bytes) + up(ea_bytes) + up(eb_bytes) + up(bal_bytes));
+  uint32_t* norm_a =
+      reinterpret_cast<uint32_t*>(base + up(qa_bytes) + up(qb_bytes) + up(ea_bytes) + up(eb_bytes) + up(bal_bytes));
+  uint32_t* norm_b = same ? norm_a : norm_a + kNormPitch * nch;
+  int32_t* Pw = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(norm_a) + up(norm_bytes));
+  DG_CUDA(cudaMemsetAsync(norm_a, 0, norm_bytes, st));
 
   // C = A B with B (K x Nc): every K index k is balanced first, row k of B by
   // 2^{-s_k} and column k of A by 2^{s_k} (exact), s_k the exponent of B's row
@@ -437,13 +687,14 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
     Br = Bt;
     ldbr = K;
   }
-  k_split_rows<<<dim3((unsigned)M, (unsigned)nch), 256, 0, st>>>(A, lda, K, s, a_lower ? 1 : 0, bal, Qa, lqa, sa,
-                                                                  Ea, nch, flag);
+  auto wide = [](const double* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 2 == 0; };
+  k_split_rows<<<dim3((unsigned)M, (unsigned)nch), 256, 0, st>>>(A, lda, K, s, a_lower ? 1 : 0, wide(A, lda) ? 1 : 0,
+                                                                  bal, Qa, lqa, sa, Ea, nch, norm_a, flag);
   count_launch();
   DG_CUDA(cudaGetLastError());
   if (!same) {
-    k_split_rows<<<dim3((unsigned)Nc, (unsigned)nch), 256, 0, st>>>(Br, ldbr, K, s, 0, nbal, Qb, lqb, sb, Eb, nch,
-                                                                     flag);
+    k_split_rows<<<dim3((unsigned)Nc, (unsigned)nch), 256, 0, st>>>(Br, ldbr, K, s, 0, wide(Br, ldbr) ? 1 : 0,
+                                                                     nbal, Qb, lqb, sb, Eb, nch, norm_b, flag);
     count_launch();
     DG_CUDA(cudaGetLastError());
   }
@@ -477,18 +728,24 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
       const int64_t k0 = (int64_t)chunk * kL;
       const int64_t kc = std::min<int64_t>(kL, K - k0);
       const int b = step & 1;
-      float* Pb = reinterpret_cast<float*>(reinterpret_cast<char*>(Pw) + (size_t)b * up(slab_set));
-      // slab of pair (i, j): M x pn, Qa_i times the panel's rows of Qb_j over this chunk,
+      int32_t* Pb = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(Pw) + (size_t)b * up(slab_set));
+      // slabs of the panel: Qa_i times the panel's rows of Qb_j over this chunk, summed per weight,
       // into buffer b once the reduction that last read it is done
       if (multi) DG_CUDA(cudaStreamWaitEvent(st, ctx->ev_reduce[b], 0));
       DG_CUDA(cudaEventRecord(ctx->ev_time[2 * step], st));
-      DG_TRY(pair_products_2sm(ctx, Qa, lqa, sa, M, Qb, lqb, sb, Nc, K, k0, kc, n0, pn, s, Pb, a_lower, tri));
+      DG_TRY(pair_products_2sm(ctx, Qa, lqa, sa, M, Qb, lqb, sb, Nc, K, k0, kc, n0, pn, s, nw, groups,
+                               norm_a + kNormPitch * chunk, norm_b + kNormPitch * chunk, Pb, a_lower, tri));
       DG_CUDA(cudaEventRecord(ctx->ev_time[2 * step + 1], st));
       if (multi) {
         DG_CUDA(cudaEventRecord(ctx->ev_pairs[b], st));
         DG_CUDA(cudaStreamWaitEvent(sr, ctx->ev_pairs[b], 0));
       }
-      DG_CUDA(launch_reduce(s, Pb, M, pn, Ea, Eb, nch, chunk, n0, C, ldc, chunk > 0 ? 1 : 0, nullptr, sr, tri));
+      const int64_t pitch = round_up(pn, 4), work = M * pitch / 4;
+      const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 16));
+      digit_reduce(nw)<<<grid, 256, 0, sr>>>(Pb, M, pn, pitch, groups, Ea, Eb, nch, chunk, n0, C, ldc,
+                                            wide(C, ldc) ? 1 : 0, chunk > 0 ? 1 : 0, tri);
+      count_launch();
+      DG_CUDA(cudaGetLastError());
       if (multi) DG_CUDA(cudaEventRecord(ctx->ev_reduce[b], sr));
     }
   }

@@ -1,0 +1,51 @@
+"""The 9-bit digits of the dense sliced products: bit for bit at the edge of the
+exact FP32 sums, at ragged drains of the accumulator (256 terms, or more where
+the digits' norms allow), at ragged K chunks and tiles, and on operands whose
+digits are all in use."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1606_03416_gb300 import dgchefsi as D
+from paper_1606_03416_gb300 import inputs as G
+
+pytestmark = pytest.mark.gpu
+
+
+def product(A, Bt, b_rows, slices=10):
+    with D.Context(G.make_blocks(G.CONFIGS["tiny_2x2x2"])) as ctx:
+        B = Bt if b_rows else np.ascontiguousarray(Bt.T)
+        out = ctx.sliced_gemm(torch.from_numpy(A.astype(np.float64)).cuda(), torch.from_numpy(B.astype(np.float64)).cuda(),
+                              b_rows=b_rows, slices=slices)
+        return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("b_rows", [True, False])
+@pytest.mark.parametrize("M,Nc,K", [(1, 1, 255), (3, 130, 256), (257, 5, 257), (70, 301, 512), (255, 257, 1030),
+                                    (40, 50, 4096), (33, 20, 4097), (129, 64, 8500)])
+def test_digits_at_their_bounds_bit_exact(M, Nc, K, b_rows):
+    """130816 = 2^17 - 256 splits (exponent 17) into q_0 = 256, q_1 = -256, so
+    products of equal-sign rows sum to +-256^3 = +-2^24 over 256 terms; rows of
+    mixed sign and a row of ones beside them. The exact products are integers
+    below 2^53."""
+    rng = np.random.default_rng(1)
+    A = np.full((M, K), 130816, dtype=np.int64)
+    Bt = np.full((Nc, K), 130816, dtype=np.int64)
+    A[1::3] *= -1
+    Bt[1::4] *= rng.choice([-1, 1], size=K)
+    if M > 2:
+        A[2] = 1
+    assert np.array_equal(product(A, Bt, b_rows), (A @ Bt.T).astype(np.float64))
+
+
+@pytest.mark.parametrize("slices", [4, 7, 10, 12])
+@pytest.mark.parametrize("M,Nc,K", [(300, 131, 4096), (64, 700, 1000), (513, 259, 5000)])
+def test_random_integers_bit_exact(M, Nc, K, slices):
+    """Random integers of 6 a and 6 b bits, a + b <= slices + 1, that `slices`
+    slices multiply exactly (the product stays below 2^53)."""
+    rng = np.random.default_rng(2)
+    a = min(slices // 2, 3)
+    b = min(slices + 1 - a, 3)
+    A = rng.integers(-(2 ** (6 * a - 1)), 2 ** (6 * a - 1), size=(M, K))
+    Bt = rng.integers(-(2 ** (6 * b - 1)), 2 ** (6 * b - 1), size=(Nc, K))
+    assert np.array_equal(product(A, Bt, True, slices), (A @ Bt.T).astype(np.float64))
