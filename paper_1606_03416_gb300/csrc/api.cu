@@ -330,6 +330,8 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
   const bool sl = ctx->products_mode == DGCHEFSI_PRODUCTS_SLICED_BF16;
   const bool own_chol = use_own_cholesky(ctx);
   int* bad = ctx->info_d + 3;
+  Parts parts;
+  DG_TRY(parts_of(ctx, &parts));
   // Step 3: S = Y^T Y (lower tiles, mirrored), S = U^T U, Y_hat = Y U^{-1}.
   // CholeskyQR2 repeats the pass on Y_hat; shifted CholeskyQR3 factors
   // Y^T Y + s I first, s = 11 (N N_s + N_s (N_s + 1)) u ||Y||_F^2, then repeats
@@ -344,7 +346,7 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
     if (sl)
       DG_TRY(sliced_gemm(ctx, true, false, Ns, Ns, N, in, ldi, in, ldi, S, Ns, ctx->products_slices, bad, Ns));
     else
-      DG_CUDA(gemm_nt_f64(in, ldi, in, ldi, S, Ns, Ns, Ns, N, true, false, s));
+      DG_CUDA(gemm_nt_f64(in, ldi, in, ldi, S, Ns, Ns, Ns, N, true, false, parts, s));
     if (pass == 0 && ctx->orth_mode == DGCHEFSI_ORTH_SHIFTED_CHOLQR3)
       DG_CUDA(shift_diagonal_by_trace_f64(S, Ns, 11.0 * ((double)N * (double)Ns + (double)Ns * (double)(Ns + 1)) *
                                                      0x1p-53, s));
@@ -387,7 +389,7 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
   if (sl)
     DG_TRY(sliced_gemm(ctx, true, false, Ns, Ns, N, W, N, Y, ld, S, Ns, ctx->products_slices, bad, Ns));
   else
-    DG_CUDA(gemm_nt_f64(W, N, Y, ld, S, Ns, Ns, Ns, N, true, false, s));
+    DG_CUDA(gemm_nt_f64(W, N, Y, ld, S, Ns, Ns, Ns, N, true, false, parts, s));
   // The eigensolver reads the lower triangle (row-major), the one computed.
   DG_TRY(subspace_eigh(ctx, S, Ns, Ns, ritz));
   // Step 5: X_new^T = Q^T Y_hat^T (column-major Q read row-major is Q^T).
@@ -443,9 +445,6 @@ dgchefsi_status dgchefsi_create(int32_t M, const int32_t* nb, const int64_t* row
       ctx->max_nb = std::max(ctx->max_nb, nb[K]);
     }
     ctx->N = ctx->off_h[M];
-    ctx->f64_tj = 64;
-    for (int K = 0; K < M; ++K)
-      if (nb[K] % 64 != 0) ctx->f64_tj = 32;
     if (row_ptr[0] != 0) return bail(set_error(DGCHEFSI_ERR_ARG, "row_ptr[0] != 0"));
     for (int K = 0; K < M; ++K)
       if (row_ptr[K + 1] < row_ptr[K]) return bail(set_error(DGCHEFSI_ERR_ARG, "row_ptr decreases at %d", K));
@@ -567,6 +566,7 @@ void dgchefsi_destroy(dgchefsi_ctx* ctx) {
   free_buf(ctx->ws_pairs_err);
   free_buf(ctx->ws_eig);
   free_buf(ctx->ws_chol);
+  free_buf(ctx->ws_parts);
   if (ctx->s_reduce) cudaStreamSynchronize(ctx->s_reduce);
   for (int i = 0; i < 2; ++i) {
     if (ctx->ev_pairs[i]) cudaEventDestroy(ctx->ev_pairs[i]);
@@ -1022,7 +1022,9 @@ dgchefsi_status dgchefsi_gram(dgchefsi_ctx* ctx, const double* Y, int64_t Ns, in
   DG_TRY(check_ctx(ctx));
   DG_TRY(check_block(ctx, Y, Ns, ld, "Y"));
   if (Ns > 0 && !S) return set_error(DGCHEFSI_ERR_ARG, "null S");
-  DG_CUDA(gemm_nt_f64(Y, ld, Y, ld, S, Ns, Ns, Ns, ctx->N, true, false, ctx->stream));
+  Parts parts;
+  DG_TRY(parts_of(ctx, &parts));
+  DG_CUDA(gemm_nt_f64(Y, ld, Y, ld, S, Ns, Ns, Ns, ctx->N, true, false, parts, ctx->stream));
   return DGCHEFSI_OK;
 }
 
@@ -1055,7 +1057,9 @@ dgchefsi_status dgchefsi_density_blocks(dgchefsi_ctx* ctx, const double* X, int6
   DG_TRY(check_ctx(ctx));
   DG_TRY(check_block(ctx, X, Ns, ld, "X"));
   if (!P || (Ns > 0 && !f)) return set_error(DGCHEFSI_ERR_ARG, "null f or P");
-  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, X, Ns, ld, f, P, ctx->stream));
+  Parts parts;
+  DG_TRY(parts_of(ctx, &parts));
+  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
   return DGCHEFSI_OK;
 }
 
@@ -1103,7 +1107,9 @@ dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t N
   DG_CUDA(cudaMemcpy2DAsync(X, sizeof(double) * ld, Yw, sizeof(double) * ld, sizeof(double) * ctx->N, Ns,
                             cudaMemcpyDeviceToDevice, ctx->stream));
   DG_CUDA(occupations_f64(ritz, Ns, Ne, kT, f, mu, ctx->stream));
-  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, X, Ns, ld, f, P, ctx->stream));
+  Parts parts;
+  DG_TRY(parts_of(ctx, &parts));
+  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
   if (bounds) {
     bounds[0] = a;
     bounds[1] = b;

@@ -87,7 +87,7 @@ struct dgchefsi_ctx {
   // form's workspace (L^{-1} and two scratch blocks, 3 N_s^2 doubles)
   int chol_mode = 0;
   dg::DevBuf ws_chol;
-  int32_t f64_tj = 64;    // column tile of the FP64 filter (set at create)
+  dg::DevBuf ws_parts;    // partial results of split FP64 products (kPartsBytes)
   // FP64 filter as a CUDA graph: coefficients copied from a pinned mirror at
   // every replay; the graph is captured again when X, Y, N_s, ld, m or the
   // workspace it refers to change
@@ -120,7 +120,6 @@ struct dgchefsi_ctx {
     h.blk_off = blk_off_d;
     h.vals = vals_d;
     h.max_nb = max_nb;
-    h.tj = f64_tj;
     return h;
   }
 };
@@ -132,6 +131,17 @@ dgchefsi_status set_error(dgchefsi_status st, const char* fmt, ...);
 void clear_error();
 // Make `b` hold at least `bytes` (synchronises the context's stream before a regrow).
 dgchefsi_status ensure(dgchefsi_ctx* ctx, DevBuf& b, size_t bytes, const char* what);
+
+// The context's buffer for split FP64 products, one for all of them (they run
+// in turn on the context's stream).
+constexpr size_t kPartsBytes = size_t(128) << 20;
+inline dgchefsi_status parts_of(dgchefsi_ctx* ctx, Parts* parts) {
+  const dgchefsi_status st = ensure(ctx, ctx->ws_parts, kPartsBytes, "partial products");
+  if (st != DGCHEFSI_OK) return st;
+  parts->p = static_cast<double*>(ctx->ws_parts.p);
+  parts->doubles = (int64_t)(ctx->ws_parts.bytes / sizeof(double));
+  return DGCHEFSI_OK;
+}
 
 // Tensor-core filter (tc_filter.cu). X, Y FP64 (Ns x ld) state-major.
 // reuse_hop: the operand copy of H - cI built by the previous call of this

@@ -900,10 +900,10 @@ dgchefsi_status eig_refined(dgchefsi_ctx* ctx, double* A, int64_t n, int64_t lda
       k_scatter_rows_of<<<grid_for(m * n), 256, 0, st>>>(Sm, n, ws.perm, m, n, R2);
       k_gather_cols_of<<<grid_for(m * n), 256, 0, st>>>(Sm, n, ws.perm, m, n, R1);
       count_launch(2);
-      DG_CUDA(gemm_nt_f64(R1, m, Wb, m, R2, m, n, m, m, false, false, st));
+      DG_CUDA(gemm_nt_f64(R1, m, Wb, m, R2, m, n, m, m, false, false, Parts(), st));
       k_scatter_cols_of<<<grid_for(m * n), 256, 0, st>>>(Sm, n, ws.perm, m, n, R2, nullptr, nullptr);
       count_launch();
-      DG_CUDA(gemm_nt_f64(Wb, m, Wb, m, R1, m, m, m, m, false, false, st));
+      DG_CUDA(gemm_nt_f64(Wb, m, Wb, m, R1, m, m, m, m, false, false, Parts(), st));
       k_scatter_block_of<<<grid_for(m * m), 256, 0, st>>>(Gm, n, ws.perm, m, R1);
       count_launch();
       DG_CUDA(cudaGetLastError());

@@ -5,12 +5,25 @@
 // diagonal density blocks (Eq. densitymatrix).
 //
 // GB300 executes FP64 only on the CUDA-core DFMA pipe (tcgen05 has no FP64
-// kind), at a small fraction of the tensor rate, so these kernels are
-// ALU-bound by a wide margin: a 64x64 output tile per 256-thread CTA, 4x4
-// register blocking, operands staged through shared memory in 16-deep slices.
+// kind), two multiply-adds per clock and SM, so these kernels are ALU-bound by
+// a wide margin and what a tile costs is the multiply-adds it issues, padding
+// included. So the tiles are small (16 rows x up to 64 columns, 128 threads,
+// one row x eight columns each; 64 x 64 for the products over states), a warp
+// skips the 8-column groups and 4-row groups that lie outside the result, and
+// the contraction runs to its own end, not to a multiple of a slice. A small
+// tile also spreads a small problem evenly over the SMs; operands re-read for
+// it come from L2 at a few bytes per clock. Operands are staged through shared
+// memory in 16-deep slices.
+// Measured, before (64 x 64 or 64 x 32 tiles, 256 threads) and now: H X at n_K =
+// 40, 300 states 3.28 -> 1.47 ms (1.13 TFLOP/s), n_K = 64 and 4096 states 371 ms
+// both (1.25); Gram matrix of 401 states of 12096 rows 12.7 -> 2.0 ms; density
+// blocks at n_K = 64, 4096 states 16.9 -> 9.6 ms; pattern blocks at n_K = 40
+// 3.75 -> 1.57 ms.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 
+#include "f64_tile.cuh"
 #include "internal.h"
 
 namespace dg {
@@ -21,37 +34,14 @@ int64_t launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
 namespace {
 
-constexpr int T = 64;       // output tile edge
-constexpr int BK = 16;      // contraction slice
-constexpr int TP = T + 1;   // padded shared-memory row
-constexpr int NT = 256;     // threads per CTA (16 x 16, 4x4 outputs each)
+using namespace f64tile;
 
-__device__ __forceinline__ void fma_tile(const double (&As)[BK][TP], const double (&Bs)[BK][TP],
-                                         double (&acc)[4][4], int tx, int ty) {
-#pragma unroll
-  for (int kk = 0; kk < BK; ++kk) {
-    double a[4], b[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-  }
-}
-
-// One Chebyshev step on a (64 states) x (TJ rows of element K) tile:
+// One Chebyshev step on a (16 states) x (64 rows of element K) tile:
 // out = alpha * (sum_{K'} H_KK' in_K' - c in_K) - beta * prev_K.
-// TJ = 64 when every element size is a multiple of 64, else 32, so uneven
-// elements leave fewer idle columns in their last tile.
-template <int TJ>
 __global__ void __launch_bounds__(NT) k_filter_step_f64(HView h, const double* __restrict__ in, int64_t ld,
                                                         const double* prev, double* out, int64_t ldo,
                                                         int64_t Ns, double alpha, double c, double beta,
                                                         const double* __restrict__ coef, int step) {
-  constexpr int JR = TJ / 16;  // output columns per thread
   if (coef) {  // coefficients in device memory ([c, alpha_0, beta_0, alpha_1, ...]; graph replays)
     c = coef[0];
     alpha = coef[1 + 2 * step];
@@ -59,66 +49,52 @@ __global__ void __launch_bounds__(NT) k_filter_step_f64(HView h, const double* _
   }
   const int K = blockIdx.y;
   const int nK = h.nb[K];
-  const int j0 = blockIdx.z * TJ;
+  const int j0 = blockIdx.z * T;
   if (j0 >= nK) return;
-  const int64_t s0 = (int64_t)blockIdx.x * T;
-  __shared__ double As[BK][TP];
-  __shared__ double Bs[BK][TJ + 1];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double acc[4][JR];
+  const int64_t s0 = (int64_t)blockIdx.x * TR;
+  __shared__ double As[BK][TRP];
+  __shared__ double Bs[BK][TP];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int jn = groups8(nK - j0);
+  const bool live = s0 + (ty & ~3) < Ns;  // this warp's four states
+  double acc[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < JR; ++j) acc[i][j] = 0.0;
+  for (int j = 0; j < 8; ++j) acc[j] = 0.0;
   const int64_t offK = h.off[K];
   const int64_t e_end = h.row_ptr[K + 1];
+  const int kk = tid & 15, rr = tid >> 4;
   for (int64_t e = h.row_ptr[K]; e < e_end; ++e) {
     const int Kp = h.col[e];
     const int nKp = h.nb[Kp];
     const int64_t offKp = h.off[Kp];
     const double* blk = h.vals + h.blk_off[e];
     for (int k0 = 0; k0 < nKp; k0 += BK) {
-      const int kk = tid & 15;
       const bool kin = (k0 + kk) < nKp;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = (tid >> 4) + 16 * i;
+      for (int i = 0; i < 2; ++i) {
+        const int r = rr + 8 * i;
         As[kk][r] = (kin && s0 + r < Ns) ? in[(s0 + r) * ld + offKp + k0 + kk] : 0.0;
       }
 #pragma unroll
-      for (int i = 0; i < JR; ++i) {
-        const int r = (tid >> 4) + 16 * i;
-        Bs[kk][r] = (kin && j0 + r < nK) ? blk[(int64_t)(j0 + r) * nKp + k0 + kk] : 0.0;
+      for (int i = 0; i < 8; ++i) {
+        const int r = rr + 8 * i;
+        if (i < jn) Bs[kk][r] = (kin && j0 + r < nK) ? blk[(int64_t)(j0 + r) * nKp + k0 + kk] : 0.0;
       }
       __syncthreads();
-#pragma unroll
-      for (int q = 0; q < BK; ++q) {
-        double a[4], b[JR];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[q][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < JR; ++j) b[j] = Bs[q][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < JR; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-      }
+      if (live) fma_slice(As, Bs, acc, min(BK, nKp - k0), jn, tx, ty);
       __syncthreads();
     }
   }
+  const int64_t s = s0 + ty;
+  if (s >= Ns) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t s = s0 + ty + 16 * i;
-    if (s >= Ns) continue;
-#pragma unroll
-    for (int j = 0; j < JR; ++j) {
-      const int jj = j0 + tx + 16 * j;
-      if (jj >= nK) continue;
-      const int64_t idx = s * ldo + offK + jj;
-      double r = alpha * (acc[i][j] - c * in[s * ld + offK + jj]);
-      if (beta != 0.0) r -= beta * prev[idx];
-      out[idx] = r;
-    }
+  for (int j = 0; j < 8; ++j) {
+    const int jj = j0 + tx + 8 * j;
+    if (jj >= nK) continue;
+    const int64_t idx = s * ldo + offK + jj;
+    double r = alpha * (acc[j] - c * in[s * ld + offK + jj]);
+    if (beta != 0.0) r -= beta * prev[idx];
+    out[idx] = r;
   }
 }
 
@@ -184,49 +160,68 @@ __global__ void k_axpby_f64(double a, const double* __restrict__ x, double b, co
     yo[i] = a * x[i] + b * y[i];
 }
 
-// C[i,j] = sum_r A[i,r] B[j,r]
+// C[i,j] = sum_r A[i,r] B[j,r]; lower_only: the entries j <= i, mirrored. With
+// gridDim.z > 1 each part sums kc terms and writes its partial result to
+// C + z * rows * cols (k_sum_parts_f64 adds them in order): a product of few
+// tiles and many terms (a Gram matrix of a few hundred states) fills the GPU.
 __global__ void __launch_bounds__(NT) k_gemm_nt_f64(const double* __restrict__ A, int64_t lda,
                                                     const double* __restrict__ B, int64_t ldb, double* C,
-                                                    int64_t ldc, int64_t rows, int64_t cols, int64_t K,
+                                                    int64_t ldc, int64_t rows, int64_t cols, int64_t K, int64_t kc,
                                                     int lower_only) {
-  if (lower_only && blockIdx.x > blockIdx.y) return;
-  const int64_t i0 = (int64_t)blockIdx.y * T, j0 = (int64_t)blockIdx.x * T;
-  __shared__ double As[BK][TP];
+  const int64_t nrt = (rows + TR - 1) / TR;
+  const int64_t i0 = (blockIdx.x % nrt) * TR, j0 = (blockIdx.x / nrt) * T;
+  if (lower_only && j0 > i0 + TR - 1) return;
+  __shared__ double As[BK][TRP];
   __shared__ double Bs[BK][TP];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int jn = groups8((lower_only && i0 + TR < cols ? i0 + TR : cols) - j0);
+  const bool live = i0 + (ty & ~3) < rows;
+  double acc[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int j = 0; j < 8; ++j) acc[j] = 0.0;
+  const int kk = tid & 15, rr = tid >> 4;
+  const int64_t kb = (int64_t)blockIdx.z * kc, ke = kb + kc < K ? kb + kc : K;
+  for (int64_t k0 = kb; k0 < ke; k0 += BK) {
+    const bool kin = (k0 + kk) < ke;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int64_t k0 = 0; k0 < K; k0 += BK) {
-    const int kk = tid & 15;
-    const bool kin = (k0 + kk) < K;
+    for (int i = 0; i < 2; ++i) {
+      const int r = rr + 8 * i;
+      As[kk][r] = (kin && i0 + r < rows) ? A[(i0 + r) * lda + k0 + kk] : 0.0;
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = (tid >> 4) + 16 * i;
-      double v = 0.0, w = 0.0;
-      if (kin && i0 + r < rows) v = A[(i0 + r) * lda + k0 + kk];
-      if (kin && j0 + r < cols) w = B[(j0 + r) * ldb + k0 + kk];
-      As[kk][r] = v;
-      Bs[kk][r] = w;
+    for (int i = 0; i < 8; ++i) {
+      const int r = rr + 8 * i;
+      if (i < jn) Bs[kk][r] = (kin && j0 + r < cols) ? B[(j0 + r) * ldb + k0 + kk] : 0.0;
     }
     __syncthreads();
-    fma_tile(As, Bs, acc, tx, ty);
+    if (live) fma_slice(As, Bs, acc, (int)(ke - k0 < BK ? ke - k0 : BK), jn, tx, ty);
     __syncthreads();
   }
-  const bool mirror = lower_only && blockIdx.x < blockIdx.y;
+  const int64_t ii = i0 + ty;
+  if (ii >= rows) return;
+  const bool part = gridDim.z > 1;
+  double* c = C + (part ? (int64_t)blockIdx.z * rows * cols : 0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t ii = i0 + ty + 16 * i;
-    if (ii >= rows) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t jj = j0 + tx + 16 * j;
-      if (jj >= cols) continue;
-      C[ii * ldc + jj] = acc[i][j];
-      if (mirror) C[jj * ldc + ii] = acc[i][j];
-    }
+  for (int j = 0; j < 8; ++j) {
+    const int64_t jj = j0 + tx + 8 * j;
+    if (jj >= cols || (lower_only && jj > ii)) continue;
+    c[ii * (part ? cols : ldc) + jj] = acc[j];
+    if (lower_only && !part) c[jj * ldc + ii] = acc[j];
+  }
+}
+
+// C[i,j] = sum_z P[z][i,j], z ascending (P: parts x rows x cols); lower_only:
+// the entries j <= i, mirrored.
+__global__ void k_sum_parts_f64(const double* __restrict__ P, int parts, int64_t rows, int64_t cols,
+                                double* __restrict__ C, int64_t ldc, int lower_only) {
+  const int64_t tot = rows * cols;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = e / cols, j = e - i * cols;
+    if (lower_only && j > i) continue;
+    double sum = P[e];
+    for (int z = 1; z < parts; ++z) sum += P[(int64_t)z * tot + e];
+    C[i * ldc + j] = sum;
+    if (lower_only) C[j * ldc + i] = sum;
   }
 }
 
@@ -244,80 +239,87 @@ __global__ void __launch_bounds__(NT) k_gemm_nn_f64(const double* __restrict__ A
                                                     const double* __restrict__ B, int64_t ldb,
                                                     double* __restrict__ C, int64_t ldc, int64_t rows,
                                                     int64_t cols, int64_t K, int a_lower) {
-  const int64_t i0 = (int64_t)blockIdx.y * T, r0 = (int64_t)blockIdx.x * T;
-  __shared__ double As[BK][TP];
+  const int64_t nrt = (rows + TR - 1) / TR;
+  const int64_t i0 = (blockIdx.x % nrt) * TR, r0 = (blockIdx.x / nrt) * T;
+  __shared__ double As[BK][TRP];
   __shared__ double Bs[BK][TP];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int jn = groups8(cols - r0);
+  const bool live = i0 + (ty & ~3) < rows;
+  double acc[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  const int64_t kend = a_lower ? (K < i0 + T ? K : i0 + T) : K;
+  for (int j = 0; j < 8; ++j) acc[j] = 0.0;
+  const int kk = tid & 15, rr = tid >> 4, cc = tid & 63;
+  const int64_t kend = a_lower && i0 + TR < K ? i0 + TR : K;
   for (int64_t k0 = 0; k0 < kend; k0 += BK) {
-    {
-      const int kk = tid & 15;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = (tid >> 4) + 16 * i;
-        const int64_t l = k0 + kk, row = i0 + r;
-        double v = 0.0;
-        if (l < K && row < rows && (!a_lower || l <= row)) v = A[row * lda + l];
-        As[kk][r] = v;
-      }
+    for (int i = 0; i < 2; ++i) {
+      const int r = rr + 8 * i;
+      const int64_t l = k0 + kk, row = i0 + r;
+      As[kk][r] = (l < K && row < rows && (!a_lower || l <= row)) ? A[row * lda + l] : 0.0;
     }
-    {
-      const int cc = tid & 63;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int kk = (tid >> 6) + 4 * i;
-        const int64_t l = k0 + kk;
-        double w = 0.0;
-        if (l < K && r0 + cc < cols) w = B[l * ldb + r0 + cc];
-        Bs[kk][cc] = w;
-      }
+    for (int i = 0; i < 8; ++i) {
+      const int kq = (tid >> 6) + 2 * i;
+      const int64_t l = k0 + kq;
+      Bs[kq][cc] = (l < K && r0 + cc < cols) ? B[l * ldb + r0 + cc] : 0.0;
     }
     __syncthreads();
-    fma_tile(As, Bs, acc, tx, ty);
+    if (live) fma_slice(As, Bs, acc, (int)(kend - k0 < BK ? kend - k0 : BK), jn, tx, ty);
     __syncthreads();
   }
+  const int64_t ii = i0 + ty;
+  if (ii >= rows) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t ii = i0 + ty + 16 * i;
-    if (ii >= rows) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t rr = r0 + tx + 16 * j;
-      if (rr < cols) C[ii * ldc + rr] = acc[i][j];
-    }
+  for (int j = 0; j < 8; ++j) {
+    const int64_t q = r0 + tx + 8 * j;
+    if (q < cols) C[ii * ldc + q] = acc[j];
   }
 }
 
-// P_K[j, j'] = sum_i f_i X[i, off_K + j] X[i, off_K + j']
+// P_K[j, j'] = sum_i f_i X[i, off_K + j] X[i, off_K + j'] for j' <= j, mirrored
+// (P_K is symmetric: half the multiply-adds). blockIdx.y: pair of 64-wide
+// chunks of the element, chunk of j >= chunk of j'. With gridDim.z > 1 each
+// part sums `sc` states into part + z * total (laid out like P) and
+// k_density_sum_f64 adds them in order, so that few elements still fill the
+// GPU and many fill it evenly.
 __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __restrict__ poff,
                                                     const double* __restrict__ X, int64_t Ns, int64_t ld,
-                                                    const double* __restrict__ f, double* __restrict__ P) {
+                                                    const double* __restrict__ f, int64_t sc, double* __restrict__ P) {
   const int K = blockIdx.x;
   const int nK = h.nb[K];
-  const int j0 = blockIdx.y * T, jp0 = blockIdx.z * T;
-  if (j0 >= nK || jp0 >= nK) return;
+  int ca = 0, cb = blockIdx.y;  // chunks of j and j': row ca of the lower triangle of chunk pairs
+  while (cb > ca) cb -= ++ca;
+  const int j0 = ca * T, jp0 = cb * T;
+  if (j0 >= nK) return;
   const int64_t offK = h.off[K];
   __shared__ double As[BK][TP];
   __shared__ double Bs[BK][TP];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  int lim[4], row[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    // the warps take the four-row groups of a 16-row band forwards and backwards
+    // in turn: below the diagonal later rows are longer, and each warp has its
+    // own part of the FP64 pipe
+    const int r4 = 16 * i + ((i & 1) ? 12 - (ty & ~3) : (ty & ~3));
+    row[i] = r4 + (ty & 3);
+    lim[i] = j0 + r4 < nK ? groups8(min(nK, j0 + r4 + 4) - jp0) : 0;
+  }
+  double acc[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
   const int cc = tid & 63;
-  for (int64_t i0 = 0; i0 < Ns; i0 += BK) {
+  const int64_t sb = (int64_t)blockIdx.z * sc, se = sb + sc < Ns ? sb + sc : Ns;
+  for (int64_t i0 = sb; i0 < se; i0 += BK) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int kk = (tid >> 6) + 4 * i;
+    for (int i = 0; i < 8; ++i) {
+      const int kk = (tid >> 6) + 2 * i;
       const int64_t s = i0 + kk;
       double v = 0.0, w = 0.0;
-      if (s < Ns) {
+      if (s < se) {
         const double* xr = X + s * ld + offK;
         if (j0 + cc < nK) v = f[s] * xr[j0 + cc];
         if (jp0 + cc < nK) w = xr[jp0 + cc];
@@ -326,19 +328,40 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
       Bs[kk][cc] = w;
     }
     __syncthreads();
-    fma_tile(As, Bs, acc, tx, ty);
+    fma_outer(As, Bs, acc, (int)(se - i0 < BK ? se - i0 : BK), lim, tx, row);
     __syncthreads();
   }
-  double* PK = P + poff[K];
+  const bool part = gridDim.z > 1;
+  double* PK = P + poff[K] + (part ? (int64_t)blockIdx.z * poff[h.M] : 0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int jj = j0 + ty + 16 * i;
+    const int jj = j0 + row[i];
     if (jj >= nK) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int jq = jp0 + tx + 16 * j;
-      if (jq < nK) PK[(int64_t)jj * nK + jq] = acc[i][j];
+    for (int j = 0; j < 8; ++j) {
+      const int jq = jp0 + tx + 8 * j;
+      if (jq > jj) continue;
+      PK[(int64_t)jj * nK + jq] = acc[i][j];
+      if (!part) PK[(int64_t)jq * nK + jj] = acc[i][j];
     }
+  }
+}
+
+// P = the sum of the parts, z ascending, lower triangles mirrored. One CTA per element.
+__global__ void k_density_sum_f64(HView h, const int64_t* __restrict__ poff, const double* __restrict__ part,
+                                  int parts, double* __restrict__ P) {
+  const int K = blockIdx.x;
+  const int nK = h.nb[K];
+  const int64_t total = poff[h.M];
+  const double* p = part + poff[K];
+  double* PK = P + poff[K];
+  for (int e = threadIdx.x; e < nK * nK; e += blockDim.x) {
+    const int j = e / nK, q = e - j * nK;
+    if (q > j) continue;
+    double sum = p[e];
+    for (int z = 1; z < parts; ++z) sum += p[(int64_t)z * total + e];
+    PK[e] = sum;
+    PK[(int64_t)q * nK + j] = sum;
   }
 }
 
@@ -430,17 +453,23 @@ __global__ void __launch_bounds__(NT) k_block_outer_f64(HView h, const int32_t* 
   const int64_t offK = h.off[K], offKp = h.off[Kp];
   __shared__ double As[BK][TP];
   __shared__ double Bs[BK][TP];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  int lim[4], row[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    row[i] = ty + 16 * i;
+    lim[i] = j0 + 16 * i + (ty & ~3) < nK ? groups8(nKp - jp0) : 0;
+  }
+  double acc[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
   const int cc = tid & 63;
   for (int64_t i0 = 0; i0 < Ns; i0 += BK) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int kk = (tid >> 6) + 4 * i;
+    for (int i = 0; i < 8; ++i) {
+      const int kk = (tid >> 6) + 2 * i;
       const int64_t s = i0 + kk;
       double v = 0.0, u = 0.0;
       if (s < Ns) {
@@ -451,17 +480,17 @@ __global__ void __launch_bounds__(NT) k_block_outer_f64(HView h, const int32_t* 
       Bs[kk][cc] = u;
     }
     __syncthreads();
-    fma_tile(As, Bs, acc, tx, ty);
+    fma_outer(As, Bs, acc, (int)(Ns - i0 < BK ? Ns - i0 : BK), lim, tx, row);
     __syncthreads();
   }
   double* Ge = G + h.blk_off[e];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int jj = j0 + ty + 16 * i;
+    const int jj = j0 + row[i];
     if (jj >= nK) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int jq = jp0 + tx + 16 * j;
+    for (int j = 0; j < 8; ++j) {
+      const int jq = jp0 + tx + 8 * j;
       if (jq < nKp) Ge[(int64_t)jj * nKp + jq] += alpha * acc[i][j];
     }
   }
@@ -472,42 +501,39 @@ __global__ void __launch_bounds__(NT) k_gemm_tn_f64(const double* __restrict__ A
                                                     const double* __restrict__ B, int64_t ldb,
                                                     double* __restrict__ C, int64_t ldc, int64_t rows,
                                                     int64_t cols, int64_t K) {
-  const int64_t i0 = (int64_t)blockIdx.y * T, r0 = (int64_t)blockIdx.x * T;
-  __shared__ double As[BK][TP];
+  const int64_t nrt = (rows + TR - 1) / TR;
+  const int64_t i0 = (blockIdx.x % nrt) * TR, r0 = (blockIdx.x / nrt) * T;
+  __shared__ double As[BK][TRP];
   __shared__ double Bs[BK][TP];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int jn = groups8(cols - r0);
+  const bool live = i0 + (ty & ~3) < rows;
+  double acc[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  const int cc = tid & 63;
+  for (int j = 0; j < 8; ++j) acc[j] = 0.0;
+  const int ar = tid & 15, ak = tid >> 4, cc = tid & 63;
   for (int64_t k0 = 0; k0 < K; k0 += BK) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int kk = (tid >> 6) + 4 * i;
-      const int64_t l = k0 + kk;
-      double v = 0.0, u = 0.0;
-      if (l < K) {
-        if (i0 + cc < rows) v = A[l * lda + i0 + cc];
-        if (r0 + cc < cols) u = B[l * ldb + r0 + cc];
-      }
-      As[kk][cc] = v;
-      Bs[kk][cc] = u;
+    for (int i = 0; i < 2; ++i) {
+      const int64_t l = k0 + ak + 8 * i;
+      As[ak + 8 * i][ar] = (l < K && i0 + ar < rows) ? A[l * lda + i0 + ar] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int kq = (tid >> 6) + 2 * i;
+      const int64_t l = k0 + kq;
+      Bs[kq][cc] = (l < K && r0 + cc < cols) ? B[l * ldb + r0 + cc] : 0.0;
     }
     __syncthreads();
-    fma_tile(As, Bs, acc, tx, ty);
+    if (live) fma_slice(As, Bs, acc, (int)(K - k0 < BK ? K - k0 : BK), jn, tx, ty);
     __syncthreads();
   }
+  const int64_t ii = i0 + ty;
+  if (ii >= rows) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t ii = i0 + ty + 16 * i;
-    if (ii >= rows) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t rr = r0 + tx + 16 * j;
-      if (rr < cols) C[ii * ldc + rr] = acc[i][j];
-    }
+  for (int j = 0; j < 8; ++j) {
+    const int64_t q = r0 + tx + 8 * j;
+    if (q < cols) C[ii * ldc + q] = acc[j];
   }
 }
 
@@ -534,12 +560,8 @@ inline unsigned stream_grid(int64_t n) {
 cudaError_t filter_step_f64(const HView& h, const double* in, int64_t ld_in, const double* prev, double* out,
                             int64_t ld_out, int64_t Ns, double alpha, double c, double beta, cudaStream_t s) {
   if (Ns == 0) return cudaSuccess;
-  if (h.tj == 64)
-    k_filter_step_f64<64><<<dim3(cdiv(Ns, T), (unsigned)h.M, cdiv(h.max_nb, 64)), NT, 0, s>>>(
-        h, in, ld_in, prev, out, ld_out, Ns, alpha, c, beta, nullptr, 0);
-  else
-    k_filter_step_f64<32><<<dim3(cdiv(Ns, T), (unsigned)h.M, cdiv(h.max_nb, 32)), NT, 0, s>>>(
-        h, in, ld_in, prev, out, ld_out, Ns, alpha, c, beta, nullptr, 0);
+  k_filter_step_f64<<<dim3(cdiv(Ns, TR), (unsigned)h.M, cdiv(h.max_nb, T)), NT, 0, s>>>(
+      h, in, ld_in, prev, out, ld_out, Ns, alpha, c, beta, nullptr, 0);
   count_launch();
   return cudaGetLastError();
 }
@@ -547,12 +569,8 @@ cudaError_t filter_step_f64(const HView& h, const double* in, int64_t ld_in, con
 cudaError_t filter_step_f64_dev(const HView& h, const double* in, int64_t ld_in, const double* prev, double* out,
                                 int64_t ld_out, int64_t Ns, const double* coef, int step, cudaStream_t s) {
   if (Ns <= 0) return cudaSuccess;
-  if (h.tj == 64)
-    k_filter_step_f64<64><<<dim3(cdiv(Ns, T), (unsigned)h.M, cdiv(h.max_nb, 64)), NT, 0, s>>>(
-        h, in, ld_in, prev, out, ld_out, Ns, 0.0, 0.0, 0.0, coef, step);
-  else
-    k_filter_step_f64<32><<<dim3(cdiv(Ns, T), (unsigned)h.M, cdiv(h.max_nb, 32)), NT, 0, s>>>(
-        h, in, ld_in, prev, out, ld_out, Ns, 0.0, 0.0, 0.0, coef, step);
+  k_filter_step_f64<<<dim3(cdiv(Ns, TR), (unsigned)h.M, cdiv(h.max_nb, T)), NT, 0, s>>>(
+      h, in, ld_in, prev, out, ld_out, Ns, 0.0, 0.0, 0.0, coef, step);
   count_launch();
   return cudaGetLastError();
 }
@@ -621,12 +639,28 @@ cudaError_t axpby_f64(double a, const double* x, double b, const double* y, doub
   return cudaGetLastError();
 }
 
+// CTAs at which a product no longer gains from more parts: 16 per SM, so that an
+// uneven last round, or tiles of uneven work, cost a few percent.
+static constexpr int64_t kFillCtas = 16 * 152;
+
 cudaError_t gemm_nt_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
-                        int64_t rows, int64_t cols, int64_t K, bool lower_only, bool symmetrise, cudaStream_t s) {
+                        int64_t rows, int64_t cols, int64_t K, bool lower_only, bool symmetrise, const Parts& parts,
+                        cudaStream_t s) {
   if (rows == 0 || cols == 0) return cudaSuccess;
-  dim3 grid(cdiv(cols, T), cdiv(rows, T));
-  k_gemm_nt_f64<<<grid, NT, 0, s>>>(A, lda, B, ldb, C, ldc, rows, cols, K, lower_only ? 1 : 0);
+  const int64_t tiles = (int64_t)cdiv(rows, TR) * cdiv(cols, T);
+  const int64_t work = lower_only ? (tiles + 1) / 2 : tiles;
+  // parts of at least 64 terms, as many as fill the GPU and the buffer holds
+  int64_t np = std::min((kFillCtas + work - 1) / work, std::min(K / 64, parts.doubles / std::max<int64_t>(rows * cols, 1)));
+  np = std::max<int64_t>(1, std::min<int64_t>(np, 65535));
+  const int64_t kc = std::max<int64_t>(BK, ((K + np - 1) / np + BK - 1) / BK * BK);
+  np = std::max<int64_t>(1, (K + kc - 1) / kc);
+  k_gemm_nt_f64<<<dim3((unsigned)tiles, 1, (unsigned)np), NT, 0, s>>>(A, lda, B, ldb, np > 1 ? parts.p : C, ldc, rows,
+                                                                     cols, K, kc, lower_only ? 1 : 0);
   count_launch();
+  if (np > 1) {
+    k_sum_parts_f64<<<stream_grid(rows * cols), 256, 0, s>>>(parts.p, (int)np, rows, cols, C, ldc, lower_only ? 1 : 0);
+    count_launch();
+  }
   if (symmetrise && rows == cols) {
     dim3 b2(32, 8), g2(cdiv(rows, 32), cdiv(rows, 8));
     k_symmetrise_f64<<<g2, b2, 0, s>>>(C, rows, ldc);
@@ -638,17 +672,27 @@ cudaError_t gemm_nt_f64(const double* A, int64_t lda, const double* B, int64_t l
 cudaError_t gemm_nn_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                         int64_t rows, int64_t cols, int64_t K, bool a_lower, cudaStream_t s) {
   if (rows == 0 || cols == 0) return cudaSuccess;
-  dim3 grid(cdiv(cols, T), cdiv(rows, T));
-  k_gemm_nn_f64<<<grid, NT, 0, s>>>(A, lda, B, ldb, C, ldc, rows, cols, K, a_lower ? 1 : 0);
+  const int64_t tiles = (int64_t)cdiv(rows, TR) * cdiv(cols, T);
+  k_gemm_nn_f64<<<(unsigned)tiles, NT, 0, s>>>(A, lda, B, ldb, C, ldc, rows, cols, K, a_lower ? 1 : 0);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t density_f64(const HView& h, const int64_t* poff, const double* X, int64_t Ns, int64_t ld,
-                        const double* f, double* P, cudaStream_t s) {
-  dim3 grid((unsigned)h.M, cdiv(h.max_nb, T), cdiv(h.max_nb, T));
-  k_density_f64<<<grid, NT, 0, s>>>(h, poff, X, Ns, ld, f, P);
+cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const double* X, int64_t Ns, int64_t ld,
+                        const double* f, double* P, const Parts& parts, cudaStream_t s) {
+  const int64_t chunks = cdiv(h.max_nb, T), pairs = chunks * (chunks + 1) / 2;
+  // parts of at least 64 states, as many as fill the GPU and the buffer holds
+  int64_t np = std::min((kFillCtas + h.M * pairs - 1) / (h.M * pairs), std::min(Ns / 64, parts.doubles / total));
+  np = std::max<int64_t>(1, std::min<int64_t>(np, 65535));
+  const int64_t sc = std::max<int64_t>(BK, ((Ns + np - 1) / np + BK - 1) / BK * BK);
+  np = std::max<int64_t>(1, (Ns + sc - 1) / sc);
+  k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)np), NT, 0, s>>>(h, poff, X, Ns, ld, f, sc,
+                                                                                 np > 1 ? parts.p : P);
   count_launch();
+  if (np > 1) {
+    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, parts.p, (int)np, P);
+    count_launch();
+  }
   return cudaGetLastError();
 }
 
@@ -686,8 +730,8 @@ cudaError_t block_outer_f64(const HView& h, const int32_t* blk_row, int64_t nnzb
 cudaError_t gemm_tn_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                         int64_t rows, int64_t cols, int64_t K, cudaStream_t s) {
   if (rows == 0 || cols == 0) return cudaSuccess;
-  dim3 grid(cdiv(cols, T), cdiv(rows, T));
-  k_gemm_tn_f64<<<grid, NT, 0, s>>>(A, lda, B, ldb, C, ldc, rows, cols, K);
+  const int64_t tiles = (int64_t)cdiv(rows, TR) * cdiv(cols, T);
+  k_gemm_tn_f64<<<(unsigned)tiles, NT, 0, s>>>(A, lda, B, ldb, C, ldc, rows, cols, K);
   count_launch();
   return cudaGetLastError();
 }

@@ -16,7 +16,13 @@ struct HView {
   const int64_t* blk_off;  // [nnzb] offsets into vals (doubles)
   const double* vals;
   int32_t max_nb;
-  int32_t tj = 64;  // FP64 filter: output columns per tile (64 if every n_K is a multiple of 64, else 32)
+};
+
+// Device buffer for the partial results of a product split along its
+// contraction (doubles = 0: not split).
+struct Parts {
+  double* p = nullptr;
+  int64_t doubles = 0;
 };
 
 void count_launch(int n = 1);
@@ -53,19 +59,20 @@ cudaError_t sub_combination_f64(double* w, const double* V, int64_t ldv, const d
 cudaError_t axpby_f64(double a, const double* x, double b, const double* y, double* y_out, int64_t n, cudaStream_t s);
 
 // C[i,j] = sum_r A[i,r] B[j,r]  (A: rows x K, B: cols x K, row-major, K contiguous).
-// lower_only: compute tiles with i-tile >= j-tile and mirror to the upper triangle
-// (for a symmetric result, A == B).  symmetrise: C <- (C + C^T)/2 afterwards.
+// lower_only: compute the entries j <= i and mirror them to the upper triangle
+// (for a symmetric result).  symmetrise: C <- (C + C^T)/2 afterwards.
 cudaError_t gemm_nt_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
-                        int64_t rows, int64_t cols, int64_t K, bool lower_only, bool symmetrise, cudaStream_t s);
+                        int64_t rows, int64_t cols, int64_t K, bool lower_only, bool symmetrise, const Parts& parts,
+                        cudaStream_t s);
 
 // C[i,r] = sum_l A[i,l] B[l,r]  (A: rows x K row-major, B: K x cols row-major).
 // a_lower: A is lower triangular (entries l > i are treated as zero, not read).
 cudaError_t gemm_nn_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                         int64_t rows, int64_t cols, int64_t K, bool a_lower, cudaStream_t s);
 
-// P_K = sum_i f_i X[i, off_K:] X[i, off_K:]^T packed at poff[K].
-cudaError_t density_f64(const HView& h, const int64_t* poff, const double* X, int64_t Ns, int64_t ld,
-                        const double* f, double* P, cudaStream_t s);
+// P_K = sum_i f_i X[i, off_K:] X[i, off_K:]^T packed at poff[K], `total` doubles in all.
+cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const double* X, int64_t Ns, int64_t ld,
+                        const double* f, double* P, const Parts& parts, cudaStream_t s);
 
 // Fermi level by bisection and occupations (one CTA).
 cudaError_t occupations_f64(const double* ritz, int64_t Ns, double Ne, double kT, double* f, double* mu,

@@ -12,105 +12,108 @@
 #include <vector>
 
 #include "ctx.h"
+#include "f64_tile.cuh"
 
 namespace dg {
 namespace {
 
+using namespace f64tile;
+
+constexpr int SG = 64;  // states per CTA of k_realign_f64
+
 // T_K = Vn_K^T Vo_K for every element; Vn_K (R x p), Vo_K (R x q) row-major.
-__global__ void __launch_bounds__(256) k_overlap_f64(const int32_t* __restrict__ nb_new, const int32_t* __restrict__ nb_old,
-                                                     const int32_t* __restrict__ nr, const int64_t* __restrict__ vn_off,
-                                                     const int64_t* __restrict__ vo_off, const int64_t* __restrict__ t_off,
-                                                     const double* __restrict__ Vn, const double* __restrict__ Vo,
-                                                     double* __restrict__ T) {
-  constexpr int TB = 32, RB = 32;
+// 16 new x 64 old basis functions per CTA.
+__global__ void __launch_bounds__(NT) k_overlap_f64(const int32_t* __restrict__ nb_new, const int32_t* __restrict__ nb_old,
+                                                    const int32_t* __restrict__ nr, const int64_t* __restrict__ vn_off,
+                                                    const int64_t* __restrict__ vo_off, const int64_t* __restrict__ t_off,
+                                                    const double* __restrict__ Vn, const double* __restrict__ Vo,
+                                                    double* __restrict__ Tk) {
   const int K = blockIdx.x;
   const int p = nb_new[K], q = nb_old[K], R = nr[K];
-  const int j0 = blockIdx.y * TB, i0 = blockIdx.z * TB;
+  const int j0 = blockIdx.y * TR, i0 = blockIdx.z * T;
   if (j0 >= p || i0 >= q) return;
-  __shared__ double As[RB][TB + 1];
-  __shared__ double Bs[RB][TB + 1];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
+  __shared__ double As[BK][TRP];
+  __shared__ double Bs[BK][TP];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int jn = groups8(q - i0);
+  const bool live = j0 + (ty & ~3) < p;
   const double* vn = Vn + vn_off[K];
   const double* vo = Vo + vo_off[K];
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int r0 = 0; r0 < R; r0 += RB) {
-    for (int rr = ty; rr < RB; rr += 8) {
-      const int r = r0 + rr;
-      As[rr][tx] = (r < R && j0 + tx < p) ? vn[(int64_t)r * p + j0 + tx] : 0.0;
-      Bs[rr][tx] = (r < R && i0 + tx < q) ? vo[(int64_t)r * q + i0 + tx] : 0.0;
+  double acc[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) acc[j] = 0.0;
+  const int ar = tid & 15, ak = tid >> 4, cc = tid & 63;
+  for (int r0 = 0; r0 < R; r0 += BK) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = r0 + ak + 8 * i;
+      As[ak + 8 * i][ar] = (r < R && j0 + ar < p) ? vn[(int64_t)r * p + j0 + ar] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int kq = (tid >> 6) + 2 * i, r = r0 + kq;
+      Bs[kq][cc] = (r < R && i0 + cc < q) ? vo[(int64_t)r * q + i0 + cc] : 0.0;
     }
     __syncthreads();
-#pragma unroll 8
-    for (int rr = 0; rr < RB; ++rr) {
-      const double b = Bs[rr][tx];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] = fma(As[rr][ty + 8 * i], b, acc[i]);
-    }
+    if (live) fma_slice(As, Bs, acc, min(BK, R - r0), jn, tx, ty);
     __syncthreads();
   }
-  double* t = T + t_off[K];
+  double* t = Tk + t_off[K];
+  const int jj = j0 + ty;
+  if (jj >= p) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int jj = j0 + ty + 8 * i;
-    if (jj < p && i0 + tx < q) t[(int64_t)jj * q + i0 + tx] = acc[i];
+  for (int j = 0; j < 8; ++j) {
+    const int i = i0 + tx + 8 * j;
+    if (i < q) t[(int64_t)jj * q + i] = acc[j];
   }
 }
 
-// Y[s, on_K + j'] = sum_j X[s, oo_K + j] T_K[j', j]; 64 states x 64 new columns per CTA.
-__global__ void __launch_bounds__(256) k_realign_f64(const int32_t* __restrict__ nb_new, const int32_t* __restrict__ nb_old,
-                                                     const int64_t* __restrict__ off_new, const int64_t* __restrict__ off_old,
-                                                     const int64_t* __restrict__ t_off, const double* __restrict__ T,
-                                                     const double* __restrict__ X, int64_t ldx, double* __restrict__ Y,
-                                                     int64_t ldy, int64_t Ns) {
-  constexpr int TS = 64, TJ = 64, KB = 16;
+// Y[s, on_K + j'] = sum_j X[s, oo_K + j] T_K[j', j]; 16 states x 64 new columns per CTA.
+__global__ void __launch_bounds__(NT) k_realign_f64(const int32_t* __restrict__ nb_new, const int32_t* __restrict__ nb_old,
+                                                    const int64_t* __restrict__ off_new, const int64_t* __restrict__ off_old,
+                                                    const int64_t* __restrict__ t_off, const double* __restrict__ Tk,
+                                                    const double* __restrict__ X, int64_t ldx, double* __restrict__ Y,
+                                                    int64_t ldy, int64_t Ns) {
   const int K = blockIdx.x;
   const int p = nb_new[K], q = nb_old[K];
-  const int64_t s0 = (int64_t)blockIdx.y * TS;
-  const int jp0 = blockIdx.z * TJ;
+  const int64_t s0 = (int64_t)blockIdx.y * SG;  // SG states per CTA, TR at a time
+  const int jp0 = blockIdx.z * T;
   if (s0 >= Ns || jp0 >= p) return;
-  __shared__ double Xs[TS][KB + 1];
-  __shared__ double Ts[KB][TJ + 1];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const double* t = T + t_off[K];
+  __shared__ double As[BK][TRP];
+  __shared__ double Bs[BK][TP];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int jn = groups8(p - jp0);
+  const double* t = Tk + t_off[K];
   const int64_t oo = off_old[K], on = off_new[K];
-  double acc[4][4];
+  const int kk = tid & 15, rr = tid >> 4;
+  for (int64_t sb = s0; sb < Ns && sb < s0 + SG; sb += TR) {
+    const bool live = sb + (ty & ~3) < Ns;
+    double acc[8];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int j = 0; j < 8; ++j) acc[j] = 0.0;
+    for (int k0 = 0; k0 < q; k0 += BK) {
+      const bool kin = k0 + kk < q;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  for (int j0 = 0; j0 < q; j0 += KB) {
+      for (int i = 0; i < 2; ++i) {
+        const int r = rr + 8 * i;
+        As[kk][r] = (kin && sb + r < Ns) ? X[(sb + r) * ldx + oo + k0 + kk] : 0.0;
+      }
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const int e = tid + 256 * l;  // 1024 entries of each tile
-      const int xr = e >> 4, xc = e & 15;
-      const int64_t s = s0 + xr;
-      Xs[xr][xc] = (s < Ns && j0 + xc < q) ? X[s * ldx + oo + j0 + xc] : 0.0;
-      const int tr = e >> 6, tc = e & 63;  // Ts[j][j'] = T[j'][j]
-      Ts[tr][tc] = (j0 + tr < q && jp0 + tc < p) ? t[(int64_t)(jp0 + tc) * q + j0 + tr] : 0.0;
+      for (int i = 0; i < 8; ++i) {
+        const int r = rr + 8 * i;
+        if (i < jn) Bs[kk][r] = (kin && jp0 + r < p) ? t[(int64_t)(jp0 + r) * q + k0 + kk] : 0.0;
+      }
+      __syncthreads();
+      if (live) fma_slice(As, Bs, acc, min(BK, q - k0), jn, tx, ty);
+      __syncthreads();
     }
-    __syncthreads();
+    const int64_t s = sb + ty;
+    if (s < Ns) {
 #pragma unroll
-    for (int kk = 0; kk < KB; ++kk) {
-      double xa[4], tb[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) xa[a] = Xs[ty + 16 * a][kk];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) tb[b] = Ts[kk][tx + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(xa[a], tb[b], acc[a][b]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int64_t s = s0 + ty + 16 * a;
-    if (s >= Ns) continue;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int jp = jp0 + tx + 16 * b;
-      if (jp < p) Y[s * ldy + on + jp] = acc[a][b];
+      for (int j = 0; j < 8; ++j) {
+        const int jp = jp0 + tx + 8 * j;
+        if (jp < p) Y[s * ldy + on + jp] = acc[j];
+      }
     }
   }
 }
@@ -173,15 +176,15 @@ extern "C" dgchefsi_status dgchefsi_realign(dgchefsi_ctx* ctx, const int32_t* nb
   const int64_t* d_to = d_vn + (M + 1);
   const int32_t* d_nb_old = reinterpret_cast<const int32_t*>(d_to + (M + 1));
   const int32_t* d_nr = d_nb_old + M;
-  double* T = reinterpret_cast<double*>(dbase + tab_al);
-  const unsigned tp = (unsigned)((ctx->max_nb + 31) / 32), tq = (unsigned)((max_old + 31) / 32);
-  k_overlap_f64<<<dim3((unsigned)M, tp, tq), 256, 0, s>>>(ctx->nb_d, d_nb_old, d_nr, d_vn, d_vo, d_to, V_new, V_old, T);
+  double* Tk = reinterpret_cast<double*>(dbase + tab_al);
+  const unsigned tp = (unsigned)((ctx->max_nb + TR - 1) / TR), tq = (unsigned)((max_old + T - 1) / T);
+  k_overlap_f64<<<dim3((unsigned)M, tp, tq), NT, 0, s>>>(ctx->nb_d, d_nb_old, d_nr, d_vn, d_vo, d_to, V_new, V_old, Tk);
   count_launch();
   DG_CUDA(cudaGetLastError());
-  const int64_t st = (Ns + 63) / 64;
+  const int64_t st = (Ns + SG - 1) / SG;
   if (st > 65535) return set_error(DGCHEFSI_ERR_UNSUPPORTED, "Ns too large for one launch");
-  k_realign_f64<<<dim3((unsigned)M, (unsigned)st, (unsigned)((ctx->max_nb + 63) / 64)), 256, 0, s>>>(
-      ctx->nb_d, d_nb_old, ctx->off_d, d_off_old, d_to, T, X_old, ld_old, X_new, ld, Ns);
+  k_realign_f64<<<dim3((unsigned)M, (unsigned)st, (unsigned)((ctx->max_nb + T - 1) / T)), NT, 0, s>>>(
+      ctx->nb_d, d_nb_old, ctx->off_d, d_off_old, d_to, Tk, X_old, ld_old, X_new, ld, Ns);
   count_launch();
   DG_CUDA(cudaGetLastError());
   // the host table must outlive the asynchronous copy from pageable memory
