@@ -184,21 +184,32 @@ dgchefsi_status sliced_gemm_tn(dgchefsi_ctx* ctx, int64_t M, int64_t Nc, int64_t
                                const double* B, int64_t ldb, double* C, int64_t ldc, int s, int* flag);
 void sliced_destroy(dgchefsi_ctx* ctx);
 
-// Slices for the block-sparse product H X (sliced.cu). slices_of_h: the row
-// exponents E (element-padded rows) and s digit copies of H in the tensor-core
-// operand layout (brow: first row of each block, cstride: elements per copy).
-// slices_of_states: the state exponents E[Ns] and s digit copies of X in the
-// element-padded layout (cmap: padded column -> column, -1 for padding).
-// reduce_pair_slabs: C[r, cmap[c]] = the FP64 sum of the slice-pair slabs
-// (rows x cols FP32 each, pair order of the dense form) scaled by Erows[r] + Ecols[c].
-cudaError_t slices_of_h(const dgchefsi_ctx* ctx, const int32_t* blk_row, const int32_t* pnb, const int32_t* poff,
-                        const int64_t* brow, int s, __nv_bfloat16* Q, int64_t cstride, int32_t* E, int* flag,
-                        cudaStream_t st);
-cudaError_t slices_of_states(const double* X, int64_t ld, int64_t Ns, int64_t N, const int32_t* cmap, int64_t ldp,
-                             int s, __nv_bfloat16* Q, int64_t cstride, int32_t* E, int* flag, cudaStream_t st);
-dgchefsi_status reduce_pair_slabs(const float* Pw, int64_t rows, int64_t cols, const int32_t* Erows,
-                                  const int32_t* Ecols, const int32_t* cmap, double* C, int64_t ldc, int s,
-                                  cudaStream_t st);
+// Slabs of the digit weights (pair_groups below).
+struct PairGroups {
+  uint8_t count[16];  // by weight t
+  int total;
+};
+
+// Digits of the block-sparse product H X (sliced.cu). digit_counts: 9-bit digits
+// and weights for a request of `slices`. digits_of_h: the row exponents E
+// (element-padded rows) and d digit copies of H in the tensor-core operand
+// layout (brow: first row of each block, cstride: elements per copy).
+// digits_of_states: the state exponents E[Ns] and d digit copies of X in the
+// element-padded layout (slices: {padded column, column, columns, padded
+// columns} of each 64-wide slice). Both raise norm2[i] (zero before) to the
+// largest sum of squares of digit i over one slice of a row.
+// reduce_digit_slabs: C[r, cmap[c]] = the FP64 sum of the weights' slabs (rows x
+// cols INT32 each) scaled by Erows[r] + Ecols[c] (cmap -1: skipped).
+void digit_counts(int slices, int* d, int* w);
+cudaError_t digits_of_h(const dgchefsi_ctx* ctx, const int32_t* blk_row, const int32_t* pnb, const int32_t* poff,
+                        const int64_t* brow, int d, __nv_bfloat16* Q, int64_t cstride, int32_t* E, uint32_t* norm2,
+                        int* flag, cudaStream_t st);
+cudaError_t digits_of_states(const double* X, int64_t ld, int64_t Ns, int64_t N, const int4* slices, int nslices,
+                             int64_t ldp, int d, __nv_bfloat16* Q, int64_t cstride, int32_t* E, uint32_t* norm2,
+                             int* flag, cudaStream_t st);
+dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols, int w, const PairGroups& groups,
+                                   const int32_t* Erows, const int32_t* Ecols, const int32_t* cmap, double* C,
+                                   int64_t ldc, cudaStream_t st);
 // The slice-pair products of the dense sliced GEMM (pair_gemm.cu: tcgen05 on
 // pairs of SMs, cta_group::2, all pairs of the chunk in one persistent
 // launch). s digit slices per operand; the pairs i + j = t < nw (nw <= s + 1) of
@@ -210,18 +221,30 @@ dgchefsi_status reduce_pair_slabs(const float* Pw, int64_t rows, int64_t cols, c
 // and kc <= 4096; a_lower: A is lower triangular, so a row tile skips the K
 // slices past its last row. norm_a, norm_b (device, s entries): the largest sum
 // of squares of digit i over an aligned 512-entry block of a row. Enqueued only.
-// pair_groups: how many slabs each weight is split into for an M x Nc output.
+// pair_groups: how many slabs each weight is split into for an output of so many 256 x 256 tiles.
 // pair_products_begin clears the kernel's error word; pair_products_status
 // synchronises and reports a pipeline timeout.
-struct PairGroups {
-  uint8_t count[16];
-  int total;
-};
-PairGroups pair_groups(int s, int nw, int64_t M, int64_t Nc, int nsm);
+PairGroups pair_groups(int s, int nw, int64_t tiles, int nsm);
 dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, int64_t lqa, int64_t sa, int64_t M,
                                   const __nv_bfloat16* Qb, int64_t lqb, int64_t sb, int64_t Nc, int64_t K, int64_t k0,
                                   int64_t kc, int64_t n0, int64_t pn, int s, int nw, const PairGroups& groups,
                                   const uint32_t* norm_a, const uint32_t* norm_b, int32_t* Pw, bool a_lower, int64_t tri = 0);
+// The same kernel on the block-sparse H: slab = the weight's sum of Hs_i times
+// Xs_j (states s0 .. s0 + pn - 1, rows of ldp padded H rows). Hs: s digit
+// copies of H in the tensor-core operand layout (h_rows x 64, hcopy apart), Xs:
+// s digit copies of the states (Ns x ldp, xcopy apart); the plan (device):
+// groups of 256 / acc elements and their slice schedules; norm_h, norm_x: the
+// largest sum of squares of a digit over one 64-wide slice.
+struct BlockPairs {
+  const __nv_bfloat16 *Hs, *Xs;
+  int64_t hcopy, h_rows, xcopy, Ns, ldp;
+  int s, nw, acc, ngroups, maxent;
+  PairGroups groups;
+  const uint32_t *norm_h, *norm_x;
+  const int32_t *sched, *sched_ptr, *grp_elem, *pnb, *poff;
+};
+dgchefsi_status pair_products_blocks(dgchefsi_ctx* ctx, const BlockPairs& B, int64_t s0, int64_t pn, int32_t* Pw);
+bool pair_blocks_fit(int maxent, int acc);
 dgchefsi_status pair_products_begin(dgchefsi_ctx* ctx);
 dgchefsi_status pair_products_status(dgchefsi_ctx* ctx);
 // Y = H X (X, Y: Ns x ld state-major FP64) from s BF16 slices of each operand on

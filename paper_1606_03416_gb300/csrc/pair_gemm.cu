@@ -36,6 +36,12 @@
 // the time), 1510 with 512, 1660 with the norms' choice for Gaussian entries,
 // 1710 without any drain: 9.3 ms, where 55 pairs of 6-bit digits took ~16.
 //
+// BLOCKS = true multiplies the block-sparse H: the A rows of a tile are the H
+// rows of a group of elements (four of up to 64 functions, two per CTA), its K
+// slices the group's neighbour list, its B rows states. Elements that do not
+// couple to a slice's element multiply a zero tile there, 21 of 48 slices for a
+// 2 x 2 x 1 group of a 27-point stencil.
+//
 // Roles per CTA (576 threads): warp 0 lane 0 loads its halves with TMA into a
 // 6-slot ring and signals the first CTA's "full" barrier (its expect-tx counts
 // both CTAs' bytes); warp 1 lane 0 of the first CTA issues the MMAs, frees
@@ -79,6 +85,17 @@ struct PairJob {
   const uint32_t* norm_b;
   int32_t* Pw;      // slab of group g at Pw + g * M * pitch, row-major M x pitch
   int* err;
+  // Block-sparse form (BLOCKS): the A rows of a tile are the H rows of 2 G2
+  // stacked elements, acc rows each (G2 = 128 / acc per CTA), its K slices the
+  // entries of their group's schedule (the padded state column and each
+  // element's first operand row, a zero tile where it does not couple), its B
+  // rows states; the slabs are (states x padded H rows).
+  const int32_t* sched;      // entries of 1 + 2 G2 numbers
+  const int32_t* sched_ptr;  // [nmt + 1]
+  const int32_t* grp_elem;   // [nmt * 2 G2], -1 past the end
+  const int32_t* pnb;        // padded size and offset of each element
+  const int32_t* poff;
+  int G2, acc;
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -160,19 +177,23 @@ __device__ __forceinline__ int64_t nth_unit(int64_t k, int cid, int ncl) {
   return k * ncl + ((k & 1) ? ncl - 1 - cid : cid);
 }
 
-// K slices of the chunk that row tile mt needs: all of them, or for a lower
+// K slices that row tile mt needs: all of the chunk's, or for a lower
 // triangular A those up to its last row (at least one, so that the tile's
-// accumulator is written).
+// accumulator is written); the entries of its schedule in the block form.
+template <bool BLOCKS>
 __device__ __forceinline__ int slices_of_tile(const PairJob& J, int mt) {
+  if (BLOCKS) return J.sched_ptr[mt + 1] - J.sched_ptr[mt];
   if (!J.lower) return J.nk;
   const int need = (mt * 256 + 256 - J.k0 + 63) / 64;
   return max(1, min(J.nk, need));
 }
 
+template <bool BLOCKS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_slice_pairs_2sm(const PairJob J) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + PG_STAGES * PG_STAGE);
+  int32_t* sched_sh = reinterpret_cast<int32_t*>(bars + 2 * PG_STAGES + 4);  // BLOCKS: the unit's schedule (producer)
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
   __shared__ uint32_t drained_sh[2];       // epilogue warps done with their part, over all uses of a buffer
@@ -208,11 +229,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
   }
   // Any partial sum of products over 512 terms is at most |a||b|, over 2^h such
   // blocks at most 2^h |a||b| with the largest block norms (Cauchy-Schwarz):
-  // exact in FP32 while that is at most 2^24.
+  // exact in FP32 while that is at most 2^24. The block form's norms are over
+  // one 64-wide slice, so len slices give len |a||b|.
   for (int p = threadIdx.x; p < J.group[J.ngroups]; p += PG_THREADS) {
     const uint64_t sq = (uint64_t)J.norm_a[J.pair_i[p]] * J.norm_b[J.pair_j[p]];
     int len = PG_DRAIN;
-    for (int h = 0; h < 4 && sq <= 1ull << (48 - 2 * h); ++h) len *= 2;
+    if (BLOCKS) {
+      while (len < 64 && (uint64_t)((len + 1) * (len + 1)) * sq <= 1ull << 48) ++len;
+    } else {
+      for (int h = 0; h < 4 && sq <= 1ull << (48 - 2 * h); ++h) len *= 2;
+    }
     drain_sh[p] = len;
   }
   tc_fence_before();
@@ -223,16 +249,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
 
   if (warp == 0) {
     // ---------------- producer: this CTA's halves, completing on the first CTA's barrier
-    if (lane == 0) {
-      const uint32_t full_l = map_to_rank(full0, 0);
-      int c = 0;
-      bool ok = true;
-      for (int64_t k = 0, u; (u = nth_unit(k, cid, ncl)) < nunits && ok; ++k) {
-        int g, mt, nt;
-        unit_of(J, u, g, mt, nt);
-        const int ya = mt * 256 + (int)rank * 128;
-        const int yb = J.n0 + nt * 256 + (int)rank * 128;
-        const int nk = slices_of_tile(J, mt);
+    const uint32_t full_l = map_to_rank(full0, 0);
+    const int ent = 1 + 2 * J.G2;
+    int c = 0;
+    bool ok = true;
+    for (int64_t k = 0, u; (u = nth_unit(k, cid, ncl)) < nunits && ok; ++k) {
+      int g, mt, nt;
+      unit_of(J, u, g, mt, nt);
+      const int ya = mt * 256 + (int)rank * 128;
+      const int yb = J.n0 + nt * 256 + (int)rank * 128;
+      const int nk = slices_of_tile<BLOCKS>(J, mt);
+      if (BLOCKS) {
+        __syncwarp();
+        const int32_t* src = J.sched + (int64_t)J.sched_ptr[mt] * ent;
+        for (int t = lane; t < nk * ent; t += 32) sched_sh[t] = src[t];
+        __syncwarp();
+      }
+      if (lane == 0) {
         for (int p = J.group[g]; p < J.group[g + 1] && ok; ++p) {
           const CUtensorMap* am = J.maps + J.pair_i[p];
           const CUtensorMap* bm = J.maps + J.s + J.pair_j[p];
@@ -245,17 +278,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
             }
             if (leader) mbar_expect_tx(full0 + 8 * st, (uint32_t)(2 * PG_STAGE));
             const uint32_t dst = smem_u32(smem + st * PG_STAGE);
-            const int x = J.k0 + ks * (SLICE_BYTES / 2);
-            tma_load_2d_pair(dst, am, x, ya, full_l + 8 * st);
-            tma_load_2d_pair(dst + PG_HALF, bm, x, yb, full_l + 8 * st);
+            if (BLOCKS) {
+              const int32_t* e = sched_sh + ks * ent;
+              for (int q = 0; q < J.G2; ++q)
+                tma_load_2d_pair(dst + q * J.acc * SLICE_BYTES, am, 0, e[1 + rank * J.G2 + q], full_l + 8 * st);
+              tma_load_2d_pair(dst + PG_HALF, bm, e[0], yb, full_l + 8 * st);
+            } else {
+              const int x = J.k0 + ks * (SLICE_BYTES / 2);
+              tma_load_2d_pair(dst, am, x, ya, full_l + 8 * st);
+              tma_load_2d_pair(dst + PG_HALF, bm, x, yb, full_l + 8 * st);
+            }
             ++c;
           }
         }
       }
-      if (!ok) {
-        atomicOr(J.err, 1);
-        atomicExch(&abort_sh, 1);
-      }
+      if (BLOCKS) ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+    }
+    if (!ok && lane == 0) {
+      atomicOr(J.err, 1);
+      atomicExch(&abort_sh, 1);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: the first CTA of the pair only
@@ -268,7 +309,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
       for (int64_t k = 0, u; (u = nth_unit(k, cid, ncl)) < nunits && ok; ++k) {
         int g, mt, nt_;
         unit_of(J, u, g, mt, nt_);
-        const int nk = slices_of_tile(J, mt);
+        const int nk = slices_of_tile<BLOCKS>(J, mt);
         for (int p = J.group[g], k0 = 0, len = drain_sh[p]; p < J.group[g + 1] && ok; ++i) {
           const int buf = i & 1;
           const uint32_t use = (uint32_t)(i >> 1);
@@ -320,7 +361,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
     for (int64_t n = 0, u; (u = nth_unit(n, cid, ncl)) < nunits && ready; ++n) {
       int g, mt, nt;
       unit_of(J, u, g, mt, nt);
-      const int nk = slices_of_tile(J, mt);
+      const int nk = slices_of_tile<BLOCKS>(J, mt);
       int ndrain = 0;
       for (int p = J.group[g]; p < J.group[g + 1]; ++p) ndrain += (nk + drain_sh[p] - 1) / drain_sh[p];
       int sum[64];
@@ -351,14 +392,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
           for (int z = 0; z < 16; ++z) sum[16 * cc + z] += __float2int_rn(v[z]);
         }
       }
-      const int64_t r = (int64_t)mt * 256 + rank * 128 + 32 * q + lane;
-      if (!ready || r >= J.M || *(volatile int*)&abort_sh != 0) continue;
-      int32_t* out = J.Pw + ((size_t)g * (size_t)J.M + (size_t)r) * (size_t)J.pitch;
+      if (!ready || *(volatile int*)&abort_sh != 0) continue;
+      int32_t* slab = J.Pw + (size_t)g * (size_t)J.M * (size_t)J.pitch;
       const int64_t c0 = (int64_t)nt * 256 + 64 * h;
+      if (BLOCKS) {  // thread = H row, register = state: consecutive rows of one state are consecutive in the slab
+        const int local = 32 * q + lane, n = local % J.acc;
+        const int K = J.grp_elem[((int64_t)mt * 2 + rank) * J.G2 + local / J.acc];
+        if (K < 0 || n >= J.pnb[K]) continue;
+        int32_t* out = slab + J.poff[K] + n;
 #pragma unroll
-      for (int z = 0; z < 64; z += 4)  // pitch % 4 == 0: every vector is inside the row or past it
-        if (c0 + z < J.pitch)
-          *reinterpret_cast<int4*>(out + c0 + z) = make_int4(sum[z], sum[z + 1], sum[z + 2], sum[z + 3]);
+        for (int z = 0; z < 64; ++z)
+          if (c0 + z < J.M) out[(c0 + z) * J.pitch] = sum[z];
+      } else {
+        const int64_t r = (int64_t)mt * 256 + rank * 128 + 32 * q + lane;
+        if (r >= J.M) continue;
+        int32_t* out = slab + (size_t)r * (size_t)J.pitch;
+#pragma unroll
+        for (int z = 0; z < 64; z += 4)  // pitch % 4 == 0: every vector is inside the row or past it
+          if (c0 + z < J.pitch)
+            *reinterpret_cast<int4*>(out + c0 + z) = make_int4(sum[z], sum[z + 1], sum[z + 2], sum[z + 3]);
+      }
     }
   }
   tc_fence_before();
@@ -383,14 +436,14 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// BF16 matrix rows x inner (row stride `stride` elements), boxes of 64 x 128, 128-byte swizzle.
+// BF16 matrix rows x inner (row stride `stride` elements), boxes of 64 x box_rows, 128-byte swizzle.
 dgchefsi_status slice_map(CUtensorMap* map, const __nv_bfloat16* base, uint64_t inner, uint64_t rows,
-                          uint64_t stride) {
+                          uint64_t stride, uint32_t box_rows = 128) {
   auto enc = tensor_map_encoder();
   if (!enc) return set_error(DGCHEFSI_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
   cuuint64_t dims[2] = {inner, rows};
   cuuint64_t strides[1] = {stride * 2};
-  cuuint32_t box[2] = {64, 128};
+  cuuint32_t box[2] = {64, box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(base), dims, strides, box,
                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -404,11 +457,10 @@ dgchefsi_status slice_map(CUtensorMap* map, const __nv_bfloat16* base, uint64_t 
 // Pairs (i, t - i) of weight t with both digits below s.
 static int pairs_of_weight(int s, int t) { return std::max(0, std::min(t, s - 1) - std::max(0, t - s + 1) + 1); }
 
-PairGroups pair_groups(int s, int nw, int64_t M, int64_t Nc, int nsm) {
+PairGroups pair_groups(int s, int nw, int64_t tiles, int nsm) {
   // pairs per unit: all of a weight (at most 7, the INT32 bound) when there
   // are many units for the clusters; fewer when a small output would leave
   // clusters idle or waiting for the longest unit
-  const int64_t tiles = ((M + 255) / 256) * ((Nc + 255) / 256);
   const int64_t clusters = std::max(nsm / 2, 1);
   int64_t pairs = 0;
   for (int t = 0; t < nw; ++t) pairs += pairs_of_weight(s, t);
@@ -422,16 +474,76 @@ PairGroups pair_groups(int s, int nw, int64_t M, int64_t Nc, int nsm) {
   return g;
 }
 
+// Tables of a launch in one host block: 2s tensor maps (64-byte aligned), then
+// the groups (slab order: weights t descending, each weight's pairs in count[t]
+// groups of nearly equal size) and their pairs, then the tile list.
+struct PairTables {
+  std::vector<uint8_t> host;
+  CUtensorMap* maps = nullptr;
+  size_t maps_bytes = 0, tiles_at = 0;
+  int npairs = 0;
+
+  PairTables(int s, int nw, const PairGroups& groups, size_t ntiles) {
+    for (int t = 0; t < nw; ++t) npairs += pairs_of_weight(s, t);
+    const int ng = groups.total;
+    maps_bytes = sizeof(CUtensorMap) * (size_t)(2 * s);
+    tiles_at = (maps_bytes + sizeof(int32_t) * (size_t)(ng + 1 + 2 * npairs) + 15) / 16 * 16;
+    host.resize(tiles_at + sizeof(int2) * ntiles);
+    maps = reinterpret_cast<CUtensorMap*>(host.data());
+    int32_t* gp = reinterpret_cast<int32_t*>(host.data() + maps_bytes);
+    int32_t* pi = gp + ng + 1;
+    int32_t* pj = pi + npairs;
+    int n = 0, g = 0;
+    for (int t = nw - 1; t >= 0; --t) {
+      const int np = pairs_of_weight(s, t), i0 = std::max(0, t - s + 1);
+      for (int q = 0, k = 0; q < groups.count[t]; ++q) {
+        gp[g++] = n;
+        for (const int end = np * (q + 1) / groups.count[t]; k < end; ++k, ++n) {
+          pi[n] = i0 + k;
+          pj[n] = t - i0 - k;
+        }
+      }
+    }
+    gp[g] = n;
+  }
+};
+
+// Copies the tables to the device, fills what every launch shares and starts the kernel.
+static dgchefsi_status launch_pairs(dgchefsi_ctx* ctx, PairJob& J, const PairTables& T, int s, const PairGroups& groups,
+                                    bool blocks, int64_t tiles, int sched_bytes) {
+  // the context's table buffer (may be regrown here: it holds no state across launches)
+  DevBuf& tables = ctx->ws_pairs;
+  DG_TRY(ensure(ctx, tables, T.host.size(), "slice-pair tensor maps"));
+  uint8_t* tab = static_cast<uint8_t*>(tables.p);
+  // the pageable copy has been staged before it returns, so the host block may go
+  DG_CUDA(cudaMemcpyAsync(tab, T.host.data(), T.host.size(), cudaMemcpyHostToDevice, ctx->stream));
+  J.maps = reinterpret_cast<const CUtensorMap*>(tab);
+  J.group = reinterpret_cast<const int32_t*>(tab + T.maps_bytes);
+  J.pair_i = J.group + groups.total + 1;
+  J.pair_j = J.pair_i + T.npairs;
+  J.ngroups = groups.total;
+  J.s = s;
+  J.tiles = J.ntl > 0 ? reinterpret_cast<const int2*>(tab + T.tiles_at) : nullptr;
+  if (!ctx->ws_pairs_err.p) return set_error(DGCHEFSI_ERR_CUDA, "slice-pair products not begun");
+  J.err = static_cast<int*>(ctx->ws_pairs_err.p);
+  int nsm = 0;
+  DG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+  const int clusters = (int)std::min<int64_t>(tiles * groups.total, std::max(nsm / 2, 1));
+  const int smem = PG_STAGES * PG_STAGE + (2 * PG_STAGES + 4) * 8 + 1024 + sched_bytes;
+  auto kern = blocks ? k_slice_pairs_2sm<true> : k_slice_pairs_2sm<false>;
+  DG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  kern<<<2 * clusters, PG_THREADS, smem, ctx->stream>>>(J);
+  count_launch();
+  DG_CUDA(cudaGetLastError());
+  return DGCHEFSI_OK;
+}
+
 dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, int64_t lqa, int64_t sa, int64_t M,
                                   const __nv_bfloat16* Qb, int64_t lqb, int64_t sb, int64_t Nc, int64_t K, int64_t k0,
                                   int64_t kc, int64_t n0, int64_t pn, int s, int nw, const PairGroups& groups,
                                   const uint32_t* norm_a, const uint32_t* norm_b, int32_t* Pw, bool a_lower, int64_t tri) {
   if (M > 2147483647LL - 256 || Nc > 2147483647LL - 256 || K > 2147483647LL)
     return set_error(DGCHEFSI_ERR_UNSUPPORTED, "slice-pair product too large for 32-bit TMA coordinates");
-  cudaStream_t st = ctx->stream;
-  int npairs = 0;
-  for (int t = 0; t < nw; ++t) npairs += pairs_of_weight(s, t);
-  const int ng = groups.total;
   const int nmt = (int)((M + 255) / 256), nnt = (int)((pn + 255) / 256);
   // tri > 0: only entries (r, n0 + c) with n0 + c <= r mod tri are wanted (the
   // lower triangle of a symmetric product, or of each of several stacked
@@ -447,45 +559,13 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
       }
     if (tl.empty()) return DGCHEFSI_OK;
   }
-  // tables: 2s tensor maps (64-byte aligned), then groups and pairs, then the tile list
-  const size_t maps_bytes = sizeof(CUtensorMap) * (size_t)(2 * s);
-  const size_t lists_bytes = sizeof(int32_t) * (size_t)(ng + 1 + 2 * npairs);
-  const size_t tiles_at = (maps_bytes + lists_bytes + 15) / 16 * 16;
-  std::vector<uint8_t> host(tiles_at + sizeof(int2) * tl.size());
-  CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(host.data());
+  PairTables T(s, nw, groups, tl.size());
   for (int i = 0; i < s; ++i) {
-    DG_TRY(slice_map(&maps[i], Qa + (size_t)i * sa, (uint64_t)K, (uint64_t)M, (uint64_t)lqa));
-    DG_TRY(slice_map(&maps[s + i], Qb + (size_t)i * sb, (uint64_t)K, (uint64_t)Nc, (uint64_t)lqb));
+    DG_TRY(slice_map(&T.maps[i], Qa + (size_t)i * sa, (uint64_t)K, (uint64_t)M, (uint64_t)lqa));
+    DG_TRY(slice_map(&T.maps[s + i], Qb + (size_t)i * sb, (uint64_t)K, (uint64_t)Nc, (uint64_t)lqb));
   }
-  int32_t* gp = reinterpret_cast<int32_t*>(host.data() + maps_bytes);
-  int32_t* pi = gp + ng + 1;
-  int32_t* pj = pi + npairs;
-  int n = 0, g = 0;
-  for (int t = nw - 1; t >= 0; --t) {  // the pairs of weight t in count[t] groups of nearly equal size
-    const int np = pairs_of_weight(s, t), i0 = std::max(0, t - s + 1);
-    for (int q = 0, k = 0; q < groups.count[t]; ++q) {
-      gp[g++] = n;
-      for (const int end = np * (q + 1) / groups.count[t]; k < end; ++k, ++n) {
-        pi[n] = i0 + k;
-        pj[n] = t - i0 - k;
-      }
-    }
-  }
-  gp[g] = n;
-  if (!tl.empty()) std::memcpy(host.data() + tiles_at, tl.data(), sizeof(int2) * tl.size());
-  // the context's table buffer (may be regrown here: it holds no state across launches)
-  DevBuf& tables = ctx->ws_pairs;
-  DG_TRY(ensure(ctx, tables, host.size(), "slice-pair tensor maps"));
-  uint8_t* tab = static_cast<uint8_t*>(tables.p);
-  DG_CUDA(cudaMemcpyAsync(tab, host.data(), host.size(), cudaMemcpyHostToDevice, st));
-  // the pageable copy above has been staged before it returns, so `host` may go
+  if (!tl.empty()) std::memcpy(T.host.data() + T.tiles_at, tl.data(), sizeof(int2) * tl.size());
   PairJob J{};
-  J.maps = reinterpret_cast<const CUtensorMap*>(tab);
-  J.group = reinterpret_cast<const int32_t*>(tab + maps_bytes);
-  J.pair_i = J.group + ng + 1;
-  J.pair_j = J.pair_i + npairs;
-  J.ngroups = ng;
-  J.s = s;
   J.M = M;
   J.pitch = (pn + 3) / 4 * 4;
   J.n0 = (int)n0;
@@ -496,21 +576,40 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
   J.lower = a_lower ? 1 : 0;
   J.norm_a = norm_a;
   J.norm_b = norm_b;
-  J.tiles = tl.empty() ? nullptr : reinterpret_cast<const int2*>(tab + tiles_at);
   J.ntl = (int)tl.size();
   J.Pw = Pw;
-  if (!ctx->ws_pairs_err.p) return set_error(DGCHEFSI_ERR_CUDA, "slice-pair products not begun");
-  J.err = static_cast<int*>(ctx->ws_pairs_err.p);
-  int nsm = 0;
-  DG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-  const int64_t units = (J.tiles ? (int64_t)J.ntl : (int64_t)J.nmt * J.nnt) * ng;
-  const int clusters = (int)std::min<int64_t>(units, std::max(nsm / 2, 1));
-  const int smem = PG_STAGES * PG_STAGE + (2 * PG_STAGES + 4) * 8 + 1024;
-  DG_CUDA(cudaFuncSetAttribute(k_slice_pairs_2sm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  k_slice_pairs_2sm<<<2 * clusters, PG_THREADS, smem, st>>>(J);
-  count_launch();
-  DG_CUDA(cudaGetLastError());
-  return DGCHEFSI_OK;
+  return launch_pairs(ctx, J, T, s, groups, false, tl.empty() ? (int64_t)nmt * nnt : (int64_t)tl.size(), 0);
+}
+
+dgchefsi_status pair_products_blocks(dgchefsi_ctx* ctx, const BlockPairs& B, int64_t s0, int64_t pn, int32_t* Pw) {
+  PairTables T(B.s, B.nw, B.groups, 0);
+  for (int i = 0; i < B.s; ++i) {
+    DG_TRY(slice_map(&T.maps[i], B.Hs + (size_t)i * B.hcopy, 64, (uint64_t)B.h_rows, 64, (uint32_t)B.acc));
+    DG_TRY(slice_map(&T.maps[B.s + i], B.Xs + (size_t)i * B.xcopy, (uint64_t)B.ldp, (uint64_t)B.Ns, (uint64_t)B.ldp));
+  }
+  PairJob J{};
+  J.M = pn;
+  J.pitch = B.ldp;
+  J.n0 = (int)s0;
+  J.nmt = B.ngroups;
+  J.nnt = (int)((pn + 255) / 256);
+  J.norm_a = B.norm_h;
+  J.norm_b = B.norm_x;
+  J.Pw = Pw;
+  J.sched = B.sched;
+  J.sched_ptr = B.sched_ptr;
+  J.grp_elem = B.grp_elem;
+  J.pnb = B.pnb;
+  J.poff = B.poff;
+  J.G2 = 128 / B.acc;
+  J.acc = B.acc;
+  const int sched_bytes = B.maxent * (1 + 2 * J.G2) * (int)sizeof(int32_t);
+  return launch_pairs(ctx, J, T, B.s, B.groups, true, (int64_t)J.nmt * J.nnt, sched_bytes);
+}
+
+// Largest schedule (entries of 1 + 2 * 128 / acc numbers) the kernel's shared memory holds.
+bool pair_blocks_fit(int maxent, int acc) {
+  return PG_STAGES * PG_STAGE + (2 * PG_STAGES + 4) * 8 + 1024 + maxent * (1 + 256 / acc) * 4 <= 226 * 1024;
 }
 
 dgchefsi_status pair_products_begin(dgchefsi_ctx* ctx) {

@@ -31,11 +31,6 @@
 // (d = 7) the splitting term is below u L m_r n_c, the size of FP64's own
 // worst-case bound. The bound is normwise per row and column: entries far
 // below their row's maximum keep fewer significant bits than FP64.
-//
-// The block-sparse product H X (below) still multiplies one pair per launch on
-// the filter's step kernel with whole-row FP32 sums, so it keeps the 6-bit
-// digits: a[r,k] = 2^{e_r} sum_{i<s} q_i 2^{-6(i+1)}, |q_0| <= 64, |q_i| <= 32,
-// pair sums over L <= 4096 terms at most 2^24.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -85,109 +80,84 @@ __device__ __forceinline__ int decompose(double x, int64_t& M, int& E) {
   return 1;
 }
 
-// Slices of v = x 2^{-e'} (|v| < 1), where x = (-1)^neg M 2^{E - 1075} and
-// base = -1075 - e' + 6s, s <= 10: F = round(v 2^{6s}) as a 64-bit integer
-// (|F| <= 2^60, |v 2^{6s} - F| <= 1/2), then its balanced base-64 digits
-// q_{s-1}, ..., q_1 in [-32, 31] and the leading q_0 = the rest, |q_0| <= 64;
-// v = sum_i q_i 2^{-6(i+1)} up to 2^{-6s}/2. Integer arithmetic only.
-__device__ __forceinline__ void slice_fixed(int64_t M, int E, bool neg, int base, int s,
-                                            __nv_bfloat16* __restrict__ q, int64_t stride) {
-  const int sh = E + base;
-  int64_t F = 0;
-  if (M != 0) {
-    if (sh >= 0)
-      F = M << sh;
-    else if (sh > -54)
-      F = (M + (1LL << (-sh - 1))) >> (-sh);
-  }
-  if (neg) F = -F;
-  for (int i = s - 1; i >= 1; --i) {
-    const int64_t d = ((F + 32) & 63) - 32;
-    q[i * stride] = __float2bfloat16_rn((float)(int)d);
-    F = (F - d) >> 6;
-  }
-  q[0] = __float2bfloat16_rn((float)(int)F);
-}
-
-// The same digits for s > 10 (F would not fit 64 bits): v is scaled in FP64,
-// each digit rounded to nearest and subtracted (every step exact).
-__device__ __forceinline__ void slice_fp64(double v, int s, __nv_bfloat16* __restrict__ q, int64_t stride) {
-  double r = v;
-  for (int i = 0; i < s; ++i) {
-    r *= 64.0;
-    const double d = rint(r);
-    r -= d;
-    q[i * stride] = __float2bfloat16_rn((float)d);
-  }
-}
-
 __device__ __forceinline__ int warp_max(int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 
-// Four consecutive digits (|x| <= 256) to q as BF16, their squares to *norm.
-__device__ __forceinline__ void put_digits(const int (&x)[4], __nv_bfloat16* __restrict__ q, bool store,
+// C = 2 or 4 consecutive digits (|x| <= 256) to q as BF16, their squares to *norm.
+template <int C>
+__device__ __forceinline__ void put_digits(const int (&x)[C], __nv_bfloat16* __restrict__ q, bool store,
                                            uint32_t* norm) {
-  if (store) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn((float)x[0], (float)x[1]);
-    const __nv_bfloat162 hi = __floats2bfloat162_rn((float)x[2], (float)x[3]);
-    *reinterpret_cast<uint2*>(q) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+  uint32_t w[C / 2], sq = 0;
+#pragma unroll
+  for (int c = 0; c < C; c += 2) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn((float)x[c], (float)x[c + 1]);
+    w[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
+    sq += (uint32_t)(x[c] * x[c] + x[c + 1] * x[c + 1]);
   }
-  const uint32_t sq = __reduce_add_sync(0xffffffffu, (uint32_t)(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]));
+  if (store) {
+    if (C == 4)
+      *reinterpret_cast<uint2*>(q) = make_uint2(w[0], w[C / 2 - 1]);
+    else
+      *reinterpret_cast<uint32_t*>(q) = w[0];
+  }
+  sq = __reduce_add_sync(0xffffffffu, sq);
   if ((threadIdx.x & 31) == 0) atomicAdd(norm, sq);
 }
 
-// Digits i = 0 .. d - 1 of four consecutive entries, entry c = (-1)^neg M_c
-// 2^{E_c - 1075}, scaled by 2^{-e}: F = round(v 2^{9d - 1}) as a 64-bit integer
-// (d <= 7: |F| <= 2^62; |v 2^{9d-1} - F| <= 1/2), then its balanced base-512
-// digits from the last one up, the first the rest (|q_0| <= 256). Integer
-// arithmetic only; one 8-byte store per digit (where `store`). norm[i] (shared)
-// collects the squares of digit i; every lane of the warp takes part.
-__device__ __forceinline__ void digits_fixed4(const int64_t (&M)[4], const int (&sh)[4], const bool (&neg)[4], int d,
-                                              __nv_bfloat16* __restrict__ q, int64_t stride, bool store,
-                                              uint32_t* norm) {
-  int64_t F[4];
+// Digits i = 0 .. d - 1 of C consecutive entries v 2^{b} scaled by 2^{-e}
+// (|v 2^{b-e}| < 1; zero entries and `zero` give zero digits), stored at
+// q + i * stride where `store`; norm[i] (shared) collects the squares of digit
+// i; every lane of the warp takes part. One store per digit.
+// d <= 7: F = round(v 2^{9d - 1}) as a 64-bit integer (|F| <= 2^62;
+// |v 2^{9d-1} - F| <= 1/2), then its balanced base-512 digits from the last one
+// up, the first the rest (|q_0| <= 256). Integer arithmetic only.
+// d > 7 (F would not fit 64 bits): v is scaled in FP64, each digit rounded to
+// nearest and subtracted (every step exact).
+template <int C>
+__device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (&b)[C], int e, bool zero, int d,
+                                               __nv_bfloat16* __restrict__ q, int64_t stride, bool store,
+                                               uint32_t* norm) {
+  int x[C];
+  if (d <= 7) {
+    int64_t F[C];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    F[c] = 0;
-    if (M[c] != 0) {
-      if (sh[c] >= 0)
-        F[c] = M[c] << sh[c];
-      else if (sh[c] > -54)
-        F[c] = (M[c] + (1LL << (-sh[c] - 1))) >> (-sh[c]);
+    for (int c = 0; c < C; ++c) {
+      int64_t M;
+      int E;
+      F[c] = 0;
+      if (!zero && decompose(v[c], M, E) == 1) {  // |v| = M 2^{E - 1075}
+        const int sh = E + b[c] - 1075 - e + 9 * d - 1;
+        if (sh >= 0)
+          F[c] = M << sh;
+        else if (sh > -54)
+          F[c] = (M + (1LL << (-sh - 1))) >> (-sh);
+        if (v[c] < 0.0) F[c] = -F[c];
+      }
     }
-    if (neg[c]) F[c] = -F[c];
-  }
-  for (int i = d - 1; i >= 0; --i) {
-    int x[4];
+    for (int i = d - 1; i >= 0; --i) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      x[c] = (int)(i > 0 ? ((F[c] + 256) & 511) - 256 : F[c]);
-      F[c] = (F[c] - x[c]) >> 9;
+      for (int c = 0; c < C; ++c) {
+        x[c] = (int)(i > 0 ? ((F[c] + 256) & 511) - 256 : F[c]);
+        F[c] = (F[c] - x[c]) >> 9;
+      }
+      put_digits<C>(x, q + i * stride, store, norm + i);
     }
-    put_digits(x, q + i * stride, store, norm + i);
-  }
-}
-
-// The same digits for d > 7 (F would not fit 64 bits): v is scaled in FP64,
-// each digit rounded to nearest and subtracted (every step exact).
-__device__ __forceinline__ void digits_fp64x4(const double (&v)[4], int d, __nv_bfloat16* __restrict__ q,
-                                              int64_t stride, bool store, uint32_t* norm) {
-  double r[4];
+  } else {
+    double r[C];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) r[c] = v[c] * 256.0;
-  for (int i = 0; i < d; ++i) {
-    int x[4];
+    for (int c = 0; c < C; ++c) r[c] = zero || v[c] == 0.0 ? 0.0 : ldexp(v[c], b[c] - e) * 256.0;
+    for (int i = 0; i < d; ++i) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const double g = rint(r[c]);
-      r[c] = (r[c] - g) * 512.0;
-      x[c] = (int)g;
+      for (int c = 0; c < C; ++c) {
+        const double g = rint(r[c]);
+        r[c] = (r[c] - g) * 512.0;
+        x[c] = (int)g;
+      }
+      put_digits<C>(x, q + i * stride, store, norm + i);
     }
-    put_digits(x, q + i * stride, store, norm + i);
   }
 }
 
@@ -267,26 +237,13 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
     const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
     if (k0 + 1024 * u >= K) break;  // the same for the whole CTA
     uint32_t* nrm = norm[2 * u + (threadIdx.x >> 7)];
-    __nv_bfloat16* q = Q + row * ldq + k;
-    if (d <= 7) {
-      int64_t M[4];
-      int sh[4];
-      bool neg[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        int Ex = 0;
-        if (zero || decompose(v[u][c], M[c], Ex) != 1) M[c] = 0;
-        sh[c] = M[c] != 0 ? Ex + (bal ? bal[k + c] : 0) - 1075 - e + 9 * d - 1 : 0;
-        neg[c] = v[u][c] < 0.0;
-      }
-      digits_fixed4(M, sh, neg, d, q, sstride, k < K, nrm);
-    } else {
-      double r[4];
+    int b[4] = {0, 0, 0, 0};
+    if (bal) {
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        r[c] = zero || v[u][c] == 0.0 ? 0.0 : ldexp(v[u][c], (bal ? bal[k + c] : 0) - e);
-      digits_fp64x4(r, d, q, sstride, k < K, nrm);
+        if (k + c < K) b[c] = bal[k + c];
     }
+    put_all_digits<4>(v[u], b, e, zero, d, Q + row * ldq + k, sstride, k < K, nrm);
   }
   __syncthreads();
   if (threadIdx.x < d) {
@@ -320,153 +277,6 @@ __global__ void __launch_bounds__(256) k_row_exponents(const double* __restrict_
   }
 }
 
-// C[r, n0 + c] (+)= 2^{e_r + f_{n0+c} - 12} sum_t 2^{-6t} g_t,  g_t = sum_{i+j=t} P_{ij}[r, c],
-// for r < M, c < P. Pair (i, j) is slab i*S - i(i-1)/2 + j of Pw (M x P FP32).
-// Each P_ij is an exact integer of magnitude <= 2^24, so g_t is summed in
-// int32 (|g_t| <= 16 * 2^24), five consecutive t are combined exactly in int64
-// (< 2^53, exact in FP64), and the blocks meet in FP64: one rounding per 30
-// bits of weight. Every slab value is loaded once, all loads of an output
-// before any use, so the kernel streams Pw at memory speed.
-// cmap (may be null): column c of the slabs goes to column cmap[c] of C, and
-// is skipped when cmap[c] < 0 (the padding columns of the element-padded layout).
-// tri > 0: only the entries with n0 + c <= r mod tri are formed (the slice-pair
-// kernel left the tiles above that line out); the others are not read or written.
-template <int S>
-__global__ void __launch_bounds__(256) k_sliced_reduce(const float* __restrict__ Pw, int64_t M, int64_t P,
-                                                       const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb,
-                                                       int nch, int chunk, int64_t n0, double* __restrict__ C,
-                                                       int64_t ldc, int accumulate, const int32_t* __restrict__ cmap,
-                                                       int64_t tri) {
-  constexpr int NB = (S + 4) / 5;  // blocks of five t
-  const int64_t total = M * P;
-  const int64_t slab = M * P;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    if (tri > 0 && n0 + idx % P > (idx / P) % tri) continue;
-    int g[S];
-#pragma unroll
-    for (int t = 0; t < S; ++t) g[t] = 0;
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-#pragma unroll
-      for (int j = 0; j < S - i; ++j)
-        g[i + j] += __float2int_rn(__ldcs(Pw + (int64_t)(i * S - i * (i - 1) / 2 + j) * slab + idx));
-    // h = sum_b B_b 2^{-30 b}, B_b = sum_{t = 5b}^{5b+4} g_t 2^{6(5b + 4 - t)}; sum_t g_t 2^{-6t} = h 2^{-24}
-    double h = 0.0;
-#pragma unroll
-    for (int b = NB - 1; b >= 0; --b) {
-      int64_t B = 0;
-#pragma unroll
-      for (int t = 5 * b; t < 5 * b + 5; ++t) B = B * 64 + (t < S ? (int64_t)g[t] : 0);
-      h = h * 0x1p-30 + (double)B;
-    }
-    const int64_t r = idx / P;
-    const int64_t c = idx - r * P;
-    const int64_t oc = cmap ? (int64_t)cmap[c] : n0 + c;
-    if (oc < 0) continue;
-    const double v = ldexp(h, Ea[r * nch + chunk] + Eb[(n0 + c) * nch + chunk] - 12 - 24);
-    double* out = C + r * ldc + oc;
-    *out = accumulate ? *out + v : v;
-  }
-}
-
-// The same for P % 4 == 0, four consecutive outputs per thread: one 16-byte
-// load per slab instead of four 4-byte ones (same sums, same roundings).
-template <int S>
-__global__ void __launch_bounds__(256) k_sliced_reduce4(const float* __restrict__ Pw, int64_t M, int64_t P,
-                                                        const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb,
-                                                        int nch, int chunk, int64_t n0, double* __restrict__ C,
-                                                        int64_t ldc, int accumulate, const int32_t* __restrict__ cmap,
-                                                        int64_t tri) {
-  constexpr int NB = (S + 4) / 5;
-  const int64_t slab = M * P;
-  const int64_t total4 = slab / 4;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total4;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t idx = 4 * q;
-    // the four entries share a row and a 256-column tile: when the first is
-    // above the line all are, and otherwise the tile was computed
-    const int64_t rdiag = tri > 0 ? (idx / P) % tri : 0;
-    if (tri > 0 && n0 + idx % P > rdiag) continue;
-    int g[4][S];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-#pragma unroll
-      for (int t = 0; t < S; ++t) g[e][t] = 0;
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-#pragma unroll
-      for (int j = 0; j < S - i; ++j) {
-        const float4 v =
-            __ldcs(reinterpret_cast<const float4*>(Pw + (int64_t)(i * S - i * (i - 1) / 2 + j) * slab + idx));
-        g[0][i + j] += __float2int_rn(v.x);
-        g[1][i + j] += __float2int_rn(v.y);
-        g[2][i + j] += __float2int_rn(v.z);
-        g[3][i + j] += __float2int_rn(v.w);
-      }
-    const int64_t r = idx / P;
-    const int64_t c0 = idx - r * P;
-    const int er = Ea[r * nch + chunk];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      double h = 0.0;
-#pragma unroll
-      for (int b = NB - 1; b >= 0; --b) {
-        int64_t B = 0;
-#pragma unroll
-        for (int t = 5 * b; t < 5 * b + 5; ++t) B = B * 64 + (t < S ? (int64_t)g[e][t] : 0);
-        h = h * 0x1p-30 + (double)B;
-      }
-      const int64_t c = c0 + e;
-      const int64_t oc = cmap ? (int64_t)cmap[c] : n0 + c;
-      if (oc < 0 || (tri > 0 && n0 + c > rdiag)) continue;
-      const double v = ldexp(h, er + Eb[(n0 + c) * nch + chunk] - 12 - 24);
-      double* out = C + r * ldc + oc;
-      *out = accumulate ? *out + v : v;
-    }
-  }
-}
-
-typedef void (*ReduceKernel)(const float*, int64_t, int64_t, const int32_t*, const int32_t*, int, int, int64_t,
-                             double*, int64_t, int, const int32_t*, int64_t);
-
-static ReduceKernel reduce_kernel(int s) {
-  switch (s) {
-#define DG_REDUCE_CASE(n) \
-  case n: return k_sliced_reduce<n>;
-    DG_REDUCE_CASE(2) DG_REDUCE_CASE(3) DG_REDUCE_CASE(4) DG_REDUCE_CASE(5) DG_REDUCE_CASE(6)
-    DG_REDUCE_CASE(7) DG_REDUCE_CASE(8) DG_REDUCE_CASE(9) DG_REDUCE_CASE(10) DG_REDUCE_CASE(11)
-    DG_REDUCE_CASE(12) DG_REDUCE_CASE(13) DG_REDUCE_CASE(14) DG_REDUCE_CASE(15) DG_REDUCE_CASE(16)
-#undef DG_REDUCE_CASE
-    default: return nullptr;
-  }
-}
-
-static ReduceKernel reduce_kernel4(int s) {
-  switch (s) {
-#define DG_REDUCE_CASE(n) \
-  case n: return k_sliced_reduce4<n>;
-    DG_REDUCE_CASE(2) DG_REDUCE_CASE(3) DG_REDUCE_CASE(4) DG_REDUCE_CASE(5) DG_REDUCE_CASE(6)
-    DG_REDUCE_CASE(7) DG_REDUCE_CASE(8) DG_REDUCE_CASE(9) DG_REDUCE_CASE(10) DG_REDUCE_CASE(11)
-    DG_REDUCE_CASE(12) DG_REDUCE_CASE(13) DG_REDUCE_CASE(14) DG_REDUCE_CASE(15) DG_REDUCE_CASE(16)
-#undef DG_REDUCE_CASE
-    default: return nullptr;
-  }
-}
-
-// The reduction over slabs of M x P: four outputs per thread when P % 4 == 0.
-static cudaError_t launch_reduce(int s, const float* Pw, int64_t M, int64_t P, const int32_t* Ea, const int32_t* Eb,
-                                 int nch, int chunk, int64_t n0, double* C, int64_t ldc, int accumulate,
-                                 const int32_t* cmap, cudaStream_t st, int64_t tri = 0) {
-  const bool v4 = P % 4 == 0;
-  const int64_t work = v4 ? M * P / 4 : M * P;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 16));
-  (v4 ? reduce_kernel4(s) : reduce_kernel(s))<<<grid, 256, 0, st>>>(Pw, M, P, Ea, Eb, nch, chunk, n0, C, ldc,
-                                                                      accumulate, cmap, tri);
-  count_launch();
-  return cudaGetLastError();
-}
-
 // h 2^e (one rounding, as ldexp; the power of two is built from its bits when
 // it is a normal number).
 __device__ __forceinline__ double scale_pow2(double h, int e) {
@@ -483,6 +293,8 @@ __device__ __forceinline__ double scale_pow2(double h, int e) {
 // rows of C at n0 start on 16 bytes. tri > 0: only the entries with
 // n0 + c <= r mod tri are formed (the slice-pair kernel left the tiles above
 // that line out); the others are not read or written.
+// cmap (may be null): column c goes to column cmap[c] of C and is skipped when
+// that is negative (the padding columns of the element-padded layout).
 // Bound by HBM: 4 bytes read per slab and entry (28 at w = 7) and 8 written, 16
 // when a chunk is added; it runs on its own stream beside the next chunk's pairs.
 template <int W>
@@ -490,7 +302,8 @@ __global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict_
                                                       int64_t pitch, const PairGroups groups,
                                                       const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb,
                                                       int nch, int chunk, int64_t n0, double* __restrict__ C,
-                                                      int64_t ldc, int wide, int accumulate, int64_t tri) {
+                                                      int64_t ldc, int wide, int accumulate, int64_t tri,
+                                                      const int32_t* __restrict__ cmap) {
   constexpr int NB = (W + 3) / 4;
   const int64_t slab = M * pitch, quads = pitch / 4, total = M * quads;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
@@ -541,6 +354,14 @@ __global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict_
       }
       y[e] = c0 + e < P ? scale_pow2(h, er + Eb[(n0 + c0 + e) * nch + chunk]) : 0.0;
     }
+    if (cmap) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int32_t oc = c0 + e < P ? cmap[c0 + e] : -1;
+        if (oc >= 0) C[r * ldc + oc] = y[e];
+      }
+      continue;
+    }
     double* out = C + r * ldc + n0 + c0;
     if (wide && c0 + 4 <= P && (tri == 0 || n0 + c0 + 3 <= rdiag)) {
       double2* o = reinterpret_cast<double2*>(out);
@@ -562,7 +383,8 @@ __global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict_
 }
 
 typedef void (*DigitReduce)(const int32_t*, int64_t, int64_t, int64_t, const PairGroups, const int32_t*,
-                            const int32_t*, int, int, int64_t, double*, int64_t, int, int, int64_t);
+                            const int32_t*, int, int, int64_t, double*, int64_t, int, int, int64_t,
+                            const int32_t*);
 
 static DigitReduce digit_reduce(int w) {
   switch (w) {
@@ -626,7 +448,7 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
   const int nch = (int)((K + kL - 1) / kL);
   int nsm = 0;
   DG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-  const PairGroups groups = pair_groups(s, nw, M, Nc, nsm);
+  const PairGroups groups = pair_groups(s, nw, ((M + 255) / 256) * ((Nc + 255) / 256), nsm);
   const size_t slab_row = sizeof(int32_t) * (size_t)groups.total * (size_t)M;  // bytes per output column
   // Slices of A: s x M x lqa, of the right operand as rows: s x Nc x lqb (K
   // contiguous in both; the A B form transposes B first).
@@ -743,7 +565,7 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
       const int64_t pitch = round_up(pn, 4), work = M * pitch / 4;
       const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 16));
       digit_reduce(nw)<<<grid, 256, 0, sr>>>(Pb, M, pn, pitch, groups, Ea, Eb, nch, chunk, n0, C, ldc,
-                                            wide(C, ldc) ? 1 : 0, chunk > 0 ? 1 : 0, tri);
+                                            wide(C, ldc) ? 1 : 0, chunk > 0 ? 1 : 0, tri, nullptr);
       count_launch();
       DG_CUDA(cudaGetLastError());
       if (multi) DG_CUDA(cudaEventRecord(ctx->ev_reduce[b], sr));
@@ -766,17 +588,16 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
 }
 
 // ---------------------------------------------------------------------------
-// H X from slices (the block-sparse product of Rayleigh-Ritz, W = H Y_hat).
+// H X from digits (the block-sparse product of Rayleigh-Ritz, W = H Y_hat).
 // Row r of H (element K, row n) contracts over the columns of K's neighbour
 // blocks only, at most 4096 of them, so one K chunk covers every row: its
 // exponent e_r is over the whole row. Each state's exponent f_s is over all N
 // of its components (a valid bound for every row's column range). H's digits
-// are written in the block layout of the tensor-core filter's operand copy
-// of H (64-column slices of each block, element-padded rows), the states'
-// digits in its element-padded state-major layout, so the filter's step
-// kernel multiplies one slice pair per launch (alpha = 1, beta = 0) into an
-// FP32 slab, and k_sliced_reduce (with the padded-to-plain column map)
-// combines the slabs.
+// are written in the block layout of the tensor-core filter's operand copy of
+// H (64-column slices of each block, element-padded rows), the states' digits
+// in its element-padded state-major layout; the pair kernel's block form sums
+// each weight's pairs into one INT32 slab and k_digit_reduce (with the
+// padded-to-plain column map) combines the slabs.
 
 // E[poff_K + n] = frexp exponent of max_j |H[(K, n), j]| over row n of element
 // K's blocks (0 for an all-zero row, and for the padding rows n >= nb[K]).
@@ -814,54 +635,52 @@ __global__ void __launch_bounds__(256) k_h_row_exponents(const int64_t* __restri
   if (threadIdx.x == 0 && bad) atomic_flag(flag);
 }
 
-// s digit copies of H in the filter's operand layout: block e, 64-column
+// d digit copies of H in the filter's operand layout: block e, 64-column
 // slice sl, padded row n at row brow[e] + sl * pnb[K] + n of each copy (copy i
-// starts at Q + i * cstride); entries past the block (padding) are zero.
-__global__ void __launch_bounds__(256) k_build_h_slices(const int32_t* __restrict__ blk_row,
-                                                        const int32_t* __restrict__ col,
-                                                        const int64_t* __restrict__ blk_off,
-                                                        const double* __restrict__ vals,
-                                                        const int32_t* __restrict__ nb,
-                                                        const int32_t* __restrict__ pnb,
-                                                        const int32_t* __restrict__ poff,
-                                                        const int64_t* __restrict__ brow,
-                                                        const int32_t* __restrict__ E, int s,
-                                                        __nv_bfloat16* __restrict__ Q, int64_t cstride) {
-  constexpr int W = 64;
+// starts at Q + i * cstride); entries past the block (padding) are zero. A warp
+// per row of 64.
+__global__ void __launch_bounds__(256) k_h_digits(const int32_t* __restrict__ blk_row, const int32_t* __restrict__ col,
+                                                  const int64_t* __restrict__ blk_off, const double* __restrict__ vals,
+                                                  const int32_t* __restrict__ nb, const int32_t* __restrict__ pnb,
+                                                  const int32_t* __restrict__ poff, const int64_t* __restrict__ brow,
+                                                  const int32_t* __restrict__ E, int d, __nv_bfloat16* __restrict__ Q,
+                                                  int64_t cstride, uint32_t* __restrict__ norm2) {
+  __shared__ uint32_t norm[8][kNormPitch], top[kNormPitch];
   const int64_t e = blockIdx.x;
   const int K = blk_row[e], Kp = col[e];
   const int nK = nb[K], nKp = nb[Kp], pK = pnb[K];
-  const int nsl = (pnb[Kp] + W - 1) / W;
+  const int nsl = (pnb[Kp] + 63) / 64;
   const double* blk = vals + blk_off[e];
-  const int64_t total = (int64_t)nsl * pK * W;
-  for (int64_t t = threadIdx.x; t < total; t += blockDim.x) {
-    const int w = (int)(t % W);
-    const int64_t rr = t / W;
-    const int n = (int)(rr % pK);
-    const int sl = (int)(rr / pK);
-    const int jp = sl * W + w;
-    const double v = (n < nK && jp < nKp) ? blk[(int64_t)n * nKp + jp] : 0.0;
-    const int er = E[poff[K] + n];
-    __nv_bfloat16* q = Q + (brow[e] + rr) * W + w;
-    if (s <= 10) {
-      int64_t Mm = 0;
-      int Ex = 0;
-      if (decompose(v, Mm, Ex) != 1) Mm = 0;
-      slice_fixed(Mm, Ex, v < 0.0, -1075 - er + 6 * s, s, q, cstride);
-    } else {
-      slice_fp64(std::isfinite(v) ? ldexp(v, -er) : 0.0, s, q, cstride);
-    }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < kNormPitch) top[threadIdx.x] = 0;
+  __syncthreads();
+  for (int rr = warp; rr < nsl * pK; rr += 8) {
+    const int n = rr % pK, jp = (rr / pK) * 64 + 2 * lane;
+    const int b[2] = {0, 0};
+    double v[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) v[c] = (n < nK && jp + c < nKp) ? blk[(int64_t)n * nKp + jp + c] : 0.0;
+    if (lane < kNormPitch) norm[warp][lane] = 0;
+    __syncwarp();
+    put_all_digits<2>(v, b, E[poff[K] + n], false, d, Q + (brow[e] + rr) * 64 + 2 * lane, cstride, true, norm[warp]);
+    __syncwarp();
+    if (lane < d) atomicMax(&top[lane], norm[warp][lane]);
+    __syncwarp();
   }
+  __syncthreads();
+  if (threadIdx.x < d) atomicMax(norm2 + threadIdx.x, top[threadIdx.x]);
 }
 
-// s digit copies of the states X (Ns x ld, state-major) in the element-padded
-// layout (Ns x ldp per copy, copy i at Q + i * cstride); cmap[c] is the
-// column of padded column c (-1 for padding, written as zero). E[s] = frexp
-// exponent of the state's largest |entry|. One CTA per state, two passes.
-__global__ void __launch_bounds__(256) k_pack_state_slices(const double* __restrict__ X, int64_t ld, int64_t N,
-                                                           const int32_t* __restrict__ cmap, int64_t ldp, int s,
-                                                           __nv_bfloat16* __restrict__ Q, int64_t cstride,
-                                                           int32_t* __restrict__ E, int* __restrict__ flag) {
+// d digit copies of the states X (Ns x ld, state-major) in the element-padded
+// layout (Ns x ldp per copy, copy i at Q + i * cstride); slices[k] = {padded
+// column, column, columns, padded columns} of the k-th 64-wide slice. E[s] =
+// frexp exponent of the state's largest |entry|. One CTA per state, two passes,
+// a warp per slice.
+__global__ void __launch_bounds__(256) k_state_digits(const double* __restrict__ X, int64_t ld, int64_t N,
+                                                      const int4* __restrict__ slices, int nslices, int64_t ldp, int d,
+                                                      __nv_bfloat16* __restrict__ Q, int64_t cstride,
+                                                      int32_t* __restrict__ E, uint32_t* __restrict__ norm2,
+                                                      int* __restrict__ flag) {
   const int64_t st = blockIdx.x;
   const double* x = X + st * ld;
   int emax = INT_MIN;
@@ -875,10 +694,13 @@ __global__ void __launch_bounds__(256) k_pack_state_slices(const double* __restr
   }
   __shared__ int red[8];
   __shared__ int sbad;
+  __shared__ uint32_t norm[8][kNormPitch], top[kNormPitch];
   if (threadIdx.x == 0) sbad = 0;
+  if (threadIdx.x < kNormPitch) top[threadIdx.x] = 0;
   emax = warp_max(emax);
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = emax;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) red[warp] = emax;
   if (bad) sbad = 1;
   __syncthreads();
   emax = red[0];
@@ -890,47 +712,58 @@ __global__ void __launch_bounds__(256) k_pack_state_slices(const double* __restr
     E[st] = e;
     if (zero) atomic_flag(flag);
   }
-  for (int64_t c = threadIdx.x; c < ldp; c += blockDim.x) {
-    const int32_t oc = cmap[c];
-    const double v = (oc >= 0 && !zero) ? x[oc] : 0.0;
-    __nv_bfloat16* q = Q + st * ldp + c;
-    if (s <= 10) {
-      int64_t Mm = 0;
-      int Ex = 0;
-      if (decompose(v, Mm, Ex) != 1) Mm = 0;
-      slice_fixed(Mm, Ex, v < 0.0, -1075 - e + 6 * s, s, q, cstride);
-    } else {
-      slice_fp64(ldexp(v, -e), s, q, cstride);
-    }
+  for (int k = warp; k < nslices; k += 8) {
+    const int4 sl = slices[k];
+    const int j = 2 * lane;
+    const int b[2] = {0, 0};
+    double v[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) v[c] = j + c < sl.z ? x[sl.y + j + c] : 0.0;
+    if (lane < kNormPitch) norm[warp][lane] = 0;
+    __syncwarp();
+    put_all_digits<2>(v, b, e, zero, d, Q + st * ldp + sl.x + j, cstride, j < sl.w, norm[warp]);
+    __syncwarp();
+    if (lane < d) atomicMax(&top[lane], norm[warp][lane]);
+    __syncwarp();
   }
+  __syncthreads();
+  if (threadIdx.x < d) atomicMax(norm2 + threadIdx.x, top[threadIdx.x]);
 }
 
-cudaError_t slices_of_h(const dgchefsi_ctx* ctx, const int32_t* blk_row, const int32_t* pnb, const int32_t* poff,
-                        const int64_t* brow, int s, __nv_bfloat16* Q, int64_t cstride, int32_t* E, int* flag,
-                        cudaStream_t st) {
+void digit_counts(int slices, int* d, int* w) {
+  *d = digits_for(slices);
+  *w = weights_for(slices);
+}
+
+cudaError_t digits_of_h(const dgchefsi_ctx* ctx, const int32_t* blk_row, const int32_t* pnb, const int32_t* poff,
+                        const int64_t* brow, int d, __nv_bfloat16* Q, int64_t cstride, int32_t* E, uint32_t* norm2,
+                        int* flag, cudaStream_t st) {
   k_h_row_exponents<<<(unsigned)ctx->M, 256, 0, st>>>(ctx->row_ptr_d, ctx->col_d, ctx->blk_off_d, ctx->vals_d,
                                                       ctx->nb_d, pnb, poff, E, flag);
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_build_h_slices<<<(unsigned)ctx->nnzb, 256, 0, st>>>(blk_row, ctx->col_d, ctx->blk_off_d, ctx->vals_d, ctx->nb_d,
-                                                        pnb, poff, brow, E, s, Q, cstride);
+  k_h_digits<<<(unsigned)ctx->nnzb, 256, 0, st>>>(blk_row, ctx->col_d, ctx->blk_off_d, ctx->vals_d, ctx->nb_d, pnb,
+                                                  poff, brow, E, d, Q, cstride, norm2);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t slices_of_states(const double* X, int64_t ld, int64_t Ns, int64_t N, const int32_t* cmap, int64_t ldp,
-                             int s, __nv_bfloat16* Q, int64_t cstride, int32_t* E, int* flag, cudaStream_t st) {
-  k_pack_state_slices<<<(unsigned)Ns, 256, 0, st>>>(X, ld, N, cmap, ldp, s, Q, cstride, E, flag);
+cudaError_t digits_of_states(const double* X, int64_t ld, int64_t Ns, int64_t N, const int4* slices, int nslices,
+                             int64_t ldp, int d, __nv_bfloat16* Q, int64_t cstride, int32_t* E, uint32_t* norm2,
+                             int* flag, cudaStream_t st) {
+  k_state_digits<<<(unsigned)Ns, 256, 0, st>>>(X, ld, N, slices, nslices, ldp, d, Q, cstride, E, norm2, flag);
   count_launch();
   return cudaGetLastError();
 }
 
-dgchefsi_status reduce_pair_slabs(const float* Pw, int64_t rows, int64_t cols, const int32_t* Erows,
-                                  const int32_t* Ecols, const int32_t* cmap, double* C, int64_t ldc, int s,
-                                  cudaStream_t st) {
-  if (!reduce_kernel(s)) return set_error(DGCHEFSI_ERR_ARG, "slices = %d outside 2..16", s);
-  DG_CUDA(launch_reduce(s, Pw, rows, cols, Erows, Ecols, 1, 0, 0, C, ldc, 0, cmap, st));
+dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols, int w, const PairGroups& groups,
+                                   const int32_t* Erows, const int32_t* Ecols, const int32_t* cmap, double* C,
+                                   int64_t ldc, cudaStream_t st) {
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows * cols / 4 + 255) / 256, 152 * 16));
+  digit_reduce(w)<<<grid, 256, 0, st>>>(Pw, rows, cols, cols, groups, Erows, Ecols, 1, 0, 0, C, ldc, 0, 0, 0, cmap);
+  count_launch();
+  DG_CUDA(cudaGetLastError());
   return DGCHEFSI_OK;
 }
 

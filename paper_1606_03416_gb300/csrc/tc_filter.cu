@@ -4,6 +4,7 @@
 // tc_kernel.cuh (instantiated in tc_tf32.cu, tc_bf16.cu, tc_bf16x3.cu).
 #include <algorithm>
 #include <cmath>
+#include <iterator>
 #include <map>
 
 #include "tc_kernel.cuh"
@@ -263,19 +264,20 @@ struct TcState {
   int coefb_cap = 0;
   int g_stride = 0, g_nseg = 0, g_mG = 0, g_mT = 0, g_mL = 0, g_mm = 0;
   std::vector<float*> cp0, cp1, segb;
-  // H X from BF16 slices (tc_sliced_matvec): H's digits in the W = 64 operand
-  // layout (s copies), the states' digits (s copies, element-padded), the
-  // FP32 slice-pair slabs of one state panel, the exponents and the padded
-  // column map
+  // H X from BF16 digits (tc_sliced_matvec): H's digits in the W = 64 operand
+  // layout (d copies), the states' digits (d copies, element-padded), the
+  // INT32 slabs of one state panel, the exponents, the padded column map and
+  // slice table, and the largest digit norms of H and of the states
   struct {
     bool layout = false, h_built = false;
-    int h_slices = 0;
+    int h_digits = 0, nslices = 0;
     std::vector<int64_t> brow_h;
     int64_t b_rows = 0, zero_row = 0, max_row_len = 0;
     int64_t* brow_d = nullptr;
     int32_t* cmap_d = nullptr;
+    int4* slices_d = nullptr;
     int32_t* eh_d = nullptr;   // [ldp] H row exponents
-    double* coef_d = nullptr;  // {c = 0, alpha = 1, beta = 0}
+    uint32_t* norm_d = nullptr;  // [2][16]
     Plan plan;
     DevBuf Hs, Xs, Pw, ex;
   } sx;
@@ -360,7 +362,8 @@ static dgchefsi_status ensure_mode(dgchefsi_ctx* ctx, TcState& t, int mode) {
 }
 
 static dgchefsi_status make_plan(dgchefsi_ctx* ctx, const TcState& t, int G, int W,
-                                 const std::vector<int64_t>& brow_h, int64_t zero_row, Plan& out);
+                                 const std::vector<int64_t>& brow_h, int64_t zero_row, Plan& out,
+                                 const std::vector<int32_t>* order = nullptr);
 
 static dgchefsi_status get_plan(dgchefsi_ctx* ctx, TcState& t, int G, Plan** out) {
   auto it = t.plans.find(G);
@@ -377,15 +380,21 @@ static dgchefsi_status get_plan(dgchefsi_ctx* ctx, TcState& t, int G, Plan** out
 
 // Element groups and their slice schedules for an operand copy of H laid out
 // with W-column slices, blocks starting at rows brow_h and zero tiles at zero_row.
+// order (may be null): the elements of each group, -1 for none; else group eg
+// holds elements eg*G .. eg*G+G-1.
 static dgchefsi_status make_plan(dgchefsi_ctx* ctx, const TcState& t, int G, int W,
-                                 const std::vector<int64_t>& brow_h, int64_t zero_row, Plan& out) {
+                                 const std::vector<int64_t>& brow_h, int64_t zero_row, Plan& out,
+                                 const std::vector<int32_t>* order) {
   const int M = ctx->M;
   Plan pl;
   pl.G = G;
   pl.W = W;
-  pl.ngroups = (M + G - 1) / G;
+  pl.ngroups = order ? (int)(order->size() / G) : (M + G - 1) / G;
   std::vector<int32_t> grp((size_t)pl.ngroups * G, -1);
-  for (int K = 0; K < M; ++K) grp[K] = K;  // group eg holds elements eg*G .. eg*G+G-1
+  if (order)
+    grp = *order;
+  else
+    for (int K = 0; K < M; ++K) grp[K] = K;
   std::vector<int32_t> sched, sptr(pl.ngroups + 1, 0), gslots(pl.ngroups, 0);
   std::vector<uint8_t> nsub;
   for (int eg = 0; eg < pl.ngroups; ++eg) {
@@ -1114,14 +1123,70 @@ dgchefsi_status tc_grad_backward(dgchefsi_ctx* ctx, int prec, const double* Wm, 
 // in panels of 256-state multiples below it.
 static constexpr size_t kSlabBytes = size_t(8) << 30;
 
+// Groups of G = 2^k elements whose neighbour lists overlap most: singles are
+// merged into pairs, pairs into fours and so on, each group (in order) with the
+// unmerged one of the same level among its neighbours' that gives the smallest
+// union of neighbours. On a grid of 27-neighbour elements: pairs along x (36
+// neighbours), then 2 x 2 (48, against 54 for four in a row).
+static std::vector<int32_t> group_elements(const dgchefsi_ctx* ctx, int G) {
+  const int M = ctx->M;
+  std::vector<std::vector<int>> elems(M), nbrs(M);
+  for (int K = 0; K < M; ++K) {
+    elems[K] = {K};
+    nbrs[K].assign(ctx->col_h.begin() + ctx->row_ptr_h[K], ctx->col_h.begin() + ctx->row_ptr_h[K + 1]);
+  }
+  std::vector<int> owner(M);
+  for (int size = 1; size < G; size *= 2) {
+    const int n = (int)elems.size();
+    for (int g = 0; g < n; ++g)
+      for (int K : elems[g]) owner[K] = g;
+    std::vector<char> used(n, 0);
+    std::vector<std::vector<int>> e2, n2;
+    for (int g = 0; g < n; ++g) {
+      if (used[g]) continue;
+      used[g] = 1;
+      int best = -1;
+      size_t best_union = 0;
+      std::vector<int> u, best_u = nbrs[g];
+      for (int K : nbrs[g]) {
+        const int h = owner[K];
+        if (used[h] || h == best) continue;
+        u.clear();
+        std::set_union(nbrs[g].begin(), nbrs[g].end(), nbrs[h].begin(), nbrs[h].end(), std::back_inserter(u));
+        if (best < 0 || u.size() < best_union || (u.size() == best_union && h < best)) {
+          best = h;
+          best_union = u.size();
+          best_u = u;
+        }
+      }
+      std::vector<int> e = elems[g];
+      if (best >= 0) {
+        used[best] = 1;
+        e.resize(size, -1);
+        e.insert(e.end(), elems[best].begin(), elems[best].end());
+      }
+      e2.push_back(e);
+      n2.push_back(best_u);
+    }
+    elems.swap(e2);
+    nbrs.swap(n2);
+  }
+  std::vector<int32_t> out;
+  for (auto& e : elems) {
+    e.resize(G, -1);
+    out.insert(out.end(), e.begin(), e.end());
+  }
+  return out;
+}
+
 dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t Ns,
-                                 int s, int* flag, bool* used) {
+                                 int slices, int* flag, bool* used) {
   *used = false;
   if (Ns <= 0) {
     *used = true;
     return DGCHEFSI_OK;
   }
-  if (ctx->max_nb > 128 || s < 2 || s > 16) return DGCHEFSI_OK;
+  if (ctx->max_nb > 128 || slices < 2 || slices > 16) return DGCHEFSI_OK;
   if (!ctx->tc) ctx->tc = new TcState();
   TcState& t = *ctx->tc;
   DG_TRY(ensure_layout(ctx, t));
@@ -1129,8 +1194,9 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
   constexpr int W = 64;
   cudaStream_t st = ctx->stream;
   if (!sx.layout) {
-    // W = 64 block layout of the slice copies (the BF16 filter's), the longest
-    // row (padded columns of its neighbour blocks) and the padded column map
+    // W = 64 block layout of the digit copies (the BF16 filter's), the longest
+    // row (columns of its neighbour blocks), the padded column map, the slices
+    // of the states and the groups of elements
     sx.brow_h.resize(ctx->nnzb);
     int64_t r = 0;
     for (int64_t e = 0; e < ctx->nnzb; ++e) {
@@ -1145,109 +1211,90 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
       sx.max_row_len = std::max(sx.max_row_len, len);
     }
     std::vector<int32_t> cmap((size_t)t.ldp, -1);
-    for (int K = 0; K < ctx->M; ++K)
+    std::vector<int4> sl;
+    for (int K = 0; K < ctx->M; ++K) {
       for (int j = 0; j < ctx->nb_h[K]; ++j) cmap[(size_t)t.poff_h[K] + j] = (int32_t)(ctx->off_h[K] + j);
+      for (int j = 0; j < t.pnb_h[K]; j += W)
+        sl.push_back(make_int4(t.poff_h[K] + j, (int)ctx->off_h[K] + j, std::max(0, std::min(W, ctx->nb_h[K] - j)),
+                               std::min(W, t.pnb_h[K] - j)));
+    }
+    sx.nslices = (int)sl.size();
     DG_CUDA(cudaMalloc(&sx.brow_d, sizeof(int64_t) * std::max<int64_t>(ctx->nnzb, 1)));
     DG_CUDA(cudaMalloc(&sx.cmap_d, sizeof(int32_t) * (size_t)t.ldp));
+    DG_CUDA(cudaMalloc(&sx.slices_d, sizeof(int4) * sl.size()));
     DG_CUDA(cudaMalloc(&sx.eh_d, sizeof(int32_t) * (size_t)t.ldp));
-    DG_CUDA(cudaMalloc(&sx.coef_d, sizeof(double) * 3));
-    const double coef[3] = {0.0, 1.0, 0.0};
+    DG_CUDA(cudaMalloc(&sx.norm_d, sizeof(uint32_t) * 32));
     DG_CUDA(cudaMemcpy(sx.brow_d, sx.brow_h.data(), sizeof(int64_t) * ctx->nnzb, cudaMemcpyHostToDevice));
     DG_CUDA(cudaMemcpy(sx.cmap_d, cmap.data(), sizeof(int32_t) * (size_t)t.ldp, cudaMemcpyHostToDevice));
-    DG_CUDA(cudaMemcpy(sx.coef_d, coef, sizeof(coef), cudaMemcpyHostToDevice));
-    DG_TRY(make_plan(ctx, t, 128 / t.ACC, W, sx.brow_h, sx.zero_row, sx.plan));
+    DG_CUDA(cudaMemcpy(sx.slices_d, sl.data(), sizeof(int4) * sl.size(), cudaMemcpyHostToDevice));
+    const int G = 256 / t.ACC;
+    const std::vector<int32_t> order = group_elements(ctx, G);
+    DG_TRY(make_plan(ctx, t, G, W, sx.brow_h, sx.zero_row, sx.plan, &order));
     sx.layout = true;
   }
-  // every pair sum must stay an exact FP32 integer: at most 4096 terms per row
+  // the INT32 sums hold at most 4096 terms per row (7 pairs of one weight)
   if (sx.max_row_len > 4096) return DGCHEFSI_OK;
   if (sx.b_rows * (int64_t)W > ((int64_t)1 << 31) || Ns * t.ldp > ((int64_t)1 << 40)) return DGCHEFSI_OK;
-  const int G = 128 / t.ACC, T = 2;
-  FilterKernel kern = pick_kernel(MODE_BF16, G, T, t.ACC, 1);
-  if (!kern) return DGCHEFSI_OK;
-  // H's digits (once per H and slice count)
+  if (!pair_blocks_fit(sx.plan.maxent, t.ACC)) return DGCHEFSI_OK;
+  int d = 0, w = 0;
+  digit_counts(slices, &d, &w);
+  // H's digits (once per H and digit count)
   const int64_t hcopy = sx.b_rows * W;
-  if (!sx.h_built || sx.h_slices != s) {
-    if (sx.Hs.bytes < sizeof(__nv_bfloat16) * (size_t)(s * hcopy)) {
-      DG_TRY(ensure(ctx, sx.Hs, sizeof(__nv_bfloat16) * (size_t)(s * hcopy), "slices of H"));
+  if (!sx.h_built || sx.h_digits != d) {
+    if (sx.Hs.bytes < sizeof(__nv_bfloat16) * (size_t)(d * hcopy)) {
+      DG_TRY(ensure(ctx, sx.Hs, sizeof(__nv_bfloat16) * (size_t)(d * hcopy), "digits of H"));
       DG_CUDA(cudaMemsetAsync(sx.Hs.p, 0, sx.Hs.bytes, st));  // zero tiles and slack rows
     }
-    DG_CUDA(slices_of_h(ctx, t.blk_row_d, t.pnb_d, t.poff_d, sx.brow_d, s, static_cast<__nv_bfloat16*>(sx.Hs.p), hcopy,
-                        sx.eh_d, flag, st));
+    DG_CUDA(cudaMemsetAsync(sx.norm_d, 0, sizeof(uint32_t) * 16, st));
+    DG_CUDA(digits_of_h(ctx, t.blk_row_d, t.pnb_d, t.poff_d, sx.brow_d, d, static_cast<__nv_bfloat16*>(sx.Hs.p), hcopy,
+                        sx.eh_d, sx.norm_d, flag, st));
     sx.h_built = true;
-    sx.h_slices = s;
+    sx.h_digits = d;
   }
   // the states' digits and exponents
   const int64_t xcopy = Ns * t.ldp;
-  DG_TRY(ensure(ctx, sx.Xs, sizeof(__nv_bfloat16) * (size_t)(s * xcopy), "slices of the states"));
+  DG_TRY(ensure(ctx, sx.Xs, sizeof(__nv_bfloat16) * (size_t)(d * xcopy), "digits of the states"));
   DG_TRY(ensure(ctx, sx.ex, sizeof(int32_t) * (size_t)Ns, "state exponents"));
   __nv_bfloat16* Xq = static_cast<__nv_bfloat16*>(sx.Xs.p);
   int32_t* ex = static_cast<int32_t*>(sx.ex.p);
-  DG_CUDA(slices_of_states(X, ldx, Ns, ctx->N, sx.cmap_d, t.ldp, s, Xq, xcopy, ex, flag, st));
+  DG_CUDA(cudaMemsetAsync(sx.norm_d + 16, 0, sizeof(uint32_t) * 16, st));
+  DG_CUDA(digits_of_states(X, ldx, Ns, ctx->N, sx.slices_d, sx.nslices, t.ldp, d, Xq, xcopy, ex, sx.norm_d + 16, flag,
+                           st));
   // state panels whose slabs fit the cap
-  const int pairs = s * (s + 1) / 2;
-  const int64_t per_state = (int64_t)pairs * t.ldp * (int64_t)sizeof(float);
+  BlockPairs B{};
+  B.groups = pair_groups(d, w, (int64_t)sx.plan.ngroups * ((Ns + 255) / 256), t.num_sms);
+  const int64_t per_state = (int64_t)B.groups.total * t.ldp * (int64_t)sizeof(int32_t);
   int64_t P = (int64_t)(kSlabBytes / (size_t)per_state) / 256 * 256;
   if (P < 256) P = 256;
   if (P > Ns) P = Ns;
   DG_TRY(ensure(ctx, sx.Pw, (size_t)per_state * (size_t)P, "slice-pair slabs"));
-  float* Pw = static_cast<float*>(sx.Pw.p);
-  // launch configuration of the transposed step kernel (layout 1, 128-byte slots)
-  const int stage_bytes = 128 * SLICE_BYTES + 256 * SLICE_BYTES;
-  const int stages = TN_RING_BYTES / stage_bytes;
-  const int smem = stages * stage_bytes + (2 * stages + 4) * 8 + 2 * sx.plan.maxent * (1 + G) * 4 + 1024;
-  if (smem > 227 * 1024) return DGCHEFSI_OK;
-  DG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  Params p{};
-  p.sched = sx.plan.sched_d;
-  p.sched_ptr = sx.plan.sched_ptr_d;
-  p.nsub = sx.plan.nsub_d;
-  p.gslots = sx.plan.gslots_d;
-  p.grp_elem = sx.plan.grp_elem_d;
-  p.nb = ctx->nb_d;
-  p.pnb = t.pnb_d;
-  p.poff = t.poff_d;
-  p.lo_rows = 0;
-  p.ldp = t.ldp;
-  p.coef = sx.coef_d;
-  p.step = 0;
-  p.W = W;
-  p.mode = MODE_BF16;
-  p.boxn = t.boxn;
-  p.G = G;
-  p.T = T;
-  p.ACC = t.ACC;
-  p.NBUF = 2;
-  p.stages = stages;
-  p.ngroups = sx.plan.ngroups;
-  p.maxent = sx.plan.maxent;
-  p.err = t.err_d;
-  p.Hout = nullptr;
-  p.Lout = nullptr;
-  DG_CUDA(cudaMemsetAsync(t.err_d, 0, sizeof(int), st));
-  std::vector<CUtensorMap> hmap(s);
-  for (int i = 0; i < s; ++i)
-    DG_TRY(make_map(&hmap[i], static_cast<__nv_bfloat16*>(sx.Hs.p) + (size_t)i * hcopy, false, (uint64_t)W,
-                    (uint64_t)sx.b_rows, (uint32_t)W, (uint32_t)t.boxn));
+  int32_t* Pw = static_cast<int32_t*>(sx.Pw.p);
+  B.Hs = static_cast<const __nv_bfloat16*>(sx.Hs.p);
+  B.Xs = Xq;
+  B.hcopy = hcopy;
+  B.h_rows = sx.b_rows;
+  B.xcopy = xcopy;
+  B.Ns = Ns;
+  B.ldp = t.ldp;
+  B.s = d;
+  B.nw = w;
+  B.acc = t.ACC;
+  B.ngroups = sx.plan.ngroups;
+  B.maxent = sx.plan.maxent;
+  B.norm_h = sx.norm_d;
+  B.norm_x = sx.norm_d + 16;
+  B.sched = sx.plan.sched_d;
+  B.sched_ptr = sx.plan.sched_ptr_d;
+  B.grp_elem = sx.plan.grp_elem_d;
+  B.pnb = t.pnb_d;
+  B.poff = t.poff_d;
+  DG_TRY(pair_products_begin(ctx));
   for (int64_t s0 = 0; s0 < Ns; s0 += P) {
     const int64_t pn = std::min<int64_t>(P, Ns - s0);
-    p.Ns = pn;
-    p.ntg = (int)((pn + 255) / 256);
-    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)p.ngroups * p.ntg, t.num_sms);
-    for (int j = 0; j < s; ++j) {
-      CUtensorMap xmap;
-      DG_TRY(make_map(&xmap, Xq + (size_t)j * xcopy + (size_t)s0 * t.ldp, false, (uint64_t)t.ldp, (uint64_t)pn,
-                      (uint32_t)W, 256u));
-      for (int i = 0; i + j < s; ++i) {
-        p.Fout = Pw + (size_t)(i * s - i * (i - 1) / 2 + j) * (size_t)(pn * t.ldp);
-        p.Fprev = p.Fout;
-        kern<<<grid, NTHREADS, smem, st>>>(xmap, xmap, hmap[i], p);
-        count_launch();
-        DG_CUDA(cudaGetLastError());
-      }
-    }
-    DG_TRY(reduce_pair_slabs(Pw, pn, t.ldp, ex + s0, sx.eh_d, sx.cmap_d, Y + s0 * ldy, ldy, s, st));
+    DG_TRY(pair_products_blocks(ctx, B, s0, pn, Pw));
+    DG_TRY(reduce_digit_slabs(Pw, pn, t.ldp, w, B.groups, ex + s0, sx.eh_d, sx.cmap_d, Y + s0 * ldy, ldy, st));
   }
-  DG_TRY(check_err(t, st));
+  DG_TRY(pair_products_status(ctx));
   *used = true;
   return DGCHEFSI_OK;
 }
@@ -1323,7 +1370,8 @@ void tc_destroy(dgchefsi_ctx* ctx) {
   cudaFree(t.sx.brow_d);
   cudaFree(t.sx.cmap_d);
   cudaFree(t.sx.eh_d);
-  cudaFree(t.sx.coef_d);
+  cudaFree(t.sx.slices_d);
+  cudaFree(t.sx.norm_d);
   cudaFree(t.sx.Hs.p);
   cudaFree(t.sx.Xs.p);
   cudaFree(t.sx.Pw.p);
