@@ -61,6 +61,7 @@ struct dgchefsi_ctx {
   dg::DevBuf ws_sliced_t;  // transposed left operand of the A^T B form
   dg::DevBuf ws_sliced_b;  // transposed right operand of the A B form
   dg::DevBuf ws_pairs;     // tensor maps, pair and tile lists of the slice-pair kernel (regrown as needed)
+  bool pairs_deferred = false;  // sliced products only enqueue (see sliced_gemm)
   dg::DevBuf ws_pairs_err; // the slice-pair kernel's error word (its own buffer: never regrown mid-product)
   // the slab reduction of the sliced products runs on its own stream, one K
   // chunk behind the slice-pair kernel (double-buffered slabs)
@@ -174,10 +175,13 @@ void tc_destroy(dgchefsi_ctx* ctx);
 // zero and not read. flag (device int) gets 1 if an operand is not finite.
 // tri > 0: only the entries C[r, c] with c <= r mod tri are computed (the lower
 // triangle of a symmetric result, or of each of M / tri stacked ones); the
-// others are left as they were.
+// others are left as they were. subtract: C -= the product; negate: C = -product.
+// Inside a run with ctx->pairs_deferred set (by a caller that has called
+// pair_products_begin) the call is only enqueued, and the caller asks
+// pair_products_status for all of them at the end.
 dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_t M, int64_t Nc, int64_t K,
                             const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc, int s,
-                            int* flag, int64_t tri = 0);
+                            int* flag, int64_t tri = 0, bool subtract = false, bool negate = false);
 // C (M x Nc) = A^T B with A (K x M, lda) and B (K x Nc, ldb) row-major: A is
 // transposed into a library buffer, then the A B form above.
 dgchefsi_status sliced_gemm_tn(dgchefsi_ctx* ctx, int64_t M, int64_t Nc, int64_t K, const double* A, int64_t lda,

@@ -284,7 +284,7 @@ __device__ __forceinline__ double scale_pow2(double h, int e) {
   return ldexp(h, e);
 }
 
-// C[r, n0 + c] (+)= 2^{e_r + f_{n0+c} - 16} sum_t 2^{-9t} g_t for r < M, c < P,
+// C[r, n0 + c] (+)= (+-) 2^{e_r + f_{n0+c} - 16} sum_t 2^{-9t} g_t for r < M, c < P,
 // g_t the sum of weight t's count[t] INT32 slabs (M rows of `pitch` entries, t
 // descending). Four consecutive t are combined in INT64 (|g_t| < 2^32, so the
 // block is below 2^60) and converted to FP64, and the blocks meet by Horner in
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict_
                                                       int64_t pitch, const PairGroups groups,
                                                       const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb,
                                                       int nch, int chunk, int64_t n0, double* __restrict__ C,
-                                                      int64_t ldc, int wide, int accumulate, int64_t tri,
-                                                      const int32_t* __restrict__ cmap) {
+                                                      int64_t ldc, int wide, int accumulate, int negate,
+                                                      int64_t tri, const int32_t* __restrict__ cmap) {
   constexpr int NB = (W + 3) / 4;
   const int64_t slab = M * pitch, quads = pitch / 4, total = M * quads;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict_
         for (int t = 4 * b; t < 4 * b + 4; ++t) B = B * 512 + (t < W ? g[e][t] : 0);
         h = b == NB - 1 ? (double)B : h * 0x1p-36 + (double)B;
       }
-      y[e] = c0 + e < P ? scale_pow2(h, er + Eb[(n0 + c0 + e) * nch + chunk]) : 0.0;
+      y[e] = c0 + e < P ? scale_pow2(negate ? -h : h, er + Eb[(n0 + c0 + e) * nch + chunk]) : 0.0;
     }
     if (cmap) {
 #pragma unroll
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict_
 }
 
 typedef void (*DigitReduce)(const int32_t*, int64_t, int64_t, int64_t, const PairGroups, const int32_t*,
-                            const int32_t*, int, int, int64_t, double*, int64_t, int, int, int64_t,
+                            const int32_t*, int, int, int64_t, double*, int64_t, int, int, int, int64_t,
                             const int32_t*);
 
 static DigitReduce digit_reduce(int w) {
@@ -436,12 +436,13 @@ static dgchefsi_status transpose_f64(const double* X, int64_t ldx, int64_t rows,
 
 dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_t M, int64_t Nc, int64_t K,
                             const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
-                            int slices, int* flag, int64_t tri) {
+                            int slices, int* flag, int64_t tri, bool subtract, bool negate) {
   if (M <= 0 || Nc <= 0) return DGCHEFSI_OK;
   if (slices < 2 || slices > 16) return set_error(DGCHEFSI_ERR_ARG, "slices = %d outside 2..16", slices);
   const int s = digits_for(slices), nw = weights_for(slices);
   cudaStream_t st = ctx->stream;
   if (K <= 0) {
+    if (subtract) return DGCHEFSI_OK;
     DG_CUDA(cudaMemset2DAsync(C, sizeof(double) * ldc, 0, sizeof(double) * Nc, M, st));
     return DGCHEFSI_OK;
   }
@@ -520,7 +521,7 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
     count_launch();
     DG_CUDA(cudaGetLastError());
   }
-  DG_TRY(pair_products_begin(ctx));
+  if (!ctx->pairs_deferred) DG_TRY(pair_products_begin(ctx));
   cudaStream_t sr = st;
   if (multi) {
     if (!ctx->s_reduce) {
@@ -565,7 +566,8 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
       const int64_t pitch = round_up(pn, 4), work = M * pitch / 4;
       const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 16));
       digit_reduce(nw)<<<grid, 256, 0, sr>>>(Pb, M, pn, pitch, groups, Ea, Eb, nch, chunk, n0, C, ldc,
-                                            wide(C, ldc) ? 1 : 0, chunk > 0 ? 1 : 0, tri, nullptr);
+                                            wide(C, ldc) ? 1 : 0, subtract || chunk > 0 ? 1 : 0, subtract || negate ? 1 : 0, tri,
+                                            nullptr);
       count_launch();
       DG_CUDA(cudaGetLastError());
       if (multi) DG_CUDA(cudaEventRecord(ctx->ev_reduce[b], sr));
@@ -575,7 +577,8 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
     DG_CUDA(cudaEventRecord(ctx->ev_reduce[0], sr));
     DG_CUDA(cudaStreamWaitEvent(st, ctx->ev_reduce[0], 0));
   }
-  DG_TRY(pair_products_status(ctx));  // synchronises the stream
+  if (ctx->pairs_deferred) return DGCHEFSI_OK;  // the caller asks once for several products
+  DG_TRY(pair_products_status(ctx));            // synchronises the stream
   double ms = 0.0;
   for (int q = 0; q < step; ++q) {
     float t = 0.f;
@@ -761,7 +764,7 @@ dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols
                                    const int32_t* Erows, const int32_t* Ecols, const int32_t* cmap, double* C,
                                    int64_t ldc, cudaStream_t st) {
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows * cols / 4 + 255) / 256, 152 * 16));
-  digit_reduce(w)<<<grid, 256, 0, st>>>(Pw, rows, cols, cols, groups, Erows, Ecols, 1, 0, 0, C, ldc, 0, 0, 0, cmap);
+  digit_reduce(w)<<<grid, 256, 0, st>>>(Pw, rows, cols, cols, groups, Erows, Ecols, 1, 0, 0, C, ldc, 0, 0, 0, 0, cmap);
   count_launch();
   DG_CUDA(cudaGetLastError());
   return DGCHEFSI_OK;
