@@ -250,47 +250,29 @@ static dgchefsi_status bounds_impl(dgchefsi_ctx* ctx, const double* v0, int k, d
   const int64_t N = ctx->N;
   if (k > N) k = (int)N;
   const size_t nvec = (size_t)k + 1;
-  DG_TRY(ensure(ctx, ctx->ws_lanczos, sizeof(double) * (nvec * (size_t)N + (size_t)N + 72), "Lanczos basis"));
+  const size_t npart = 65 * (size_t)LZ_MAX_CTAS;
+  DG_TRY(ensure(ctx, ctx->ws_lanczos, sizeof(double) * (nvec * (size_t)N + (size_t)N + npart + 130), "Lanczos basis"));
   double* V = static_cast<double*>(ctx->ws_lanczos.p);
   double* w = V + nvec * (size_t)N;
-  double* sc = w + N;  // device scalars [72]
+  double* part = w + N;
+  double* out = part + npart;
   cudaStream_t s = ctx->stream;
-  double host[72];
-  auto fetch = [&](int n) -> dgchefsi_status {
-    DG_CUDA(cudaMemcpyAsync(host, sc, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
-    DG_CUDA(cudaStreamSynchronize(s));
-    return DGCHEFSI_OK;
-  };
-  DG_CUDA(dots_f64(v0, 0, 1, v0, N, sc, s));
-  DG_TRY(fetch(1));
-  const double nrm = std::sqrt(host[0]);
+  double host[130];
+  DG_CUDA(lanczos_f64(ctx->view(), v0, k, V, w, part, ctx->n_values, out, s));
+  DG_CUDA(cudaMemcpyAsync(host, out, sizeof(double) * (size_t)(2 + 2 * k), cudaMemcpyDeviceToHost, s));
+  DG_CUDA(cudaStreamSynchronize(s));
+  const double nrm = host[0];
   if (!(nrm > 0.0) || !std::isfinite(nrm)) return set_error(DGCHEFSI_ERR_ARG, "Lanczos start vector is zero or not finite");
-  DG_CUDA(axpby_f64(1.0 / nrm, v0, 0.0, v0, V, N, s));
+  const int steps = (int)host[1];
   std::vector<double> al, be;
-  double beta_prev = 0.0, beta_last = 0.0;
-  const HView h = ctx->view();
-  for (int j = 0; j < k; ++j) {
-    double* vj = V + (size_t)j * N;
-    DG_CUDA(spmv_f64(h, vj, w, s));
-    if (j > 0) DG_CUDA(axpby_f64(-beta_prev, vj - N, 1.0, w, w, N, s));
-    DG_CUDA(dots_f64(vj, 0, 1, w, N, sc, s));
-    DG_TRY(fetch(1));
-    const double alpha = host[0];
-    DG_CUDA(axpby_f64(-alpha, vj, 1.0, w, w, N, s));
-    DG_CUDA(dots_f64(V, N, j + 1, w, N, sc, s));
-    DG_CUDA(sub_combination_f64(w, V, N, sc, j + 1, N, s));
-    DG_CUDA(dots_f64(w, 0, 1, w, N, sc + 64, s));
-    DG_CUDA(cudaMemcpyAsync(host, sc + 64, sizeof(double), cudaMemcpyDeviceToHost, s));
-    DG_CUDA(cudaStreamSynchronize(s));
-    const double beta = std::sqrt(host[0]);
-    al.push_back(alpha);
-    beta_last = beta;
+  double beta_last = 0.0;
+  for (int j = 0; j < steps; ++j) {
+    const double alpha = host[2 + 2 * j], beta = host[3 + 2 * j];
     if (!std::isfinite(alpha) || !std::isfinite(beta))
       return set_error(DGCHEFSI_ERR_NONFINITE, "Lanczos produced a non-finite coefficient");
-    if (j == k - 1 || beta == 0.0) break;
-    be.push_back(beta);
-    DG_CUDA(axpby_f64(1.0 / beta, w, 0.0, w, vj + N, N, s));
-    beta_prev = beta;
+    al.push_back(alpha);
+    beta_last = beta;
+    if (j + 1 < steps) be.push_back(beta);
   }
   const int n = (int)al.size();
   const double tmax = tridiag_eig(al, be, n);

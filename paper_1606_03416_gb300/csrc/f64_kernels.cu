@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cooperative_groups.h>
 
 #include "f64_tile.cuh"
 #include "internal.h"
@@ -98,11 +99,12 @@ __global__ void __launch_bounds__(NT) k_filter_step_f64(HView h, const double* _
   }
 }
 
-// y = H x: one warp per row of H, lanes stride over each neighbour block's row.
-__global__ void k_spmv_f64(HView h, const double* __restrict__ x, double* __restrict__ y) {
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Row `row` of H times x, by one warp (the sum in every lane). The lanes fetch
+// the descriptors of up to 32 neighbour blocks at once, so that the loads of
+// the blocks' rows, not a chain of descriptor loads per block, are in flight.
+// (x is no __restrict__ pointer: the Lanczos kernel reads what other CTAs wrote.)
+__device__ __forceinline__ double warp_row_product(const HView& h, const double* x, int64_t row) {
   const int lane = threadIdx.x & 31;
-  if (row >= h.N) return;
   int lo = 0, hi = h.M;  // find K with off[K] <= row < off[K+1]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -111,16 +113,59 @@ __global__ void k_spmv_f64(HView h, const double* __restrict__ x, double* __rest
   const int K = lo;
   const int j = (int)(row - h.off[K]);
   double sum = 0.0;
-  for (int64_t e = h.row_ptr[K]; e < h.row_ptr[K + 1]; ++e) {
-    const int Kp = h.col[e];
-    const int nKp = h.nb[Kp];
-    const double* brow = h.vals + h.blk_off[e] + (int64_t)j * nKp;
-    const double* xs = x + h.off[Kp];
-    for (int jp = lane; jp < nKp; jp += 32) sum = fma(brow[jp], xs[jp], sum);
+  const int64_t e1 = h.row_ptr[K + 1];
+  for (int64_t e0 = h.row_ptr[K]; e0 < e1; e0 += 32) {
+    const int cnt = e1 - e0 < 32 ? (int)(e1 - e0) : 32;
+    int n = 0;
+    const double *brow = nullptr, *xs = nullptr;
+    if (lane < cnt) {
+      const int Kp = h.col[e0 + lane];
+      n = h.nb[Kp];
+      brow = h.vals + h.blk_off[e0 + lane] + (int64_t)j * n;
+      xs = x + h.off[Kp];
+    }
+    for (int q0 = 0; q0 < cnt; q0 += 4) {  // four blocks' loads, then their multiply-adds
+      double bv[4][2], xv[4][2];
+      int nq[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = min(q0 + u, cnt - 1);
+        nq[u] = __shfl_sync(0xffffffffu, n, q);
+        const double* bq = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(brow), q));
+        const double* xq = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(xs), q));
+        if (q0 + u >= cnt) nq[u] = 0;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const bool in = lane + 32 * c < nq[u];
+          bv[u][c] = in ? bq[lane + 32 * c] : 0.0;
+          xv[u][c] = in ? xq[lane + 32 * c] : 0.0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (nq[u] > 0) sum = fma(bv[u][0], xv[u][0], sum);
+        if (nq[u] > 32) sum = fma(bv[u][1], xv[u][1], sum);
+      }
+    }
+    if (__any_sync(0xffffffffu, n > 64))  // elements of more than 64 functions: the rest of their rows
+      for (int q = 0; q < cnt; ++q) {
+        const int nq = __shfl_sync(0xffffffffu, n, q);
+        const double* bq = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(brow), q));
+        const double* xq = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(xs), q));
+        for (int jp = lane + 64; jp < nq; jp += 32) sum = fma(bq[jp], xq[jp], sum);
+      }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (lane == 0) y[row] = sum;
+  return sum;
+}
+
+// y = H x: one warp per row of H.
+__global__ void k_spmv_f64(HView h, const double* __restrict__ x, double* __restrict__ y) {
+  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (row >= h.N) return;
+  const double sum = warp_row_product(h, x, row);
+  if ((threadIdx.x & 31) == 0) y[row] = sum;
 }
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
@@ -158,6 +203,125 @@ __global__ void k_sub_combination_f64(double* __restrict__ w, const double* __re
 __global__ void k_axpby_f64(double a, const double* __restrict__ x, double b, const double* y, double* yo, int64_t n) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     yo[i] = a * x[i] + b * y[i];
+}
+
+// All k Lanczos steps with full re-orthogonalisation in one cooperative launch
+// (a step by launches: ~8 of them and two host round trips, 65 us on a 256-row
+// H). Each CTA owns a range of rows of every vector; what crosses CTAs are the
+// dot products: each CTA writes its part to `part` (entry l of CTA b at l * grid
+// + b), and after a grid barrier every CTA adds the parts in the same order, so
+// all hold the same bits. Per step: w = H v_j - beta v_{j-1}, alpha = v_j . w |
+// w -= alpha v_j, c = V^T w | w -= V c, beta = |w| | v_{j+1} = w / beta, with a
+// barrier at each bar. V: k + 1 vectors, w: one. out: [0] |v0|, [1] steps taken,
+// [2 + 2 j] alpha_j, [3 + 2 j] beta_j. Stops after a zero or non-finite beta.
+// Bound by the row products (0.45 GB and 57 M multiply-adds per step on the
+// 8x8x8 H, ~0.1 ms of the FP64 pipe) or, on small H, by the barriers.
+// FP64 adds are few and far between: one warp adds the parts, takes the root and
+// the reciprocal for its CTA (a warp's FP64 instruction takes 16 clocks of the
+// SM whatever its lanes do, ~150 until its result can be used).
+constexpr int LZ_THREADS = 1024;
+
+__device__ __forceinline__ double lz_warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sum of entry l's parts, by one warp.
+__device__ __forceinline__ double lz_total(const double* part, int l) {
+  double v = 0.0;
+  for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32) v += __ldcg(part + (int64_t)l * gridDim.x + b);
+  return lz_warp_sum(v);
+}
+
+__global__ void __launch_bounds__(LZ_THREADS, 1) k_lanczos_f64(HView h, const double* __restrict__ v0, int k, double* V,
+                                                               double* w, double* part, double* out) {
+  namespace cg = cooperative_groups;
+  cg::grid_group grid = cg::this_grid();
+  __shared__ double red[LZ_THREADS / 32], coef[64], tot[2];
+  const int64_t N = h.N;
+  const int64_t r0 = N * blockIdx.x / gridDim.x, r1 = N * (blockIdx.x + 1) / gridDim.x;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nt = blockDim.x, nw = nt >> 5;
+  const bool first = blockIdx.x == 0 && t == 0;
+  // tot[0] = the total of a dot product of which v is this thread's part, or its
+  // root and tot[1] the reciprocal of that
+  auto all_sum = [&](double v, bool root) {
+    v = lz_warp_sum(v);
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+      const double p = lz_warp_sum(lane < nw ? red[lane] : 0.0);
+      if (lane == 0) __stcg(part + blockIdx.x, p);
+    }
+    grid.sync();
+    if (warp == 0) {
+      double s = lz_total(part, 0);
+      if (root) s = sqrt(s);
+      if (lane == 0) {
+        tot[0] = s;
+        if (root) tot[1] = 1.0 / s;
+      }
+    }
+    __syncthreads();
+  };
+  double s = 0.0;
+  for (int64_t i = r0 + t; i < r1; i += nt) s = fma(v0[i], v0[i], s);
+  all_sum(s, true);
+  const double nrm = tot[0];
+  if (first) {
+    out[0] = nrm;
+    out[1] = 0.0;
+  }
+  if (!(nrm > 0.0) || !isfinite(nrm)) return;  // the same in every CTA
+  double inv = tot[1], beta = 0.0;
+  for (int64_t i = r0 + t; i < r1; i += nt) V[i] = v0[i] * inv;
+  for (int j = 0; j < k; ++j) {
+    const double* vj = V + (int64_t)j * N;
+    grid.sync();  // v_j complete, and the parts of the last total read
+    s = 0.0;
+    for (int64_t i = r0 + warp; i < r1; i += nw) {
+      double y = warp_row_product(h, vj, i);
+      if (lane == 0) {
+        if (j > 0) y -= beta * vj[i - N];
+        w[i] = y;
+        s = fma(vj[i], y, s);
+      }
+    }
+    all_sum(s, false);
+    const double alpha = tot[0];
+    for (int64_t i = r0 + t; i < r1; i += nt) w[i] -= alpha * vj[i];
+    __syncthreads();
+    for (int l = warp; l <= j; l += nw) {  // parts 1 .. j + 1: entry 0 may still be read
+      double c = 0.0;
+      for (int64_t i = r0 + lane; i < r1; i += 32) c = fma(V[(int64_t)l * N + i], w[i], c);
+      c = lz_warp_sum(c);
+      if (lane == 0) __stcg(part + (int64_t)(l + 1) * gridDim.x + blockIdx.x, c);
+    }
+    grid.sync();
+    for (int l = warp; l <= j; l += nw) {
+      const double c = lz_total(part, l + 1);
+      if (lane == 0) coef[l] = c;
+    }
+    __syncthreads();
+    s = 0.0;
+    for (int64_t i = r0 + t; i < r1; i += nt) {
+      double acc = 0.0;
+      for (int l = 0; l <= j; ++l) acc = fma(coef[l], V[(int64_t)l * N + i], acc);
+      const double x = w[i] - acc;
+      w[i] = x;
+      s = fma(x, x, s);
+    }
+    all_sum(s, true);
+    beta = tot[0];
+    inv = tot[1];
+    if (first) {
+      out[1] = j + 1;
+      out[2 + 2 * j] = alpha;
+      out[3 + 2 * j] = beta;
+    }
+    if (j == k - 1 || beta == 0.0 || !isfinite(alpha) || !isfinite(beta)) return;  // the same in every CTA
+    for (int64_t i = r0 + t; i < r1; i += nt) V[(int64_t)(j + 1) * N + i] = w[i] * inv;
+  }
 }
 
 // C[i,j] = sum_r A[i,r] B[j,r]; lower_only: the entries j <= i, mirrored. With
@@ -373,10 +537,20 @@ __device__ __forceinline__ double fermi(double x) {
   return 1.0 / (1.0 + exp(x));
 }
 
-// Fermi level by bisection and occupations; one CTA of 256 threads.
+// Fermi level by bisection and occupations, by one cluster of up to 8 CTAs of
+// 256 threads. Each CTA sums the occupations of its share of the states; the
+// parts meet through distributed shared memory in one order, so every CTA takes
+// the same branch. Bound by the FP64 exponentials of ~45 halvings (one SM does
+// two multiply-adds per clock: 1.71 ms for 4096 states on one CTA that took the
+// exponential of every state), so a state further than 45 kT from the level
+// counts as 0 or 1, off by e^-45 < 2^-64, in the halvings.
+constexpr int OCC_CTAS = 8;
 __global__ void __launch_bounds__(256) k_occupations_f64(const double* __restrict__ lam, int64_t Ns, double Ne,
                                                         double kT, double* __restrict__ f, double* __restrict__ mu_out) {
-  __shared__ double red[256];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int nct = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  __shared__ double red[256], part[2];
   double vmin = INFINITY, vmax = -INFINITY;
   for (int64_t i = threadIdx.x; i < Ns; i += blockDim.x) {
     vmin = fmin(vmin, lam[i]);
@@ -399,17 +573,32 @@ __global__ void __launch_bounds__(256) k_occupations_f64(const double* __restric
   double hi = red[0] + 50.0 * kT;
   __syncthreads();
   const double tol = 1e-13 * Ne;
+  // Ns states off by e^-45 each are below tol / 100 unless almost nothing is occupied
+  const double far = Ne >= 1e-4 * (double)Ns ? 45.0 * kT : INFINITY;
   double mu = 0.5 * (lo + hi);
+  const int64_t first = (int64_t)rank * blockDim.x + threadIdx.x, step = (int64_t)nct * blockDim.x;
   for (int it = 0; it < 200; ++it) {
     mu = 0.5 * (lo + hi);
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < Ns; i += blockDim.x) s += fermi((lam[i] - mu) / kT);
-    const double count = 2.0 * block_sum(s, red);
+    for (int64_t i = first; i < Ns; i += step) {
+      const double x = lam[i] - mu;
+      if (x < -far)
+        s += 1.0;
+      else if (!(x > far))
+        s += fermi(x / kT);
+    }
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) part[it & 1] = s;  // the other buffer may still be read
+    cl.sync();
+    double total = 0.0;
+    for (int c = 0; c < nct; ++c) total += *cl.map_shared_rank(&part[it & 1], c);
+    const double count = 2.0 * total;
     if (fabs(count - Ne) <= tol) break;
     if (count < Ne) lo = mu; else hi = mu;
   }
-  for (int64_t i = threadIdx.x; i < Ns; i += blockDim.x) f[i] = fermi((lam[i] - mu) / kT);
-  if (threadIdx.x == 0) *mu_out = mu;
+  for (int64_t i = first; i < Ns; i += step) f[i] = fermi((lam[i] - mu) / kT);
+  if (rank == 0 && threadIdx.x == 0) *mu_out = mu;
+  cl.sync();  // no CTA leaves while another reads its part
 }
 
 __global__ void k_shift_diag_f64(double* A, int64_t n, double coef) {
@@ -617,6 +806,24 @@ cudaError_t spmv_f64(const HView& h, const double* x, double* y, cudaStream_t s)
   return cudaGetLastError();
 }
 
+cudaError_t lanczos_f64(const HView& h, const double* v0, int k, double* V, double* w, double* part, int64_t nnz,
+                        double* out, cudaStream_t s) {
+  // one CTA per 8 rows (or 16 K entries of H), at most one per SM; a warp per row
+  // while there are few, else 1024 threads for the loads in flight
+  int64_t g = std::min<int64_t>(std::max<int64_t>(nnz / 16384, h.N / 8) + 1, LZ_MAX_CTAS);
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  g = std::max<int64_t>(1, std::min<int64_t>(g, nsm));
+  HView hv = h;
+  void* args[] = {&hv, &v0, &k, &V, &w, &part, &out};
+  const unsigned threads = h.N / g <= 8 ? 256 : LZ_THREADS;
+  e = cudaLaunchCooperativeKernel((const void*)k_lanczos_f64, dim3((unsigned)g), dim3(threads), args, 0, s);
+  count_launch();
+  return e;
+}
+
 cudaError_t dots_f64(const double* V, int64_t ldv, int nv, const double* w, int64_t n, double* out, cudaStream_t s) {
   if (nv <= 0) return cudaSuccess;
   k_dots_f64<<<nv, 256, 0, s>>>(V, ldv, w, n, out);
@@ -698,9 +905,21 @@ cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, cons
 
 cudaError_t occupations_f64(const double* ritz, int64_t Ns, double Ne, double kT, double* f, double* mu,
                             cudaStream_t s) {
-  k_occupations_f64<<<1, 256, 0, s>>>(ritz, Ns, Ne, kT, f, mu);
+  // one CTA per 256 states up to a cluster of 8
+  const unsigned ctas = (unsigned)std::max<int64_t>(1, std::min<int64_t>(OCC_CTAS, (Ns + 255) / 256));
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = ctas;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_occupations_f64, ritz, Ns, Ne, kT, f, mu);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t shift_diagonal_by_trace_f64(double* A, int64_t n, double coef, cudaStream_t s) {

@@ -51,6 +51,13 @@ cudaError_t preload_lanczos_kernels();
 // y = H x for one vector (Lanczos).
 cudaError_t spmv_f64(const HView& h, const double* x, double* y, cudaStream_t s);
 
+// k Lanczos steps (k <= 64) from v0 in one cooperative launch. V: (k + 1) N, w:
+// N, part: 65 LZ_MAX_CTAS, out: 2 + 2 k doubles, all device; nnz: stored entries
+// of H. out: |v0|, steps taken, then alpha_j, beta_j.
+constexpr int LZ_MAX_CTAS = 256;
+cudaError_t lanczos_f64(const HView& h, const double* v0, int k, double* V, double* w, double* part, int64_t nnz,
+                        double* out, cudaStream_t s);
+
 // out[l] = V_l . w for l < nv, V_l = V + l*ldv (deterministic block reductions).
 cudaError_t dots_f64(const double* V, int64_t ldv, int nv, const double* w, int64_t n, double* out, cudaStream_t s);
 // w -= sum_l coef[l] V_l   (coef on the device)
