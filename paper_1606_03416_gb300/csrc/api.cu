@@ -282,7 +282,8 @@ static dgchefsi_status bounds_impl(dgchefsi_ctx* ctx, const double* v0, int k, d
   return DGCHEFSI_OK;
 }
 
-static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t ld, double* ritz) {
+// X_new goes to `out` (row stride ld): Y itself, or a block that does not overlap it.
+static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t ld, double* ritz, double* out) {
   const int64_t N = ctx->N;
   cudaStream_t s = ctx->stream;
   DG_TRY(ensure(ctx, ctx->ws_rr, sizeof(double) * (size_t)Ns * (size_t)N, "Rayleigh-Ritz block"));
@@ -376,9 +377,9 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
   DG_TRY(subspace_eigh(ctx, S, Ns, Ns, ritz));
   // Step 5: X_new^T = Q^T Y_hat^T (column-major Q read row-major is Q^T).
   if (sl)
-    DG_TRY(sliced_gemm(ctx, false, false, Ns, N, Ns, S, Ns, W, N, Y, ld, ctx->products_slices, bad));
+    DG_TRY(sliced_gemm(ctx, false, false, Ns, N, Ns, S, Ns, W, N, out, ld, ctx->products_slices, bad));
   else
-    DG_CUDA(gemm_nn_f64(S, Ns, W, N, Y, ld, Ns, N, Ns, false, s));
+    DG_CUDA(gemm_nn_f64(S, Ns, W, N, out, ld, Ns, N, Ns, false, s));
   DG_CUDA(check_finite_f64(ritz, Ns, ctx->info_d + 3, s));
   DG_CUDA(cudaMemcpyAsync(info, ctx->info_d, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
   DG_CUDA(cudaStreamSynchronize(s));
@@ -1018,7 +1019,7 @@ dgchefsi_status dgchefsi_rayleigh_ritz(dgchefsi_ctx* ctx, double* Y, int64_t Ns,
   if (Ns > ctx->N) return set_error(DGCHEFSI_ERR_ARG, "Ns (%lld) > N (%lld)", (long long)Ns, (long long)ctx->N);
   if (Ns > 2147483647LL) return set_error(DGCHEFSI_ERR_UNSUPPORTED, "Ns too large for the dense eigensolver");
   if (Ns == 0) return DGCHEFSI_OK;
-  return rr_impl(ctx, Y, Ns, ld, ritz);
+  return rr_impl(ctx, Y, Ns, ld, ritz, Y);
 }
 
 dgchefsi_status dgchefsi_occupations(dgchefsi_ctx* ctx, const double* ritz, int64_t Ns, double Ne, double kT,
@@ -1085,9 +1086,7 @@ dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t N
     DG_TRY(filter_f64(ctx, X, Yw, Ns, ld, m, a, b, a0));
   else
     DG_TRY(filter_tc(ctx, prec, X, Yw, Ns, ld, m, a, b, a0));
-  DG_TRY(rr_impl(ctx, Yw, Ns, ld, ritz));
-  DG_CUDA(cudaMemcpy2DAsync(X, sizeof(double) * ld, Yw, sizeof(double) * ld, sizeof(double) * ctx->N, Ns,
-                            cudaMemcpyDeviceToDevice, ctx->stream));
+  DG_TRY(rr_impl(ctx, Yw, Ns, ld, ritz, X));
   DG_CUDA(occupations_f64(ritz, Ns, Ne, kT, f, mu, ctx->stream));
   Parts parts;
   DG_TRY(parts_of(ctx, &parts));
