@@ -86,16 +86,17 @@ __device__ __forceinline__ int warp_max(int v) {
   return v;
 }
 
-// C = 2 or 4 consecutive digits (|x| <= 256) to q as BF16, their squares to *norm.
+// C = 2 or 4 consecutive digits (integers, |f| <= 256) to q as BF16, their squares to *norm.
 template <int C>
-__device__ __forceinline__ void put_digits(const int (&x)[C], __nv_bfloat16* __restrict__ q, bool store,
+__device__ __forceinline__ void put_digits(const float (&f)[C], __nv_bfloat16* __restrict__ q, bool store,
                                            uint32_t* norm) {
-  uint32_t w[C / 2], sq = 0;
+  uint32_t w[C / 2];
+  float sq = 8388608.f;  // 2^23: the low bits of the sum's pattern are the integer sum (below 2^19)
 #pragma unroll
   for (int c = 0; c < C; c += 2) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn((float)x[c], (float)x[c + 1]);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(f[c], f[c + 1]);
     w[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
-    sq += (uint32_t)(x[c] * x[c] + x[c + 1] * x[c + 1]);
+    sq = fmaf(f[c], f[c], fmaf(f[c + 1], f[c + 1], sq));
   }
   if (store) {
     if (C == 4)
@@ -103,8 +104,8 @@ __device__ __forceinline__ void put_digits(const int (&x)[C], __nv_bfloat16* __r
     else
       *reinterpret_cast<uint32_t*>(q) = w[0];
   }
-  sq = __reduce_add_sync(0xffffffffu, sq);
-  if ((threadIdx.x & 31) == 0) atomicAdd(norm, sq);
+  const uint32_t sum = __reduce_add_sync(0xffffffffu, __float_as_uint(sq) & 0x7fffffu);
+  if ((threadIdx.x & 31) == 0) atomicAdd(norm, sum);
 }
 
 // Digits i = 0 .. d - 1 of C consecutive entries v 2^{b} scaled by 2^{-e}
@@ -112,38 +113,43 @@ __device__ __forceinline__ void put_digits(const int (&x)[C], __nv_bfloat16* __r
 // q + i * stride where `store`; norm[i] (shared) collects the squares of digit
 // i; every lane of the warp takes part. One store per digit.
 // d <= 7: F = round(v 2^{9d - 1}) as a 64-bit integer (|F| <= 2^62;
-// |v 2^{9d-1} - F| <= 1/2), then its balanced base-512 digits from the last one
-// up, the first the rest (|q_0| <= 256). Integer arithmetic only.
+// |v 2^{9d-1} - F| <= 1/2), then its balanced base-512 digits: with 256 added at
+// the weight of every digit but the first, digit i + 256 is a 9-bit field of the
+// sum and the first digit its rest (|q_0| <= 256). Each field becomes a float by
+// its bit pattern (2^23 + field) and one subtraction: a conversion from integer
+// would run at a quarter of that rate.
 // d > 7 (F would not fit 64 bits): v is scaled in FP64, each digit rounded to
 // nearest and subtracted (every step exact).
 template <int C>
 __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (&b)[C], int e, bool zero, int d,
                                                __nv_bfloat16* __restrict__ q, int64_t stride, bool store,
                                                uint32_t* norm) {
-  int x[C];
+  float f[C];
   if (d <= 7) {
+    // 256 (1 + 512 + ... + 512^{d-2})
+    const int64_t bias = (int64_t)((0x0040201008040201ULL & ((1ULL << (9 * (d - 1))) - 1)) << 8);
     int64_t F[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       int64_t M;
       int E;
-      F[c] = 0;
-      if (!zero && decompose(v[c], M, E) == 1) {  // |v| = M 2^{E - 1075}
-        const int sh = E + b[c] - 1075 - e + 9 * d - 1;
-        if (sh >= 0)
-          F[c] = M << sh;
-        else if (sh > -54)
-          F[c] = (M + (1LL << (-sh - 1))) >> (-sh);
-        if (v[c] < 0.0) F[c] = -F[c];
+      F[c] = bias;
+      if (!zero && decompose(v[c], M, E) == 1) {  // |v| = M 2^{E - 1075}, M < 2^53
+        // right shift of M 2^10 by r leaves one bit for the rounding; r >= 0 because |v 2^{b-e}| < 1
+        const int r = 1075 + e + 10 - E - b[c] - 9 * d;
+        const int64_t a = r < 64 ? (int64_t)((((unsigned long long)M << 10) >> r) + 1) >> 1 : 0;
+        F[c] += v[c] < 0.0 ? -a : a;
       }
     }
     for (int i = d - 1; i >= 0; --i) {
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        x[c] = (int)(i > 0 ? ((F[c] + 256) & 511) - 256 : F[c]);
-        F[c] = (F[c] - x[c]) >> 9;
+        const uint32_t lo = (uint32_t)F[c];
+        f[c] = i > 0 ? __uint_as_float((lo & 511u) | 0x4B000000u) - 8388864.f  // 2^23 + 256
+                     : __uint_as_float((lo + 512u) + 0x4B000000u) - 8389120.f; // the rest, -256 .. 256
+        F[c] >>= 9;
       }
-      put_digits<C>(x, q + i * stride, store, norm + i);
+      put_digits<C>(f, q + i * stride, store, norm + i);
     }
   } else {
     double r[C];
@@ -154,9 +160,9 @@ __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (
       for (int c = 0; c < C; ++c) {
         const double g = rint(r[c]);
         r[c] = (r[c] - g) * 512.0;
-        x[c] = (int)g;
+        f[c] = (float)g;
       }
-      put_digits<C>(x, q + i * stride, store, norm + i);
+      put_digits<C>(f, q + i * stride, store, norm + i);
     }
   }
 }
@@ -174,7 +180,9 @@ __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (
 // keep its FP32 sums over 512 terms or more instead of 256.
 // Bound by HBM: 8 bytes read and 2 d written per entry, in 32- and 8-byte
 // pieces per thread (2-byte stores of single entries took twice the time).
-__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X, int64_t ldx, int64_t K, int d,
+constexpr int kSplitThreads = 256;
+
+__global__ void __launch_bounds__(kSplitThreads) k_split_rows(const double* __restrict__ X, int64_t ldx, int64_t K, int d,
                                                     int lower, int wide, const int32_t* __restrict__ bal,
                                                     __nv_bfloat16* __restrict__ Q, int64_t ldq, int64_t sstride,
                                                     int32_t* __restrict__ E, int nch, uint32_t* __restrict__ norm2,
@@ -183,12 +191,13 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
   const int chunk = blockIdx.y;
   const int64_t k0 = (int64_t)chunk * kL;
   const int64_t kend = lower && row + 1 < K ? row + 1 : K;  // entries from here on are zero
-  double v[4][4];
+  constexpr int NT = kSplitThreads, NU = 1024 / NT;  // groups of four entries per thread
+  double v[NU][4];
   int emax = INT_MIN;
   bool bad = false;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
+  for (int u = 0; u < NU; ++u) {
+    const int64_t k = k0 + 4 * (threadIdx.x + NT * u);
     const double* x = X + row * ldx + k;
     if (wide && k + 4 <= kend) {
       const double2 a = *reinterpret_cast<const double2*>(x), b = *reinterpret_cast<const double2*>(x + 2);
@@ -202,8 +211,8 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
     }
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
+  for (int u = 0; u < NU; ++u) {
+    const int64_t k = k0 + 4 * (threadIdx.x + NT * u);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       int64_t M;
@@ -213,7 +222,7 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
       if (z == 1) emax = max(emax, Ex + (bal ? bal[k + c] : 0));
     }
   }
-  __shared__ int red[8];
+  __shared__ int red[NT / 32];
   __shared__ int sbad;
   __shared__ uint32_t norm[8][kNormPitch];  // by 512-entry block and digit
   if (threadIdx.x == 0) sbad = 0;
@@ -225,7 +234,7 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
   __syncthreads();
   emax = red[0];
 #pragma unroll
-  for (int w = 1; w < 8; ++w) emax = max(emax, red[w]);
+  for (int w = 1; w < NT / 32; ++w) emax = max(emax, red[w]);
   const bool zero = sbad != 0;
   const int e = (emax == INT_MIN || zero) ? 0 : emax - 1022;
   if (threadIdx.x == 0) {
@@ -233,10 +242,10 @@ __global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ X
     if (zero) atomic_flag(flag);
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int64_t k = k0 + 4 * (threadIdx.x + 256 * u);
-    if (k0 + 1024 * u >= K) break;  // the same for the whole CTA
-    uint32_t* nrm = norm[2 * u + (threadIdx.x >> 7)];
+  for (int u = 0; u < NU; ++u) {
+    const int64_t k = k0 + 4 * (threadIdx.x + NT * u);
+    if (k0 + 4 * NT * u >= K) break;  // the same for the whole CTA
+    uint32_t* nrm = norm[(threadIdx.x + NT * u) >> 7];
     int b[4] = {0, 0, 0, 0};
     if (bal) {
 #pragma unroll
@@ -511,12 +520,12 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
     ldbr = K;
   }
   auto wide = [](const double* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 2 == 0; };
-  k_split_rows<<<dim3((unsigned)M, (unsigned)nch), 256, 0, st>>>(A, lda, K, s, a_lower ? 1 : 0, wide(A, lda) ? 1 : 0,
+  k_split_rows<<<dim3((unsigned)M, (unsigned)nch), kSplitThreads, 0, st>>>(A, lda, K, s, a_lower ? 1 : 0, wide(A, lda) ? 1 : 0,
                                                                   bal, Qa, lqa, sa, Ea, nch, norm_a, flag);
   count_launch();
   DG_CUDA(cudaGetLastError());
   if (!same) {
-    k_split_rows<<<dim3((unsigned)Nc, (unsigned)nch), 256, 0, st>>>(Br, ldbr, K, s, 0, wide(Br, ldbr) ? 1 : 0,
+    k_split_rows<<<dim3((unsigned)Nc, (unsigned)nch), kSplitThreads, 0, st>>>(Br, ldbr, K, s, 0, wide(Br, ldbr) ? 1 : 0,
                                                                      nbal, Qb, lqb, sb, Eb, nch, norm_b, flag);
     count_launch();
     DG_CUDA(cudaGetLastError());
