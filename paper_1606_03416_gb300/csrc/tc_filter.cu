@@ -603,6 +603,9 @@ static dgchefsi_status prepare_launch(dgchefsi_ctx* ctx, TcState& t, int mode, i
   const int W = f32 ? 32 : 64;
   Plan* pl = nullptr;
   DG_TRY(get_plan(ctx, t, G, &pl));
+  // up to 128 states the second tile of a unit is empty: the one-tile kernel of
+  // the same group loads and multiplies half as much, in twice the ring slots
+  if (layout == 0 && T == 2 && Ns <= BM) T = 1;
   L.kern = pick_kernel(mode, G, T, t.ACC, layout);
   if (!L.kern)
     return set_error(DGCHEFSI_ERR_UNSUPPORTED, "no filter kernel for G=%d T=%d ACC=%d layout %d", G, T, t.ACC, layout);
@@ -616,7 +619,7 @@ static dgchefsi_status prepare_launch(dgchefsi_ctx* ctx, TcState& t, int mode, i
                   layout == 2));
   const int na = mode == MODE_BF16X3 ? 2 : 1;
   const int stage_bytes = layout >= 1 ? na * (128 * sb + 256 * sb) : na * (T * A_BYTES + G * t.ACC * SLICE_BYTES);
-  const int stages = layout >= 1 ? TN_RING_BYTES / stage_bytes : (mode == MODE_BF16X3 ? STAGES / 2 : STAGES);
+  const int stages = layout >= 1 ? TN_RING_BYTES / stage_bytes : ring_slots(stage_bytes);
   L.smem = stages * stage_bytes + (2 * stages + 4) * 8 + 2 * pl->maxent * (1 + G) * 4 + 1024;
   if (L.smem > 227 * 1024) return set_error(DGCHEFSI_ERR_UNSUPPORTED, "filter schedule too large for shared memory");
   DG_CUDA(cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem));
@@ -652,6 +655,27 @@ static dgchefsi_status prepare_launch(dgchefsi_ctx* ctx, TcState& t, int mode, i
   return DGCHEFSI_OK;
 }
 
+// Launch of a step kernel. One of at most half the SMs may start before the work
+// ahead of it on the stream has finished (it waits for that itself, see
+// wait_for_previous_grid): its set-up runs on idle SMs. A step that fills the
+// GPU has none, and lost 2 % where its CTAs came to sit as SMs became free.
+static cudaError_t start_step(const Launch& L, int num_sms, const CUtensorMap& A0, const CUtensorMap& A1,
+                              const Params& p, cudaStream_t s) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = L.grid;
+  cfg.blockDim = dim3(NTHREADS);
+  cfg.dynamicSmemBytes = (size_t)L.smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 2 * (int)L.grid.x <= num_sms ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, L.kern, A0, A1, L.B, p);
+  count_launch();
+  return e;
+}
+
 // Step k: Y_{k+1} from Y_k (buffer k%2) and Y_{k-1} (buffer (k+1)%2).
 static dgchefsi_status launch_step(dgchefsi_ctx* ctx, TcState& t, int mode, Launch& L, int k, cudaStream_t s) {
   const int cur = k & 1, nxt = cur ^ 1;
@@ -661,9 +685,7 @@ static dgchefsi_status launch_step(dgchefsi_ctx* ctx, TcState& t, int mode, Laun
   p.Fout = static_cast<float*>(t.F[nxt].p);
   p.Hout = mode == MODE_TF32 ? nullptr : static_cast<__nv_bfloat16*>(t.Sh[nxt].p);
   p.Lout = mode == MODE_BF16X3 ? static_cast<__nv_bfloat16*>(t.Sl[nxt].p) : nullptr;
-  L.kern<<<L.grid, NTHREADS, L.smem, s>>>(L.A0[cur], L.A1[cur], L.B, p);
-  count_launch();
-  DG_CUDA(cudaGetLastError());
+  DG_CUDA(start_step(L, t.num_sms, L.A0[cur], L.A1[cur], p, s));
   (void)ctx;
   return DGCHEFSI_OK;
 }
@@ -691,9 +713,7 @@ static dgchefsi_status launch_io(TcState& t, int mode, Launch& L, int k, const d
   p.Fout = io.Fout;
   p.Hout = mode == MODE_TF32 ? nullptr : io.Hout;
   p.Lout = mode == MODE_BF16X3 ? io.Lout : nullptr;
-  L.kern<<<L.grid, NTHREADS, L.smem, s>>>(A0, A1, L.B, p);
-  count_launch();
-  DG_CUDA(cudaGetLastError());
+  DG_CUDA(start_step(L, t.num_sms, A0, A1, p, s));
   return DGCHEFSI_OK;
 }
 
@@ -1364,7 +1384,9 @@ dgchefsi_status tc_set_shape(dgchefsi_ctx* ctx, int prec, int G, int T, int layo
     if (t.force_tgb[mode] < 0) t.tgb[mode] = -1;
     return DGCHEFSI_OK;
   }
-  if (!pick_kernel(mode, G, T, t.ACC, layout))
+  bool known = false;
+  for (const auto& sh : SHAPES) known = known || (sh[0] == G && sh[1] == T && sh[2] == t.ACC && sh[3] == layout);
+  if (!known || !pick_kernel(mode, G, T, t.ACC, layout))
     return set_error(DGCHEFSI_ERR_UNSUPPORTED, "no kernel for G=%d T=%d layout %d with accumulator width %d", G, T,
                      layout, t.ACC);
   t.forceG[mode] = G;

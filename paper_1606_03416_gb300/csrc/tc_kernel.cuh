@@ -52,7 +52,11 @@ constexpr int BM = 128;           // states per tile (MMA M)
 constexpr int SLICE_BYTES = 128;  // K extent of one ring slot in bytes (one swizzle row)
 constexpr int NTHREADS = 320;  // producer warp, MMA warp, 8 epilogue warps
 constexpr int EPI_WARPS = 8;
-constexpr int STAGES = 4;       // ring slots (each T A-tiles + G B-tiles)
+// Ring slots (each T A-tiles + G B-tiles, hi and lo in BF16X3) of layout 0: the
+// largest power of two up to 8 that fits 192 KB.
+constexpr int ring_slots(int slot_bytes) {
+  return 8 * slot_bytes <= 192 * 1024 ? 8 : (4 * slot_bytes <= 192 * 1024 ? 4 : 2);
+}
 constexpr int ZERO_TILES = 64;  // zero B tiles for non-coupling elements, spread over L2
 constexpr int A_BYTES = BM * SLICE_BYTES;
 constexpr int TN_RING_BYTES = 192 * 1024;  // ring of the transposed kernel (any slot size)
@@ -156,6 +160,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+
+// Programmatic dependent launch: a step is launched while the previous one runs,
+// sets up its barriers and tensor memory on the SMs that are free or become
+// free, and waits here until the previous grid has completed and its writes are
+// visible. Nothing that a previous grid writes is read, and nothing that it
+// reads is written, before. Ten steps of a small filter (8 elements, 48 states):
+// 134 us without this, 108 with it and one-tile units (see pick_shape).
+__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
@@ -299,10 +312,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // BF16X3 keeps the hi and lo copies of both operands in one ring slot (its
   // three products reuse them), so its slots are twice as large and half as many.
   constexpr int NA = MODE_ == MODE_BF16X3 ? 2 : 1;
-  constexpr int S = MODE_ == MODE_BF16X3 ? STAGES / 2 : STAGES;
   constexpr int b_bytes = ACC * SLICE_BYTES;  // one element's B tile: ACC rows of 128 bytes
   constexpr int a_part = NA * T * A_BYTES;    // [A hi x T][A lo x T]
   constexpr int stage_bytes = a_part + NA * G * b_bytes;  // then [B hi x G][B lo x G]
+  constexpr int S = ring_slots(stage_bytes);
   constexpr uint32_t NMMA = (uint32_t)(G * ACC);  // the G elements' B tiles are stacked along N
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
   // per-role copies of the current group's slice entries (producer, MMA issuer)
@@ -338,6 +351,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
+  let_next_grid_launch();    // only now: this CTA holds its tensor memory, which the next one waits for
+  wait_for_previous_grid();  // everything above overlaps the previous step's end
 
   if (warp == 0) {
     // ---------------- producer: TMA into the ring (lane 0 issues; the warp copies schedules)
@@ -589,6 +604,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
+  let_next_grid_launch();    // only now: this CTA holds its tensor memory, which the next one waits for
+  wait_for_previous_grid();  // everything above overlaps the previous step's end
 
   if (warp == 0) {
     // ---------------- producer
@@ -812,6 +829,11 @@ FilterKernel pick_shape(int G, int T, int ACC, int layout) {
   if (G == 2 && T == 1 && ACC == 64) return k_filter_step_tc<MODE_, 2, 1, 64>;
   if (G == 4 && T == 2 && ACC == 32) return k_filter_step_tc<MODE_, 4, 2, 32>;
   if (G == 2 && T == 2 && ACC == 32) return k_filter_step_tc<MODE_, 2, 2, 32>;
+  // the one-tile forms of the two-tile shapes, for at most 128 states
+  if (G == 4 && T == 1 && ACC == 32) return k_filter_step_tc<MODE_, 4, 1, 32>;
+  if (G == 2 && T == 1 && ACC == 32) return k_filter_step_tc<MODE_, 2, 1, 32>;
+  if (G == 1 && T == 1 && ACC == 64) return k_filter_step_tc<MODE_, 1, 1, 64>;
+  if (G == 1 && T == 1 && ACC == 128) return k_filter_step_tc<MODE_, 1, 1, 128>;
   if (G == 2 && T == 1 && ACC == 128) return k_filter_step_tc<MODE_, 2, 1, 128>;
   if (G == 1 && T == 2 && ACC == 128) return k_filter_step_tc<MODE_, 1, 2, 128>;
   return nullptr;
