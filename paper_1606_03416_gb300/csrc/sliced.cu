@@ -293,100 +293,145 @@ __device__ __forceinline__ double scale_pow2(double h, int e) {
   return ldexp(h, e);
 }
 
+// (hi 2^36 + lo) 2^e, rounded once to nearest even, in integer instructions:
+// |hi| 2^36 + |lo| < 2^126. A result below the normal range goes through ldexp.
+__device__ __forceinline__ double round_pow2(int64_t hi, int64_t lo, int e) {
+  const __int128 v = ((__int128)hi << 36) + lo;
+  const bool neg = v < 0;
+  const unsigned __int128 u = neg ? -(unsigned __int128)v : (unsigned __int128)v;
+  uint64_t uh = (uint64_t)(u >> 64), ul = (uint64_t)u;
+  int E = 127 + e;  // exponent of the leading bit
+  if (uh == 0) {
+    uh = ul;
+    ul = 0;
+    E -= 64;
+  }
+  if (uh == 0) return 0.0;
+  const int n = __clzll((long long)uh);
+  const uint64_t top = n == 0 ? uh : (uh << n) | (ul >> (64 - n));  // leading bit at 63
+  E -= n;
+  const uint32_t rest = ((uint32_t)top & 0x7ffu) << 1 | ((ul << n) != 0);  // below the last of 53 bits
+  const uint64_t m = top >> 11;
+  const uint64_t up = rest + ((uint32_t)m & 1u) > 0x800u;
+  double y;
+  if (E > -1023 && E < 1023)
+    y = __longlong_as_double((long long)(((uint64_t)(E + 1022) << 52) + m + up));  // m's leading bit adds the 1
+  else
+    y = ldexp((double)(m + up), E - 52);
+  return neg ? -y : y;
+}
+
 // C[r, n0 + c] (+)= (+-) 2^{e_r + f_{n0+c} - 16} sum_t 2^{-9t} g_t for r < M, c < P,
 // g_t the sum of weight t's count[t] INT32 slabs (M rows of `pitch` entries, t
 // descending). Four consecutive t are combined in INT64 (|g_t| < 2^32, so the
-// block is below 2^60) and converted to FP64, and the blocks meet by Horner in
-// 2^{-36}: one rounding of each block and one per step.
-// Four consecutive outputs per thread, one 16-byte load per slab; wide: the
-// rows of C at n0 start on 16 bytes. tri > 0: only the entries with
+// block is below 2^60). Up to w = 8 the two blocks meet in 128 bits and the sum
+// is rounded once, all in integer instructions; above that the blocks are
+// converted and meet by Horner in 2^{-36}, one rounding of each and one per step.
+// ONE: one slab per weight, all W loads before any use.
+// Two consecutive outputs per thread, so a warp's stores are contiguous; wide:
+// the rows of C at n0 start on 16 bytes. tri > 0: only the entries with
 // n0 + c <= r mod tri are formed (the slice-pair kernel left the tiles above
 // that line out); the others are not read or written.
 // cmap (may be null): column c goes to column cmap[c] of C and is skipped when
 // that is negative (the padding columns of the element-padded layout).
 // Bound by HBM: 4 bytes read per slab and entry (28 at w = 7) and 8 written, 16
-// when a chunk is added; it runs on its own stream beside the next chunk's pairs.
-template <int W>
-__global__ void __launch_bounds__(256) k_digit_reduce(const int32_t* __restrict__ Pw, int64_t M, int64_t P,
-                                                      int64_t pitch, const PairGroups groups,
-                                                      const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb,
-                                                      int nch, int chunk, int64_t n0, double* __restrict__ C,
-                                                      int64_t ldc, int wide, int accumulate, int negate,
-                                                      int64_t tri, const int32_t* __restrict__ cmap) {
+// when a chunk is added; on products of several chunks it runs on its own stream
+// beside the next chunk's pairs. 4096 x 32768, w = 7: 0.84 ms, 5.7 TB/s. With the
+// conversions, the Horner step and the scaling on the FP64 pipe (2 a clock and SM,
+// about five an entry) 1.26 ms; integers but four outputs a thread (16-byte loads,
+// 100 registers) 1.09 ms; two outputs with a division for the row 0.93 ms.
+template <int W, bool ONE>
+__global__ void __launch_bounds__(256, 4)
+    k_digit_reduce(const int32_t* __restrict__ Pw, int64_t M, int64_t P, int64_t pitch, const PairGroups groups,
+                   const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb, int nch, int chunk, int64_t n0,
+                   double* __restrict__ C, int64_t ldc, int wide, int accumulate, int negate, int64_t tri,
+                   const int32_t* __restrict__ cmap) {
   constexpr int NB = (W + 3) / 4;
-  const int64_t slab = M * pitch, quads = pitch / 4, total = M * quads;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = q / quads, c0 = 4 * (q - r * quads);
-    // the four entries share a row and a 256-column tile: when the first is
-    // above the line all are, and otherwise the tile was computed
-    const int64_t rdiag = tri > 0 ? r % tri : 0;
+  const int64_t half = M * pitch / 2;
+  const uint32_t pairs = (uint32_t)(pitch / 2), stride = gridDim.x * blockDim.x;
+  const uint32_t q0 = blockIdx.x * blockDim.x + threadIdx.x;
+  // row and column pair of q, carried along: no division per output
+  const uint32_t dr = stride / pairs, dc = stride - dr * pairs;
+  uint32_t r = q0 / pairs, c = q0 - r * pairs;
+  for (int64_t q = q0; q < half; q += stride, r += dr, c += dc) {
+    if (c >= pairs) {
+      c -= pairs;
+      ++r;
+    }
+    const int64_t c0 = 2 * (int64_t)c;
+    // the two entries share a row and a 256-column tile: when the first is
+    // above the line both are, and otherwise the tile was computed
+    const int64_t rdiag = tri > 0 ? r % (uint32_t)tri : 0;
     if (tri > 0 && n0 + c0 > rdiag) continue;
-    const int4* p = reinterpret_cast<const int4*>(Pw + 4 * q);
-    int64_t g[4][W];
-    if (groups.total == W) {  // one slab per weight: all loads before any use
-      int4 v[W];
+    const int2* p = reinterpret_cast<const int2*>(Pw) + q;
+    const bool second = c0 + 1 < P;
+    if (c0 >= P) continue;  // the pitch's padding
+    const int er = Ea[(int64_t)r * nch + chunk] - 16 - 27;
+    const int ec[2] = {er + Eb[(n0 + c0) * nch + chunk], second ? er + Eb[(n0 + c0 + 1) * nch + chunk] : 0};
+    int2 v[ONE ? W : 1];  // one slab per weight: all loads before any use
+    int64_t g[2][ONE ? 1 : W];
+    if constexpr (ONE) {
 #pragma unroll
-      for (int t = 0; t < W; ++t) v[t] = __ldcs(p + (int64_t)(W - 1 - t) * (slab / 4));
-#pragma unroll
-      for (int t = 0; t < W; ++t) {
-        g[0][t] = v[t].x;
-        g[1][t] = v[t].y;
-        g[2][t] = v[t].z;
-        g[3][t] = v[t].w;
-      }
+      for (int t = W - 1; t >= 0; --t, p += half) v[t] = __ldcs(p);
     } else {
 #pragma unroll
       for (int t = W - 1; t >= 0; --t) {
-        g[0][t] = g[1][t] = g[2][t] = g[3][t] = 0;
-        for (int k = 0; k < groups.count[t]; ++k, p += slab / 4) {
-          const int4 v = __ldcs(p);
-          g[0][t] += v.x;
-          g[1][t] += v.y;
-          g[2][t] += v.z;
-          g[3][t] += v.w;
+        g[0][t] = g[1][t] = 0;
+        for (int k = 0; k < groups.count[t]; ++k, p += half) {
+          const int2 x = __ldcs(p);
+          g[0][t] += x.x;
+          g[1][t] += x.y;
         }
       }
     }
-    const int er = Ea[r * nch + chunk] - 16 - 27;
-    double y[4];
+    const auto sum_of = [&](int t, int e) -> int64_t {
+      if (t >= W) return 0;
+      if constexpr (ONE) return e == 0 ? v[t].x : v[t].y;
+      else return g[e][t];
+    };
+    double y[2];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < 2; ++e) {
       // B_b = sum_{t = 4b}^{4b+3} g_t 2^{9(4b + 3 - t)}; sum_t g_t 2^{-9t} = 2^{-27} sum_b B_b 2^{-36b}
-      double h = 0.0;
+      int64_t B[NB];
 #pragma unroll
-      for (int b = NB - 1; b >= 0; --b) {
-        int64_t B = 0;
+      for (int b = 0; b < NB; ++b) {
+        B[b] = 0;
 #pragma unroll
-        for (int t = 4 * b; t < 4 * b + 4; ++t) B = B * 512 + (t < W ? g[e][t] : 0);
-        h = b == NB - 1 ? (double)B : h * 0x1p-36 + (double)B;
+        for (int t = 4 * b; t < 4 * b + 4; ++t) B[b] = B[b] * 512 + sum_of(t, e);
       }
-      y[e] = c0 + e < P ? scale_pow2(negate ? -h : h, er + Eb[(n0 + c0 + e) * nch + chunk]) : 0.0;
+      if constexpr (NB <= 2) {
+        y[e] = round_pow2(B[0], NB == 2 ? B[NB - 1] : 0, ec[e] - 36);
+      } else {
+        double h = (double)B[NB - 1];
+#pragma unroll
+        for (int b = NB - 2; b >= 0; --b) h = h * 0x1p-36 + (double)B[b];
+        y[e] = scale_pow2(h, ec[e]);
+      }
+      if (negate) y[e] = -y[e];
     }
     if (cmap) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int32_t oc = c0 + e < P ? cmap[c0 + e] : -1;
-        if (oc >= 0) C[r * ldc + oc] = y[e];
+      const int32_t oc = cmap[c0], od = second ? cmap[c0 + 1] : -1;
+      double* o = C + r * ldc + oc;
+      if (oc >= 0 && od == oc + 1 && (reinterpret_cast<uintptr_t>(o) & 15) == 0) {
+        *reinterpret_cast<double2*>(o) = make_double2(y[0], y[1]);
+      } else {
+        if (oc >= 0) *o = y[0];
+        if (od >= 0) C[r * ldc + od] = y[1];
       }
       continue;
     }
-    double* out = C + r * ldc + n0 + c0;
-    if (wide && c0 + 4 <= P && (tri == 0 || n0 + c0 + 3 <= rdiag)) {
-      double2* o = reinterpret_cast<double2*>(out);
+    double* o = C + r * ldc + n0 + c0;
+    if (wide && second && (tri == 0 || n0 + c0 + 1 <= rdiag)) {
       if (accumulate) {
-        const double2 a = o[0], b = o[1];
+        const double2 a = *reinterpret_cast<const double2*>(o);
         y[0] += a.x;
         y[1] += a.y;
-        y[2] += b.x;
-        y[3] += b.y;
       }
-      o[0] = make_double2(y[0], y[1]);
-      o[1] = make_double2(y[2], y[3]);
+      *reinterpret_cast<double2*>(o) = make_double2(y[0], y[1]);
     } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (c0 + e < P && (tri == 0 || n0 + c0 + e <= rdiag)) out[e] = accumulate ? out[e] + y[e] : y[e];
+      o[0] = accumulate ? o[0] + y[0] : y[0];
+      if (second && (tri == 0 || n0 + c0 + 1 <= rdiag)) o[1] = accumulate ? o[1] + y[1] : y[1];
     }
   }
 }
@@ -395,18 +440,20 @@ typedef void (*DigitReduce)(const int32_t*, int64_t, int64_t, int64_t, const Pai
                             const int32_t*, int, int, int64_t, double*, int64_t, int, int, int, int64_t,
                             const int32_t*);
 
+// the kernel of w weights; one: one slab per weight
+template <bool ONE>
 static DigitReduce digit_reduce(int w) {
   switch (w) {
-    case 2: return k_digit_reduce<2>;
-    case 3: return k_digit_reduce<3>;
-    case 4: return k_digit_reduce<4>;
-    case 5: return k_digit_reduce<5>;
-    case 6: return k_digit_reduce<6>;
-    case 7: return k_digit_reduce<7>;
-    case 8: return k_digit_reduce<8>;
-    case 9: return k_digit_reduce<9>;
-    case 10: return k_digit_reduce<10>;
-    case 11: return k_digit_reduce<11>;
+    case 2: return k_digit_reduce<2, ONE>;
+    case 3: return k_digit_reduce<3, ONE>;
+    case 4: return k_digit_reduce<4, ONE>;
+    case 5: return k_digit_reduce<5, ONE>;
+    case 6: return k_digit_reduce<6, ONE>;
+    case 7: return k_digit_reduce<7, ONE>;
+    case 8: return k_digit_reduce<8, ONE>;
+    case 9: return k_digit_reduce<9, ONE>;
+    case 10: return k_digit_reduce<10, ONE>;
+    case 11: return k_digit_reduce<11, ONE>;
     default: return nullptr;
   }
 }
@@ -572,11 +619,12 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
         DG_CUDA(cudaEventRecord(ctx->ev_pairs[b], st));
         DG_CUDA(cudaStreamWaitEvent(sr, ctx->ev_pairs[b], 0));
       }
-      const int64_t pitch = round_up(pn, 4), work = M * pitch / 4;
+      const int64_t pitch = round_up(pn, 4), work = M * pitch / 2;
       const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 16));
-      digit_reduce(nw)<<<grid, 256, 0, sr>>>(Pb, M, pn, pitch, groups, Ea, Eb, nch, chunk, n0, C, ldc,
-                                            wide(C, ldc) ? 1 : 0, subtract || chunk > 0 ? 1 : 0, subtract || negate ? 1 : 0, tri,
-                                            nullptr);
+      const DigitReduce reduce = groups.total == nw ? digit_reduce<true>(nw) : digit_reduce<false>(nw);
+      reduce<<<grid, 256, 0, sr>>>(Pb, M, pn, pitch, groups, Ea, Eb, nch, chunk, n0, C, ldc,
+                                wide(C, ldc) ? 1 : 0, subtract || chunk > 0 ? 1 : 0, subtract || negate ? 1 : 0, tri,
+                                nullptr);
       count_launch();
       DG_CUDA(cudaGetLastError());
       if (multi) DG_CUDA(cudaEventRecord(ctx->ev_reduce[b], sr));
@@ -772,8 +820,9 @@ cudaError_t digits_of_states(const double* X, int64_t ld, int64_t Ns, int64_t N,
 dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols, int w, const PairGroups& groups,
                                    const int32_t* Erows, const int32_t* Ecols, const int32_t* cmap, double* C,
                                    int64_t ldc, cudaStream_t st) {
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows * cols / 4 + 255) / 256, 152 * 16));
-  digit_reduce(w)<<<grid, 256, 0, st>>>(Pw, rows, cols, cols, groups, Erows, Ecols, 1, 0, 0, C, ldc, 0, 0, 0, 0, cmap);
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows * cols / 2 + 255) / 256, 152 * 16));
+  const DigitReduce reduce = groups.total == w ? digit_reduce<true>(w) : digit_reduce<false>(w);
+  reduce<<<grid, 256, 0, st>>>(Pw, rows, cols, cols, groups, Erows, Ecols, 1, 0, 0, C, ldc, 0, 0, 0, 0, cmap);
   count_launch();
   DG_CUDA(cudaGetLastError());
   return DGCHEFSI_OK;

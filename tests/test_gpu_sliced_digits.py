@@ -1,7 +1,7 @@
 """The 9-bit digits of the dense sliced products: bit for bit at the edge of the
 exact FP32 sums, at ragged drains of the accumulator (256 terms, or more where
-the digits' norms allow), at ragged K chunks and tiles, and on operands whose
-digits are all in use."""
+the digits' norms allow), at ragged K chunks and tiles, on operands whose
+digits are all in use, and the one rounding of the digit sums."""
 import numpy as np
 import pytest
 import torch
@@ -49,3 +49,23 @@ def test_random_integers_bit_exact(M, Nc, K, slices):
     A = rng.integers(-(2 ** (6 * a - 1)), 2 ** (6 * a - 1), size=(M, K))
     Bt = rng.integers(-(2 ** (6 * b - 1)), 2 ** (6 * b - 1), size=(Nc, K))
     assert np.array_equal(product(A, Bt, True, slices), (A @ Bt.T).astype(np.float64))
+
+
+@pytest.mark.parametrize("slices", [10, 11])
+@pytest.mark.parametrize("M,Nc,K,e", [(1, 1, 700, 0), (5, 7, 700, -537), (40, 301, 300, 400), (257, 64, 513, -40)])
+def test_sums_are_rounded_once(M, Nc, K, e, slices):
+    """Integers of 27 bits have four digits at most and no pair of them is
+    dropped, so the sum (up to 64 bits) is exact before its only rounding:
+    the result is the nearest double, ties to even. e scales both operands by
+    2^e; at -537 small integers end as exact subnormals. One K chunk."""
+    rng = np.random.default_rng(3)
+    top = 2 ** 27 if e != -537 else 2 ** 8
+    A = rng.integers(-top, top, size=(M, K))
+    Bt = rng.integers(-top, top, size=(Nc, K))
+    if M > 1:
+        A[1] = 0
+        Bt[::3] = abs(Bt[::3])
+        A[0] = abs(A[0])
+    exact = A.astype(object) @ Bt.T.astype(object)
+    want = np.array([[float(x) for x in row] for row in exact])
+    assert np.array_equal(product(A * 2.0 ** e, Bt * 2.0 ** e, True, slices), np.ldexp(want, 2 * e))
