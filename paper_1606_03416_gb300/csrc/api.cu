@@ -1088,9 +1088,14 @@ dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t N
     DG_TRY(filter_tc(ctx, prec, X, Yw, Ns, ld, m, a, b, a0));
   DG_TRY(rr_impl(ctx, Yw, Ns, ld, ritz, X));
   DG_CUDA(occupations_f64(ritz, Ns, Ne, kT, f, mu, ctx->stream));
-  Parts parts;
-  DG_TRY(parts_of(ctx, &parts));
-  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
+  bool done = false;
+  if (ctx->products_mode == DGCHEFSI_PRODUCTS_SLICED_BF16 && density_digits_fit(ctx, Ns))
+    DG_TRY(density_digits(ctx, X, Ns, ld, f, P, &done));
+  if (!done) {
+    Parts parts;
+    DG_TRY(parts_of(ctx, &parts));
+    DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
+  }
   if (bounds) {
     bounds[0] = a;
     bounds[1] = b;

@@ -188,6 +188,13 @@ dgchefsi_status sliced_gemm_tn(dgchefsi_ctx* ctx, int64_t M, int64_t Nc, int64_t
                                const double* B, int64_t ldb, double* C, int64_t ldc, int s, int* flag);
 void sliced_destroy(dgchefsi_ctx* ctx);
 
+// density_digits: P = the packed density blocks from digits (f >= 0), for the
+// sizes density_digits_fit accepts; done = false where the FP64 form has to be
+// used after all (no workspace, or an entry that is not finite). Synchronises.
+bool density_digits_fit(const dgchefsi_ctx* ctx, int64_t Ns);
+dgchefsi_status density_digits(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P,
+                               bool* done);
+
 // Slabs of the digit weights (pair_groups below).
 struct PairGroups {
   uint8_t count[16];  // by weight t
@@ -226,6 +233,8 @@ dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols
 // slices past its last row. norm_a, norm_b (device, s entries): the largest sum
 // of squares of digit i over an aligned 512-entry block of a row. Enqueued only.
 // pair_groups: how many slabs each weight is split into for an output of so many 256 x 256 tiles.
+// pair_products_diag: the 256 x 256 blocks on the diagonal of Q Q^T only (slabs
+// of rows x 256), with the digits of one operand.
 // pair_products_begin clears the kernel's error word; pair_products_status
 // synchronises and reports a pipeline timeout.
 PairGroups pair_groups(int s, int nw, int64_t tiles, int nsm);
@@ -233,6 +242,9 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
                                   const __nv_bfloat16* Qb, int64_t lqb, int64_t sb, int64_t Nc, int64_t K, int64_t k0,
                                   int64_t kc, int64_t n0, int64_t pn, int s, int nw, const PairGroups& groups,
                                   const uint32_t* norm_a, const uint32_t* norm_b, int32_t* Pw, bool a_lower, int64_t tri = 0);
+dgchefsi_status pair_products_diag(dgchefsi_ctx* ctx, const __nv_bfloat16* Q, int64_t lq, int64_t sq, int64_t rows,
+                                   int64_t K, int64_t k0, int64_t kc, int s, int nw, const PairGroups& groups,
+                                   const uint32_t* norm, int32_t* Pw);
 // The same kernel on the block-sparse H: slab = the weight's sum of Hs_i times
 // Xs_j (states s0 .. s0 + pn - 1, rows of ldp padded H rows). Hs: s digit
 // copies of H in the tensor-core operand layout (h_rows x 64, hcopy apart), Xs:

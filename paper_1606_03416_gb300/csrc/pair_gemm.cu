@@ -79,6 +79,8 @@ struct PairJob {
   int n0, k0, nk;   // first B row, first K column, 64-wide K slices of the chunk
   int nmt, nnt;     // 256-row tiles along M and along the panel
   int lower;        // A is lower triangular: a row tile stops at the chunk's last K slice it reaches
+  int diag;         // > 0: the B rows of row tile mt start at 256 mt (nnt = 1, slabs of 256 columns);
+                    // 2: the units of one tile back to back, not those of one group
   const int2* tiles;  // null: every (row tile, column tile); else the ntl tiles to compute
   int ntl;
   const uint32_t* norm_a;  // [s] largest sum of squares of digit i over 512 terms of a row of A, of B
@@ -165,6 +167,12 @@ __device__ __forceinline__ void unit_of(const PairJob& J, int64_t u, int& g, int
     return;
   }
   const int64_t ntiles = (int64_t)J.nmt * J.nnt;
+  if (J.diag == 2) {
+    mt = (int)(u / J.ngroups);
+    g = (int)(u - (int64_t)mt * J.ngroups);
+    nt = 0;
+    return;
+  }
   g = (int)(u / ntiles);
   const int64_t tile = u - (int64_t)g * ntiles;
   mt = (int)(tile % J.nmt);
@@ -257,7 +265,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
       int g, mt, nt;
       unit_of(J, u, g, mt, nt);
       const int ya = mt * 256 + (int)rank * 128;
-      const int yb = J.n0 + nt * 256 + (int)rank * 128;
+      const int yb = J.n0 + (J.diag ? mt : nt) * 256 + (int)rank * 128;
       const int nk = slices_of_tile<BLOCKS>(J, mt);
       if (BLOCKS) {
         __syncwarp();
@@ -579,6 +587,36 @@ dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, in
   J.ntl = (int)tl.size();
   J.Pw = Pw;
   return launch_pairs(ctx, J, T, s, groups, false, tl.empty() ? (int64_t)nmt * nnt : (int64_t)tl.size(), 0);
+}
+
+dgchefsi_status pair_products_diag(dgchefsi_ctx* ctx, const __nv_bfloat16* Q, int64_t lq, int64_t sq, int64_t rows,
+                                   int64_t K, int64_t k0, int64_t kc, int s, int nw, const PairGroups& groups,
+                                   const uint32_t* norm, int32_t* Pw) {
+  if (rows > 2147483647LL - 256 || K > 2147483647LL)
+    return set_error(DGCHEFSI_ERR_UNSUPPORTED, "slice-pair product too large for 32-bit TMA coordinates");
+  PairTables T(s, nw, groups, 0);
+  for (int i = 0; i < s; ++i) {
+    DG_TRY(slice_map(&T.maps[i], Q + (size_t)i * sq, (uint64_t)K, (uint64_t)rows, (uint64_t)lq));
+    T.maps[s + i] = T.maps[i];
+  }
+  PairJob J{};
+  J.M = rows;
+  J.pitch = 256;
+  J.k0 = (int)k0;
+  J.nk = (int)((kc + 63) / 64);
+  J.nmt = (int)((rows + 255) / 256);
+  J.nnt = 1;
+  // A tile's digits are read by its own units only. While the chunk's digits fit
+  // L2 a few times over, the order by groups (longest first) has the shorter last
+  // wave: 36 tiles of 1001 terms (129 MB) 114 us, 165 by tiles. Above that a
+  // tile's units run side by side and share its reads: 128 tiles of 4096 terms
+  // (3.8 GB) 2.00 -> 1.55 ms, 64 of 2000 (459 MB) 0.48 -> 0.39, 25 of 4096
+  // (367 MB) 0.37 -> 0.35, 39 of 2000 (280 MB) 0.32 by groups, 0.34 by tiles.
+  J.diag = 2 * (double)rows * (double)kc * s > 320e6 ? 2 : 1;
+  J.norm_a = norm;
+  J.norm_b = norm;
+  J.Pw = Pw;
+  return launch_pairs(ctx, J, T, s, groups, false, J.nmt, 0);
 }
 
 dgchefsi_status pair_products_blocks(dgchefsi_ctx* ctx, const BlockPairs& B, int64_t s0, int64_t pn, int32_t* Pw) {

@@ -321,12 +321,32 @@ __device__ __forceinline__ double round_pow2(int64_t hi, int64_t lo, int e) {
   return neg ? -y : y;
 }
 
+// 2^{e + 27} sum_{t < W} 2^{-9t} sum_of(t), |sum_of(t)| < 2^32. Four consecutive t
+// are combined in INT64 (the block is below 2^60). Up to W = 8 the two blocks
+// meet in 128 bits and the sum is rounded once, all in integer instructions;
+// above that the blocks are converted and meet by Horner in 2^{-36}, one
+// rounding of each and one per step.
+template <int W, class Sums>
+__device__ __forceinline__ double digits_to_double(const Sums& sum_of, int e) {
+  constexpr int NB = (W + 3) / 4;
+  // B_b = sum_{t = 4b}^{4b+3} g_t 2^{9(4b + 3 - t)}; sum_t g_t 2^{-9t} = 2^{-27} sum_b B_b 2^{-36b}
+  int64_t B[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    B[b] = 0;
+#pragma unroll
+    for (int t = 4 * b; t < 4 * b + 4; ++t) B[b] = B[b] * 512 + (t < W ? sum_of(t) : 0);
+  }
+  if constexpr (NB <= 2) return round_pow2(B[0], NB == 2 ? B[NB - 1] : 0, e - 36);
+  double h = (double)B[NB - 1];
+#pragma unroll
+  for (int b = NB - 2; b >= 0; --b) h = h * 0x1p-36 + (double)B[b];
+  return scale_pow2(h, e);
+}
+
 // C[r, n0 + c] (+)= (+-) 2^{e_r + f_{n0+c} - 16} sum_t 2^{-9t} g_t for r < M, c < P,
 // g_t the sum of weight t's count[t] INT32 slabs (M rows of `pitch` entries, t
-// descending). Four consecutive t are combined in INT64 (|g_t| < 2^32, so the
-// block is below 2^60). Up to w = 8 the two blocks meet in 128 bits and the sum
-// is rounded once, all in integer instructions; above that the blocks are
-// converted and meet by Horner in 2^{-36}, one rounding of each and one per step.
+// descending).
 // ONE: one slab per weight, all W loads before any use.
 // Two consecutive outputs per thread, so a warp's stores are contiguous; wide:
 // the rows of C at n0 start on 16 bytes. tri > 0: only the entries with
@@ -346,7 +366,6 @@ __global__ void __launch_bounds__(256, 4)
                    const int32_t* __restrict__ Ea, const int32_t* __restrict__ Eb, int nch, int chunk, int64_t n0,
                    double* __restrict__ C, int64_t ldc, int wide, int accumulate, int negate, int64_t tri,
                    const int32_t* __restrict__ cmap) {
-  constexpr int NB = (W + 3) / 4;
   const int64_t half = M * pitch / 2;
   const uint32_t pairs = (uint32_t)(pitch / 2), stride = gridDim.x * blockDim.x;
   const uint32_t q0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -384,30 +403,15 @@ __global__ void __launch_bounds__(256, 4)
         }
       }
     }
-    const auto sum_of = [&](int t, int e) -> int64_t {
-      if (t >= W) return 0;
-      if constexpr (ONE) return e == 0 ? v[t].x : v[t].y;
-      else return g[e][t];
-    };
     double y[2];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      // B_b = sum_{t = 4b}^{4b+3} g_t 2^{9(4b + 3 - t)}; sum_t g_t 2^{-9t} = 2^{-27} sum_b B_b 2^{-36b}
-      int64_t B[NB];
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        B[b] = 0;
-#pragma unroll
-        for (int t = 4 * b; t < 4 * b + 4; ++t) B[b] = B[b] * 512 + sum_of(t, e);
-      }
-      if constexpr (NB <= 2) {
-        y[e] = round_pow2(B[0], NB == 2 ? B[NB - 1] : 0, ec[e] - 36);
-      } else {
-        double h = (double)B[NB - 1];
-#pragma unroll
-        for (int b = NB - 2; b >= 0; --b) h = h * 0x1p-36 + (double)B[b];
-        y[e] = scale_pow2(h, ec[e]);
-      }
+      y[e] = digits_to_double<W>(
+          [&](int t) -> int64_t {
+            if constexpr (ONE) return e == 0 ? v[t].x : v[t].y;
+            else return g[e][t];
+          },
+          ec[e]);
       if (negate) y[e] = -y[e];
     }
     if (cmap) {
@@ -825,6 +829,171 @@ dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols
   reduce<<<grid, 256, 0, st>>>(Pw, rows, cols, cols, groups, Erows, Ecols, 1, 0, 0, C, ldc, 0, 0, 0, 0, cmap);
   count_launch();
   DG_CUDA(cudaGetLastError());
+  return DGCHEFSI_OK;
+}
+
+// ---------------------------------------------------------------------------
+// The density blocks P_K = sum_i f_i x_i x_i^T (f >= 0) from digits: the rows of
+// Z = (sqrt(f_i) x_i)^T are packed into 256-row tiles, whole elements one after
+// another, and the pair kernel multiplies each tile with itself only. Bound by
+// HBM: per row and state 16 bytes for Z, 8 + 14 for its digits and the pairs'
+// reads of them (a tile's digits serve that tile only). FP64 tiles do n + 1
+// operations there (the rule is in density_digits_fit).
+// 8 x 8 x 8 elements of 64, 4096 states: 9.66 ms on the FP64 cores; here 0.44 for
+// Z, 0.67 for the digits, 1.55 for the pairs, 0.04 for the blocks. Largest error
+// against 64-bit mantissas, relative to sqrt(P_jj P_j'j'): 1.0e-16, FP64 1.9e-15.
+
+// Zt[p, i] = sf[i] X[i, col[p]], 0 where col[p] < 0; 32 x 32 tiles, 32 x 8 threads.
+__global__ void __launch_bounds__(256) k_density_rows(const double* __restrict__ X, int64_t ldx, int64_t Ns,
+                                                      const int32_t* __restrict__ col, const double* __restrict__ sf,
+                                                      double* __restrict__ Zt, int64_t ldz) {
+  __shared__ double tile[32][33];
+  const int64_t p0 = (int64_t)blockIdx.x * 32, i0 = (int64_t)blockIdx.y * 32;
+  const int32_t c = col[p0 + threadIdx.x];
+  for (int j = threadIdx.y; j < 32; j += 8) {
+    const int64_t i = i0 + j;
+    tile[j][threadIdx.x] = i < Ns && c >= 0 ? X[i * ldx + c] * sf[i] : 0.0;
+  }
+  __syncthreads();
+  for (int j = threadIdx.y; j < 32; j += 8)
+    if (i0 + threadIdx.x < ldz) Zt[(p0 + j) * ldz + i0 + threadIdx.x] = tile[threadIdx.x][j];
+}
+
+__global__ void k_sqrt(const double* __restrict__ f, int64_t n, double* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = sqrt(f[i]);
+}
+
+// P_K (+)= element K's block of its tile's slabs (rows x 256 each): its rows and
+// columns start at row prow[K] of the packed rows. blockIdx.x: element.
+template <int W>
+__global__ void __launch_bounds__(256) k_density_reduce(const int32_t* __restrict__ nb, const int64_t* __restrict__ poff,
+                                                        const int32_t* __restrict__ prow,
+                                                        const int32_t* __restrict__ Pw, int64_t rows,
+                                                        const PairGroups groups, const int32_t* __restrict__ E, int nch,
+                                                        int chunk, double* __restrict__ P) {
+  const int K = blockIdx.x, n = nb[K], r0 = prow[K], c0 = r0 & 255;
+  double* out = P + poff[K];
+  for (int q = blockIdx.y * 256 + threadIdx.x; q < n * n; q += 256 * gridDim.y) {
+    const int j = q / n, jp = q - j * n;
+    const int32_t* p = Pw + (int64_t)(r0 + j) * 256 + c0 + jp;
+    int64_t g[W];
+#pragma unroll
+    for (int t = W - 1; t >= 0; --t) {
+      g[t] = 0;
+      for (int k = 0; k < groups.count[t]; ++k, p += rows * 256) g[t] += *p;
+    }
+    const int e = E[(int64_t)(r0 + j) * nch + chunk] + E[(int64_t)(r0 + jp) * nch + chunk] - 16 - 27;
+    const double y = digits_to_double<W>([&](int t) -> int64_t { return g[t]; }, e);
+    out[q] = chunk > 0 ? out[q] + y : y;
+  }
+}
+
+typedef void (*DensityReduce)(const int32_t*, const int64_t*, const int32_t*, const int32_t*, int64_t, const PairGroups,
+                              const int32_t*, int, int, double*);
+
+static DensityReduce density_reduce(int w) {
+  switch (w) {
+    case 7: return k_density_reduce<7>;
+    case 8: return k_density_reduce<8>;
+    case 9: return k_density_reduce<9>;
+    case 10: return k_density_reduce<10>;
+    case 11: return k_density_reduce<11>;
+    default: return nullptr;
+  }
+}
+
+// Elements in order, each whole in one 256-row tile; rows of Z in all.
+static int64_t pack_density_rows(const dgchefsi_ctx* ctx, std::vector<int32_t>* prow) {
+  int64_t r = 0;
+  for (int K = 0; K < ctx->M; ++K) {
+    const int n = ctx->nb_h[K];
+    if (r / 256 != (r + n - 1) / 256) r = round_up(r, 256);
+    if (prow) (*prow)[K] = (int32_t)r;
+    r += n;
+  }
+  return round_up(r, 256);
+}
+
+bool density_digits_fit(const dgchefsi_ctx* ctx, int64_t Ns) {
+  int64_t sq = 0;
+  for (int K = 0; K < ctx->M; ++K) {
+    if (ctx->nb_h[K] > 256) return false;
+    sq += (int64_t)ctx->nb_h[K] * ctx->nb_h[K];
+  }
+  const int64_t rows = pack_density_rows(ctx, nullptr);
+  // Both forms per row of Z and state: n + 1 FP64 operations, or some 50 bytes and
+  // 28 pairs of a 256-wide row whatever n is. Kernel time, FP64 and digits, us:
+  // n = 8, 1.4 M row-states 77 / 75; n = 16, 8.2 M 338 / 248; n = 40, 0.8 M 67 / 90;
+  // n = 64, 4.1 M 431 / 145; n = 40..120, 20 M 2040 / 590; n = 64, 134 M 9660 / 2700.
+  return rows < 1 << 30 && Ns < 1 << 20 && sq >= 16 * rows && rows * Ns >= 1 << 21;
+}
+
+dgchefsi_status density_digits(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P,
+                               bool* done) {
+  *done = false;
+  const int slices = std::max(ctx->products_slices, 10), s = digits_for(slices), nw = weights_for(slices);
+  cudaStream_t st = ctx->stream;
+  const DensityReduce reduce = density_reduce(nw);
+  if (!reduce) return DGCHEFSI_OK;
+  std::vector<int32_t> prow(ctx->M);
+  const int64_t max_nb = ctx->view().max_nb;
+  const int64_t rows = pack_density_rows(ctx, &prow);
+  const int nch = (int)((Ns + kL - 1) / kL);
+  const int64_t ldz = round_up(Ns, 2), lq = round_up(Ns, 8), sq = rows * lq;
+  int nsm = 0;
+  DG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+  const PairGroups groups = pair_groups(s, nw, rows / 256, nsm);
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t q_bytes = up(sizeof(__nv_bfloat16) * (size_t)(s * sq)), e_bytes = up(sizeof(int32_t) * (size_t)(rows * nch));
+  const size_t n_bytes = up(sizeof(uint32_t) * (size_t)(kNormPitch * nch) + sizeof(int));
+  const size_t c_bytes = up(sizeof(int32_t) * (size_t)rows), k_bytes = up(sizeof(int32_t) * (size_t)ctx->M);
+  const size_t s_bytes = up(sizeof(double) * (size_t)Ns);
+  const size_t w_bytes = sizeof(int32_t) * (size_t)groups.total * (size_t)rows * 256;
+  // the buffers of the rotation before it, larger only where the packing pads; without the memory, the FP64 form
+  if (ensure(ctx, ctx->ws_sliced_b, sizeof(double) * (size_t)(rows * ldz), "density rows") != DGCHEFSI_OK ||
+      ensure(ctx, ctx->ws_sliced, q_bytes + e_bytes + n_bytes + c_bytes + k_bytes + s_bytes + w_bytes,
+             "density digits") != DGCHEFSI_OK) {
+    clear_error();
+    return DGCHEFSI_OK;
+  }
+  char* at = static_cast<char*>(ctx->ws_sliced.p);
+  auto take = [&](size_t bytes) { char* p = at; at += bytes; return p; };
+  __nv_bfloat16* Q = reinterpret_cast<__nv_bfloat16*>(take(q_bytes));
+  int32_t* E = reinterpret_cast<int32_t*>(take(e_bytes));
+  uint32_t* norm = reinterpret_cast<uint32_t*>(take(n_bytes));
+  int* flag = reinterpret_cast<int*>(norm + kNormPitch * nch);
+  int32_t* col_d = reinterpret_cast<int32_t*>(take(c_bytes));
+  int32_t* prow_d = reinterpret_cast<int32_t*>(take(k_bytes));
+  double* sf = reinterpret_cast<double*>(take(s_bytes));
+  int32_t* Pw = reinterpret_cast<int32_t*>(at);
+  double* Zt = static_cast<double*>(ctx->ws_sliced_b.p);
+  std::vector<int32_t> col(rows, -1);
+  for (int K = 0; K < ctx->M; ++K)
+    for (int j = 0; j < ctx->nb_h[K]; ++j) col[prow[K] + j] = (int32_t)(ctx->off_h[K] + j);
+  DG_CUDA(cudaMemcpyAsync(col_d, col.data(), sizeof(int32_t) * (size_t)rows, cudaMemcpyHostToDevice, st));
+  DG_CUDA(cudaMemcpyAsync(prow_d, prow.data(), sizeof(int32_t) * (size_t)ctx->M, cudaMemcpyHostToDevice, st));
+  DG_CUDA(cudaMemsetAsync(norm, 0, n_bytes, st));
+  k_sqrt<<<(unsigned)((Ns + 255) / 256), 256, 0, st>>>(f, Ns, sf);
+  k_density_rows<<<dim3((unsigned)(rows / 32), (unsigned)((Ns + 31) / 32)), dim3(32, 8), 0, st>>>(X, ld, Ns, col_d, sf,
+                                                                                              Zt, ldz);
+  k_split_rows<<<dim3((unsigned)rows, (unsigned)nch), kSplitThreads, 0, st>>>(Zt, ldz, Ns, s, 0, 1, nullptr, Q, lq, sq, E,
+                                                                              nch, norm, flag);
+  count_launch(3);
+  DG_CUDA(cudaGetLastError());
+  DG_TRY(pair_products_begin(ctx));
+  const unsigned ctas = (unsigned)((max_nb * max_nb + 1023) / 1024);  // four entries a thread
+  for (int chunk = 0; chunk < nch; ++chunk) {
+    const int64_t k0 = (int64_t)chunk * kL, kc = std::min<int64_t>(kL, Ns - k0);
+    DG_TRY(pair_products_diag(ctx, Q, lq, sq, rows, Ns, k0, kc, s, nw, groups, norm + kNormPitch * chunk, Pw));
+    reduce<<<dim3((unsigned)ctx->M, ctas), 256, 0, st>>>(ctx->nb_d, ctx->poff_d, prow_d, Pw, rows, groups, E, nch, chunk, P);
+    count_launch();
+    DG_CUDA(cudaGetLastError());
+  }
+  int bad = 0;  // a state or an occupation that is not finite: the FP64 form spreads it as it did
+  DG_CUDA(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+  DG_TRY(pair_products_status(ctx));  // synchronises the stream
+  *done = bad == 0;
   return DGCHEFSI_OK;
 }
 
