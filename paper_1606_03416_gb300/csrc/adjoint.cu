@@ -67,8 +67,7 @@ extern "C" dgchefsi_status dgchefsi_set_values(dgchefsi_ctx* ctx, const double* 
   if (!values) return set_error(DGCHEFSI_ERR_ARG, "null values");
   DG_CUDA(cudaMemcpyAsync(ctx->vals_d, values, sizeof(double) * (size_t)ctx->n_values, cudaMemcpyDeviceToDevice,
                           ctx->stream));
-  if (ctx->tc) tc_destroy(ctx);  // operand copies of H are rebuilt from the new values
-  return DGCHEFSI_OK;
+  return tc_values_changed(ctx);  // operand copies of H are rebuilt from the new values
 }
 
 extern "C" dgchefsi_status dgchefsi_energy_grad(dgchefsi_ctx* ctx, int prec, const double* X, int64_t Ns, int64_t ld,

@@ -168,6 +168,12 @@ dgchefsi_status tc_grad_forward(dgchefsi_ctx* ctx, int prec, const double* X, in
 dgchefsi_status tc_grad_backward(dgchefsi_ctx* ctx, int prec, const double* Wm, int64_t Ns, int m, int stride,
                                  double* H_bar, double* X_bar, int64_t ld_xbar);
 void tc_destroy(dgchefsi_ctx* ctx);
+// After new values of H: everything built from the old ones and what was tuned
+// or captured with them goes, as in tc_destroy; the layout of the pattern, the
+// plan and the buffers of the sliced H X stay (H's digits are split anew): a
+// gradient's forward and backward call spent 1.2 of 64.4 ms (4 x 4 x 4 elements of
+// 40, 300 states) on making them again.
+dgchefsi_status tc_values_changed(dgchefsi_ctx* ctx);
 
 // C (M x Nc, row-major, ldc) = A B^T (b_rows: B is Nc x K) or A B (B is K x Nc),
 // A (M x K, lda) row-major, all FP64, computed from s exact BF16 slices per

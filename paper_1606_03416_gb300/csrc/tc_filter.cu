@@ -6,6 +6,8 @@
 #include <cmath>
 #include <iterator>
 #include <map>
+#include <new>
+#include <utility>
 
 #include "tc_kernel.cuh"
 
@@ -285,6 +287,7 @@ struct Plan {
 
 struct TcState {
   int64_t Ns = -1, ldp = 0;
+  bool unused = false;  // nothing has run since new values of H
   int mode = -1;  // precision the operand copy of H is laid out for
   int boxn = 16, ACC = 64, num_sms = 0;
   std::vector<int32_t> pnb_h, poff_h, blk_row_h;
@@ -358,6 +361,7 @@ static void free_plan(Plan& pl) {
 }
 
 static dgchefsi_status ensure_layout(dgchefsi_ctx* ctx, TcState& t) {
+  t.unused = false;
   if (!t.pnb_h.empty()) return DGCHEFSI_OK;
   const int M = ctx->M;
   t.pnb_h.resize(M);
@@ -1194,7 +1198,7 @@ dgchefsi_status tc_grad_backward(dgchefsi_ctx* ctx, int prec, const double* Wm, 
   return check_err(t, s);
 }
 
-// Workspace cap of the FP32 slice-pair slabs of the sliced H X; the states run
+// Workspace cap of the INT32 weight slabs of the sliced H X; the states run
 // in panels of 256-state multiples below it.
 static constexpr size_t kSlabBytes = size_t(8) << 30;
 
@@ -1411,7 +1415,7 @@ dgchefsi_status tc_get_unit_order(dgchefsi_ctx* ctx, int prec, int* tgb) {
 }
 
 dgchefsi_status tc_get_shape(dgchefsi_ctx* ctx, int prec, int* G, int* T, int* ACC, int* layout) {
-  if (!ctx->tc) {
+  if (!ctx->tc || ctx->tc->unused) {
     *G = *T = *ACC = *layout = 0;
     return DGCHEFSI_OK;
   }
@@ -1421,6 +1425,34 @@ dgchefsi_status tc_get_shape(dgchefsi_ctx* ctx, int prec, int* G, int* T, int* A
   *T = t.forceG[mode] ? t.forceT[mode] : t.shapeT[mode];
   *layout = t.forceG[mode] ? t.forceL[mode] : t.shapeL[mode];
   *ACC = t.ACC;
+  return DGCHEFSI_OK;
+}
+
+dgchefsi_status tc_values_changed(dgchefsi_ctx* ctx) {
+  if (!ctx->tc) return DGCHEFSI_OK;
+  // what is freed may still be read, and the caller may go on in another stream
+  DG_CUDA(cudaStreamSynchronize(ctx->stream));
+  TcState& t = *ctx->tc;
+  TcState* n = new (std::nothrow) TcState();
+  if (n && !t.pnb_h.empty()) {
+    std::swap(n->pnb_h, t.pnb_h);
+    std::swap(n->poff_h, t.poff_h);
+    std::swap(n->blk_row_h, t.blk_row_h);
+    std::swap(n->pnb_d, t.pnb_d);
+    std::swap(n->poff_d, t.poff_d);
+    std::swap(n->blk_row_d, t.blk_row_d);
+    std::swap(n->brow_d, t.brow_d);
+    std::swap(n->err_d, t.err_d);
+    std::swap(n->sx, t.sx);
+    n->ldp = t.ldp;
+    n->boxn = t.boxn;
+    n->ACC = t.ACC;
+    n->num_sms = t.num_sms;
+    n->sx.h_built = false;
+    n->unused = true;
+  }
+  tc_destroy(ctx);
+  ctx->tc = n;
   return DGCHEFSI_OK;
 }
 
