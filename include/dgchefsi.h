@@ -266,7 +266,9 @@ dgchefsi_status dgchefsi_set_orthonormalisation(dgchefsi_ctx* ctx, int mode);
  *           below the FP64 worst-case bound for rows of similar magnitude
  * ERR_ARG for another mode or slice count. In the sliced form H Y_hat runs
  * from slices too (dgchefsi_sliced_matvec) when H fits that form, else on the
- * FP64 cores.
+ * FP64 cores, and dgchefsi_cycle forms its density blocks P_KK from slices (at
+ * least 10; sqrt(f_i) x_i split once) where that is faster: elements of 16
+ * functions and more on average, none above 256, and enough states.
  * dgchefsi_energy_grad follows the same setting for its forward products
  * (H Y_hat included) and the dense products of its adjoint (Z = U^{-1} Q,
  * W_m = Z (2 G R^T)); dgchefsi_gram always uses FP64 products. */
@@ -444,13 +446,14 @@ dgchefsi_status dgchefsi_sliced_timing(dgchefsi_ctx* ctx, double* pairs_ms, int6
  * product of Eq. matvec_3 (y_K = sum over K' in N(K) of H_{K;K'} x_{K'}) that
  * the Rayleigh-Ritz step (Alg. 1 step 4, H Y_hat) runs when the context's
  * subspace products are DGCHEFSI_PRODUCTS_SLICED_BF16. Each row of H (element
- * K, row n) is split into `slices` 6-bit digits with one exponent e_r for the
- * whole row, which contracts over at most 4096 columns (the columns of K's
- * neighbour blocks), so every slice-pair product is an exact FP32 integer;
- * each state with one exponent f_s over all its N entries. The slice pairs
- * (i + j <= slices - 1) run on the tensor-core filter's block-sparse step
- * kernel, one pair per launch, into FP32 workspace (state panels under 8 GB),
- * and are summed in FP64 as in dgchefsi_sliced_gemm. Error of Y[s, r]: at most
+ * K, row n) is split into 9-bit digits worth `slices` 6-bit ones (as in
+ * dgchefsi_sliced_gemm) with one exponent e_r for the whole row, which
+ * contracts over at most 4096 columns (the columns of K's neighbour blocks);
+ * each state with one exponent f_s over all its N entries. The pairs of digits
+ * run on the dense form's kernel, tile rows = the H rows of a few neighbouring
+ * elements, exact in FP32 and INT32, into one INT32 slab per digit weight
+ * (workspace; state panels under 8 GB), and the slabs are summed as in
+ * dgchefsi_sliced_gemm. Error of Y[s, r]: at most
  * L m_r n_s (2^{-6 slices} (slices + 4) + 6 u), L = the row's column count,
  * m_r and n_s the row's and the state's largest |entry|.
  *   X  device (Ns x ld) state-major, FP64;  Y  device (Ns x ld) out, must not overlap X

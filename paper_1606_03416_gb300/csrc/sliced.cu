@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <cmath>
 #include <climits>
+#include <new>
 
 #include "ctx.h"
 
@@ -936,9 +937,16 @@ dgchefsi_status density_digits(dgchefsi_ctx* ctx, const double* X, int64_t Ns, i
   cudaStream_t st = ctx->stream;
   const DensityReduce reduce = density_reduce(nw);
   if (!reduce) return DGCHEFSI_OK;
-  std::vector<int32_t> prow(ctx->M);
   const int64_t max_nb = ctx->view().max_nb;
-  const int64_t rows = pack_density_rows(ctx, &prow);
+  std::vector<int32_t> prow, col;
+  int64_t rows = 0;
+  try {
+    prow.resize(ctx->M);
+    rows = pack_density_rows(ctx, &prow);
+    col.assign(rows, -1);
+  } catch (const std::bad_alloc&) {
+    return DGCHEFSI_OK;
+  }
   const int nch = (int)((Ns + kL - 1) / kL);
   const int64_t ldz = round_up(Ns, 2), lq = round_up(Ns, 8), sq = rows * lq;
   int nsm = 0;
@@ -968,7 +976,6 @@ dgchefsi_status density_digits(dgchefsi_ctx* ctx, const double* X, int64_t Ns, i
   double* sf = reinterpret_cast<double*>(take(s_bytes));
   int32_t* Pw = reinterpret_cast<int32_t*>(at);
   double* Zt = static_cast<double*>(ctx->ws_sliced_b.p);
-  std::vector<int32_t> col(rows, -1);
   for (int K = 0; K < ctx->M; ++K)
     for (int j = 0; j < ctx->nb_h[K]; ++j) col[prow[K] + j] = (int32_t)(ctx->off_h[K] + j);
   DG_CUDA(cudaMemcpyAsync(col_d, col.data(), sizeof(int32_t) * (size_t)rows, cudaMemcpyHostToDevice, st));
