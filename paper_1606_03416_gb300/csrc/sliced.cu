@@ -87,8 +87,40 @@ __device__ __forceinline__ int warp_max(int v) {
   return v;
 }
 
-// C = 2 or 4 consecutive digits (integers, |f| <= 256) to q as BF16, their squares to *norm.
-template <int C>
+// Largest bit pattern of |x[0]| .. |x[n - 1]| (the order of the magnitudes, NaN
+// and infinity above the rest), to all 256 threads of the CTA. Four loads of 16
+// bytes before their use: a pass over a row waits on memory, not on instructions.
+__device__ __forceinline__ unsigned long long cta_max_bits(const double* __restrict__ x, int64_t n) {
+  unsigned long long m = 0;
+  const auto take = [&](double v) { m = max(m, (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL); };
+  int64_t c0 = 0;
+  if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+    const double2* x2 = reinterpret_cast<const double2*>(x);
+    for (; c0 + 2048 <= n; c0 += 2048) {
+      double2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = x2[c0 / 2 + threadIdx.x + 256 * u];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        take(v[u].x);
+        take(v[u].y);
+      }
+    }
+  }
+  for (int64_t c = c0 + threadIdx.x; c < n; c += 256) take(x[c]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  __shared__ unsigned long long red[8];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = max(m, red[w]);
+  return m;
+}
+
+// C = 2 or 4 consecutive digits (integers, |f| <= 256) to q as BF16, their squares to *norm
+// (HALF: each half of the warp has its own norm).
+template <int C, bool HALF>
 __device__ __forceinline__ void put_digits(const float (&f)[C], __nv_bfloat16* __restrict__ q, bool store,
                                            uint32_t* norm) {
   uint32_t w[C / 2];
@@ -105,8 +137,9 @@ __device__ __forceinline__ void put_digits(const float (&f)[C], __nv_bfloat16* _
     else
       *reinterpret_cast<uint32_t*>(q) = w[0];
   }
-  const uint32_t sum = __reduce_add_sync(0xffffffffu, __float_as_uint(sq) & 0x7fffffu);
-  if ((threadIdx.x & 31) == 0) atomicAdd(norm, sum);
+  const uint32_t mask = HALF ? 0xffffu << (threadIdx.x & 16) : 0xffffffffu;
+  const uint32_t sum = __reduce_add_sync(mask, __float_as_uint(sq) & 0x7fffffu);
+  if ((threadIdx.x & (HALF ? 15 : 31)) == 0) atomicAdd(norm, sum);
 }
 
 // Digits i = 0 .. d - 1 of C consecutive entries v 2^{b} scaled by 2^{-e}
@@ -121,7 +154,7 @@ __device__ __forceinline__ void put_digits(const float (&f)[C], __nv_bfloat16* _
 // would run at a quarter of that rate.
 // d > 7 (F would not fit 64 bits): v is scaled in FP64, each digit rounded to
 // nearest and subtracted (every step exact).
-template <int C>
+template <int C, bool HALF = false>
 __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (&b)[C], int e, bool zero, int d,
                                                __nv_bfloat16* __restrict__ q, int64_t stride, bool store,
                                                uint32_t* norm) {
@@ -150,7 +183,7 @@ __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (
                      : __uint_as_float((lo + 512u) + 0x4B000000u) - 8389120.f; // the rest, -256 .. 256
         F[c] >>= 9;
       }
-      put_digits<C>(f, q + i * stride, store, norm + i);
+      put_digits<C, HALF>(f, q + i * stride, store, norm + i);
     }
   } else {
     double r[C];
@@ -163,7 +196,7 @@ __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (
         r[c] = (r[c] - g) * 512.0;
         f[c] = (float)g;
       }
-      put_digits<C>(f, q + i * stride, store, norm + i);
+      put_digits<C, HALF>(f, q + i * stride, store, norm + i);
     }
   }
 }
@@ -265,24 +298,16 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_rows(const double* __re
 }
 
 // bal[k] = frexp exponent of max_c |X[k, c]| (X row-major K x C), 0 for a row
-// with no finite nonzero entry, and nbal[k] = -bal[k]. One CTA per row.
+// of zeros or with an entry that is not finite, and nbal[k] = -bal[k]. One CTA per
+// row. Bound by HBM: 4096 x 32768 0.16 ms, 6.5 TB/s (0.26 with one 8-byte load at a time).
 __global__ void __launch_bounds__(256) k_row_exponents(const double* __restrict__ X, int64_t ldx, int64_t C,
                                                        int32_t* __restrict__ bal, int32_t* __restrict__ nbal) {
   const int64_t k = blockIdx.x;
-  int emax = INT_MIN;
-  for (int64_t c = threadIdx.x; c < C; c += 256) {
+  const double top = __longlong_as_double((long long)cta_max_bits(X + k * ldx, C));
+  if (threadIdx.x == 0) {
     int64_t M;
     int Ex;
-    if (decompose(X[k * ldx + c], M, Ex) == 1) emax = max(emax, Ex);
-  }
-  emax = warp_max(emax);
-  __shared__ int red[8];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = emax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) emax = max(emax, red[w]);
-    emax = max(emax, red[0]);
-    bal[k] = emax == INT_MIN ? 0 : emax - 1022;
+    bal[k] = decompose(top, M, Ex) == 1 ? Ex - 1022 : 0;
     nbal[k] = -bal[k];
   }
 }
@@ -739,8 +764,10 @@ __global__ void __launch_bounds__(256) k_h_digits(const int32_t* __restrict__ bl
 // d digit copies of the states X (Ns x ld, state-major) in the element-padded
 // layout (Ns x ldp per copy, copy i at Q + i * cstride); slices[k] = {padded
 // column, column, columns, padded columns} of the k-th 64-wide slice. E[s] =
-// frexp exponent of the state's largest |entry|. One CTA per state, two passes,
-// a warp per slice.
+// frexp exponent of the state's largest |entry|. One CTA per state, two passes;
+// in the second a half warp takes a slice, four entries a lane.
+// 4096 states of 32768: 0.81 ms; 1.65 with a warp per slice and two entries a
+// lane, whose reductions, counters and 4-byte stores took the time.
 __global__ void __launch_bounds__(256) k_state_digits(const double* __restrict__ X, int64_t ld, int64_t N,
                                                       const int4* __restrict__ slices, int nslices, int64_t ldp, int d,
                                                       __nv_bfloat16* __restrict__ Q, int64_t cstride,
@@ -748,47 +775,42 @@ __global__ void __launch_bounds__(256) k_state_digits(const double* __restrict__
                                                       int* __restrict__ flag) {
   const int64_t st = blockIdx.x;
   const double* x = X + st * ld;
-  int emax = INT_MIN;
-  bool bad = false;
-  for (int64_t c = threadIdx.x; c < N; c += blockDim.x) {
-    int64_t Mm;
-    int Ex;
-    const int k = decompose(x[c], Mm, Ex);
-    if (k == 2) bad = true;
-    if (k == 1) emax = max(emax, Ex);
-  }
-  __shared__ int red[8];
-  __shared__ int sbad;
-  __shared__ uint32_t norm[8][kNormPitch], top[kNormPitch];
-  if (threadIdx.x == 0) sbad = 0;
+  __shared__ uint32_t norm[16][kNormPitch], top[kNormPitch];
   if (threadIdx.x < kNormPitch) top[threadIdx.x] = 0;
-  emax = warp_max(emax);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[warp] = emax;
-  if (bad) sbad = 1;
-  __syncthreads();
-  emax = red[0];
-#pragma unroll
-  for (int w = 1; w < 8; ++w) emax = max(emax, red[w]);
-  const bool zero = sbad != 0;
-  const int e = (emax == INT_MIN || zero) ? 0 : emax - 1022;
+  int64_t Mm;
+  int Ex;
+  const int kind = decompose(__longlong_as_double((long long)cta_max_bits(x, N)), Mm, Ex);  // synchronises
+  const bool zero = kind == 2;
+  const int e = kind == 1 ? Ex - 1022 : 0;
   if (threadIdx.x == 0) {
     E[st] = e;
     if (zero) atomic_flag(flag);
   }
-  for (int k = warp; k < nslices; k += 8) {
+  const int half = threadIdx.x >> 4, l = threadIdx.x & 15;
+  for (int k0 = 0; k0 < nslices; k0 += 16) {
+    // the last slices: a half warp without one repeats the last and stores nothing
+    const int k = min(k0 + half, nslices - 1);
     const int4 sl = slices[k];
-    const int j = 2 * lane;
-    const int b[2] = {0, 0};
-    double v[2];
+    const int j = 4 * l;
+    const int b[4] = {0, 0, 0, 0};
+    const double* xs = x + sl.y + j;
+    double v[4];
+    if (j + 4 <= sl.z && (reinterpret_cast<uintptr_t>(xs) & 15) == 0) {
+      const double2 a = *reinterpret_cast<const double2*>(xs), c = *reinterpret_cast<const double2*>(xs + 2);
+      v[0] = a.x;
+      v[1] = a.y;
+      v[2] = c.x;
+      v[3] = c.y;
+    } else {
 #pragma unroll
-    for (int c = 0; c < 2; ++c) v[c] = j + c < sl.z ? x[sl.y + j + c] : 0.0;
-    if (lane < kNormPitch) norm[warp][lane] = 0;
+      for (int c = 0; c < 4; ++c) v[c] = j + c < sl.z ? xs[c] : 0.0;
+    }
+    if (l < kNormPitch) norm[half][l] = 0;
     __syncwarp();
-    put_all_digits<2>(v, b, e, zero, d, Q + st * ldp + sl.x + j, cstride, j < sl.w, norm[warp]);
+    put_all_digits<4, true>(v, b, e, zero, d, Q + st * ldp + sl.x + j, cstride, j < sl.w && k0 + half < nslices,
+                            norm[half]);
     __syncwarp();
-    if (lane < d) atomicMax(&top[lane], norm[warp][lane]);
+    if (l < d) atomicMax(&top[l], norm[half][l]);
     __syncwarp();
   }
   __syncthreads();

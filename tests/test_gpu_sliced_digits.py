@@ -69,3 +69,22 @@ def test_sums_are_rounded_once(M, Nc, K, e, slices):
     exact = A.astype(object) @ Bt.T.astype(object)
     want = np.array([[float(x) for x in row] for row in exact])
     assert np.array_equal(product(A * 2.0 ** e, Bt * 2.0 ** e, True, slices), np.ldexp(want, 2 * e))
+
+
+@pytest.mark.parametrize("grid,nb,Ns,ld_more", [((1, 1, 1), 5, 1, 0), ((3, 2, 2), (17, 31), 9, 1), ((4, 2, 2), 64, 5, 0),
+                                                ((3, 3, 2), 70, 4, 3), ((5, 7, 1), (40, 120), 3, 1)])
+def test_state_digits_bit_exact(grid, nb, Ns, ld_more):
+    """Integer H and states (products far below 2^53) on states of 1 to 58
+    slices of 64, slices that are not full, rows and elements that start on 8 or 16
+    bytes: the sliced H X equals the FP64 product bit for bit."""
+    cfg = G.scaled_copy(G.CONFIGS["sheet2d_24x20" if grid[2] == 1 else "bulk3d_8x8x8"], grid=grid, nb=nb, Ns=Ns)
+    H = G.make_blocks(cfg)
+    rng = np.random.default_rng(5)
+    X = torch.zeros((Ns, H.N + ld_more), dtype=torch.float64, device="cuda")
+    X[:, : H.N] = torch.from_numpy(rng.integers(-2 ** 20, 2 ** 20, size=(Ns, H.N)).astype(np.float64)).cuda()
+    with D.Context(H) as ctx:
+        ctx.set_values(torch.from_numpy(np.round(H.values * 64)).cuda())
+        W, V = torch.zeros_like(X), torch.zeros_like(X)
+        ctx.sliced_matvec(X[:, : H.N], W[:, : H.N])
+        ctx.matvec(X[:, : H.N], V[:, : H.N])
+        assert torch.equal(W, V)
