@@ -1449,8 +1449,8 @@ dgchefsi_status tc_values_changed(dgchefsi_ctx* ctx) {
     n->ACC = t.ACC;
     n->num_sms = t.num_sms;
     n->sx.h_built = false;
-    n->unused = true;
   }
+  if (n) n->unused = true;
   tc_destroy(ctx);
   ctx->tc = n;
   return DGCHEFSI_OK;
