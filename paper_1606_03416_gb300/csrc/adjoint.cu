@@ -177,10 +177,7 @@ extern "C" dgchefsi_status dgchefsi_energy_grad(dgchefsi_ctx* ctx, int prec, con
   // read (the Cholesky factorisation and the eigensolver)
   auto prod_nt = [&](const double* A_, const double* B_, double* C_) -> dgchefsi_status {
     if (sl) return sliced_gemm(ctx, true, false, Ns, Ns, N, A_, N, B_, N, C_, Ns, nsl, bad, Ns);
-    Parts parts;
-    DG_TRY(parts_of(ctx, &parts));
-    DG_CUDA(gemm_nt_f64(A_, N, B_, N, C_, Ns, Ns, Ns, N, true, false, parts, s));
-    return DGCHEFSI_OK;
+    return sym_product_f64(ctx, A_, N, B_, N, C_, Ns, Ns, N);
   };
   auto prod_nn = [&](const double* A_, const double* B_, int64_t ldb_, int64_t cols, double* C_, int64_t ldc_,
                      bool lower) -> dgchefsi_status {  // C = A B, A N_s x N_s, K = N_s

@@ -49,6 +49,43 @@ dgchefsi_status ensure(dgchefsi_ctx* ctx, DevBuf& b, size_t bytes, const char* w
   return DGCHEFSI_OK;
 }
 
+dgchefsi_status parts_begin(dgchefsi_ctx* ctx, Parts* parts) {
+  *parts = Parts();
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return DGCHEFSI_OK;
+  }
+  DG_TRY(ensure(ctx, ctx->ws_parts, kPartsBytes, "partial products"));
+  if (!ctx->ev_parts)
+    DG_CUDA(cudaEventCreateWithFlags(&ctx->ev_parts, cudaEventDisableTiming));
+  else
+    DG_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_parts, 0));
+  parts->p = static_cast<double*>(ctx->ws_parts.p);
+  parts->doubles = (int64_t)(ctx->ws_parts.bytes / sizeof(double));
+  return DGCHEFSI_OK;
+}
+
+dgchefsi_status parts_end(dgchefsi_ctx* ctx, const Parts& parts) {
+  if (parts.p) DG_CUDA(cudaEventRecord(ctx->ev_parts, ctx->stream));
+  return DGCHEFSI_OK;
+}
+
+dgchefsi_status sym_product_f64(dgchefsi_ctx* ctx, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
+                                int64_t ldc, int64_t n, int64_t K) {
+  Parts parts;
+  DG_TRY(parts_begin(ctx, &parts));
+  DG_CUDA(gemm_nt_f64(A, lda, B, ldb, C, ldc, n, n, K, true, false, parts, ctx->stream));
+  return parts_end(ctx, parts);
+}
+
+dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P) {
+  Parts parts;
+  DG_TRY(parts_begin(ctx, &parts));
+  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
+  return parts_end(ctx, parts);
+}
+
 static void free_buf(DevBuf& b) {
   if (b.p) cudaFree(b.p);
   b.p = nullptr;
@@ -313,8 +350,6 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
   const bool sl = ctx->products_mode == DGCHEFSI_PRODUCTS_SLICED_BF16;
   const bool own_chol = use_own_cholesky(ctx);
   int* bad = ctx->info_d + 3;
-  Parts parts;
-  DG_TRY(parts_of(ctx, &parts));
   // Step 3: S = Y^T Y (lower tiles, mirrored), S = U^T U, Y_hat = Y U^{-1}.
   // CholeskyQR2 repeats the pass on Y_hat; shifted CholeskyQR3 factors
   // Y^T Y + s I first, s = 11 (N N_s + N_s (N_s + 1)) u ||Y||_F^2, then repeats
@@ -329,7 +364,7 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
     if (sl)
       DG_TRY(sliced_gemm(ctx, true, false, Ns, Ns, N, in, ldi, in, ldi, S, Ns, ctx->products_slices, bad, Ns));
     else
-      DG_CUDA(gemm_nt_f64(in, ldi, in, ldi, S, Ns, Ns, Ns, N, true, false, parts, s));
+      DG_TRY(sym_product_f64(ctx, in, ldi, in, ldi, S, Ns, Ns, N));
     if (pass == 0 && ctx->orth_mode == DGCHEFSI_ORTH_SHIFTED_CHOLQR3)
       DG_CUDA(shift_diagonal_by_trace_f64(S, Ns, 11.0 * ((double)N * (double)Ns + (double)Ns * (double)(Ns + 1)) *
                                                      0x1p-53, s));
@@ -372,7 +407,7 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
   if (sl)
     DG_TRY(sliced_gemm(ctx, true, false, Ns, Ns, N, W, N, Y, ld, S, Ns, ctx->products_slices, bad, Ns));
   else
-    DG_CUDA(gemm_nt_f64(W, N, Y, ld, S, Ns, Ns, Ns, N, true, false, parts, s));
+    DG_TRY(sym_product_f64(ctx, W, N, Y, ld, S, Ns, Ns, N));
   // The eigensolver reads the lower triangle (row-major), the one computed.
   DG_TRY(subspace_eigh(ctx, S, Ns, Ns, ritz));
   // Step 5: X_new^T = Q^T Y_hat^T (column-major Q read row-major is Q^T).
@@ -549,7 +584,8 @@ void dgchefsi_destroy(dgchefsi_ctx* ctx) {
   free_buf(ctx->ws_pairs_err);
   free_buf(ctx->ws_eig);
   free_buf(ctx->ws_chol);
-  free_buf(ctx->ws_parts);
+  free_buf(ctx->ws_parts);  // waits for the device, and so for its last user on whatever stream
+  if (ctx->ev_parts) cudaEventDestroy(ctx->ev_parts);
   if (ctx->s_reduce) cudaStreamSynchronize(ctx->s_reduce);
   for (int i = 0; i < 2; ++i) {
     if (ctx->ev_pairs[i]) cudaEventDestroy(ctx->ev_pairs[i]);
@@ -1005,10 +1041,7 @@ dgchefsi_status dgchefsi_gram(dgchefsi_ctx* ctx, const double* Y, int64_t Ns, in
   DG_TRY(check_ctx(ctx));
   DG_TRY(check_block(ctx, Y, Ns, ld, "Y"));
   if (Ns > 0 && !S) return set_error(DGCHEFSI_ERR_ARG, "null S");
-  Parts parts;
-  DG_TRY(parts_of(ctx, &parts));
-  DG_CUDA(gemm_nt_f64(Y, ld, Y, ld, S, Ns, Ns, Ns, ctx->N, true, false, parts, ctx->stream));
-  return DGCHEFSI_OK;
+  return sym_product_f64(ctx, Y, ld, Y, ld, S, Ns, Ns, ctx->N);
 }
 
 dgchefsi_status dgchefsi_rayleigh_ritz(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t ld, double* ritz) {
@@ -1040,10 +1073,7 @@ dgchefsi_status dgchefsi_density_blocks(dgchefsi_ctx* ctx, const double* X, int6
   DG_TRY(check_ctx(ctx));
   DG_TRY(check_block(ctx, X, Ns, ld, "X"));
   if (!P || (Ns > 0 && !f)) return set_error(DGCHEFSI_ERR_ARG, "null f or P");
-  Parts parts;
-  DG_TRY(parts_of(ctx, &parts));
-  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
-  return DGCHEFSI_OK;
+  return density_blocks_f64(ctx, X, Ns, ld, f, P);
 }
 
 dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t Ns, int64_t ld, int m, double Ne,
@@ -1091,11 +1121,7 @@ dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t N
   bool done = false;
   if (ctx->products_mode == DGCHEFSI_PRODUCTS_SLICED_BF16 && density_digits_fit(ctx, Ns))
     DG_TRY(density_digits(ctx, X, Ns, ld, f, P, &done));
-  if (!done) {
-    Parts parts;
-    DG_TRY(parts_of(ctx, &parts));
-    DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
-  }
+  if (!done) DG_TRY(density_blocks_f64(ctx, X, Ns, ld, f, P));
   if (bounds) {
     bounds[0] = a;
     bounds[1] = b;

@@ -89,6 +89,7 @@ struct dgchefsi_ctx {
   int chol_mode = 0;
   dg::DevBuf ws_chol;
   dg::DevBuf ws_parts;    // partial results of split FP64 products (kPartsBytes)
+  cudaEvent_t ev_parts = nullptr;  // after the last of them that was enqueued
   // FP64 filter as a CUDA graph: coefficients copied from a pinned mirror at
   // every replay; the graph is captured again when X, Y, N_s, ld, m or the
   // workspace it refers to change
@@ -133,16 +134,19 @@ void clear_error();
 // Make `b` hold at least `bytes` (synchronises the context's stream before a regrow).
 dgchefsi_status ensure(dgchefsi_ctx* ctx, DevBuf& b, size_t bytes, const char* what);
 
-// The context's buffer for split FP64 products, one for all of them (they run
-// in turn on the context's stream).
+// The context's buffer for split FP64 products, one for all of them. The calls
+// that use it may be asynchronous and the context's stream may change between
+// them (dgchefsi_set_stream), so parts_begin makes the stream wait for the last
+// product's sum and parts_end records this one's.
 constexpr size_t kPartsBytes = size_t(128) << 20;
-inline dgchefsi_status parts_of(dgchefsi_ctx* ctx, Parts* parts) {
-  const dgchefsi_status st = ensure(ctx, ctx->ws_parts, kPartsBytes, "partial products");
-  if (st != DGCHEFSI_OK) return st;
-  parts->p = static_cast<double*>(ctx->ws_parts.p);
-  parts->doubles = (int64_t)(ctx->ws_parts.bytes / sizeof(double));
-  return DGCHEFSI_OK;
-}
+dgchefsi_status parts_begin(dgchefsi_ctx* ctx, Parts* parts);
+dgchefsi_status parts_end(dgchefsi_ctx* ctx, const Parts& parts);
+
+// The symmetric n x n product C = A B^T (gemm_nt_f64, lower triangle mirrored)
+// and the packed density blocks (density_f64) on the context's stream.
+dgchefsi_status sym_product_f64(dgchefsi_ctx* ctx, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
+                                int64_t ldc, int64_t n, int64_t K);
+dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P);
 
 // Tensor-core filter (tc_filter.cu). X, Y FP64 (Ns x ld) state-major.
 // reuse_hop: the operand copy of H - cI built by the previous call of this
