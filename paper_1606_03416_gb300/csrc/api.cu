@@ -49,40 +49,52 @@ dgchefsi_status ensure(dgchefsi_ctx* ctx, DevBuf& b, size_t bytes, const char* w
   return DGCHEFSI_OK;
 }
 
-dgchefsi_status parts_begin(dgchefsi_ctx* ctx, Parts* parts) {
-  *parts = Parts();
+// The context's buffer of partial sums for a call on its stream, null where
+// there is none to have: a capture, or no memory (128 MB that the call can do
+// without). The exchange lets cudaMalloc run beside another stream's capture.
+static dgchefsi_status parts_begin(dgchefsi_ctx* ctx, double** p) {
+  *p = nullptr;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return DGCHEFSI_OK;
   }
-  DG_TRY(ensure(ctx, ctx->ws_parts, kPartsBytes, "partial products"));
+  if (!ctx->ws_parts.p) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    DG_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    const dgchefsi_status st = ensure(ctx, ctx->ws_parts, kPartsBytes, "partial products");
+    DG_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    if (st != DGCHEFSI_OK) {
+      clear_error();
+      return DGCHEFSI_OK;
+    }
+  }
   if (!ctx->ev_parts)
     DG_CUDA(cudaEventCreateWithFlags(&ctx->ev_parts, cudaEventDisableTiming));
   else
     DG_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_parts, 0));
-  parts->p = static_cast<double*>(ctx->ws_parts.p);
-  parts->doubles = (int64_t)(ctx->ws_parts.bytes / sizeof(double));
+  *p = static_cast<double*>(ctx->ws_parts.p);
   return DGCHEFSI_OK;
 }
 
-dgchefsi_status parts_end(dgchefsi_ctx* ctx, const Parts& parts) {
+static dgchefsi_status parts_end(dgchefsi_ctx* ctx, const Parts& parts) {
   if (parts.p) DG_CUDA(cudaEventRecord(ctx->ev_parts, ctx->stream));
   return DGCHEFSI_OK;
 }
 
 dgchefsi_status sym_product_f64(dgchefsi_ctx* ctx, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
                                 int64_t ldc, int64_t n, int64_t K) {
-  Parts parts;
-  DG_TRY(parts_begin(ctx, &parts));
+  Parts parts{nullptr, (int64_t)(kPartsBytes / sizeof(double))};
+  if (gemm_nt_parts(n, n, K, true, parts.doubles) > 1) DG_TRY(parts_begin(ctx, &parts.p));
   DG_CUDA(gemm_nt_f64(A, lda, B, ldb, C, ldc, n, n, K, true, false, parts, ctx->stream));
   return parts_end(ctx, parts);
 }
 
 dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P) {
-  Parts parts;
-  DG_TRY(parts_begin(ctx, &parts));
-  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, ctx->poff_h[ctx->M], X, Ns, ld, f, P, parts, ctx->stream));
+  Parts parts{nullptr, (int64_t)(kPartsBytes / sizeof(double))};
+  const int64_t total = ctx->poff_h[ctx->M];
+  if (density_parts(ctx->view(), total, Ns, parts.doubles) > 1) DG_TRY(parts_begin(ctx, &parts.p));
+  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, total, X, Ns, ld, f, P, parts, ctx->stream));
   return parts_end(ctx, parts);
 }
 

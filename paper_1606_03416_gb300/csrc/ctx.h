@@ -134,13 +134,12 @@ void clear_error();
 // Make `b` hold at least `bytes` (synchronises the context's stream before a regrow).
 dgchefsi_status ensure(dgchefsi_ctx* ctx, DevBuf& b, size_t bytes, const char* what);
 
-// The context's buffer for split FP64 products, one for all of them. The calls
-// that use it may be asynchronous and the context's stream may change between
-// them (dgchefsi_set_stream), so parts_begin makes the stream wait for the last
-// product's sum and parts_end records this one's.
+// Size of the context's buffer for split FP64 products, one for all of them. The
+// calls that use it may be asynchronous and the context's stream may change
+// between them (dgchefsi_set_stream), so each waits on its stream for the event
+// of the last one that used it. Without the buffer (no memory; a stream capture,
+// whose replays no such event orders) the parts are added one after another.
 constexpr size_t kPartsBytes = size_t(128) << 20;
-dgchefsi_status parts_begin(dgchefsi_ctx* ctx, Parts* parts);
-dgchefsi_status parts_end(dgchefsi_ctx* ctx, const Parts& parts);
 
 // The symmetric n x n product C = A B^T (gemm_nt_f64, lower triangle mirrored)
 // and the packed density blocks (density_f64) on the context's stream.

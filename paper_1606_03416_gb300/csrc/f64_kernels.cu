@@ -324,14 +324,19 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) k_lanczos_f64(HView h, const do
   }
 }
 
-// C[i,j] = sum_r A[i,r] B[j,r]; lower_only: the entries j <= i, mirrored. With
-// gridDim.z > 1 each part sums kc terms and writes its partial result to
-// C + z * rows * cols (k_sum_parts_f64 adds them in order): a product of few
-// tiles and many terms (a Gram matrix of a few hundred states) fills the GPU.
+// What a product split along its contraction does with part z's result:
+// written as the whole one (part 0), to the z-th block of the buffer of parts
+// (another kernel adds these in order), or added to the parts before it.
+enum PartTo { kWrite, kBuffer, kAdd };
+
+// C[i,j] = sum_r A[i,r] B[j,r]; lower_only: the entries j <= i, mirrored. Part z =
+// z0 + blockIdx.z sums kc terms; in a buffer (C + z * rows * cols, added by
+// k_sum_parts_f64) all parts run at once: a product of few tiles and many terms (a
+// Gram matrix of a few hundred states) fills the GPU.
 __global__ void __launch_bounds__(NT) k_gemm_nt_f64(const double* __restrict__ A, int64_t lda,
                                                     const double* __restrict__ B, int64_t ldb, double* C,
                                                     int64_t ldc, int64_t rows, int64_t cols, int64_t K, int64_t kc,
-                                                    int lower_only) {
+                                                    int lower_only, int z0, PartTo to) {
   const int64_t nrt = (rows + TR - 1) / TR;
   const int64_t i0 = (blockIdx.x % nrt) * TR, j0 = (blockIdx.x / nrt) * T;
   if (lower_only && j0 > i0 + TR - 1) return;
@@ -344,7 +349,7 @@ __global__ void __launch_bounds__(NT) k_gemm_nt_f64(const double* __restrict__ A
 #pragma unroll
   for (int j = 0; j < 8; ++j) acc[j] = 0.0;
   const int kk = tid & 15, rr = tid >> 4;
-  const int64_t kb = (int64_t)blockIdx.z * kc, ke = kb + kc < K ? kb + kc : K;
+  const int64_t z = z0 + (int64_t)blockIdx.z, kb = z * kc, ke = kb + kc < K ? kb + kc : K;
   for (int64_t k0 = kb; k0 < ke; k0 += BK) {
     const bool kin = (k0 + kk) < ke;
 #pragma unroll
@@ -363,14 +368,16 @@ __global__ void __launch_bounds__(NT) k_gemm_nt_f64(const double* __restrict__ A
   }
   const int64_t ii = i0 + ty;
   if (ii >= rows) return;
-  const bool part = gridDim.z > 1;
-  double* c = C + (part ? (int64_t)blockIdx.z * rows * cols : 0);
+  const bool part = to == kBuffer;
+  double* c = C + (part ? z * rows * cols : 0);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int64_t jj = j0 + tx + 8 * j;
     if (jj >= cols || (lower_only && jj > ii)) continue;
-    c[ii * (part ? cols : ldc) + jj] = acc[j];
-    if (lower_only && !part) c[jj * ldc + ii] = acc[j];
+    double* o = c + ii * (part ? cols : ldc) + jj;
+    const double v = to == kAdd ? *o + acc[j] : acc[j];
+    *o = v;
+    if (lower_only && !part) c[jj * ldc + ii] = v;
   }
 }
 
@@ -443,13 +450,14 @@ __global__ void __launch_bounds__(NT) k_gemm_nn_f64(const double* __restrict__ A
 
 // P_K[j, j'] = sum_i f_i X[i, off_K + j] X[i, off_K + j'] for j' <= j, mirrored
 // (P_K is symmetric: half the multiply-adds). blockIdx.y: pair of 64-wide
-// chunks of the element, chunk of j >= chunk of j'. With gridDim.z > 1 each
-// part sums `sc` states into part + z * total (laid out like P) and
-// k_density_sum_f64 adds them in order, so that few elements still fill the
+// chunks of the element, chunk of j >= chunk of j'. Part z = z0 + blockIdx.z
+// sums `sc` states; in a buffer (P + z * total, laid out like P, added by
+// k_density_sum_f64) all parts run at once, so that few elements still fill the
 // GPU and many fill it evenly.
 __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __restrict__ poff,
                                                     const double* __restrict__ X, int64_t Ns, int64_t ld,
-                                                    const double* __restrict__ f, int64_t sc, double* __restrict__ P) {
+                                                    const double* __restrict__ f, int64_t sc, double* __restrict__ P,
+                                                    int z0, PartTo to) {
   const int K = blockIdx.x;
   const int nK = h.nb[K];
   int ca = 0, cb = blockIdx.y;  // chunks of j and j': row ca of the lower triangle of chunk pairs
@@ -476,7 +484,7 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
   const int cc = tid & 63;
-  const int64_t sb = (int64_t)blockIdx.z * sc, se = sb + sc < Ns ? sb + sc : Ns;
+  const int64_t z = z0 + (int64_t)blockIdx.z, sb = z * sc, se = sb + sc < Ns ? sb + sc : Ns;
   for (int64_t i0 = sb; i0 < se; i0 += BK) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -495,8 +503,8 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
     fma_outer(As, Bs, acc, (int)(se - i0 < BK ? se - i0 : BK), lim, tx, row);
     __syncthreads();
   }
-  const bool part = gridDim.z > 1;
-  double* PK = P + poff[K] + (part ? (int64_t)blockIdx.z * poff[h.M] : 0);
+  const bool part = to == kBuffer;
+  double* PK = P + poff[K] + (part ? z * poff[h.M] : 0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int jj = j0 + row[i];
@@ -505,8 +513,10 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
     for (int j = 0; j < 8; ++j) {
       const int jq = jp0 + tx + 8 * j;
       if (jq > jj) continue;
-      PK[(int64_t)jj * nK + jq] = acc[i][j];
-      if (!part) PK[(int64_t)jq * nK + jj] = acc[i][j];
+      double* o = PK + (int64_t)jj * nK + jq;
+      const double v = to == kAdd ? *o + acc[i][j] : acc[i][j];
+      *o = v;
+      if (!part) PK[(int64_t)jq * nK + jj] = v;
     }
   }
 }
@@ -850,23 +860,52 @@ cudaError_t axpby_f64(double a, const double* x, double b, const double* y, doub
 // uneven last round, or tiles of uneven work, cost a few percent.
 static constexpr int64_t kFillCtas = 16 * 152;
 
+// Parts of at least 64 of n terms, as many as give kFillCtas CTAs (of `ctas` a
+// part) and as `most` allows: their number and their length, a multiple of BK.
+struct Split {
+  int64_t np, len;
+};
+static Split split_of(int64_t n, int64_t ctas, int64_t most) {
+  int64_t np = std::min((kFillCtas + ctas - 1) / ctas, std::min(n / 64, most));
+  np = std::max<int64_t>(1, std::min<int64_t>(np, 65535));
+  const int64_t len = std::max<int64_t>(BK, ((n + np - 1) / np + BK - 1) / BK * BK);
+  return {std::max<int64_t>(1, (n + len - 1) / len), len};
+}
+
+static Split gemm_nt_split(int64_t rows, int64_t cols, int64_t K, bool lower_only, int64_t doubles) {
+  const int64_t tiles = (int64_t)cdiv(rows, TR) * cdiv(cols, T);
+  return split_of(K, lower_only ? (tiles + 1) / 2 : tiles, doubles / std::max<int64_t>(rows * cols, 1));
+}
+
+static Split density_split(const HView& h, int64_t total, int64_t Ns, int64_t doubles) {
+  const int64_t chunks = cdiv(h.max_nb, T);
+  return split_of(Ns, h.M * (chunks * (chunks + 1) / 2), doubles / total);
+}
+
+int64_t gemm_nt_parts(int64_t rows, int64_t cols, int64_t K, bool lower_only, int64_t doubles) {
+  return rows == 0 || cols == 0 ? 1 : gemm_nt_split(rows, cols, K, lower_only, doubles).np;
+}
+
+int64_t density_parts(const HView& h, int64_t total, int64_t Ns, int64_t doubles) {
+  return density_split(h, total, Ns, doubles).np;
+}
+
 cudaError_t gemm_nt_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                         int64_t rows, int64_t cols, int64_t K, bool lower_only, bool symmetrise, const Parts& parts,
                         cudaStream_t s) {
   if (rows == 0 || cols == 0) return cudaSuccess;
-  const int64_t tiles = (int64_t)cdiv(rows, TR) * cdiv(cols, T);
-  const int64_t work = lower_only ? (tiles + 1) / 2 : tiles;
-  // parts of at least 64 terms, as many as fill the GPU and the buffer holds
-  int64_t np = std::min((kFillCtas + work - 1) / work, std::min(K / 64, parts.doubles / std::max<int64_t>(rows * cols, 1)));
-  np = std::max<int64_t>(1, std::min<int64_t>(np, 65535));
-  const int64_t kc = std::max<int64_t>(BK, ((K + np - 1) / np + BK - 1) / BK * BK);
-  np = std::max<int64_t>(1, (K + kc - 1) / kc);
-  k_gemm_nt_f64<<<dim3((unsigned)tiles, 1, (unsigned)np), NT, 0, s>>>(A, lda, B, ldb, np > 1 ? parts.p : C, ldc, rows,
-                                                                     cols, K, kc, lower_only ? 1 : 0);
-  count_launch();
-  if (np > 1) {
-    k_sum_parts_f64<<<stream_grid(rows * cols), 256, 0, s>>>(parts.p, (int)np, rows, cols, C, ldc, lower_only ? 1 : 0);
-    count_launch();
+  const unsigned tiles = cdiv(rows, TR) * cdiv(cols, T);
+  const Split sp = gemm_nt_split(rows, cols, K, lower_only, parts.doubles);
+  const int lower = lower_only ? 1 : 0;
+  if (sp.np > 1 && parts.p) {
+    k_gemm_nt_f64<<<dim3(tiles, 1, (unsigned)sp.np), NT, 0, s>>>(A, lda, B, ldb, parts.p, ldc, rows, cols, K, sp.len,
+                                                                lower, 0, kBuffer);
+    k_sum_parts_f64<<<stream_grid(rows * cols), 256, 0, s>>>(parts.p, (int)sp.np, rows, cols, C, ldc, lower);
+    count_launch(2);
+  } else {
+    for (int z = 0; z < (int)sp.np; ++z)
+      k_gemm_nt_f64<<<tiles, NT, 0, s>>>(A, lda, B, ldb, C, ldc, rows, cols, K, sp.len, lower, z, z == 0 ? kWrite : kAdd);
+    count_launch((int)sp.np);
   }
   if (symmetrise && rows == cols) {
     dim3 b2(32, 8), g2(cdiv(rows, 32), cdiv(rows, 8));
@@ -888,17 +927,17 @@ cudaError_t gemm_nn_f64(const double* A, int64_t lda, const double* B, int64_t l
 cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const double* X, int64_t Ns, int64_t ld,
                         const double* f, double* P, const Parts& parts, cudaStream_t s) {
   const int64_t chunks = cdiv(h.max_nb, T), pairs = chunks * (chunks + 1) / 2;
-  // parts of at least 64 states, as many as fill the GPU and the buffer holds
-  int64_t np = std::min((kFillCtas + h.M * pairs - 1) / (h.M * pairs), std::min(Ns / 64, parts.doubles / total));
-  np = std::max<int64_t>(1, std::min<int64_t>(np, 65535));
-  const int64_t sc = std::max<int64_t>(BK, ((Ns + np - 1) / np + BK - 1) / BK * BK);
-  np = std::max<int64_t>(1, (Ns + sc - 1) / sc);
-  k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)np), NT, 0, s>>>(h, poff, X, Ns, ld, f, sc,
-                                                                                 np > 1 ? parts.p : P);
-  count_launch();
-  if (np > 1) {
-    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, parts.p, (int)np, P);
-    count_launch();
+  const Split sp = density_split(h, total, Ns, parts.doubles);
+  if (sp.np > 1 && parts.p) {
+    k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)sp.np), NT, 0, s>>>(h, poff, X, Ns, ld, f, sp.len,
+                                                                                      parts.p, 0, kBuffer);
+    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, parts.p, (int)sp.np, P);
+    count_launch(2);
+  } else {
+    for (int z = 0; z < (int)sp.np; ++z)
+      k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs), NT, 0, s>>>(h, poff, X, Ns, ld, f, sp.len, P, z,
+                                                                       z == 0 ? kWrite : kAdd);
+    count_launch((int)sp.np);
   }
   return cudaGetLastError();
 }

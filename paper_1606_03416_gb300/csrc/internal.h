@@ -19,11 +19,16 @@ struct HView {
 };
 
 // Device buffer for the partial results of a product split along its
-// contraction (doubles = 0: not split).
+// contraction. doubles: what it holds, 0 to have the product not split; with p
+// null the product is split all the same (same bits), its parts launched one
+// after another.
 struct Parts {
   double* p = nullptr;
   int64_t doubles = 0;
 };
+// Parts of the products below for a buffer of so many doubles, 1: not split.
+int64_t gemm_nt_parts(int64_t rows, int64_t cols, int64_t K, bool lower_only, int64_t doubles);
+int64_t density_parts(const HView& h, int64_t total, int64_t Ns, int64_t doubles);
 
 void count_launch(int n = 1);
 
