@@ -525,6 +525,7 @@ dgchefsi_status sliced_gemm(dgchefsi_ctx* ctx, bool b_rows, bool a_lower, int64_
                             int slices, int* flag, int64_t tri, bool subtract, bool negate) {
   if (M <= 0 || Nc <= 0) return DGCHEFSI_OK;
   if (slices < 2 || slices > 16) return set_error(DGCHEFSI_ERR_ARG, "slices = %d outside 2..16", slices);
+  tri = std::min(tri, M);  // r mod tri = r from there on; the reduction's rows and tri are 32-bit numbers
   const int s = digits_for(slices), nw = weights_for(slices);
   cudaStream_t st = ctx->stream;
   if (K <= 0) {
