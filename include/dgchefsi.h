@@ -488,7 +488,7 @@ dgchefsi_status dgchefsi_density_blocks(dgchefsi_ctx* ctx, const double* X, int6
  * x_{i;K'}^T for every stored block (K, K'), FP64.
  *   X  device (Ns x ld) state-major;  f  device [Ns]
  *   P  device [n_values] out, laid out like H's values (block e at blk_off[e],
- *      row-major n_K x n_K'); the diagonal blocks equal dgchefsi_density_blocks'.
+ *      row-major n_K x n_K'); the diagonal blocks are dgchefsi_density_blocks', bit for bit.
  * Asynchronous on the context's stream. */
 dgchefsi_status dgchefsi_density_pattern(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld,
                                          const double* f, double* P);

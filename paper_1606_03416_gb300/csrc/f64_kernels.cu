@@ -454,8 +454,9 @@ __global__ void __launch_bounds__(NT) k_gemm_nn_f64(const double* __restrict__ A
 // sums `sc` states; in a buffer (P + z * total, laid out like P, added by
 // k_density_sum_f64) all parts run at once, so that few elements still fill the
 // GPU and many fill it evenly.
+// Element K's block goes to P + pout[K] (poff[K] in a buffer).
 __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __restrict__ poff,
-                                                    const double* __restrict__ X, int64_t Ns, int64_t ld,
+                                                    const int64_t* __restrict__ pout, const double* __restrict__ X, int64_t Ns, int64_t ld,
                                                     const double* __restrict__ f, int64_t sc, double* __restrict__ P,
                                                     int z0, PartTo to) {
   const int K = blockIdx.x;
@@ -504,7 +505,7 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
     __syncthreads();
   }
   const bool part = to == kBuffer;
-  double* PK = P + poff[K] + (part ? z * poff[h.M] : 0);
+  double* PK = P + (part ? poff[K] + z * poff[h.M] : pout[K]);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int jj = j0 + row[i];
@@ -522,13 +523,13 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
 }
 
 // P = the sum of the parts, z ascending, lower triangles mirrored. One CTA per element.
-__global__ void k_density_sum_f64(HView h, const int64_t* __restrict__ poff, const double* __restrict__ part,
-                                  int parts, double* __restrict__ P) {
+__global__ void k_density_sum_f64(HView h, const int64_t* __restrict__ poff, const int64_t* __restrict__ pout,
+                                  const double* __restrict__ part, int parts, double* __restrict__ P) {
   const int K = blockIdx.x;
   const int nK = h.nb[K];
   const int64_t total = poff[h.M];
   const double* p = part + poff[K];
-  double* PK = P + poff[K];
+  double* PK = P + pout[K];
   for (int e = threadIdx.x; e < nK * nK; e += blockDim.x) {
     const int j = e / nK, q = e - j * nK;
     if (q > j) continue;
@@ -638,14 +639,15 @@ __global__ void k_check_finite_f64(const double* __restrict__ x, int64_t n, int*
 
 
 // G_e += alpha * sum_s w_s A[s, off_K + j] B[s, off_K' + j'] for every stored
-// block e = (K, K') (w may be null: unit weights).
+// block e = (K, K') (w may be null: unit weights), or every one with K != K'.
 __global__ void __launch_bounds__(NT) k_block_outer_f64(HView h, const int32_t* __restrict__ blk_row,
                                                         const double* __restrict__ A, int64_t lda,
                                                         const double* __restrict__ B, int64_t ldb,
                                                         const double* __restrict__ w, double alpha, int64_t Ns,
-                                                        double* __restrict__ G) {
+                                                        double* __restrict__ G, int off_diagonal) {
   const int64_t e = blockIdx.x;
   const int K = blk_row[e], Kp = h.col[e];
+  if (off_diagonal && K == Kp) return;
   const int nK = h.nb[K], nKp = h.nb[Kp];
   const int j0 = blockIdx.y * T, jp0 = blockIdx.z * T;
   if (j0 >= nK || jp0 >= nKp) return;
@@ -924,18 +926,18 @@ cudaError_t gemm_nn_f64(const double* A, int64_t lda, const double* B, int64_t l
   return cudaGetLastError();
 }
 
-cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const double* X, int64_t Ns, int64_t ld,
-                        const double* f, double* P, const Parts& parts, cudaStream_t s) {
+cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const int64_t* pout, const double* X,
+                        int64_t Ns, int64_t ld, const double* f, double* P, const Parts& parts, cudaStream_t s) {
   const int64_t chunks = cdiv(h.max_nb, T), pairs = chunks * (chunks + 1) / 2;
   const Split sp = density_split(h, total, Ns, parts.doubles);
   if (sp.np > 1 && parts.p) {
-    k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)sp.np), NT, 0, s>>>(h, poff, X, Ns, ld, f, sp.len,
-                                                                                      parts.p, 0, kBuffer);
-    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, parts.p, (int)sp.np, P);
+    k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)sp.np), NT, 0, s>>>(h, poff, pout, X, Ns, ld, f,
+                                                                                      sp.len, parts.p, 0, kBuffer);
+    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, pout, parts.p, (int)sp.np, P);
     count_launch(2);
   } else {
     for (int z = 0; z < (int)sp.np; ++z)
-      k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs), NT, 0, s>>>(h, poff, X, Ns, ld, f, sp.len, P, z,
+      k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs), NT, 0, s>>>(h, poff, pout, X, Ns, ld, f, sp.len, P, z,
                                                                        z == 0 ? kWrite : kAdd);
     count_launch((int)sp.np);
   }
@@ -977,10 +979,10 @@ cudaError_t zero_strict_upper_f64(double* A, int64_t n, int64_t lda, cudaStream_
 
 cudaError_t block_outer_f64(const HView& h, const int32_t* blk_row, int64_t nnzb, const double* A, int64_t lda,
                             const double* B, int64_t ldb, const double* w, double alpha, int64_t Ns, double* G,
-                            cudaStream_t s) {
+                            bool off_diagonal, cudaStream_t s) {
   if (nnzb == 0) return cudaSuccess;
   dim3 grid((unsigned)nnzb, cdiv(h.max_nb, T), cdiv(h.max_nb, T));
-  k_block_outer_f64<<<grid, NT, 0, s>>>(h, blk_row, A, lda, B, ldb, w, alpha, Ns, G);
+  k_block_outer_f64<<<grid, NT, 0, s>>>(h, blk_row, A, lda, B, ldb, w, alpha, Ns, G, off_diagonal ? 1 : 0);
   count_launch();
   return cudaGetLastError();
 }
