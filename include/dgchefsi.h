@@ -517,7 +517,9 @@ dgchefsi_status dgchefsi_realign(dgchefsi_ctx* ctx, const int32_t* nb_old, const
 
 /* One full CheFSI cycle (Alg. 1) plus occupations and density blocks:
  * bounds -> filter -> Cholesky-QR -> Rayleigh-Ritz -> rotation -> f, mu -> P_KK.
- *   X          device (Ns x ld): in = starting block, out = X_new
+ *   X          device (Ns x ld): in = starting block, out = X_new; as it was
+ *              after ERR_NOT_SPD, ERR_NO_CONVERGENCE and ERR_NONFINITE, so that
+ *              the cycle can be repeated with another solver
  *   prev_ritz  host [Ns] or NULL. Filter bounds: b from k_lanczos Lanczos steps
  *              started at v0 (device [N]); a = max(prev_ritz), a0 = min(prev_ritz);
  *              on the first cycle (NULL) a0 = theta_min and a = a0 + (b-a0) Ns/N.

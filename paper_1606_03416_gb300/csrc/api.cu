@@ -332,7 +332,8 @@ static dgchefsi_status bounds_impl(dgchefsi_ctx* ctx, const double* v0, int k, d
   return DGCHEFSI_OK;
 }
 
-// X_new goes to `out` (row stride ld): Y itself, or a block that does not overlap it.
+// X_new goes to `out` (row stride ld): Y itself, or a block that does not overlap
+// it, which is then written only once every earlier step has succeeded.
 static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t ld, double* ritz, double* out) {
   const int64_t N = ctx->N;
   cudaStream_t s = ctx->stream;
@@ -423,19 +424,28 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
     DG_TRY(sym_product_f64(ctx, W, N, Y, ld, S, Ns, Ns, N));
   // The eigensolver reads the lower triangle (row-major), the one computed.
   DG_TRY(subspace_eigh(ctx, S, Ns, Ns, ritz));
+  auto check = [&]() -> dgchefsi_status {
+    DG_CUDA(check_finite_f64(ritz, Ns, bad, s));
+    DG_CUDA(cudaMemcpyAsync(info, ctx->info_d, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    DG_CUDA(cudaStreamSynchronize(s));
+    if (info[1] != 0) return set_error(DGCHEFSI_ERR_NOT_SPD, "triangular inverse failed (info %d)", info[1]);
+    if (info[2] != 0) return set_error(DGCHEFSI_ERR_NO_CONVERGENCE, "dense eigensolver failed (info %d)", info[2]);
+    if (info[3] != 0)
+      return set_error(DGCHEFSI_ERR_NONFINITE, sl ? "non-finite Ritz value or Rayleigh-Ritz operand" : "non-finite Ritz value");
+    return DGCHEFSI_OK;
+  };
+  if (out != Y) {
+    // what the sliced rotation would raise the flag for: its operands are the
+    // eigenvectors and Y_hat, and Y_hat was an operand of H_hat
+    if (sl) DG_CUDA(check_finite_f64(S, Ns * Ns, bad, s));
+    DG_TRY(check());
+  }
   // Step 5: X_new^T = Q^T Y_hat^T (column-major Q read row-major is Q^T).
   if (sl)
     DG_TRY(sliced_gemm(ctx, false, false, Ns, N, Ns, S, Ns, W, N, out, ld, ctx->products_slices, bad));
   else
     DG_CUDA(gemm_nn_f64(S, Ns, W, N, out, ld, Ns, N, Ns, false, s));
-  DG_CUDA(check_finite_f64(ritz, Ns, ctx->info_d + 3, s));
-  DG_CUDA(cudaMemcpyAsync(info, ctx->info_d, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
-  DG_CUDA(cudaStreamSynchronize(s));
-  if (info[1] != 0) return set_error(DGCHEFSI_ERR_NOT_SPD, "triangular inverse failed (info %d)", info[1]);
-  if (info[2] != 0) return set_error(DGCHEFSI_ERR_NO_CONVERGENCE, "dense eigensolver failed (info %d)", info[2]);
-  if (info[3] != 0)
-    return set_error(DGCHEFSI_ERR_NONFINITE, sl ? "non-finite Ritz value or Rayleigh-Ritz operand" : "non-finite Ritz value");
-  return DGCHEFSI_OK;
+  return out == Y ? check() : DGCHEFSI_OK;
 }
 
 }  // namespace dg
