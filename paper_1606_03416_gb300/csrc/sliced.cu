@@ -143,7 +143,8 @@ __device__ __forceinline__ void put_digits(const float (&f)[C], __nv_bfloat16* _
 }
 
 // Digits i = 0 .. d - 1 of C consecutive entries v 2^{b} scaled by 2^{-e}
-// (|v 2^{b-e}| < 1; zero entries and `zero` give zero digits), stored at
+// (|v 2^{b-e}| < 1; zero entries, `zero` and, beside an entry that is not finite,
+// entries above that give zero digits), stored at
 // q + i * stride where `store`; norm[i] (shared) collects the squares of digit
 // i; every lane of the warp takes part. One store per digit.
 // d <= 7: F = round(v 2^{9d - 1}) as a 64-bit integer (|F| <= 2^62;
@@ -169,9 +170,9 @@ __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (
       int E;
       F[c] = bias;
       if (!zero && decompose(v[c], M, E) == 1) {  // |v| = M 2^{E - 1075}, M < 2^53
-        // right shift of M 2^10 by r leaves one bit for the rounding; r >= 0 because |v 2^{b-e}| < 1
+        // right shift of M 2^10 by r leaves one bit for the rounding; r >= 0 where |v 2^{b-e}| < 1
         const int r = 1075 + e + 10 - E - b[c] - 9 * d;
-        const int64_t a = r < 64 ? (int64_t)((((unsigned long long)M << 10) >> r) + 1) >> 1 : 0;
+        const int64_t a = (unsigned)r < 64u ? (int64_t)((((unsigned long long)M << 10) >> r) + 1) >> 1 : 0;
         F[c] += v[c] < 0.0 ? -a : a;
       }
     }
@@ -188,7 +189,10 @@ __device__ __forceinline__ void put_all_digits(const double (&v)[C], const int (
   } else {
     double r[C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) r[c] = zero || v[c] == 0.0 ? 0.0 : ldexp(v[c], b[c] - e) * 256.0;
+    for (int c = 0; c < C; ++c) {
+      const double y = zero || v[c] == 0.0 ? 0.0 : ldexp(v[c], b[c] - e);
+      r[c] = fabs(y) < 1.0 ? y * 256.0 : 0.0;
+    }
     for (int i = 0; i < d; ++i) {
 #pragma unroll
       for (int c = 0; c < C; ++c) {

@@ -1319,7 +1319,9 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
   digit_counts(slices, &d, &w);
   // H's digits (once per H and digit count)
   const int64_t hcopy = sx.b_rows * W;
-  if (!sx.h_built || sx.h_digits != d) {
+  const bool build = !sx.h_built || sx.h_digits != d;
+  if (build) {
+    sx.h_built = false;
     if (sx.Hs.bytes < sizeof(__nv_bfloat16) * (size_t)(d * hcopy)) {
       DG_TRY(ensure(ctx, sx.Hs, sizeof(__nv_bfloat16) * (size_t)(d * hcopy), "digits of H"));
       DG_CUDA(cudaMemsetAsync(sx.Hs.p, 0, sx.Hs.bytes, st));  // zero tiles and slack rows
@@ -1327,8 +1329,6 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
     DG_CUDA(cudaMemsetAsync(sx.norm_d, 0, sizeof(uint32_t) * 16, st));
     DG_CUDA(digits_of_h(ctx, t.blk_row_d, t.pnb_d, t.poff_d, sx.brow_d, d, static_cast<__nv_bfloat16*>(sx.Hs.p), hcopy,
                         sx.eh_d, sx.norm_d, flag, st));
-    sx.h_built = true;
-    sx.h_digits = d;
   }
   // the states' digits and exponents
   const int64_t xcopy = Ns * t.ldp;
@@ -1374,6 +1374,13 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
     DG_TRY(reduce_digit_slabs(Pw, pn, t.ldp, w, B.groups, ex + s0, sx.eh_d, sx.cmap_d, Y + s0 * ldy, ldy, st));
   }
   DG_TRY(pair_products_status(ctx));
+  if (build) {  // kept only without a non-finite entry: the flag is raised where the digits are formed
+    int bad = 0;
+    DG_CUDA(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DG_CUDA(cudaStreamSynchronize(st));
+    sx.h_built = bad == 0;
+    sx.h_digits = d;
+  }
   *used = true;
   return DGCHEFSI_OK;
 }
