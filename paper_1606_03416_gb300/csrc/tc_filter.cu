@@ -607,9 +607,26 @@ static dgchefsi_status prepare_launch(dgchefsi_ctx* ctx, TcState& t, int mode, i
   const int W = f32 ? 32 : 64;
   Plan* pl = nullptr;
   DG_TRY(get_plan(ctx, t, G, &pl));
+  const int na = mode == MODE_BF16X3 ? 2 : 1;
+  const int sched_bytes = 2 * pl->maxent * (1 + G) * 4;
+  const auto slot_bytes = [&](int tiles) { return na * (tiles * A_BYTES + G * t.ACC * SLICE_BYTES); };  // layout 0
+  const auto smem_bytes = [&](int stages, int slot) { return stages * slot + (2 * stages + 4) * 8 + sched_bytes + 1024; };
+  constexpr int kSmem = 227 * 1024;
+  const int sb = layout == 2 ? 64 : SLICE_BYTES;  // ring-slot K extent in bytes
+  int stage_bytes = layout >= 1 ? na * (128 * sb + 256 * sb) : slot_bytes(T);
+  int stages = layout >= 1 ? TN_RING_BYTES / stage_bytes : ring_slots(stage_bytes);
+  if (smem_bytes(stages, stage_bytes) > kSmem)
+    return set_error(DGCHEFSI_ERR_UNSUPPORTED, "filter schedule too large for shared memory");
   // up to 128 states the second tile of a unit is empty: the one-tile kernel of
-  // the same group loads and multiplies half as much, in twice the ring slots
-  if (layout == 0 && T == 2 && Ns <= BM) T = 1;
+  // the same group loads and multiplies half as much, in a ring of more slots. A
+  // shape has to fit with two tiles all the same (it may be used for more states
+  // later), and with one where that ring is the larger one (1 KB of the limit is
+  // left for the kernel's static part).
+  if (layout == 0 && T == 2 && Ns <= BM && smem_bytes(ring_slots(slot_bytes(1)), slot_bytes(1)) <= kSmem - 1024) {
+    T = 1;
+    stage_bytes = slot_bytes(T);
+    stages = ring_slots(stage_bytes);
+  }
   L.kern = pick_kernel(mode, G, T, t.ACC, layout);
   if (!L.kern)
     return set_error(DGCHEFSI_ERR_UNSUPPORTED, "no filter kernel for G=%d T=%d ACC=%d layout %d", G, T, t.ACC, layout);
@@ -618,14 +635,9 @@ static dgchefsi_status prepare_launch(dgchefsi_ctx* ctx, TcState& t, int mode, i
     DG_TRY(bind_iterate(t, mode, layout, Ns, static_cast<float*>(t.F[i].p), static_cast<__nv_bfloat16*>(t.Sh[i].p),
                         static_cast<__nv_bfloat16*>(t.Sl[i].p), &L.A0[i], &L.A1[i]));
   const uint64_t brows_total = (uint64_t)t.b_rows * (mode == MODE_BF16X3 ? 2 : 1);
-  const int sb = layout == 2 ? 64 : SLICE_BYTES;  // ring-slot K extent in bytes
   DG_TRY(make_map(&L.B, t.Hop.p, f32, (uint64_t)W, brows_total, (uint32_t)(W * sb / SLICE_BYTES), (uint32_t)t.boxn,
                   layout == 2));
-  const int na = mode == MODE_BF16X3 ? 2 : 1;
-  const int stage_bytes = layout >= 1 ? na * (128 * sb + 256 * sb) : na * (T * A_BYTES + G * t.ACC * SLICE_BYTES);
-  const int stages = layout >= 1 ? TN_RING_BYTES / stage_bytes : ring_slots(stage_bytes);
-  L.smem = stages * stage_bytes + (2 * stages + 4) * 8 + 2 * pl->maxent * (1 + G) * 4 + 1024;
-  if (L.smem > 227 * 1024) return set_error(DGCHEFSI_ERR_UNSUPPORTED, "filter schedule too large for shared memory");
+  L.smem = smem_bytes(stages, stage_bytes);
   DG_CUDA(cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem));
   Params& p = L.p;
   p = Params{};
