@@ -271,7 +271,6 @@ struct BlockPairs {
   const int32_t *sched, *sched_ptr, *grp_elem, *pnb, *poff;
 };
 dgchefsi_status pair_products_blocks(dgchefsi_ctx* ctx, const BlockPairs& B, int64_t s0, int64_t pn, int32_t* Pw);
-bool pair_blocks_fit(int maxent, int acc);
 dgchefsi_status pair_products_begin(dgchefsi_ctx* ctx);
 dgchefsi_status pair_products_status(dgchefsi_ctx* ctx);
 // Y = H X (X, Y: Ns x ld state-major FP64) from s BF16 slices of each operand on

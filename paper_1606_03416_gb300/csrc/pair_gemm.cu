@@ -98,6 +98,7 @@ struct PairJob {
   const int32_t* pnb;        // padded size and offset of each element
   const int32_t* poff;
   int G2, acc;
+  int sched_in_smem;  // a unit's schedule is copied to shared memory; else read where it is
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -267,11 +268,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
       const int ya = mt * 256 + (int)rank * 128;
       const int yb = J.n0 + (J.diag ? mt : nt) * 256 + (int)rank * 128;
       const int nk = slices_of_tile<BLOCKS>(J, mt);
+      const int32_t* sched = nullptr;
       if (BLOCKS) {
-        __syncwarp();
-        const int32_t* src = J.sched + (int64_t)J.sched_ptr[mt] * ent;
-        for (int t = lane; t < nk * ent; t += 32) sched_sh[t] = src[t];
-        __syncwarp();
+        sched = J.sched + (int64_t)J.sched_ptr[mt] * ent;
+        if (J.sched_in_smem) {
+          __syncwarp();
+          for (int t = lane; t < nk * ent; t += 32) sched_sh[t] = sched[t];
+          __syncwarp();
+          sched = sched_sh;
+        }
       }
       if (lane == 0) {
         for (int p = J.group[g]; p < J.group[g + 1] && ok; ++p) {
@@ -287,7 +292,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
             if (leader) mbar_expect_tx(full0 + 8 * st, (uint32_t)(2 * PG_STAGE));
             const uint32_t dst = smem_u32(smem + st * PG_STAGE);
             if (BLOCKS) {
-              const int32_t* e = sched_sh + ks * ent;
+              const int32_t* e = sched + ks * ent;
               for (int q = 0; q < J.G2; ++q)
                 tma_load_2d_pair(dst + q * J.acc * SLICE_BYTES, am, 0, e[1 + rank * J.G2 + q], full_l + 8 * st);
               tma_load_2d_pair(dst + PG_HALF, bm, e[0], yb, full_l + 8 * st);
@@ -641,13 +646,11 @@ dgchefsi_status pair_products_blocks(dgchefsi_ctx* ctx, const BlockPairs& B, int
   J.poff = B.poff;
   J.G2 = 128 / B.acc;
   J.acc = B.acc;
-  const int sched_bytes = B.maxent * (1 + 2 * J.G2) * (int)sizeof(int32_t);
-  return launch_pairs(ctx, J, T, B.s, B.groups, true, (int64_t)J.nmt * J.nnt, sched_bytes);
-}
-
-// Largest schedule (entries of 1 + 2 * 128 / acc numbers) the kernel's shared memory holds.
-bool pair_blocks_fit(int maxent, int acc) {
-  return PG_STAGES * PG_STAGE + (2 * PG_STAGES + 4) * 8 + 1024 + maxent * (1 + 256 / acc) * 4 <= 226 * 1024;
+  // a schedule longer than what the ring leaves (930 entries of groups of 8 elements) stays in global memory
+  int64_t sched_bytes = (int64_t)B.maxent * (1 + 2 * J.G2) * (int64_t)sizeof(int32_t);
+  J.sched_in_smem = PG_STAGES * PG_STAGE + (2 * PG_STAGES + 4) * 8 + 1024 + sched_bytes <= 226 * 1024 ? 1 : 0;
+  if (!J.sched_in_smem) sched_bytes = 0;
+  return launch_pairs(ctx, J, T, B.s, B.groups, true, (int64_t)J.nmt * J.nnt, (int)sched_bytes);
 }
 
 dgchefsi_status pair_products_begin(dgchefsi_ctx* ctx) {

@@ -1326,7 +1326,6 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
   // the INT32 sums hold at most 4096 terms per row (7 pairs of one weight)
   if (sx.max_row_len > 4096) return DGCHEFSI_OK;
   if (sx.b_rows * (int64_t)W > ((int64_t)1 << 31) || Ns * t.ldp > ((int64_t)1 << 40)) return DGCHEFSI_OK;
-  if (!pair_blocks_fit(sx.plan.maxent, t.ACC)) return DGCHEFSI_OK;
   int d = 0, w = 0;
   digit_counts(slices, &d, &w);
   // H's digits (once per H and digit count)
