@@ -4,11 +4,11 @@
 // tc_kernel.cuh (instantiated in tc_tf32.cu, tc_bf16.cu, tc_bf16x3.cu).
 #include <algorithm>
 #include <cmath>
-#include <iterator>
 #include <map>
 #include <new>
 #include <utility>
 
+#include "element_groups.h"
 #include "tc_kernel.cuh"
 
 namespace dg {
@@ -1214,62 +1214,6 @@ dgchefsi_status tc_grad_backward(dgchefsi_ctx* ctx, int prec, const double* Wm, 
 // in panels of 256-state multiples below it.
 static constexpr size_t kSlabBytes = size_t(8) << 30;
 
-// Groups of G = 2^k elements whose neighbour lists overlap most: singles are
-// merged into pairs, pairs into fours and so on, each group (in order) with the
-// unmerged one of the same level among its neighbours' that gives the smallest
-// union of neighbours. On a grid of 27-neighbour elements: pairs along x (36
-// neighbours), then 2 x 2 (48, against 54 for four in a row).
-static std::vector<int32_t> group_elements(const dgchefsi_ctx* ctx, int G) {
-  const int M = ctx->M;
-  std::vector<std::vector<int>> elems(M), nbrs(M);
-  for (int K = 0; K < M; ++K) {
-    elems[K] = {K};
-    nbrs[K].assign(ctx->col_h.begin() + ctx->row_ptr_h[K], ctx->col_h.begin() + ctx->row_ptr_h[K + 1]);
-  }
-  std::vector<int> owner(M);
-  for (int size = 1; size < G; size *= 2) {
-    const int n = (int)elems.size();
-    for (int g = 0; g < n; ++g)
-      for (int K : elems[g]) owner[K] = g;
-    std::vector<char> used(n, 0);
-    std::vector<std::vector<int>> e2, n2;
-    for (int g = 0; g < n; ++g) {
-      if (used[g]) continue;
-      used[g] = 1;
-      int best = -1;
-      size_t best_union = 0;
-      std::vector<int> u, best_u = nbrs[g];
-      for (int K : nbrs[g]) {
-        const int h = owner[K];
-        if (used[h] || h == best) continue;
-        u.clear();
-        std::set_union(nbrs[g].begin(), nbrs[g].end(), nbrs[h].begin(), nbrs[h].end(), std::back_inserter(u));
-        if (best < 0 || u.size() < best_union || (u.size() == best_union && h < best)) {
-          best = h;
-          best_union = u.size();
-          best_u = u;
-        }
-      }
-      std::vector<int> e = elems[g];
-      if (best >= 0) {
-        used[best] = 1;
-        e.resize(size, -1);
-        e.insert(e.end(), elems[best].begin(), elems[best].end());
-      }
-      e2.push_back(e);
-      n2.push_back(best_u);
-    }
-    elems.swap(e2);
-    nbrs.swap(n2);
-  }
-  std::vector<int32_t> out;
-  for (auto& e : elems) {
-    e.resize(G, -1);
-    out.insert(out.end(), e.begin(), e.end());
-  }
-  return out;
-}
-
 dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t Ns,
                                  int slices, int* flag, bool* used) {
   *used = false;
@@ -1284,10 +1228,9 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
   auto& sx = t.sx;
   constexpr int W = 64;
   cudaStream_t st = ctx->stream;
-  if (!sx.layout) {
-    // W = 64 block layout of the digit copies (the BF16 filter's), the longest
-    // row (columns of its neighbour blocks), the padded column map, the slices
-    // of the states and the groups of elements
+  if (sx.brow_h.empty()) {
+    // W = 64 block layout of the digit copies (the BF16 filter's) and the longest
+    // row (columns of its neighbour blocks)
     sx.brow_h.resize(ctx->nnzb);
     int64_t r = 0;
     for (int64_t e = 0; e < ctx->nnzb; ++e) {
@@ -1301,6 +1244,12 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
       for (int64_t e = ctx->row_ptr_h[K]; e < ctx->row_ptr_h[K + 1]; ++e) len += ctx->nb_h[ctx->col_h[e]];
       sx.max_row_len = std::max(sx.max_row_len, len);
     }
+  }
+  // the INT32 sums hold at most 4096 terms per row (7 pairs of one weight)
+  if (sx.max_row_len > 4096) return DGCHEFSI_OK;
+  if (sx.b_rows * (int64_t)W > ((int64_t)1 << 31) || Ns * t.ldp > ((int64_t)1 << 40)) return DGCHEFSI_OK;
+  if (!sx.layout) {
+    // the padded column map, the slices of the states and the groups of elements
     std::vector<int32_t> cmap((size_t)t.ldp, -1);
     std::vector<int4> sl;
     for (int K = 0; K < ctx->M; ++K) {
@@ -1319,13 +1268,10 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
     DG_CUDA(cudaMemcpy(sx.cmap_d, cmap.data(), sizeof(int32_t) * (size_t)t.ldp, cudaMemcpyHostToDevice));
     DG_CUDA(cudaMemcpy(sx.slices_d, sl.data(), sizeof(int4) * sl.size(), cudaMemcpyHostToDevice));
     const int G = 256 / t.ACC;
-    const std::vector<int32_t> order = group_elements(ctx, G);
+    const std::vector<int32_t> order = group_elements(ctx->M, ctx->row_ptr_h.data(), ctx->col_h.data(), G);
     DG_TRY(make_plan(ctx, t, G, W, sx.brow_h, sx.zero_row, sx.plan, &order));
     sx.layout = true;
   }
-  // the INT32 sums hold at most 4096 terms per row (7 pairs of one weight)
-  if (sx.max_row_len > 4096) return DGCHEFSI_OK;
-  if (sx.b_rows * (int64_t)W > ((int64_t)1 << 31) || Ns * t.ldp > ((int64_t)1 << 40)) return DGCHEFSI_OK;
   int d = 0, w = 0;
   digit_counts(slices, &d, &w);
   // H's digits (once per H and digit count)
