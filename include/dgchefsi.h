@@ -267,8 +267,11 @@ dgchefsi_status dgchefsi_set_orthonormalisation(dgchefsi_ctx* ctx, int mode);
  * ERR_ARG for another mode or slice count. In the sliced form H Y_hat runs
  * from slices too (dgchefsi_sliced_matvec) when H fits that form, else on the
  * FP64 cores, and dgchefsi_cycle forms its density blocks P_KK from slices (at
- * least 10; sqrt(f_i) x_i split once) where that is faster: elements of 16
- * functions and more on average, none above 256, and enough states.
+ * least 10; sqrt(f_i) x_i split once) where that is faster: elements of about 16
+ * functions and more on average, none above 256, and enough states. An entry is
+ * then within (5 + N_s / 20) 2^-53 sqrt(P_jj P_j'j'), a normwise bound where the
+ * FP64 sum of dgchefsi_density_blocks has (N_s + 1) 2^-53 sum_i f_i
+ * |x_ij x_ij'|; without the memory for it the cycle uses that form.
  * dgchefsi_energy_grad follows the same setting for its forward products
  * (H Y_hat included) and the dense products of its adjoint (Z = U^{-1} Q,
  * W_m = Z (2 G R^T)); dgchefsi_gram always uses FP64 products. */
