@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/dgchefsi.h"
+#include "digit_rules.h"
 #include "internal.h"
 
 namespace dg {
@@ -206,14 +207,7 @@ bool density_digits_fit(const dgchefsi_ctx* ctx, int64_t Ns);
 dgchefsi_status density_digits(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P,
                                bool* done);
 
-// Slabs of the digit weights (pair_groups below).
-struct PairGroups {
-  uint8_t count[16];  // by weight t
-  int total;
-};
-
-// Digits of the block-sparse product H X (sliced.cu). digit_counts: 9-bit digits
-// and weights for a request of `slices`. digits_of_h: the row exponents E
+// Digits of the block-sparse product H X (sliced.cu). digits_of_h: the row exponents E
 // (element-padded rows) and d digit copies of H in the tensor-core operand
 // layout (brow: first row of each block, cstride: elements per copy).
 // digits_of_states: the state exponents E[Ns] and d digit copies of X in the
@@ -222,7 +216,6 @@ struct PairGroups {
 // largest sum of squares of digit i over one slice of a row.
 // reduce_digit_slabs: C[r, cmap[c]] = the FP64 sum of the weights' slabs (rows x
 // cols INT32 each) scaled by Erows[r] + Ecols[c] (cmap -1: skipped).
-void digit_counts(int slices, int* d, int* w);
 cudaError_t digits_of_h(const dgchefsi_ctx* ctx, const int32_t* blk_row, const int32_t* pnb, const int32_t* poff,
                         const int64_t* brow, int d, __nv_bfloat16* Q, int64_t cstride, int32_t* E, uint32_t* norm2,
                         int* flag, cudaStream_t st);
@@ -243,12 +236,10 @@ dgchefsi_status reduce_digit_slabs(const int32_t* Pw, int64_t rows, int64_t cols
 // and kc <= 4096; a_lower: A is lower triangular, so a row tile skips the K
 // slices past its last row. norm_a, norm_b (device, s entries): the largest sum
 // of squares of digit i over an aligned 512-entry block of a row. Enqueued only.
-// pair_groups: how many slabs each weight is split into for an output of so many 256 x 256 tiles.
 // pair_products_diag: the 256 x 256 blocks on the diagonal of Q Q^T only (slabs
 // of rows x 256), with the digits of one operand.
 // pair_products_begin clears the kernel's error word; pair_products_status
 // synchronises and reports a pipeline timeout.
-PairGroups pair_groups(int s, int nw, int64_t tiles, int nsm);
 dgchefsi_status pair_products_2sm(dgchefsi_ctx* ctx, const __nv_bfloat16* Qa, int64_t lqa, int64_t sa, int64_t M,
                                   const __nv_bfloat16* Qb, int64_t lqb, int64_t sb, int64_t Nc, int64_t K, int64_t k0,
                                   int64_t kc, int64_t n0, int64_t pn, int s, int nw, const PairGroups& groups,

@@ -65,8 +65,6 @@ constexpr int PG_THREADS = 32 * (2 + PG_EPI_WARPS);
 constexpr int PG_HALF = 128 * SLICE_BYTES;  // 128 rows x 64 BF16 of one operand
 constexpr int PG_STAGE = 2 * PG_HALF;       // A half + B half per CTA
 constexpr int PG_STAGES = 6;
-constexpr int PG_DRAIN = 4;       // K slices (64 terms each) per accumulator: 256 * 2^16 = 2^24
-constexpr int PG_MAXPAIRS = 66;   // 11 digits
 
 struct PairJob {
   const CUtensorMap* maps;  // device, 64-byte aligned: [s] maps of A_i, then [s] maps of B_j
@@ -206,7 +204,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
   __shared__ uint32_t drained_sh[2];       // epilogue warps done with their part, over all uses of a buffer
-  __shared__ int drain_sh[PG_MAXPAIRS];    // K slices per accumulator of each pair
+  __shared__ int drain_sh[kMaxPairs];    // K slices per accumulator of each pair
 
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
@@ -236,20 +234,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1) k_sli
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  // Any partial sum of products over 512 terms is at most |a||b|, over 2^h such
-  // blocks at most 2^h |a||b| with the largest block norms (Cauchy-Schwarz):
-  // exact in FP32 while that is at most 2^24. The block form's norms are over
-  // one 64-wide slice, so len slices give len |a||b|.
-  for (int p = threadIdx.x; p < J.group[J.ngroups]; p += PG_THREADS) {
-    const uint64_t sq = (uint64_t)J.norm_a[J.pair_i[p]] * J.norm_b[J.pair_j[p]];
-    int len = PG_DRAIN;
-    if (BLOCKS) {
-      while (len < 64 && (uint64_t)((len + 1) * (len + 1)) * sq <= 1ull << 48) ++len;
-    } else {
-      for (int h = 0; h < 4 && sq <= 1ull << (48 - 2 * h); ++h) len *= 2;
-    }
-    drain_sh[p] = len;
-  }
+  for (int p = threadIdx.x; p < J.group[J.ngroups]; p += PG_THREADS)
+    drain_sh[p] = drain_slices((uint64_t)J.norm_a[J.pair_i[p]] * J.norm_b[J.pair_j[p]], BLOCKS);
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // barriers of both CTAs initialised before any remote use
@@ -467,26 +453,6 @@ dgchefsi_status slice_map(CUtensorMap* map, const __nv_bfloat16* base, uint64_t 
 
 }  // namespace
 
-// Pairs (i, t - i) of weight t with both digits below s.
-static int pairs_of_weight(int s, int t) { return std::max(0, std::min(t, s - 1) - std::max(0, t - s + 1) + 1); }
-
-PairGroups pair_groups(int s, int nw, int64_t tiles, int nsm) {
-  // pairs per unit: all of a weight (at most 7, the INT32 bound) when there
-  // are many units for the clusters; fewer when a small output would leave
-  // clusters idle or waiting for the longest unit
-  const int64_t clusters = std::max(nsm / 2, 1);
-  int64_t pairs = 0;
-  for (int t = 0; t < nw; ++t) pairs += pairs_of_weight(s, t);
-  const int64_t avg = (pairs * tiles + clusters - 1) / clusters;
-  const int cap = (int)std::min<int64_t>(7, std::max<int64_t>(1, (avg + 1) / 2));
-  PairGroups g{};
-  for (int t = 0; t < nw; ++t) {
-    g.count[t] = (uint8_t)((pairs_of_weight(s, t) + cap - 1) / cap);
-    g.total += g.count[t];
-  }
-  return g;
-}
-
 // Tables of a launch in one host block: 2s tensor maps (64-byte aligned), then
 // the groups (slab order: weights t descending, each weight's pairs in count[t]
 // groups of nearly equal size) and their pairs, then the tile list.
@@ -511,7 +477,7 @@ struct PairTables {
       const int np = pairs_of_weight(s, t), i0 = std::max(0, t - s + 1);
       for (int q = 0, k = 0; q < groups.count[t]; ++q) {
         gp[g++] = n;
-        for (const int end = np * (q + 1) / groups.count[t]; k < end; ++k, ++n) {
+        for (const int end = group_end(np, q, groups.count[t]); k < end; ++k, ++n) {
           pi[n] = i0 + k;
           pj[n] = t - i0 - k;
         }

@@ -26,7 +26,7 @@
 // Error per chunk (row and column maxima m_r, n_c over the chunk): the
 // remainders after d digits and the dropped pairs contribute at most
 // L 2^{e_r + f_c} 2^{-9d} (d + 2) <= 4 L m_r n_c 2^{-9d} (d + 2), which
-// digits_for keeps below L m_r n_c 2^{-6s} (s + 4); the FP64 steps and the sum
+// digits_for (digit_rules.h) keeps below L m_r n_c 2^{-6s} (s + 4); the FP64 steps and the sum
 // over chunks add at most (5 + chunks) u L m_r n_c, u = 2^{-53}. For s = 10
 // (d = 7) the splitting term is below u L m_r n_c, the size of FP64's own
 // worst-case bound. The bound is normwise per row and column: entries far
@@ -43,19 +43,7 @@
 namespace dg {
 
 static constexpr int64_t kL = 4096;     // K chunk: one exponent per row and chunk; INT32 holds 7 pairs of it
-static constexpr int kNormPitch = 16;  // digit norms of a chunk (at most 11 digits)
-// For a request of s 6-bit slices (2 <= s <= 16): the number of 9-bit digits,
-// 9 d >= 6 s + 1, so that their remainders are below those of the slices; and
-// the number of weights t = i + j kept, w >= d. w is d, or d + 1 where integer
-// operands that s slices multiply exactly need it to stay exact: operands of a
-// and b slices, a + b <= s + 1, have at most 6 (a + b) bits between them (53
-// when the result is representable) and ceil((bits + 1) / 9) digits each, and
-// the pair of their last digits is kept when those counts sum to at most w + 1.
-static int digits_for(int s) { return (6 * s + 9) / 9; }
-static int weights_for(int s) {
-  const int bits = std::min(6 * (s + 1), 53);
-  return std::min(std::max(digits_for(s), (bits + 18) / 9 - 1), std::max(s, digits_for(s)));
-}
+static constexpr int kNormPitch = 16;  // digit norms of a chunk (at most kMaxDigits)
 
 __device__ __forceinline__ void atomic_flag(int* flag) {
   if (flag) atomicOr(flag, 1);
@@ -820,11 +808,6 @@ __global__ void __launch_bounds__(256) k_state_digits(const double* __restrict__
   }
   __syncthreads();
   if (threadIdx.x < d) atomicMax(norm2 + threadIdx.x, top[threadIdx.x]);
-}
-
-void digit_counts(int slices, int* d, int* w) {
-  *d = digits_for(slices);
-  *w = weights_for(slices);
 }
 
 cudaError_t digits_of_h(const dgchefsi_ctx* ctx, const int32_t* blk_row, const int32_t* pnb, const int32_t* poff,

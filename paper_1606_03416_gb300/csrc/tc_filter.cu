@@ -1272,8 +1272,7 @@ dgchefsi_status tc_sliced_matvec(dgchefsi_ctx* ctx, const double* X, int64_t ldx
     DG_TRY(make_plan(ctx, t, G, W, sx.brow_h, sx.zero_row, sx.plan, &order));
     sx.layout = true;
   }
-  int d = 0, w = 0;
-  digit_counts(slices, &d, &w);
+  const int d = digits_for(slices), w = weights_for(slices);
   // H's digits (once per H and digit count)
   const int64_t hcopy = sx.b_rows * W;
   const bool build = !sx.h_built || sx.h_digits != d;
