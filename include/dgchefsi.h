@@ -136,7 +136,8 @@ dgchefsi_status dgchefsi_bounds(dgchefsi_ctx* ctx, const double* v0, int k,
  * start at zero (each call writes every entry it reads), but calls whose work
  * overlaps on the GPU (other threads or streams) race on it and must be
  * serialised by the caller.
- * Arguments, results and synchronisation are those of dgchefsi_bounds. */
+ * Arguments and synchronisation are those of dgchefsi_bounds; the results agree
+ * to rounding (the same steps, with sums in another order). */
 dgchefsi_status dgchefsi_bounds_static(dgchefsi_ctx* ctx, const double* v0, int k,
                                        double* b_upper, double* theta_min);
 
@@ -195,7 +196,9 @@ dgchefsi_status dgchefsi_filter_graph(dgchefsi_ctx* ctx, int prec, const double*
  * this H's accumulator width and keeps the fastest. Setting a shape without a
  * kernel returns DGCHEFSI_ERR_UNSUPPORTED. */
 dgchefsi_status dgchefsi_set_tile_shape(dgchefsi_ctx* ctx, int prec, int G, int T, int layout);
-/* The shape in use (all 0 if not chosen yet) and the accumulator width. */
+/* The shape in use (all 0 if not chosen yet) and the accumulator width. Up to 128
+ * states a layout-0 shape with T = 2 runs with T = 1 (its second tile would hold no
+ * state); T = 2 is reported all the same. */
 dgchefsi_status dgchefsi_get_tile_shape(dgchefsi_ctx* ctx, int prec, int* G, int* T, int* ACC, int* layout);
 
 /* Order in which the persistent tensor-core filter walks its work units: the
@@ -212,7 +215,12 @@ dgchefsi_status dgchefsi_get_unit_order(dgchefsi_ctx* ctx, int prec, int* tgb);
 /* Overlap matrix S = Y^T Y of a block (the first product of Cholesky-QR,
  * Alg. 1 step 3), FP64: the tiles on and below the diagonal are computed and
  * mirrored, so S is exactly symmetric.
- *   Y  device (Ns x ld) state-major;  S  device out, row-major Ns x Ns. */
+ *   Y  device (Ns x ld) state-major;  S  device out, row-major Ns x Ns.
+ * A product of few tiles and many terms is summed in parts (the same ones at every
+ * call with these sizes), in a buffer of 128 MB of the context: calls on
+ * two streams wait for one another's parts. Without the memory, and in a stream
+ * capture, the parts run one after another: the same bits, later. The same holds
+ * for dgchefsi_density_blocks and dgchefsi_density_pattern. */
 dgchefsi_status dgchefsi_gram(dgchefsi_ctx* ctx, const double* Y, int64_t Ns, int64_t ld, double* S);
 
 /* Cholesky-QR and Rayleigh-Ritz (Alg. 1 steps 3-5; Sec. III.B.2), all FP64:
@@ -538,7 +546,9 @@ dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t N
 
 /* Replace the values of H (same block pattern) from a device array laid out
  * like `values` at create: [n_values] doubles. The caller keeps H symmetric
- * (not re-checked). Operand copies used by the tensor-core filter are rebuilt. */
+ * (not re-checked). Operand copies used by the tensor-core filter are rebuilt;
+ * what depends on the pattern alone, and up to 1 GB of the sliced H X's buffers,
+ * stays. */
 dgchefsi_status dgchefsi_set_values(dgchefsi_ctx* ctx, const double* values);
 
 /* Band energy of one cycle and its gradient. The paper does not differentiate

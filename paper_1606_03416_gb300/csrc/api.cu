@@ -300,14 +300,13 @@ static dgchefsi_status bounds_impl(dgchefsi_ctx* ctx, const double* v0, int k, d
   const int64_t N = ctx->N;
   if (k > N) k = (int)N;
   const size_t nvec = (size_t)k + 1;
-  const size_t npart = 65 * (size_t)LZ_MAX_CTAS;
-  DG_TRY(ensure(ctx, ctx->ws_lanczos, sizeof(double) * (nvec * (size_t)N + (size_t)N + npart + 130), "Lanczos basis"));
+  DG_TRY(ensure(ctx, ctx->ws_lanczos, sizeof(double) * (nvec * (size_t)N + (size_t)N + LZ_PARTS + LZ_OUT), "Lanczos basis"));
   double* V = static_cast<double*>(ctx->ws_lanczos.p);
   double* w = V + nvec * (size_t)N;
   double* part = w + N;
-  double* out = part + npart;
+  double* out = part + LZ_PARTS;
   cudaStream_t s = ctx->stream;
-  double host[130];
+  double host[LZ_OUT];
   DG_CUDA(lanczos_f64(ctx->view(), v0, k, V, w, part, ctx->n_values, out, s));
   DG_CUDA(cudaMemcpyAsync(host, out, sizeof(double) * (size_t)(2 + 2 * k), cudaMemcpyDeviceToHost, s));
   DG_CUDA(cudaStreamSynchronize(s));
@@ -413,8 +412,8 @@ static dgchefsi_status rr_impl(dgchefsi_ctx* ctx, double* Y, int64_t Ns, int64_t
   // symmetric up to rounding and the eigensolver reads one triangle (row-major
   // lower = column-major upper), so only the tiles on and below the diagonal
   // are computed.
-  // With sliced products H Y_hat also runs from BF16 slices, on the
-  // tensor-core filter's block-sparse step kernel, when H fits that form.
+  // With sliced products H Y_hat also runs from BF16 slices, on the block form of
+  // the pair kernel, when H fits that form.
   bool hx_sliced = false;
   if (sl) DG_TRY(tc_sliced_matvec(ctx, W, N, Y, ld, Ns, ctx->products_slices, bad, &hx_sliced));
   if (!hx_sliced) DG_CUDA(filter_step_f64(ctx->view(), W, N, nullptr, Y, ld, Ns, 1.0, 0.0, 0.0, s));
@@ -669,7 +668,7 @@ dgchefsi_status dgchefsi_bounds(dgchefsi_ctx* ctx, const double* v0, int k, doub
   clear_error();
   DG_TRY(check_ctx(ctx));
   if (!v0 || !b_upper) return set_error(DGCHEFSI_ERR_ARG, "null v0 or b_upper");
-  if (k < 1 || k > 64) return set_error(DGCHEFSI_ERR_ARG, "k = %d outside 1..64", k);
+  if (k < 1 || k > LZ_MAX_STEPS) return set_error(DGCHEFSI_ERR_ARG, "k = %d outside 1..64", k);
   return bounds_impl(ctx, v0, k, b_upper, theta_min);
 }
 

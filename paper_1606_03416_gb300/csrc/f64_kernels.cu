@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) k_lanczos_f64(HView h, const do
                                                                double* w, double* part, double* out) {
   namespace cg = cooperative_groups;
   cg::grid_group grid = cg::this_grid();
-  __shared__ double red[LZ_THREADS / 32], coef[64], tot[2];
+  __shared__ double red[LZ_THREADS / 32], coef[LZ_MAX_STEPS], tot[2];
   const int64_t N = h.N;
   const int64_t r0 = N * blockIdx.x / gridDim.x, r1 = N * (blockIdx.x + 1) / gridDim.x;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nt = blockDim.x, nw = nt >> 5;

@@ -56,10 +56,13 @@ cudaError_t preload_lanczos_kernels();
 // y = H x for one vector (Lanczos).
 cudaError_t spmv_f64(const HView& h, const double* x, double* y, cudaStream_t s);
 
-// k Lanczos steps (k <= 64) from v0 in one cooperative launch. V: (k + 1) N, w:
-// N, part: 65 LZ_MAX_CTAS, out: 2 + 2 k doubles, all device; nnz: stored entries
-// of H. out: |v0|, steps taken, then alpha_j, beta_j.
-constexpr int LZ_MAX_CTAS = 256;
+// k Lanczos steps (k <= LZ_MAX_STEPS) from v0 in one cooperative launch. V: (k + 1)
+// N, w: N, part: LZ_PARTS (the CTAs' parts of k + 1 dot products at a time), out: 2
+// + 2 k doubles, all device; nnz: stored entries of H. out: |v0|, steps taken, then
+// alpha_j, beta_j.
+constexpr int LZ_MAX_STEPS = 64, LZ_MAX_CTAS = 256;
+constexpr int LZ_PARTS = (LZ_MAX_STEPS + 1) * LZ_MAX_CTAS;
+constexpr int LZ_OUT = 2 + 2 * LZ_MAX_STEPS;
 cudaError_t lanczos_f64(const HView& h, const double* v0, int k, double* V, double* w, double* part, int64_t nnz,
                         double* out, cudaStream_t s);
 

@@ -5,7 +5,10 @@
 // a loop that cannot absorb the device-wide synchronisation of cudaMalloc /
 // cudaFree. For them the Krylov basis of the bound lives in one fixed
 // file-scope device array instead of the context's grow-only workspace. The
-// arithmetic and launch sequence are those of dgchefsi_bounds.
+// steps are those of dgchefsi_bounds, one kernel per operation: its one cooperative
+// launch needs room for the CTAs' partial sums, which would take from the largest
+// requests the array serves. Sums are added in another order, so the two agree to
+// rounding.
 #include <cmath>
 #include <mutex>
 

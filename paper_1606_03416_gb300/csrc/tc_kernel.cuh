@@ -166,7 +166,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
 // free, and waits here until the previous grid has completed and its writes are
 // visible. Nothing that a previous grid writes is read, and nothing that it
 // reads is written, before. Ten steps of a small filter (8 elements, 48 states):
-// 134 us without this, 108 with it and one-tile units (see pick_shape).
+// 134 us without this, 108 with it and one-tile units (prepare_launch in tc_filter.cu).
 __device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
