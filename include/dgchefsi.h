@@ -220,7 +220,7 @@ dgchefsi_status dgchefsi_get_unit_order(dgchefsi_ctx* ctx, int prec, int* tgb);
  * call with these sizes), in a buffer of 128 MB of the context: calls on
  * two streams wait for one another's parts. Without the memory, and in a stream
  * capture, the parts run one after another: the same bits, later. The same holds
- * for dgchefsi_density_blocks and dgchefsi_density_pattern. */
+ * for dgchefsi_density_blocks. */
 dgchefsi_status dgchefsi_gram(dgchefsi_ctx* ctx, const double* Y, int64_t Ns, int64_t ld, double* S);
 
 /* Cholesky-QR and Rayleigh-Ritz (Alg. 1 steps 3-5; Sec. III.B.2), all FP64:

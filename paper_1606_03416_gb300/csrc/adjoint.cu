@@ -261,7 +261,7 @@ extern "C" dgchefsi_status dgchefsi_energy_grad(dgchefsi_ctx* ctx, int prec, con
   double* Hb = H_bar;
   if (Hb) {
     DG_CUDA(cudaMemsetAsync(Hb, 0, sizeof(double) * (size_t)ctx->n_values, s));
-    DG_CUDA(block_outer_f64(h, ctx->blk_row_d, ctx->nnzb, XN, N, XN, N, g, 1.0, Ns, Hb, false, s));
+    DG_CUDA(block_outer_f64(h, ctx->blk_row_d, ctx->nnzb, XN, N, XN, N, g, 1.0, Ns, Hb, 0, s));
   }
   // Y~bar = 2 R G Z^T, in state-major form Y~bar^T = Z (2 G R^T), Z^T = Q^T L
   DG_CUDA(scaled_residual_f64(HXN, XN, N, lam, g, 2.0, Ns, N, T0, N, s));
@@ -290,7 +290,7 @@ extern "C" dgchefsi_status dgchefsi_energy_grad(dgchefsi_ctx* ctx, int prec, con
     }
     for (int k = k1 - 1; k >= k0; --k) {
       if (Hb) DG_CUDA(block_outer_f64(h, ctx->blk_row_d, ctx->nnzb, Wcur, N, seg[k - k0], N, nullptr, cf.alpha[k], Ns,
-                                      Hb, false, s));
+                                      Hb, 0, s));
       const double bnext = (k + 1 < m) ? cf.beta[k + 1] : 0.0;
       // W_k = alpha_k (H - cI) W_{k+1} - beta_{k+1} W_{k+2}, written over W_{k+2}
       double* out = Wprev;

@@ -90,12 +90,12 @@ dgchefsi_status sym_product_f64(dgchefsi_ctx* ctx, const double* A, int64_t lda,
   return parts_end(ctx, parts);
 }
 
-dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P,
-                                   const int64_t* pout) {
+dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P) {
   Parts parts{nullptr, (int64_t)(kPartsBytes / sizeof(double))};
   const int64_t total = ctx->poff_h[ctx->M];
-  if (density_parts(ctx->view(), total, Ns, parts.doubles) > 1) DG_TRY(parts_begin(ctx, &parts.p));
-  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, total, pout, X, Ns, ld, f, P, parts, ctx->stream));
+  int64_t len = 0;
+  if (density_parts(ctx->view(), total, Ns, parts.doubles, &len) > 1) DG_TRY(parts_begin(ctx, &parts.p));
+  DG_CUDA(density_f64(ctx->view(), ctx->poff_d, total, X, Ns, ld, f, P, parts, ctx->stream));
   return parts_end(ctx, parts);
 }
 
@@ -552,25 +552,19 @@ dgchefsi_status dgchefsi_create(int32_t M, const int32_t* nb, const int64_t* row
       (st = dmalloc((void**)&ctx->blk_off_d, sizeof(int64_t) * ctx->nnzb)) ||
       (st = dmalloc((void**)&ctx->vals_d, sizeof(double) * n_values)) ||
       (st = dmalloc((void**)&ctx->poff_d, sizeof(int64_t) * (M + 1))) ||
-      (st = dmalloc((void**)&ctx->diag_off_d, sizeof(int64_t) * M)) ||
       (st = dmalloc((void**)&ctx->blk_row_d, sizeof(int32_t) * std::max<int64_t>(ctx->nnzb, 1))) ||
       (st = dmalloc((void**)&ctx->info_d, sizeof(int) * 4)))
     return bail(st);
   auto h2d = [&](void* d, const void* h, size_t bytes) { return cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice); };
   std::vector<int32_t> blk_row(ctx->nnzb);
-  std::vector<int64_t> diag_off(M);
   for (int K = 0; K < M; ++K)
-    for (int64_t e = row_ptr[K]; e < row_ptr[K + 1]; ++e) {
-      blk_row[e] = K;
-      if (col[e] == K) diag_off[K] = blk_off[e];
-    }
+    for (int64_t e = row_ptr[K]; e < row_ptr[K + 1]; ++e) blk_row[e] = K;
   if (ctx->nnzb > 0 && h2d(ctx->blk_row_d, blk_row.data(), sizeof(int32_t) * ctx->nnzb))
     return bail(set_error(DGCHEFSI_ERR_CUDA, "copy of the block rows to the device failed"));
   if (h2d(ctx->nb_d, nb, sizeof(int32_t) * M) || h2d(ctx->off_d, ctx->off_h.data(), sizeof(int64_t) * (M + 1)) ||
       h2d(ctx->row_ptr_d, row_ptr, sizeof(int64_t) * (M + 1)) || h2d(ctx->col_d, col, sizeof(int32_t) * ctx->nnzb) ||
       h2d(ctx->blk_off_d, blk_off, sizeof(int64_t) * ctx->nnzb) ||
       h2d(ctx->vals_d, values, sizeof(double) * n_values) ||
-      h2d(ctx->diag_off_d, diag_off.data(), sizeof(int64_t) * M) ||
       h2d(ctx->poff_d, ctx->poff_h.data(), sizeof(int64_t) * (M + 1)))
     return bail(set_error(DGCHEFSI_ERR_CUDA, "copy of H to the device failed"));
   if (cusolverDnCreate(&ctx->solver) != CUSOLVER_STATUS_SUCCESS)
@@ -595,7 +589,6 @@ void dgchefsi_destroy(dgchefsi_ctx* ctx) {
   cudaFree(ctx->blk_off_d);
   cudaFree(ctx->vals_d);
   cudaFree(ctx->poff_d);
-  cudaFree(ctx->diag_off_d);
   cudaFree(ctx->blk_row_d);
   cudaFree(ctx->info_d);
   free_buf(ctx->ws_filter);
@@ -1102,7 +1095,7 @@ dgchefsi_status dgchefsi_density_blocks(dgchefsi_ctx* ctx, const double* X, int6
   DG_TRY(check_ctx(ctx));
   DG_TRY(check_block(ctx, X, Ns, ld, "X"));
   if (!P || (Ns > 0 && !f)) return set_error(DGCHEFSI_ERR_ARG, "null f or P");
-  return density_blocks_f64(ctx, X, Ns, ld, f, P, ctx->poff_d);
+  return density_blocks_f64(ctx, X, Ns, ld, f, P);
 }
 
 dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t Ns, int64_t ld, int m, double Ne,
@@ -1150,7 +1143,7 @@ dgchefsi_status dgchefsi_cycle(dgchefsi_ctx* ctx, int prec, double* X, int64_t N
   bool done = false;
   if (ctx->products_mode == DGCHEFSI_PRODUCTS_SLICED_BF16 && density_digits_fit(ctx, Ns))
     DG_TRY(density_digits(ctx, X, Ns, ld, f, P, &done));
-  if (!done) DG_TRY(density_blocks_f64(ctx, X, Ns, ld, f, P, ctx->poff_d));
+  if (!done) DG_TRY(density_blocks_f64(ctx, X, Ns, ld, f, P));
   if (bounds) {
     bounds[0] = a;
     bounds[1] = b;

@@ -43,7 +43,6 @@ struct dgchefsi_ctx {
   int64_t* blk_off_d = nullptr;
   double* vals_d = nullptr;
   int64_t* poff_d = nullptr;  // packed density-block offsets
-  int64_t* diag_off_d = nullptr;  // offsets of the diagonal blocks in H's values
   int32_t* blk_row_d = nullptr;  // element row of each stored block
   // workspace
   dg::DevBuf ws_filter;   // filter ping-pong partner (Ns x ld FP64)
@@ -144,11 +143,10 @@ dgchefsi_status ensure(dgchefsi_ctx* ctx, DevBuf& b, size_t bytes, const char* w
 constexpr size_t kPartsBytes = size_t(128) << 20;
 
 // The symmetric n x n product C = A B^T (gemm_nt_f64, lower triangle mirrored)
-// and the density blocks (density_f64; block K at P + pout[K]) on the context's stream.
+// and the packed density blocks (density_f64) on the context's stream.
 dgchefsi_status sym_product_f64(dgchefsi_ctx* ctx, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
                                 int64_t ldc, int64_t n, int64_t K);
-dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P,
-                                   const int64_t* pout);
+dgchefsi_status density_blocks_f64(dgchefsi_ctx* ctx, const double* X, int64_t Ns, int64_t ld, const double* f, double* P);
 
 // Tensor-core filter (tc_filter.cu). X, Y FP64 (Ns x ld) state-major.
 // reuse_hop: the operand copy of H - cI built by the previous call of this

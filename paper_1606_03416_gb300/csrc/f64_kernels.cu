@@ -454,9 +454,8 @@ __global__ void __launch_bounds__(NT) k_gemm_nn_f64(const double* __restrict__ A
 // sums `sc` states; in a buffer (P + z * total, laid out like P, added by
 // k_density_sum_f64) all parts run at once, so that few elements still fill the
 // GPU and many fill it evenly.
-// Element K's block goes to P + pout[K] (poff[K] in a buffer).
 __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __restrict__ poff,
-                                                    const int64_t* __restrict__ pout, const double* __restrict__ X, int64_t Ns, int64_t ld,
+                                                    const double* __restrict__ X, int64_t Ns, int64_t ld,
                                                     const double* __restrict__ f, int64_t sc, double* __restrict__ P,
                                                     int z0, PartTo to) {
   const int K = blockIdx.x;
@@ -505,7 +504,7 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
     __syncthreads();
   }
   const bool part = to == kBuffer;
-  double* PK = P + (part ? poff[K] + z * poff[h.M] : pout[K]);
+  double* PK = P + poff[K] + (part ? z * poff[h.M] : 0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int jj = j0 + row[i];
@@ -523,13 +522,13 @@ __global__ void __launch_bounds__(NT) k_density_f64(HView h, const int64_t* __re
 }
 
 // P = the sum of the parts, z ascending, lower triangles mirrored. One CTA per element.
-__global__ void k_density_sum_f64(HView h, const int64_t* __restrict__ poff, const int64_t* __restrict__ pout,
-                                  const double* __restrict__ part, int parts, double* __restrict__ P) {
+__global__ void k_density_sum_f64(HView h, const int64_t* __restrict__ poff, const double* __restrict__ part,
+                                  int parts, double* __restrict__ P) {
   const int K = blockIdx.x;
   const int nK = h.nb[K];
   const int64_t total = poff[h.M];
   const double* p = part + poff[K];
-  double* PK = P + pout[K];
+  double* PK = P + poff[K];
   for (int e = threadIdx.x; e < nK * nK; e += blockDim.x) {
     const int j = e / nK, q = e - j * nK;
     if (q > j) continue;
@@ -639,18 +638,21 @@ __global__ void k_check_finite_f64(const double* __restrict__ x, int64_t n, int*
 
 
 // G_e += alpha * sum_s w_s A[s, off_K + j] B[s, off_K' + j'] for every stored
-// block e = (K, K') (w may be null: unit weights), or every one with K != K'.
+// block e = (K, K') (w may be null: unit weights). DIAG (A = B, G zero, alpha 1): the
+// blocks with K = K' are formed as k_density_f64 does, in parts of diag_len states
+// added in order, the entries j' <= j mirrored, so that they have its bits.
+template <bool DIAG>
 __global__ void __launch_bounds__(NT) k_block_outer_f64(HView h, const int32_t* __restrict__ blk_row,
                                                         const double* __restrict__ A, int64_t lda,
                                                         const double* __restrict__ B, int64_t ldb,
                                                         const double* __restrict__ w, double alpha, int64_t Ns,
-                                                        double* __restrict__ G, int off_diagonal) {
+                                                        double* __restrict__ G, int64_t diag_len) {
   const int64_t e = blockIdx.x;
   const int K = blk_row[e], Kp = h.col[e];
-  if (off_diagonal && K == Kp) return;
+  const bool diag = DIAG && K == Kp;
   const int nK = h.nb[K], nKp = h.nb[Kp];
   const int j0 = blockIdx.y * T, jp0 = blockIdx.z * T;
-  if (j0 >= nK || jp0 >= nKp) return;
+  if (j0 >= nK || jp0 >= nKp || (diag && jp0 > j0)) return;
   const int64_t offK = h.off[K], offKp = h.off[Kp];
   __shared__ double As[BK][TP];
   __shared__ double Bs[BK][TP];
@@ -659,40 +661,49 @@ __global__ void __launch_bounds__(NT) k_block_outer_f64(HView h, const int32_t* 
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     row[i] = ty + 16 * i;
-    lim[i] = j0 + 16 * i + (ty & ~3) < nK ? groups8(nKp - jp0) : 0;
+    const int r4 = j0 + 16 * i + (ty & ~3);
+    lim[i] = r4 < nK ? groups8((diag ? min(nK, r4 + 4) : nKp) - jp0) : 0;
   }
   double acc[4][8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
   const int cc = tid & 63;
-  for (int64_t i0 = 0; i0 < Ns; i0 += BK) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int kk = (tid >> 6) + 2 * i;
-      const int64_t s = i0 + kk;
-      double v = 0.0, u = 0.0;
-      if (s < Ns) {
-        if (j0 + cc < nK) v = (w ? w[s] : 1.0) * A[s * lda + offK + j0 + cc];
-        if (jp0 + cc < nKp) u = B[s * ldb + offKp + jp0 + cc];
-      }
-      As[kk][cc] = v;
-      Bs[kk][cc] = u;
-    }
-    __syncthreads();
-    fma_outer(As, Bs, acc, (int)(Ns - i0 < BK ? Ns - i0 : BK), lim, tx, row);
-    __syncthreads();
-  }
   double* Ge = G + h.blk_off[e];
+  const int64_t len = DIAG && diag ? diag_len : Ns;
+  for (int64_t sb = 0; sb < Ns; sb += len) {
+    const int64_t se = sb + len < Ns ? sb + len : Ns;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int jj = j0 + row[i];
-    if (jj >= nK) continue;
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int jq = jp0 + tx + 8 * j;
-      if (jq < nKp) Ge[(int64_t)jj * nKp + jq] += alpha * acc[i][j];
+      for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
+    for (int64_t i0 = sb; i0 < se; i0 += BK) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int kk = (tid >> 6) + 2 * i;
+        const int64_t s = i0 + kk;
+        double v = 0.0, u = 0.0;
+        if (s < se) {
+          if (j0 + cc < nK) v = (w ? w[s] : 1.0) * A[s * lda + offK + j0 + cc];
+          if (jp0 + cc < nKp) u = B[s * ldb + offKp + jp0 + cc];
+        }
+        As[kk][cc] = v;
+        Bs[kk][cc] = u;
+      }
+      __syncthreads();
+      fma_outer(As, Bs, acc, (int)(se - i0 < BK ? se - i0 : BK), lim, tx, row);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int jj = j0 + row[i];
+      if (jj >= nK) continue;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int jq = jp0 + tx + 8 * j;
+        if (jq >= nKp || (diag && jq > jj)) continue;
+        double* o = Ge + (int64_t)jj * nKp + jq;
+        const double v = DIAG ? (sb == 0 ? acc[i][j] : *o + acc[i][j]) : *o + alpha * acc[i][j];
+        *o = v;
+        if (diag) Ge[(int64_t)jq * nKp + jj] = v;
+      }
     }
   }
 }
@@ -888,8 +899,10 @@ int64_t gemm_nt_parts(int64_t rows, int64_t cols, int64_t K, bool lower_only, in
   return rows == 0 || cols == 0 ? 1 : gemm_nt_split(rows, cols, K, lower_only, doubles).np;
 }
 
-int64_t density_parts(const HView& h, int64_t total, int64_t Ns, int64_t doubles) {
-  return density_split(h, total, Ns, doubles).np;
+int64_t density_parts(const HView& h, int64_t total, int64_t Ns, int64_t doubles, int64_t* len) {
+  const Split sp = density_split(h, total, Ns, doubles);
+  *len = sp.len;
+  return sp.np;
 }
 
 cudaError_t gemm_nt_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
@@ -926,18 +939,18 @@ cudaError_t gemm_nn_f64(const double* A, int64_t lda, const double* B, int64_t l
   return cudaGetLastError();
 }
 
-cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const int64_t* pout, const double* X,
-                        int64_t Ns, int64_t ld, const double* f, double* P, const Parts& parts, cudaStream_t s) {
+cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const double* X, int64_t Ns, int64_t ld,
+                        const double* f, double* P, const Parts& parts, cudaStream_t s) {
   const int64_t chunks = cdiv(h.max_nb, T), pairs = chunks * (chunks + 1) / 2;
   const Split sp = density_split(h, total, Ns, parts.doubles);
   if (sp.np > 1 && parts.p) {
-    k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)sp.np), NT, 0, s>>>(h, poff, pout, X, Ns, ld, f,
-                                                                                      sp.len, parts.p, 0, kBuffer);
-    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, pout, parts.p, (int)sp.np, P);
+    k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs, (unsigned)sp.np), NT, 0, s>>>(h, poff, X, Ns, ld, f, sp.len,
+                                                                                      parts.p, 0, kBuffer);
+    k_density_sum_f64<<<(unsigned)h.M, 256, 0, s>>>(h, poff, parts.p, (int)sp.np, P);
     count_launch(2);
   } else {
     for (int z = 0; z < (int)sp.np; ++z)
-      k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs), NT, 0, s>>>(h, poff, pout, X, Ns, ld, f, sp.len, P, z,
+      k_density_f64<<<dim3((unsigned)h.M, (unsigned)pairs), NT, 0, s>>>(h, poff, X, Ns, ld, f, sp.len, P, z,
                                                                        z == 0 ? kWrite : kAdd);
     count_launch((int)sp.np);
   }
@@ -979,10 +992,13 @@ cudaError_t zero_strict_upper_f64(double* A, int64_t n, int64_t lda, cudaStream_
 
 cudaError_t block_outer_f64(const HView& h, const int32_t* blk_row, int64_t nnzb, const double* A, int64_t lda,
                             const double* B, int64_t ldb, const double* w, double alpha, int64_t Ns, double* G,
-                            bool off_diagonal, cudaStream_t s) {
+                            int64_t diag_len, cudaStream_t s) {
   if (nnzb == 0) return cudaSuccess;
   dim3 grid((unsigned)nnzb, cdiv(h.max_nb, T), cdiv(h.max_nb, T));
-  k_block_outer_f64<<<grid, NT, 0, s>>>(h, blk_row, A, lda, B, ldb, w, alpha, Ns, G, off_diagonal ? 1 : 0);
+  if (diag_len > 0)
+    k_block_outer_f64<true><<<grid, NT, 0, s>>>(h, blk_row, A, lda, B, ldb, w, alpha, Ns, G, diag_len);
+  else
+    k_block_outer_f64<false><<<grid, NT, 0, s>>>(h, blk_row, A, lda, B, ldb, w, alpha, Ns, G, 0);
   count_launch();
   return cudaGetLastError();
 }

@@ -26,9 +26,9 @@ struct Parts {
   double* p = nullptr;
   int64_t doubles = 0;
 };
-// Parts of the products below for a buffer of so many doubles, 1: not split.
+// Parts of the products below for a buffer of so many doubles, 1: not split; len: states a part.
 int64_t gemm_nt_parts(int64_t rows, int64_t cols, int64_t K, bool lower_only, int64_t doubles);
-int64_t density_parts(const HView& h, int64_t total, int64_t Ns, int64_t doubles);
+int64_t density_parts(const HView& h, int64_t total, int64_t Ns, int64_t doubles, int64_t* len);
 
 void count_launch(int n = 1);
 
@@ -85,20 +85,20 @@ cudaError_t gemm_nt_f64(const double* A, int64_t lda, const double* B, int64_t l
 cudaError_t gemm_nn_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                         int64_t rows, int64_t cols, int64_t K, bool a_lower, cudaStream_t s);
 
-// P_K = sum_i f_i X[i, off_K:] X[i, off_K:]^T at P + pout[K]; poff: the packed
-// offsets, `total` doubles in all (the layout of a buffer of parts).
-cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const int64_t* pout, const double* X,
-                        int64_t Ns, int64_t ld, const double* f, double* P, const Parts& parts, cudaStream_t s);
+// P_K = sum_i f_i X[i, off_K:] X[i, off_K:]^T packed at poff[K], `total` doubles in all.
+cudaError_t density_f64(const HView& h, const int64_t* poff, int64_t total, const double* X, int64_t Ns, int64_t ld,
+                        const double* f, double* P, const Parts& parts, cudaStream_t s);
 
 // Fermi level by bisection and occupations (one cluster of CTAs).
 cudaError_t occupations_f64(const double* ritz, int64_t Ns, double Ne, double kT, double* f, double* mu,
                             cudaStream_t s);
 
 // G_e += alpha * sum_s w_s A[s, off_K + j] B[s, off_K' + j'] for every stored block e = (K, K')
-// (values layout of H; w may be null), off_diagonal: for those with K != K' only.
+// (values layout of H; w may be null). diag_len > 0, with A = B, G = 0 and alpha = 1: the
+// diagonal blocks have density_f64's bits, diag_len its part length (density_parts).
 cudaError_t block_outer_f64(const HView& h, const int32_t* blk_row, int64_t nnzb, const double* A, int64_t lda,
                             const double* B, int64_t ldb, const double* w, double alpha, int64_t Ns, double* G,
-                            bool off_diagonal, cudaStream_t s);
+                            int64_t diag_len, cudaStream_t s);
 // C[i,r] = sum_l A[l,i] B[l,r]  (A: K x rows row-major, B: K x cols row-major).
 cudaError_t gemm_tn_f64(const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                         int64_t rows, int64_t cols, int64_t K, cudaStream_t s);

@@ -201,7 +201,9 @@ extern "C" dgchefsi_status dgchefsi_density_pattern(dgchefsi_ctx* ctx, const dou
   if (ld < ctx->N) return set_error(DGCHEFSI_ERR_ARG, "ld < N");
   cudaStream_t s = ctx->stream;
   DG_CUDA(cudaMemsetAsync(P, 0, sizeof(double) * (size_t)ctx->n_values, s));
-  DG_CUDA(block_outer_f64(ctx->view(), ctx->blk_row_d, ctx->nnzb, X, ld, X, ld, f, 1.0, Ns, P, true, s));
-  // the diagonal blocks by the kernel of dgchefsi_density_blocks: its bits
-  return density_blocks_f64(ctx, X, Ns, ld, f, P, ctx->diag_off_d);
+  // the diagonal blocks with the bits of dgchefsi_density_blocks
+  int64_t len = 0;
+  density_parts(ctx->view(), ctx->poff_h[ctx->M], Ns, (int64_t)(kPartsBytes / sizeof(double)), &len);
+  DG_CUDA(block_outer_f64(ctx->view(), ctx->blk_row_d, ctx->nnzb, X, ld, X, ld, f, 1.0, Ns, P, len, s));
+  return DGCHEFSI_OK;
 }
