@@ -20,7 +20,10 @@
  * Streams: all device work is enqueued on the context's stream (set at create,
  *        changeable with dgchefsi_set_stream). A call returns once its work is
  *        enqueued, except where it says it synchronises (it returns host
- *        scalars or checks a device status).
+ *        scalars or checks a device status). Of the calls that do not, matvec,
+ *        occupations, gram, density_blocks and density_pattern may be in flight
+ *        on several streams at a time; the FP64 filters use the context's
+ *        workspace, so work on another stream has to wait for them.
  * Ownership: the context owns its copy of H and all workspace; callers own
  *        every buffer they pass. No call dereferences a caller pointer after it
  *        returns (the graph form remembers the addresses of its last capture
