@@ -142,6 +142,11 @@ def _block(X: torch.Tensor, N: int, name: str):
     return X.shape[0], max(ld, N)
 
 
+def _like(Ns: int, N: int, ld: int, device) -> torch.Tensor:
+    """A new block (Ns, N) with rows ld apart, for calls whose output has the input's row stride."""
+    return torch.empty_strided((Ns, N), (ld, 1), dtype=torch.float64, device=device)
+
+
 def _stream() -> int:
     return torch.cuda.current_stream().cuda_stream
 
@@ -269,7 +274,9 @@ class Context:
         """The filter replayed from a CUDA graph (captured on first use); any precision."""
         Ns, ld = _block(X, self.N, "X")
         if Y is None:
-            Y = torch.empty_like(X)
+            Y = _like(Ns, self.N, ld, X.device)
+        if _block(Y, self.N, "Y") != (Ns, ld):
+            raise ValueError("X and Y need the same shape and stride")
         self._sync_stream()
         _check(_lib.dgchefsi_filter_graph(self._h, PRECISIONS[prec], _ptr(X), _ptr(Y), Ns, ld, int(m), float(a),
                                           float(b), float(a0)))
@@ -492,7 +499,7 @@ class Context:
         ritz = torch.empty(Ns, dtype=torch.float64, device=dev)
         Hb = torch.empty(int(n_values if n_values is not None else self.n_values), dtype=torch.float64,
                          device=dev) if grad else None
-        Xb = torch.empty_like(X) if grad else None
+        Xb = _like(Ns, self.N, ld, dev) if grad else None
         E = C.c_double()
         self._sync_stream()
         _check(_lib.dgchefsi_energy_grad(self._h, PRECISIONS[prec], _ptr(X), Ns, ld, int(m), float(a), float(b), float(a0),
