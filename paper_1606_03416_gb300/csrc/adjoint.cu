@@ -146,15 +146,20 @@ extern "C" dgchefsi_status dgchefsi_energy_grad(dgchefsi_ctx* ctx, int prec, con
     DG_TRY(copy_blk(T0, N, X, ld));
     DG_TRY(filter_tc(ctx, prec, T0, Yt, Ns, N, m, a, b, a0));
   } else {
-    // Y_0 = X (caller layout ld); iterates in T0/T1/T2 rotation (ld = N)
+    // Y_0 = X; iterates in T0/T1/T2 rotation (ld = N). The second step reads X at
+    // the row stride of its output: padded rows are copied first, to the buffer
+    // that the third step is the first to write.
     double* rot[3] = {T0, T1, T2};
     const double* prev = nullptr;
     const double* cur = X;
-    int64_t ldc = ld;
+    if (ld != N) {
+      DG_TRY(copy_blk(T2, N, X, ld));
+      cur = T2;
+    }
     if (want_grad) DG_TRY(copy_blk(cp0[0], N, X, ld));
     for (int k = 0; k < m; ++k) {
       double* out = (k == m - 1) ? Yt : rot[k % 3];
-      DG_CUDA(filter_step_f64(h, cur, ldc, k == 0 ? nullptr : prev, out, N, Ns, cf.alpha[k], cf.c,
+      DG_CUDA(filter_step_f64(h, cur, N, k == 0 ? nullptr : prev, out, N, Ns, cf.alpha[k], cf.c,
                               k == 0 ? 0.0 : cf.beta[k], s));
       const int kk = k + 1;  // index of the iterate just produced
       if (want_grad && kk < m) {
@@ -163,7 +168,6 @@ extern "C" dgchefsi_status dgchefsi_energy_grad(dgchefsi_ctx* ctx, int prec, con
       }
       prev = cur;
       cur = out;
-      ldc = N;
     }
   }
   // ---- Cholesky-QR and Rayleigh-Ritz, keeping U^{-T} (L) and Q^T (row-major views).

@@ -21,12 +21,14 @@ def blocks(Ns=9, pad=5):
     return H, X, wide, wide[:, :H.N]
 
 
-@pytest.mark.parametrize("prec", ["bf16x3"])
-def test_gradient(prec):
+@pytest.mark.parametrize("m", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("prec", ["f64", "bf16x3"])
+def test_gradient(prec, m):
     H, X, wide, Xs = blocks()
     with D.Context(H) as ctx:
-        E, ritz, Hb, Xb = ctx.energy_grad(X, 4, 5.0, 46.0, -1.8, 9.0, 0.3, prec=prec)
-        Es, ritzs, Hbs, Xbs = ctx.energy_grad(Xs, 4, 5.0, 46.0, -1.8, 9.0, 0.3, prec=prec)
+        E, ritz, Hb, Xb = ctx.energy_grad(X, m, 5.0, 46.0, -1.8, 9.0, 0.3, prec=prec)
+        Es, ritzs, Hbs, Xbs = ctx.energy_grad(Xs, m, 5.0, 46.0, -1.8, 9.0, 0.3, prec=prec)
+        assert ctx.energy_grad(Xs, m, 5.0, 46.0, -1.8, 9.0, 0.3, grad=False, prec=prec)[0] == E
     assert Xbs.stride() == Xs.stride() and Xbs.shape == X.shape
     assert Es == E and torch.equal(ritzs, ritz) and torch.equal(Hbs, Hb) and torch.equal(Xbs, Xb)
     assert bool((wide[:, H.N:] == 7.0).all())
