@@ -139,7 +139,9 @@ def _block(X: torch.Tensor, N: int, name: str):
     if X.shape[1] != N or (X.shape[0] > 1 and X.stride(1) != 1) or (X.shape[0] > 0 and X.stride(1) != 1):
         raise ValueError(f"{name} must have shape (N_s, {N}) with unit column stride")
     ld = X.stride(0) if X.shape[0] > 1 else N
-    return X.shape[0], max(ld, N)
+    if ld < N:
+        raise ValueError(f"{name} must not have overlapping rows")
+    return X.shape[0], ld
 
 
 def _like(Ns: int, N: int, ld: int, device) -> torch.Tensor:
@@ -258,7 +260,9 @@ class Context:
             raise TypeError("X must be a 2-D float64 CPU tensor (N_s, N)")
         if X.shape[1] != self.N or (X.shape[0] > 0 and X.stride(1) != 1):
             raise ValueError(f"X must have shape (N_s, {self.N}) with unit column stride")
-        ld = max(X.stride(0) if X.shape[0] > 1 else self.N, self.N)
+        ld = X.stride(0) if X.shape[0] > 1 else self.N
+        if ld < self.N:
+            raise ValueError("X must not have overlapping rows")
         if Y is None:
             Y = torch.empty(X.shape, dtype=torch.float64, pin_memory=X.is_pinned())
         if Y.device.type != "cpu" or Y.dtype != torch.float64 or Y.shape != X.shape or \

@@ -47,3 +47,16 @@ def test_graph_filter(prec):
             ctx.filter_graph(X, 4, 5.0, 46.0, -1.8, prec=prec, Y=wide[:, :H.N])
         with pytest.raises(ValueError):
             ctx.filter_graph(X, 4, 5.0, 46.0, -1.8, prec=prec, Y=torch.empty_like(X)[:-1])
+
+
+def test_overlapping_rows_are_refused():
+    """An expanded row has stride 0: it was read as a block of rows N apart."""
+    H, X, wide, Xs = blocks()
+    with D.Context(H) as ctx:
+        for bad in (X[:1].expand(4, H.N), X.reshape(-1).as_strided((4, H.N), (H.N - 1, 1))):
+            for call in (ctx.gram, ctx.matvec, lambda x: ctx.energy_grad(x, 2, 5.0, 46.0, -1.8, 2.0, 0.3)):
+                with pytest.raises(ValueError):
+                    call(bad)
+            with pytest.raises(ValueError):
+                ctx.filter_host(bad.cpu()[:1].expand(4, H.N), 2, 5.0, 46.0, -1.8)
+        assert ctx.gram(X[:1].expand(1, H.N)).shape == (1, 1)
